@@ -1,6 +1,5 @@
 // Network kernels other than the tensor-core GEMM: the fp32 check-mode GEMM, token embedding,
-// LayerNorm, the two small attentions, the output head, the toy MLP and the closed-form Gaussian
-// denoiser.  T is the activation type: float in the fp32 check mode, bf16 in the production mode.
+// LayerNorm, the two small attentions, the output head and the closed-form Gaussian denoiser.  T is the activation type: float in the fp32 check mode, bf16 in the production mode.
 #pragma once
 #include "common.cuh"
 #include "gemm_tcgen05.cuh"
@@ -782,58 +781,6 @@ __global__ void head_kernel(const float* __restrict__ h, const float* __restrict
     const float e = head_out<VEC>(v, W_outT + (size_t)a * d, b_out[a], lane);
     if (lane == 0) o[a] = e;
   }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Toy MLP denoiser (fp32): input [latent | sinusoidal(tau) | obs], SiLU hidden layers, linear head.
-// One block per candidate; weights [in, out] so that a warp reads a weight row coalesced.
-// ------------------------------------------------------------------------------------------------
-constexpr int MLP_MAX_LAYERS = 8;
-struct MlpWeights {
-  int n_lin;                 // hidden layers + 1
-  int dims[MLP_MAX_LAYERS + 2];
-  const float* W[MLP_MAX_LAYERS + 1];
-  const float* b[MLP_MAX_LAYERS + 1];
-  int temb;
-  const float* temb_table;   // [T, temb]
-};
-
-__global__ void mlp_forward_kernel(MlpWeights w, CandMap cm, const float* __restrict__ obs, int obs_len, int D,
-                                   int Tsteps) {
-  pdl_trigger();
-  pdl_wait();
-  extern __shared__ float sm[];
-  const int n = blockIdx.x;
-  if (n >= cand_count(cm, gridDim.x)) return;
-  int b, c;
-  cand_decode(cm, n, b, c);
-  int tau = cm.t[b] - cm.koff - c;
-  tau = max(0, min(Tsteps - 1, tau));
-  int maxw = 0;
-  for (int l = 0; l <= w.n_lin; ++l) maxw = max(maxw, w.dims[l]);
-  float* cur = sm;
-  float* nxt = sm + maxw;
-  const float* x = cm.xin + b * cm.x_stride_b + (long long)c * D;
-  for (int i = threadIdx.x; i < w.dims[0]; i += blockDim.x) {
-    float v;
-    if (i < D) v = x[i];
-    else if (i < D + w.temb) v = w.temb_table[tau * w.temb + (i - D)];
-    else v = obs[(size_t)item_of(cm.item, b) * obs_len + (i - D - w.temb)];
-    cur[i] = v;
-  }
-  __syncthreads();
-  for (int l = 0; l < w.n_lin; ++l) {
-    const int nin = w.dims[l], nout = w.dims[l + 1];
-    for (int j = threadIdx.x; j < nout; j += blockDim.x) {
-      float a = w.b[l][j];
-      for (int i = 0; i < nin; ++i) a += cur[i] * w.W[l][(size_t)i * nout + j];
-      nxt[j] = (l + 1 < w.n_lin) ? silu(a) : a;
-    }
-    __syncthreads();
-    float* tmp = cur; cur = nxt; nxt = tmp;
-  }
-  float* o = cm.eout + b * cm.e_stride_b + (long long)c * D;
-  for (int i = threadIdx.x; i < D; i += blockDim.x) o[i] = cur[i];
 }
 
 // Closed-form denoiser of iid N(m0, s0^2) data: eps = sqrt(1-abar)(x - sqrt(abar) m0)/(abar s0^2 + 1 - abar).

@@ -19,6 +19,7 @@
 #include "common.cuh"
 #include "gemm_tcgen05.cuh"
 #include "net_kernels.cuh"
+#include "mlp_kernels.cuh"
 #include "round_kernels.cuh"
 #include "drafter_cluster.cuh"
 #include "sched_kernel.cuh"
@@ -1121,6 +1122,40 @@ int forward(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, cudaStream_t s, 
   return r;
 }
 
+// How the MLP kernels cover n latents.  One latent per cluster while that leaves SMs free (a weight is read once per
+// latent), four beyond a quarter of the SMs (it is then read once per four); CTAs per cluster doubled while a CTA's share
+// of the largest layer exceeds 32 KB -- about 500 clocks of L2 reads, what a cluster barrier costs -- and the SMs last.
+struct MlpShape { int R, cs; size_t smem; };
+MlpShape mlp_shape(const tsdp_ctx* c, const Net& n, int latents) {
+  MlpShape sh{1, 1, 0};
+  const int mw = mlp_max_width(n.mlp);
+  if (latents > c->num_sms / 4 && mlp_smem_bytes(mw, 4) + 4 * sizeof(float) * c->D <= MLP_MAX_SMEM) sh.R = 4;
+  size_t big = 0;
+  for (int l = 0; l < n.mlp.n_lin; ++l) big = std::max(big, (size_t)n.mlp.dims[l] * n.mlp.dims[l + 1] * sizeof(float));
+  const int groups = (latents + sh.R - 1) / sh.R;
+  while (sh.cs < 8 && big > (size_t)sh.cs * 32 * 1024 && groups * sh.cs * 2 <= c->num_sms) sh.cs *= 2;
+  sh.smem = mlp_smem_bytes(mw, sh.R) + (size_t)sh.R * sizeof(float) * c->D;
+  return sh;
+}
+
+// K draft steps of B slots with the MLP drafter in one launch.
+int launch_mlp_rollout(tsdp_ctx* c, int B, int K, cudaStream_t s) {
+  const Net& n = c->net[TSDP_DRAFT];
+  const MlpShape sh = mlp_shape(c, n, B);
+  const int groups = (B + sh.R - 1) / sh.R;
+  const long long xs_b = (long long)(c->cfg.max_K + 1) * c->D, ms_b = (long long)(c->cfg.max_K > 0 ? c->cfg.max_K : 1) * c->D;
+  prof_begin(c, s, 5, 0.0);
+#define MLP_CASE(RR) launch_kernel_cluster(c, mlp_rollout_kernel<RR>, dim3(groups * sh.cs), dim3(MLP_THREADS), sh.smem, s, sh.cs, n.mlp, c->S,       \
+                                           c->xt, xs_b, c->muhat, ms_b, c->t, c->seed, c->sched_on ? c->envp : nullptr, c->item, c->obs, \
+                                           c->cfg.obs_tokens * c->cfg.obs_dim, c->D, B, K, c->cfg.T, sh.cs)
+  if (sh.R == 4) MLP_CASE(4); else MLP_CASE(1);
+#undef MLP_CASE
+  prof_end(c, s);
+  c->launches_per_round_tmp++;
+  CU_TRY(c, cudaGetLastError());
+  return TSDP_OK;
+}
+
 int forward_arch(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, cudaStream_t s) {
   const int D = c->D;
   switch (n.cfg.arch) {
@@ -1134,11 +1169,13 @@ int forward_arch(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, cudaStream_
       return TSDP_OK;
     }
     case TSDP_ARCH_MLP: {
-      int maxw = 0;
-      for (int l = 0; l <= n.mlp.n_lin; ++l) maxw = n.mlp.dims[l] > maxw ? n.mlp.dims[l] : maxw;
+      const MlpShape sh = mlp_shape(c, n, n_cand);
+      const int groups = (n_cand + sh.R - 1) / sh.R;
       prof_begin(c, s, 5, 0.0);
-      TSDP_LAUNCH(c, (mlp_forward_kernel), n_cand, 256, 2 * maxw * sizeof(float), s, n.mlp, cm, c->obs, c->cfg.obs_tokens * c->cfg.obs_dim,
-                                                                        D, c->cfg.T);
+#define MLP_CASE(RR) launch_kernel_cluster(c, mlp_forward_kernel<RR>, dim3(groups * sh.cs), dim3(MLP_THREADS), sh.smem, s, sh.cs, n.mlp, cm, \
+                                           c->obs, c->cfg.obs_tokens * c->cfg.obs_dim, D, c->cfg.T, n_cand, sh.cs)
+      if (sh.R == 4) MLP_CASE(4); else MLP_CASE(1);
+#undef MLP_CASE
       prof_end(c, s);
       c->launches_per_round_tmp++;
       CU_TRY(c, cudaGetLastError());
@@ -1274,9 +1311,11 @@ int enqueue_round(tsdp_ctx* c, int B, int K, cudaStream_t s, bool dbg) {
       if (r) return r;
     }
   }
+  const bool mlp_draft = K > 0 && c->net[TSDP_DRAFT].cfg.arch == TSDP_ARCH_MLP;
+  if (mlp_draft && (r = launch_mlp_rollout(c, B, K, s))) return r;
   // transformer drafter, layer by layer: its head, the draft step and the next step's embedding are one kernel
   const bool fused_tail = c->net[TSDP_DRAFT].cfg.arch == TSDP_ARCH_XFMR && c->cfg.A <= 32;
-  for (int k = 1; k <= K && !cluster_draft; ++k) {
+  for (int k = 1; k <= K && !cluster_draft && !mlp_draft; ++k) {
     CandMap cm{c->xt + (long long)(k - 1) * D, xs_b, c->eps_d, (long long)D, c->t, 1, k - 1, c->item,
                compact ? c->plan_order : nullptr, compact ? c->plan_dn + k : nullptr};     // the slots still drafting at step k
     c->prof_gemm_cat = 6;
@@ -1621,6 +1660,9 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
     fprintf(stderr, "tsdp_init: the persistent cluster drafter does not fit this configuration\n");
     return fail(TSDP_ERR_UNSUPPORTED);
   }
+  for (const void* fn : {(const void*)mlp_forward_kernel<1>, (const void*)mlp_forward_kernel<4>, (const void*)mlp_rollout_kernel<1>,
+                         (const void*)mlp_rollout_kernel<4>})
+    INIT_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_MAX_SMEM));
   INIT_TRY(cudaFuncSetAttribute(cross_attn_ctx_mma_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, cx_smem_bytes<32>(256)));
   INIT_TRY(cudaFuncSetAttribute(cross_attn_ctx_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, cx_smem_bytes<64>(256)));
   INIT_TRY(cudaFuncSetAttribute(cross_attn_ctx_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, cx_smem_bytes<128>(256)));
