@@ -14,9 +14,10 @@ constexpr int TSDP_PLAN_MAXK = 32;      // = TSDP_MAX_K of the C ABI
 // [B, Kmax+1, D]; slot 0 is the current latent x.
 __global__ void init_chunk_kernel(float* __restrict__ xt, long long xs_b, int* __restrict__ t, int B, int D,
                                   int T, const uint64_t* __restrict__ seedp, int* __restrict__ round_idx, int* __restrict__ n_done,
-                                  int* __restrict__ item, int* __restrict__ queue_head) {
+                                  int* __restrict__ item, int* __restrict__ queue_head, int* __restrict__ item_counts, int n_requests) {
   pdl_trigger();
   pdl_wait();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 4 * n_requests; i += gridDim.x * blockDim.x) item_counts[i] = 0;
   const uint64_t seed = *seedp;
   const int b = blockIdx.x;
   const int nq = (D + 3) >> 2;
@@ -199,6 +200,26 @@ __device__ __forceinline__ void store_quad(float* __restrict__ p, int q, int D, 
   }
 }
 
+// End of a round, by the last block of the acceptance kernel: the round index advances and the host learns, through one
+// mapped 64-bit word, how many rounds are complete (upper half) and how many reverse steps the slot that is furthest
+// behind still needs (lower half; 0: every request is finished).  blocks, t_left: device words that are zero between
+// rounds; blocks null: no round bookkeeping (the allocation-free entry point).
+struct RoundEnd {
+  int *blocks, *t_left, *round_idx;
+  volatile unsigned long long* host;
+};
+__device__ __forceinline__ void round_end(const RoundEnd& e, int t_after) {      // one thread of every block
+  if (e.blocks == nullptr) return;
+  if (t_after >= 0) atomicMax(e.t_left, t_after + 1);
+  __threadfence();
+  if (atomicAdd(e.blocks, 1) != (int)gridDim.x - 1) return;
+  __threadfence();
+  const int left = atomicExch(e.t_left, 0), idx = *e.round_idx + 1;
+  *e.blocks = 0;
+  *e.round_idx = idx;
+  *e.host = ((unsigned long long)idx << 32) | (unsigned long long)left;
+}
+
 // Fused verification tail, one block per environment, one warp per drafted step.
 //   warp k-1 (k = 1..K_eff): mu_k = posterior mean of (x~_{k-1}, eps_{k-1}) at tau = t-k+1;
 //       d = (mu^_k - mu_k) / (s sigma_tau);  log alpha = -1/2 |d|^2 - <d, xi_tau>   (Sec. 3.2)
@@ -214,11 +235,11 @@ __global__ void accept_kernel(DdpmTables S, float* __restrict__ xt, long long xs
                               const float* __restrict__ muhat, long long ms_b,
                               const float* __restrict__ eps, long long es_b, int* __restrict__ t, int K, int D,
                               const uint64_t* __restrict__ seedp, const RoundParams* __restrict__ sched, int n_sched,
-                              const int* __restrict__ round_idx, float* __restrict__ actions,
+                              const int* round_idx, float* __restrict__ actions,
                               int* __restrict__ n_done, DevStats* __restrict__ stats, float draft_nfe,
                               float* __restrict__ dbg_logalpha, int* __restrict__ dbg_jstar,
                               const EnvParams* __restrict__ envp, int* __restrict__ item, int* __restrict__ queue_head,
-                              const int* __restrict__ n_items, int* __restrict__ item_counts) {
+                              const int* __restrict__ n_items, int* __restrict__ item_counts, RoundEnd rend) {
   pdl_trigger();
   pdl_wait();
   __shared__ float s_la[32], s_s1[32], s_s2[32];
@@ -228,7 +249,10 @@ __global__ void accept_kernel(DdpmTables S, float* __restrict__ xt, long long xs
   const int b = blockIdx.x;
   const int tb = t[b];
   if (tb < 0) {
-    if (dbg_jstar && threadIdx.x == 0) dbg_jstar[b] = -1;
+    if (threadIdx.x == 0) {
+      if (dbg_jstar) dbg_jstar[b] = -1;
+      round_end(rend, -1);
+    }
     return;
   }
   const int r = min(*round_idx, n_sched - 1);
@@ -381,8 +405,11 @@ __global__ void accept_kernel(DdpmTables S, float* __restrict__ xt, long long xs
           if (4 * q + jj < D) xo[4 * q + jj] = z[jj];
       }
       if (threadIdx.x == 0) { item[b] = next; t[b] = S.T - 1; }
+      if (threadIdx.x == 0) round_end(rend, S.T - 1);
+      return;
     }
   }
+  if (threadIdx.x == 0) round_end(rend, t_new);
 }
 
 // Intermediate ("process") reward of the scheduler's training signal, Sec. 3.3 "Reward function":
@@ -398,16 +425,6 @@ __global__ void process_reward_kernel(const int* __restrict__ item_counts, int n
   const float a = n_draft > 0 ? (float)n_acc / (float)n_draft : 0.f;
   const float e = n_diff > 0 ? (float)n_acc / (float)n_diff : 0.f;
   reward[i] = (a + e) * lam;
-}
-
-// End of a round: advance the schedule index and publish the number of finished chunks where the
-// host can read it.
-__global__ void round_end_kernel(int* __restrict__ round_idx, const int* __restrict__ n_done,
-                                 volatile int* __restrict__ host_done) {
-  pdl_trigger();
-  pdl_wait();
-  *round_idx += 1;
-  *host_done = *n_done;
 }
 
 }  // namespace tsdp

@@ -98,9 +98,12 @@ struct tsdp_ctx {
   size_t items_cap = 0;
   uint64_t* seed = nullptr;
   int *round_idx = nullptr, *n_done = nullptr, *status = nullptr;
-  int* host_done = nullptr;                   // mapped pinned
+  int *round_blocks = nullptr, *t_left = nullptr;        // end-of-round bookkeeping of the acceptance kernel (RoundEnd)
+  unsigned long long* host_prog = nullptr;    // mapped pinned: rounds complete << 32 | reverse steps still needed
+  int* status_host = nullptr;                 // pinned copy of the status word at the end of a chunk call
+  // parameters of a call, one buffer and one copy: seed (8 bytes), number of requests (4 + 4), the round table behind it
   RoundParams* sched = nullptr;               // device, capacity TSDP_MAX_T + 1
-  RoundParams* sched_host = nullptr;          // pinned staging
+  uint8_t *params = nullptr, *params_host = nullptr;     // the whole buffer on the device, its pinned staging
   DevStats* stats = nullptr;
   float* dbg_logalpha = nullptr;
   int* dbg_jstar = nullptr;
@@ -1357,10 +1360,10 @@ int enqueue_round(tsdp_ctx* c, int B, int K, cudaStream_t s, bool dbg) {
   TSDP_LAUNCH(c, (accept_kernel), B, warps * 32, 0, s, c->S, c->xt, xs_b, c->muhat, ms_b, c->eps, xs_b, c->t, K, D, c->seed, c->sched,
                                          TSDP_MAX_T + 1, c->round_idx, c->actions, c->n_done, c->stats, c->cfg.draft_nfe,
                                          dbg ? c->dbg_logalpha : nullptr, dbg ? c->dbg_jstar : nullptr,
-                                         c->sched_on ? c->envp : nullptr, c->item, c->queue_head, c->n_items, c->item_counts);
+                                         c->sched_on ? c->envp : nullptr, c->item, c->queue_head, c->n_items, c->item_counts,
+                                         RoundEnd{c->round_blocks, c->t_left, c->round_idx, c->host_prog});
   prof_end(c, s);
-  TSDP_LAUNCH(c, (round_end_kernel), 1, 1, 0, s, c->round_idx, c->n_done, c->host_done);
-  c->launches_per_round_tmp += 2;
+  c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
   return TSDP_OK;
 }
@@ -1417,19 +1420,41 @@ bool accept_ok(const tsdp_accept_t* a) {
   return a && (a->mode == 0 || a->mode == 1) && a->sigma_scale > 0.f && (a->mode == 0 || (a->lambda > 0.f && a->lambda <= 1.f));
 }
 
-// Upload the per-round parameter table: entry r for round r, the last entry repeating.
-int upload_schedule(tsdp_ctx* c, int K, const tsdp_accept_t& acc, cudaStream_t s, bool ignore_user_schedule) {
+constexpr size_t PARAMS_HEAD = 16;
+constexpr size_t PARAMS_BYTES = PARAMS_HEAD + sizeof(RoundParams) * (TSDP_MAX_T + 1);
+
+// Upload the parameters of a call: seed, number of requests and the round table (entry r for round r, the last entry
+// repeating).
+int upload_params(tsdp_ctx* c, int K, const tsdp_accept_t& acc, uint64_t seed, int n_requests, cudaStream_t s, bool ignore_user_schedule) {
+  memcpy(c->params_host, &seed, sizeof(seed));
+  memcpy(c->params_host + 8, &n_requests, sizeof(int));
+  RoundParams* tab = reinterpret_cast<RoundParams*>(c->params_host + PARAMS_HEAD);
   const int n = ignore_user_schedule ? 0 : (int)c->sched_K.size();
-  for (int r = 0; r <= TSDP_MAX_T; ++r) {
-    if (n > 0) {
-      const int i = r < n ? r : n - 1;
-      fill_round_params(&c->sched_host[r], c->sched_K[i], c->sched_acc[i]);
-    } else {
-      fill_round_params(&c->sched_host[r], K, acc);
-    }
-  }
-  CU_TRY(c, cudaMemcpyAsync(c->sched, c->sched_host, sizeof(RoundParams) * (TSDP_MAX_T + 1), cudaMemcpyHostToDevice, s));
+  for (int r = 0; r < n; ++r) fill_round_params(&tab[r], c->sched_K[r], c->sched_acc[r]);
+  RoundParams last;
+  if (n > 0) last = tab[n - 1];
+  else fill_round_params(&last, K, acc);
+  for (int r = n; r <= TSDP_MAX_T; ++r) tab[r] = last;
+  CU_TRY(c, cudaMemcpyAsync(c->params, c->params_host, PARAMS_BYTES, cudaMemcpyHostToDevice, s));
   return TSDP_OK;
+}
+
+// Wait until at least `rounds` rounds of the running call are complete and return the progress word.  The word is
+// polled, so that the host reacts within a microsecond; the stream is asked now and then in case it failed.
+int wait_progress(tsdp_ctx* c, cudaStream_t s, unsigned long long rounds, unsigned long long* out) {
+  volatile unsigned long long* p = c->host_prog;
+  for (unsigned i = 1;; ++i) {
+    unsigned long long v = *p;
+    if ((v >> 32) >= rounds) { *out = v; return TSDP_OK; }
+    if (i % 4096 != 0) continue;
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e == cudaErrorNotReady) continue;
+    CU_TRY(c, e);
+    v = *p;                                  // everything issued has finished: the word is final
+    if ((v >> 32) >= rounds) { *out = v; return TSDP_OK; }
+    c->last_error = "a round finished without reporting its progress";
+    return TSDP_ERR_CUDA;
+  }
 }
 
 }  // namespace
@@ -1535,17 +1560,17 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
   st |= dev_alloc(c, c->allocs, &c->actions, B * D);
   st |= dev_alloc(c, c->allocs, &c->obs, B * (size_t)cfg->obs_tokens * cfg->obs_dim + 1);
   st |= dev_alloc(c, c->allocs, &c->t, B);
-  st |= dev_alloc(c, c->allocs, &c->seed, 1);
+  st |= dev_alloc(c, c->allocs, &c->params, PARAMS_BYTES);
   st |= dev_alloc(c, c->allocs, &c->round_idx, 1);
   st |= dev_alloc(c, c->allocs, &c->n_done, 1);
   st |= dev_alloc(c, c->allocs, &c->status, 1);
-  st |= dev_alloc(c, c->allocs, &c->sched, TSDP_MAX_T + 1);
+  st |= dev_alloc(c, c->allocs, &c->round_blocks, 1);
+  st |= dev_alloc(c, c->allocs, &c->t_left, 1);
   st |= dev_alloc(c, c->allocs, &c->stats, 1);
   st |= dev_alloc(c, c->allocs, &c->dbg_logalpha, B * Km);
   st |= dev_alloc(c, c->allocs, &c->dbg_jstar, B);
   st |= dev_alloc(c, c->allocs, &c->item, B);
   st |= dev_alloc(c, c->allocs, &c->queue_head, 1);
-  st |= dev_alloc(c, c->allocs, &c->n_items, 1);
   c->items_cap = B;
   st |= dev_alloc(c, c->allocs, &c->envp, B);
   st |= dev_alloc(c, c->allocs, &c->progress, B);
@@ -1561,9 +1586,13 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
   st |= dev_alloc(c, c->allocs, &c->distill_terms, 5 * B);
   st |= dev_alloc(c, c->allocs, &c->distill_res, 8);
   if (st) return fail(TSDP_ERR_CUDA);
-  INIT_TRY(cudaHostAlloc(reinterpret_cast<void**>(&c->host_done), sizeof(int), cudaHostAllocMapped));
-  *c->host_done = 0;
-  INIT_TRY(cudaHostAlloc(reinterpret_cast<void**>(&c->sched_host), sizeof(RoundParams) * (TSDP_MAX_T + 1), cudaHostAllocDefault));
+  c->seed = reinterpret_cast<uint64_t*>(c->params);
+  c->n_items = reinterpret_cast<int*>(c->params + 8);
+  c->sched = reinterpret_cast<RoundParams*>(c->params + PARAMS_HEAD);
+  INIT_TRY(cudaHostAlloc(reinterpret_cast<void**>(&c->host_prog), sizeof(unsigned long long), cudaHostAllocMapped));
+  *c->host_prog = 0;
+  INIT_TRY(cudaHostAlloc(reinterpret_cast<void**>(&c->params_host), PARAMS_BYTES, cudaHostAllocDefault));
+  INIT_TRY(cudaHostAlloc(reinterpret_cast<void**>(&c->status_host), sizeof(int), cudaHostAllocDefault));
   INIT_TRY(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   INIT_TRY(cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
   INIT_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
@@ -1713,8 +1742,9 @@ void tsdp_destroy(tsdp_ctx* c) {
   for (cudaEvent_t e : c->prof_ev) cudaEventDestroy(e);
   dev_free_pool(c, c->allocs);
   for (int w = 0; w < 2; ++w) dev_free_pool(c, c->net[w].allocs);
-  if (c->host_done) cudaFreeHost(c->host_done);
-  if (c->sched_host) cudaFreeHost(c->sched_host);
+  if (c->host_prog) cudaFreeHost(c->host_prog);
+  if (c->params_host) cudaFreeHost(c->params_host);
+  if (c->status_host) cudaFreeHost(c->status_host);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -2259,11 +2289,9 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
   CU_TRY(c, cudaEventRecord(c->ev_chunk0, s));
   if (obs_n)
     CU_TRY(c, cudaMemcpyAsync(c->obs, obs, obs_n * sizeof(float), obs_on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
-  CU_TRY(c, cudaMemcpyAsync(c->seed, &seed, sizeof(seed), cudaMemcpyHostToDevice, s));
-  CU_TRY(c, cudaMemcpyAsync(c->n_items, &N, sizeof(int), cudaMemcpyHostToDevice, s));
-  CU_TRY(c, cudaMemsetAsync(c->item_counts, 0, sizeof(int) * 4 * (size_t)N, s));
   c->items_last = N;
-  if ((r = upload_schedule(c, K, *acc, s, false))) return r;
+  *c->host_prog = 0;                         // nothing of an earlier call is in flight: every call ends with a synchronise
+  if ((r = upload_params(c, K, *acc, seed, N, s, false))) return r;
   if (c->sched_on) {
     // the scheduler network reads the new observation, the previous chunk's actions and the progress; it
     // runs on a side stream beside the chunk set-up and joins before the first round
@@ -2276,31 +2304,42 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
     c->launches++;
   }
   const long long xs_b = (long long)(c->cfg.max_K + 1) * D;
-  init_chunk_kernel<<<B, 128, 0, s>>>(c->xt, xs_b, c->t, B, D, T, c->seed, c->round_idx, c->n_done, c->item, c->queue_head);
+  init_chunk_kernel<<<B, 128, 0, s>>>(c->xt, xs_b, c->t, B, D, T, c->seed, c->round_idx, c->n_done, c->item, c->queue_head,
+                                    c->item_counts, N);
   CU_TRY(c, cudaGetLastError());
   c->launches_per_round_tmp = 0;
   if ((r = prepare_obs(c, c->net[TSDP_BASE], N, s))) return r;
   if ((r = prepare_obs(c, c->net[TSDP_DRAFT], N, s))) return r;
   c->launches += 1 + c->launches_per_round_tmp;
-  // Rounds.  A request cannot finish before its drafted windows could have covered T steps, so the
-  // completion flag is only read once the slots could have worked through all N requests.
   if (c->sched_on) CU_TRY(c, cudaStreamWaitEvent(s, c->ev_join, 0));
+  // Rounds, issued ahead of their results: a round takes a slot at most K + 1 reverse steps further, so the next round is
+  // surely needed while the slots cannot have worked through all N requests yet (`budget`), or while the slot that was
+  // furthest behind after the last completed round the host knows of needs more steps than the rounds in flight can
+  // take.  Only where neither holds does the host wait for a newer result; the GPU idles between two rounds only
+  // near the end of a call.
   const int n_sched = (int)c->sched_K.size();
+  auto round_K = [&](long long r) { return n_sched > 0 ? c->sched_K[r < n_sched ? r : n_sched - 1] : K; };
   const long long waves = ((long long)N + B - 1) / B;
   long long budget = (long long)T * N / B;
   const long long max_rounds = (long long)(T + 1) * waves + 1;
-  for (long long round = 0; round < max_rounds; ++round) {
-    const int Kr = n_sched > 0 ? c->sched_K[round < n_sched ? round : n_sched - 1] : K;
-    if ((r = run_round(c, B, Kr, s))) return r;
-    c->rounds++;
-    budget -= Kr + 1;
-    if (budget <= 0) {
-      CU_TRY(c, cudaStreamSynchronize(s));
-      if (*c->host_done >= N) break;
+  long long known = 0, left = T, in_flight = 0;      // rounds known to be complete, steps needed after them, steps the others may take
+  for (long long round = 0; round < max_rounds;) {
+    if (budget > 0 || left > in_flight) {
+      const int Kr = round_K(round);
+      if ((r = run_round(c, B, Kr, s))) return r;
+      c->rounds++; round++;
+      budget -= Kr + 1; in_flight += Kr + 1;
+      continue;
     }
+    if (known == round) break;                       // left == 0: every request is finished
+    unsigned long long v = 0;
+    if ((r = wait_progress(c, s, (unsigned long long)known + 1, &v))) return r;
+    for (; known < (long long)(v >> 32); ++known) in_flight -= round_K(known) + 1;
+    left = (long long)(v & 0xffffffffull);
   }
   CU_TRY(c, cudaMemcpyAsync(actions, c->actions, (size_t)N * D * sizeof(float),
                             actions_on_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, s));
+  CU_TRY(c, cudaMemcpyAsync(c->status_host, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU_TRY(c, cudaEventRecord(c->ev_chunk1, s));
   CU_TRY(c, cudaStreamSynchronize(s));
   {   // device time of this call, copies included, into the latency ring
@@ -2311,7 +2350,7 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
       if (c->lat_n < c->lat_ring.size()) c->lat_n++;
     }
   }
-  return check_status(c);
+  return *c->status_host != 0 ? check_status(c) : TSDP_OK;
 }
 
 int tsdp_sample_chunk(tsdp_ctx* c, const float* d_obs, int B, int K, const tsdp_accept_t* acc, uint64_t seed,
@@ -2345,8 +2384,7 @@ int tsdp_round(tsdp_ctx* c, const float* d_obs, int B, int K, const tsdp_accept_
   const size_t K1 = c->cfg.max_K + 1, Km = c->cfg.max_K > 0 ? c->cfg.max_K : 1;
   int r;
   if (obs_n) CU_TRY(c, cudaMemcpyAsync(c->obs, d_obs, obs_n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  CU_TRY(c, cudaMemcpyAsync(c->seed, &seed, sizeof(seed), cudaMemcpyHostToDevice, s));
-  if ((r = upload_schedule(c, K, *acc, s, true))) return r;
+  if ((r = upload_params(c, K, *acc, seed, B, s, true))) return r;
   CU_TRY(c, cudaMemsetAsync(c->round_idx, 0, sizeof(int), s));
   CU_TRY(c, cudaMemsetAsync(c->n_done, 0, sizeof(int), s));
   {   // every slot serves the request of its own index and nothing is waiting
@@ -2354,7 +2392,6 @@ int tsdp_round(tsdp_ctx* c, const float* d_obs, int B, int K, const tsdp_accept_
     for (int b = 0; b < B; ++b) ident[b] = b;
     CU_TRY(c, cudaMemcpyAsync(c->item, ident.data(), sizeof(int) * B, cudaMemcpyHostToDevice, s));
     CU_TRY(c, cudaMemcpyAsync(c->queue_head, &B, sizeof(int), cudaMemcpyHostToDevice, s));
-    CU_TRY(c, cudaMemcpyAsync(c->n_items, &B, sizeof(int), cudaMemcpyHostToDevice, s));
     CU_TRY(c, cudaMemsetAsync(c->item_counts, 0, sizeof(int) * 4 * (size_t)B, s));
     c->items_last = B;
   }
@@ -2753,7 +2790,8 @@ int tsdp_verify_commit_static(int device, int T, float beta0, float beta1, float
   if (warps < 4) warps = 4;
   if (warps > 16) warps = 16;
   accept_kernel<<<B, warps * 32, 0, s>>>(S, d_xt, xs_b, d_muhat, ms_b, d_eps, xs_b, dt, K, D, dseed, drp, 1, dround,
-                                         d_actions, ddone, st, draft_nfe, d_logalpha, dj, nullptr, nullptr, nullptr, nullptr, nullptr);
+                                         d_actions, ddone, st, draft_nfe, d_logalpha, dj, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                         RoundEnd{});
   ST_TRY(cudaGetLastError());
   ST_TRY(cudaMemcpyAsync(h_t_new, dt, sizeof(int) * B, cudaMemcpyDeviceToHost, s));
   ST_TRY(cudaMemcpyAsync(h_jstar, dj, sizeof(int) * B, cudaMemcpyDeviceToHost, s));
