@@ -63,7 +63,7 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   const uint32_t sQ = base, sK = base + CXT_OFF_K, sVt = base + CXT_OFF_VT, bar0 = base + CXT_OFF_BAR;
   const uint32_t bar_kv = bar0, bar_q0 = bar0 + 8, bar_s = bar0 + 24, bar_p = bar0 + 32, bar_o = bar0 + 40, bar_or = bar0 + 48;
   const uint32_t tmem_slot = bar0 + 64;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     ptx::mbar_init(bar_kv, 1); ptx::mbar_init(bar_q0, 1); ptx::mbar_init(bar_q0 + 8, 1);
     ptx::mbar_init(bar_s, 1); ptx::mbar_init(bar_p, 256); ptx::mbar_init(bar_o, 1); ptx::mbar_init(bar_or, 256);
@@ -132,7 +132,7 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   const int hc = Tc / 2;                                    // score columns per softmax thread; a multiple of 16
   if (ok && n_tiles > 0) {
     if (warp == 8) {
-      if (lane == 0) {
+      if (ptx::elect_one()) {
         const uint32_t idesc1 = umma_idesc_bf16(Tc, 128), idesc2 = umma_idesc_bf16(64, 128);
         for (int i = 0; i < n_tiles; ++i) {
           const uint32_t qb = sQ + (uint32_t)(i & 1) * CXT_Q_BYTES;

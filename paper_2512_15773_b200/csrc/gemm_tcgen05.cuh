@@ -41,8 +41,13 @@ constexpr int GEMM_THREADS = 320;
 constexpr int GEMM_EPI_WARPS = 8;
 constexpr long long GEMM_WAIT_CYCLES = 2000000000ll;   // about one second of SM clock
 
-__host__ __device__ constexpr int gemm_stages(int BN) { return BN >= 192 ? 4 : (BN >= 128 ? 6 : 8); }
-__host__ __device__ constexpr int gemm_stage_bytes(int BN) { return GEMM_BM * GEMM_BK * 2 + BN * GEMM_BK * 2; }
+// k-blocks per pipeline stage.  A round of the issue loops (wait, loads or MMAs, arrive) takes about 336 clocks, the tensor
+// core 160 - 192 clocks per k-block for tiles up to 64 wide (operand reads from shared memory), so there a stage holds two
+// k-blocks and a round issues twice as much: 0.177 -> 0.135 us per k-block at BN = 64 (0.177 -> 0.130 at BN = 32).  At 128 two of
+// them leave only three stages and tie, wider tiles are bound by the MMAs (512 clocks per k-block at BN = 256).
+__host__ __device__ constexpr int gemm_stage_kb(int BN) { return BN <= 64 ? 2 : 1; }
+__host__ __device__ constexpr int gemm_stages(int BN) { return BN >= 192 ? 4 : (BN == 128 ? 6 : (BN == 64 ? 4 : 5)); }
+__host__ __device__ constexpr int gemm_stage_bytes(int BN) { return gemm_stage_kb(BN) * (GEMM_BM * GEMM_BK * 2 + BN * GEMM_BK * 2); }
 constexpr int GEMM_STAGING_BYTES = 2 * 128 * 128;   // one 128-row x 128-byte chunk per column half
 constexpr int GEMM_ATTN_BN = 192;                   // [Q | K | V] of one 64-wide head
 constexpr int GEMM_ATTN_P = 64 + 8;                 // row pitch (elements) of the staged Q / K / V tiles
@@ -62,7 +67,9 @@ __host__ __device__ constexpr int gemm_smem_bytes(int BN) {
 // HALF of the W tile, so a stage is smaller and the ring deeper.
 // The smaller stages also leave room for two staging chunks per column half, so that the epilogue does not have to
 // wait for its previous TMA store (which queues behind the operand loads) before it fills the next chunk.
-__host__ __device__ constexpr int gemm_stage_bytes_cg(int BN, int CG) { return GEMM_BM * GEMM_BK * 2 + (BN / CG) * GEMM_BK * 2; }
+__host__ __device__ constexpr int gemm_stage_bytes_cg(int BN, int CG) {
+  return CG == 2 ? GEMM_BM * GEMM_BK * 2 + (BN / CG) * GEMM_BK * 2 : gemm_stage_bytes(BN);
+}
 __host__ __device__ constexpr int gemm_stages_cg(int BN, int CG) { return CG == 2 ? (BN == GEMM_ATTN_BN ? 6 : 5) : gemm_stages(BN); }
 __host__ __device__ constexpr int gemm_staging_bufs(int CG) { return CG == 2 ? 2 : 1; }      // per column half
 __host__ __device__ constexpr int gemm_epi_smem_bytes_cg(int BN, int CG) {
@@ -106,6 +113,14 @@ __device__ __forceinline__ bool mbar_wait_thread(uint32_t bar, uint32_t parity, 
 // .sync.aligned section alone.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, long long limit = GEMM_WAIT_CYCLES) {
   return __all_sync(0xffffffffu, mbar_wait_thread(bar, parity, limit)) != 0;
+}
+// One lane of a converged warp, chosen by the hardware.  Under this predicate the compiler knows that a single thread
+// runs and issues tcgen05 / TMA instructions directly; under `lane == 0` it wraps each of them in a loop over the active
+// lanes (measured per k-block of four MMAs, wait and commit: 231 clocks against 467 for tiles up to 64 wide).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile(
@@ -363,7 +378,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   constexpr int STAGES = gemm_stages_cg(BN, CG);
   constexpr int A_BYTES = GEMM_BM * GEMM_BK * 2;
   constexpr int B_ROWS = BN / CG;                      // rows of the W tile this CTA stages
+  constexpr int SK = CG == 2 ? 1 : gemm_stage_kb(BN);  // k-blocks per stage, each [A | W] one behind the other
   constexpr int STAGE_BYTES = gemm_stage_bytes_cg(BN, CG);
+  constexpr int KB_BYTES = STAGE_BYTES / SK;
   static_assert(CG == 1 || CG == 2, "CG");
   static_assert(CG == 1 || BN == 256 || BN == GEMM_ATTN_BN, "pair form: wide tiles only");
   constexpr int ACC = BN == GEMM_ATTN_BN ? 256 : BN;          // column distance of the two accumulator buffers
@@ -387,7 +404,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       reinterpret_cast<volatile uint32_t*>(smem_raw + (tmem_slot - ptx::smem_u32(smem_raw)));
   float* sbias = reinterpret_cast<float*>(smem_raw + (bar0 + 256u - ptx::smem_u32(smem_raw)));    // behind the barriers
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int tiles_n = g.N / BN;
   const int kblocks = g.K / GEMM_BK;
   const uint32_t rank = CG == 2 ? ptx::cluster_rank() : 0u;     // 0: the pair's leader
@@ -422,28 +439,38 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       int stage = 0; uint32_t phase = 0;
       for (int unit = tile0; unit < n_tiles && ok; unit += tile_step) {
         const int tile = unit / S, part = unit - tile * S;
         const int tm = (tile / tiles_n) * CG + (int)rank, tn = tile % tiles_n;
         const int kb0 = part * kblocks / S, kb1 = (part + 1) * kblocks / S;
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (int kb = kb0; kb < kb1; kb += SK) {
           if (!ptx::mbar_wait_thread(empty_bar(stage), phase ^ 1u, wlim)) { ok = false; break; }
           if (!(g.withhold_first_stage && blockIdx.x == 0 && unit == 0 && kb == 0)) {
-            const uint32_t sa = base + stage * STAGE_BYTES;
-            const int kcol = kb * GEMM_BK;
-            const int ax = g.conv_c ? kcol % g.conv_c : kcol, ay = tm * GEMM_BM + (g.conv_c ? kcol / g.conv_c : 0);
+            const uint32_t s0 = base + stage * STAGE_BYTES;
+            const int nk = SK == 1 ? 1 : min(SK, kb1 - kb);
             if (CG == 2) {
               // the leader's barrier counts the bytes of both CTAs' loads of this stage
               if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), STAGE_BYTES * 2);
-              const uint32_t fb = ptx::mapa_rank(full_bar(stage), 0);
-              ptx::tma_load_2d_pair(sa, &tmA, ax, ay, fb);
-              ptx::tma_load_2d_pair(sa + A_BYTES, &tmB, kb * GEMM_BK, tn * BN + (int)rank * B_ROWS, fb);
             } else {
-              ptx::mbar_expect_tx(full_bar(stage), STAGE_BYTES);
-              ptx::tma_load_2d(sa, &tmA, ax, ay, full_bar(stage));
-              ptx::tma_load_2d(sa + A_BYTES, &tmB, kb * GEMM_BK, tn * BN, full_bar(stage));
+              ptx::mbar_expect_tx(full_bar(stage), nk * KB_BYTES);
+            }
+#pragma unroll
+            for (int j = 0; j < SK; ++j) {
+              if (j < nk) {
+                const uint32_t sa = s0 + j * KB_BYTES;
+                const int kcol = (kb + j) * GEMM_BK;
+                const int ax = g.conv_c ? kcol % g.conv_c : kcol, ay = tm * GEMM_BM + (g.conv_c ? kcol / g.conv_c : 0);
+                if (CG == 2) {
+                  const uint32_t fb = ptx::mapa_rank(full_bar(stage), 0);
+                  ptx::tma_load_2d_pair(sa, &tmA, ax, ay, fb);
+                  ptx::tma_load_2d_pair(sa + A_BYTES, &tmB, kcol, tn * BN + (int)rank * B_ROWS, fb);
+                } else {
+                  ptx::tma_load_2d(sa, &tmA, ax, ay, full_bar(stage));
+                  ptx::tma_load_2d(sa + A_BYTES, &tmB, kcol, tn * BN, full_bar(stage));
+                }
+              }
             }
           }
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -451,7 +478,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {      // in a pair only the leader issues
+    if (rank == 0 && ptx::elect_one()) {      // in a pair only the leader issues
       int stage = 0; uint32_t phase = 0; int it = 0;
       for (int unit = tile0; unit < n_tiles && ok; unit += tile_step, ++it) {
         const int part = unit % S;
@@ -460,15 +487,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (!ptx::mbar_wait_thread(tempty_bar(as), aphase ^ 1u, wlim)) { ok = false; break; }
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * ACC);
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (int kb = kb0; kb < kb1; kb += SK) {
           if (!ptx::mbar_wait_thread(full_bar(stage), phase, wlim)) { ok = false; break; }
           ptx::tc_fence_after();
-          const uint32_t sa = base + stage * STAGE_BYTES;
-          const uint64_t da = umma_desc_sw128(sa), db = umma_desc_sw128(sa + A_BYTES);
+          const uint32_t s0 = base + stage * STAGE_BYTES;
 #pragma unroll
-          for (int k = 0; k < GEMM_BK / 16; ++k) {
-            if (CG == 2) ptx::tc_mma_bf16_pair(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), IDESC, (kb > kb0 || k) ? 1u : 0u);
-            else ptx::tc_mma_bf16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), IDESC, (kb > kb0 || k) ? 1u : 0u);
+          for (int j = 0; j < SK; ++j) {
+            if (SK > 1 && kb + j >= kb1) break;
+            const uint64_t da = umma_desc_sw128(s0 + j * KB_BYTES), db = umma_desc_sw128(s0 + j * KB_BYTES + A_BYTES);
+#pragma unroll
+            for (int k = 0; k < GEMM_BK / 16; ++k) {
+              const uint32_t acc = (kb > kb0 || j || k) ? 1u : 0u;
+              if (CG == 2) ptx::tc_mma_bf16_pair(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), IDESC, acc);
+              else ptx::tc_mma_bf16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), IDESC, acc);
+            }
           }
           if (CG == 2) ptx::tc_commit_pair(empty_bar(stage)); else ptx::tc_commit(empty_bar(stage));
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
