@@ -122,6 +122,11 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
   return p != 0;
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -154,6 +159,11 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster_addr) : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar_cluster_addr) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar_cluster_addr) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols) : "memory");
@@ -295,10 +305,13 @@ struct GemmArgs {
   const int* t;
   int C, koff, H, Tsteps;
   int lda;              // row pitch of A in elements (CUDA-core GEMM; the tensor-core one has it in its tensor map)
-  // Kernel-5 convolution over a zero-padded channels-last tensor [rows, conv_c] (0: plain GEMM): logical A row m
-  // is the 5 conv_c elements starting at tensor row m, so k-block kb is tensor rows m + tap, columns
-  // [c0, c0 + 64) with tap = (64 kb) / conv_c, c0 = (64 kb) % conv_c; conv_c is a multiple of 64.
-  int conv_c;
+  // Convolution over a zero-padded channels-last tensor [n, conv_l + 4, conv_c] (conv_c = 0: plain GEMM): logical A row
+  // n conv_l + l is the K contiguous elements starting at padded position l + conv_off of candidate n (kernel 5: K = 5 conv_c,
+  // conv_off = 0; pointwise: K = conv_c, conv_off = 2).  A's tensor map is three-dimensional (channel, position,
+  // candidate) with boxes of 64 channels x conv_l positions x tile_rows / conv_l candidates, so k-block kb is the box
+  // at channel (64 kb) % conv_c, position conv_off + (64 kb) / conv_c; the padding rows cost nothing.
+  int conv_c, conv_l, conv_off;
+  int tile_rows;        // rows of an output tile: 128, or the largest multiple of conv_l that is not larger
   // Rows that really exist when the forward runs on a compacted candidate list: min(M, *live.n * live.mul + live.add)
   // (live.n null: M).  The tensor maps keep their full extent; tiles beyond the live rows are simply not visited.
   LiveRows live;
@@ -309,13 +322,14 @@ struct GemmArgs {
   // `status`, drains and returns; every other CTA finishes its tiles as usual.
   int withhold_first_stage;
   int causal;           // EPI_ATTN: causal mask of the fused 16-token self-attention
-  // Split reduction (narrow tiles with the plain-store epilogue, EPI_F32 only; 0 or 1: off): the k-blocks of every
+  // Split reduction (EPI_F32 only; 0 or 1: off): the k-blocks of every
   // tile are cut into `ksplit` contiguous parts, each a work unit of its own whose partial sums go to the buffer
   // out + part * split_stride (elements); the bias goes into part 0.  The consumer adds the parts in a fixed order,
   // so the result does not depend on which CTA ran which part.  For deep reductions over few rows (the convolutions
   // of a small batch), where the tiles alone occupy a fraction of the SMs.
   int ksplit;
   long long split_stride;
+  int split_rows;       // split_stride in rows of the output (tiles that leave through TMA): a multiple of tile_rows
 };
 
 __device__ __forceinline__ const float* gate_row(const GemmArgs& g, int row) {
@@ -428,8 +442,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   const long long wlim = g.wait_cycles > 0 ? g.wait_cycles : GEMM_WAIT_CYCLES;
   pdl_wait();      // operands, bias, the output and the live-row count belong to earlier kernels of the stream
   const int M = live_rows(g.live, g.M);
-  const int tiles_m = (M + GEMM_BM * CG - 1) / (GEMM_BM * CG);     // tiles of 128 CG rows
-  const int S = g.ksplit > 1 ? g.ksplit : 1;                       // parts of the reduction (plain-store epilogue only)
+  const int TR = g.tile_rows;
+  const int tiles_m = (M + TR * CG - 1) / (TR * CG);               // tiles of TR CG rows
+  const int S = g.ksplit > 1 ? g.ksplit : 1;                       // parts of the reduction
   const int n_tiles = tiles_m * tiles_n * S;                       // work units: (tile, part), part fastest
   const int tile0 = blockIdx.x / CG, tile_step = gridDim.x / CG;      // both CTAs of a pair walk the same tiles
   // an epilogue warp hands accumulator buffer `as` back: the barrier that the MMA warp waits on lives in the leader
@@ -441,10 +456,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   if (warp == 0) {
     if (ptx::elect_one()) {
       int stage = 0; uint32_t phase = 0;
+      const int a_missing = A_BYTES - TR * GEMM_BK * 2;          // rows of a k-block that no load fills (never stored)
       for (int unit = tile0; unit < n_tiles && ok; unit += tile_step) {
         const int tile = unit / S, part = unit - tile * S;
         const int tm = (tile / tiles_n) * CG + (int)rank, tn = tile % tiles_n;
         const int kb0 = part * kblocks / S, kb1 = (part + 1) * kblocks / S;
+        // convolution: position and channel of the next box, candidate of the tile
+        int ctap = g.conv_c ? kb0 * GEMM_BK / g.conv_c : 0, cx = kb0 * GEMM_BK - ctap * g.conv_c;
+        const int cz = g.conv_c ? tm * (TR / g.conv_l) : 0;
         for (int kb = kb0; kb < kb1; kb += SK) {
           if (!ptx::mbar_wait_thread(empty_bar(stage), phase ^ 1u, wlim)) { ok = false; break; }
           if (!(g.withhold_first_stage && blockIdx.x == 0 && unit == 0 && kb == 0)) {
@@ -452,24 +471,26 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const int nk = SK == 1 ? 1 : min(SK, kb1 - kb);
             if (CG == 2) {
               // the leader's barrier counts the bytes of both CTAs' loads of this stage
-              if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), STAGE_BYTES * 2);
+              if (rank == 0) ptx::mbar_expect_tx(full_bar(stage), (STAGE_BYTES - a_missing) * 2);
             } else {
-              ptx::mbar_expect_tx(full_bar(stage), nk * KB_BYTES);
+              ptx::mbar_expect_tx(full_bar(stage), nk * (KB_BYTES - a_missing));
             }
 #pragma unroll
             for (int j = 0; j < SK; ++j) {
               if (j < nk) {
                 const uint32_t sa = s0 + j * KB_BYTES;
                 const int kcol = (kb + j) * GEMM_BK;
-                const int ax = g.conv_c ? kcol % g.conv_c : kcol, ay = tm * GEMM_BM + (g.conv_c ? kcol / g.conv_c : 0);
                 if (CG == 2) {
                   const uint32_t fb = ptx::mapa_rank(full_bar(stage), 0);
-                  ptx::tma_load_2d_pair(sa, &tmA, ax, ay, fb);
+                  if (g.conv_c) ptx::tma_load_3d_pair(sa, &tmA, cx, ctap + g.conv_off, cz, fb);
+                  else ptx::tma_load_2d_pair(sa, &tmA, kcol, tm * GEMM_BM, fb);
                   ptx::tma_load_2d_pair(sa + A_BYTES, &tmB, kcol, tn * BN + (int)rank * B_ROWS, fb);
                 } else {
-                  ptx::tma_load_2d(sa, &tmA, ax, ay, full_bar(stage));
+                  if (g.conv_c) ptx::tma_load_3d(sa, &tmA, cx, ctap + g.conv_off, cz, full_bar(stage));
+                  else ptx::tma_load_2d(sa, &tmA, kcol, tm * GEMM_BM, full_bar(stage));
                   ptx::tma_load_2d(sa + A_BYTES, &tmB, kcol, tn * BN, full_bar(stage));
                 }
+                if (g.conv_c && (cx += GEMM_BK) == g.conv_c) { cx = 0; ++ctap; }
               }
             }
           }
@@ -611,14 +632,14 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       float* sb = sbias + half * 128;
       const bool bias_lane = g.bias != nullptr && r < COLS;
       float bias_next = 0.f;
-      if (bias_lane && tile0 < n_tiles) bias_next = __ldg(g.bias + (tile0 % tiles_n) * BN + half * COLS + r);
-      constexpr int NPART = COLS / 32;       // 32-column parts of this half
-      for (int tile = tile0; tile < n_tiles; tile += tile_step, ++it) {
+      if (bias_lane && tile0 < n_tiles) bias_next = __ldg(g.bias + ((tile0 / S) % tiles_n) * BN + half * COLS + r);
+      for (int unit = tile0; unit < n_tiles; unit += tile_step, ++it) {
+        const int tile = unit / S, kpart = unit - tile * S;
         const int tm = (tile / tiles_n) * CG + (int)rank, tn = tile % tiles_n;
         const int as = it & 1; const uint32_t aphase = (it >> 1) & 1;
         if (bias_lane) {         // the previous tile's reads of `sb` lie before its last staging barrier
           sb[r] = bias_next;
-          if (tile + tile_step < n_tiles) bias_next = __ldg(g.bias + ((tile + tile_step) % tiles_n) * BN + half * COLS + r);
+          if (unit + tile_step < n_tiles) bias_next = __ldg(g.bias + (((unit + tile_step) / S) % tiles_n) * BN + half * COLS + r);
         }
         // the row's gate values of the first part, in flight while the accumulator is awaited
         float4 gq[8];
@@ -658,7 +679,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             float2 f2[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) f2[i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-            if (g.bias) {
+            if (g.bias && kpart == 0) {
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
                 const float4 bb = reinterpret_cast<const float4*>(sb + col_t)[i];
@@ -706,7 +727,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
           ptx::fence_async_smem();
           ptx::named_bar_sync(bar_id, 128);
           if (issuer) {
-            const int x = tn * BN + half * COLS + ch * CW, y = tm * GEMM_BM;
+            const int x = tn * BN + half * COLS + ch * CW, y = kpart * g.split_rows + tm * TR;
             if (EPI == EPI_RESID || EPI == EPI_GATE) ptx::tma_reduce_add_2d(&tmC, x, y, stg);
             else ptx::tma_store_2d(&tmC, x, y, stg);
             ptx::bulk_commit();
@@ -729,7 +750,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
         if (!ptx::mbar_wait_warp(tfull_bar(as), aphase, wlim)) { ok = false; break; }
         ptx::tc_fence_after();
-        const int row = tm * GEMM_BM + quad * 32 + lane;
+        const int row = quad * 32 + lane < TR ? tm * TR + quad * 32 + lane : M;      // rows past the tile are nobody's
         const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(as * ACC + half * COLS);
 #pragma unroll
         for (int c = 0; c < COLS; c += 16) {

@@ -23,7 +23,9 @@ gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ W, GemmA
   for (int k0 = 0; k0 < g.K; k0 += 16) {
     for (int i = threadIdx.x; i < 64 * 16; i += 256) {
       const int r = i >> 4, k = i & 15;
-      As[k][r] = (m0 + r < g.M && k0 + k < g.K) ? A[(size_t)(m0 + r) * g.lda + k0 + k] : 0.f;
+      const int row = m0 + r;
+      const size_t arow = g.conv_c ? (size_t)(row / g.conv_l) * (g.conv_l + 4) + row % g.conv_l + g.conv_off : row;
+      As[k][r] = (row < g.M && k0 + k < g.K) ? A[arow * g.lda + k0 + k] : 0.f;
       Ws[k][r] = (n0 + r < g.N && k0 + k < g.K) ? W[(size_t)(n0 + r) * g.K + k0 + k] : 0.f;
     }
     __syncthreads();

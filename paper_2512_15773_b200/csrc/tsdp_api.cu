@@ -76,7 +76,7 @@ struct Net {
   float *bh = nullptr, *gh = nullptr, *beh = nullptr;
   // UNET activations (zero-padded channels-last tensors, see unet_kernels.cuh), allocated at init
   struct UWs { void *X0 = nullptr, *E = nullptr, *M1 = nullptr, *M2 = nullptr, *HB = nullptr;
-               void *TMP[4] = {}, *D[4] = {}, *CAT[4] = {}, *P[4] = {}, *U1[4] = {}, *U2[4] = {};
+               void *TMP[4] = {}, *D[4] = {}, *CAT[4] = {}, *P[4] = {}, *U1[4] = {}, *U2 = nullptr;
                float *Y = nullptr, *R = nullptr; size_t Y_cap = 0; } uw;
   std::vector<void*> allocs;
 };
@@ -116,7 +116,7 @@ struct tsdp_ctx {
   // graphs and tensor maps
   struct GraphRec { cudaGraphExec_t exec; int launches; };
   std::map<std::tuple<int, int>, GraphRec> graphs;
-  std::map<std::tuple<const void*, int, int, int, int, int, int>, CUtensorMap> maps;
+  std::map<std::tuple<const void*, int, int, int, int, int, int, int>, CUtensorMap> maps;
   std::map<void*, size_t> guards;             // device buffer -> its size: the guard bytes sit right behind it
   EncodeTiledFn encode = nullptr;
   cudaStream_t cap_stream = nullptr;
@@ -343,7 +343,7 @@ size_t sched_weights_count(const tsdp_config_t& cfg) {
 // `ld` elements apart; esz = 2 (bf16) or 4 (fp32).  The box is box_cols x box_rows (box_cols * esz = 128).
 int get_map(tsdp_ctx* c, const void* ptr, int esz, int rows, int cols, int ld, int box_cols, int box_rows,
             CUtensorMap* out) {
-  auto key = std::make_tuple(ptr, esz, rows, cols, ld, box_cols, box_rows);
+  auto key = std::make_tuple(ptr, esz, rows, cols, ld, box_cols, box_rows, 0);
   auto it = c->maps.find(key);
   if (it != c->maps.end()) { *out = it->second; return TSDP_OK; }
   CUtensorMap m;
@@ -363,6 +363,28 @@ int get_map(tsdp_ctx* c, const void* ptr, int esz, int rows, int cols, int ld, i
   return TSDP_OK;
 }
 
+// The A operand of a convolution: a bf16 tensor [n, positions, C] as boxes of 64 channels x L positions x nb candidates.
+int get_map_conv(tsdp_ctx* c, const void* ptr, int n, int positions, int C, int L, int nb, CUtensorMap* out) {
+  auto key = std::make_tuple(ptr, 2, n, C, positions, L, nb, 3);
+  auto it = c->maps.find(key);
+  if (it != c->maps.end()) { *out = it->second; return TSDP_OK; }
+  CUtensorMap m;
+  cuuint64_t gdim[3] = {(cuuint64_t)C, (cuuint64_t)positions, (cuuint64_t)n};
+  cuuint64_t gstr[2] = {(cuuint64_t)C * 2, (cuuint64_t)positions * C * 2};
+  cuuint32_t box[3] = {(cuuint32_t)GEMM_BK, (cuuint32_t)L, (cuuint32_t)nb};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = c->encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), gdim, gstr, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    c->last_error = "cuTensorMapEncodeTiled failed with code " + std::to_string((int)r);
+    return TSDP_ERR_CUDA;
+  }
+  c->maps[key] = m;
+  *out = m;
+  return TSDP_OK;
+}
+
 // Rows a GEMM of the forward being enqueued really processes, as far as the host knows (profiling mode reads the
 // round's plan back); otherwise the dense count.
 int gemm_rows_known(const tsdp_ctx* c, const GemmArgs& g) {
@@ -371,10 +393,17 @@ int gemm_rows_known(const tsdp_ctx* c, const GemmArgs& g) {
   return v < 0 ? 0 : (v < g.M ? v : g.M);
 }
 
+GemmArgs gemm_args(tsdp_ctx* c, int M, int N, int K, const float* bias, void* out, int ldo) {
+  GemmArgs g{};
+  g.M = M; g.N = N; g.K = K; g.bias = bias; g.out = out; g.ldo = ldo; g.status = c->status;
+  g.C = 1; g.H = 1; g.Tsteps = 1; g.lda = K; g.conv_l = 1; g.tile_rows = GEMM_BM;
+  return g;
+}
+
 template <int BN, int EPI>
 int launch_tc(tsdp_ctx* c, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const GemmArgs& g,
               cudaStream_t s) {
-  const int tiles = ((g.M + GEMM_BM - 1) / GEMM_BM) * (g.N / BN) * (g.ksplit > 1 ? g.ksplit : 1);
+  const int tiles = ((g.M + g.tile_rows - 1) / g.tile_rows) * (g.N / BN) * (g.ksplit > 1 ? g.ksplit : 1);
   const int grid = tiles < c->num_sms ? tiles : c->num_sms;
   prof_begin(c, s, c->prof_gemm_cat, 2.0 * gemm_rows_known(c, g) * g.N * g.K);
   TSDP_LAUNCH(c, (gemm_tcgen05_kernel<BN, EPI>), grid, GEMM_THREADS, gemm_smem_bytes(BN), s, ma, mb, mc, g);
@@ -388,7 +417,7 @@ int launch_tc(tsdp_ctx* c, const CUtensorMap& ma, const CUtensorMap& mb, const C
 template <int EPI>
 int launch_tc_pair(tsdp_ctx* c, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const GemmArgs& g,
                    cudaStream_t s) {
-  const int tiles = ((g.M + 2 * GEMM_BM - 1) / (2 * GEMM_BM)) * (g.N / 256);
+  const int tiles = ((g.M + 2 * g.tile_rows - 1) / (2 * g.tile_rows)) * (g.N / 256);
   const int pairs = tiles < c->pair_clusters ? tiles : c->pair_clusters;
   prof_begin(c, s, c->prof_gemm_cat, 2.0 * gemm_rows_known(c, g) * g.N * g.K);
   launch_kernel_cluster(c, gemm_tcgen05_kernel<256, EPI, 2>, dim3(2 * pairs), dim3(GEMM_THREADS), (size_t)gemm_smem_bytes_cg(256, 2), s, 2,
@@ -461,21 +490,38 @@ int pick_bn(int M, int N, int num_sms) {
   return 0;
 }
 
-// Parts into which the reduction of a convolution GEMM [M x N x K] -> fp32 is split (1: not at all).  With a small batch
-// the deep levels of the UNet are a handful of narrow tiles (16 - 32 CTAs) that each walk 80 - 160 k-blocks one after the
-// other: cutting the k range puts those k-blocks on otherwise idle SMs, each part writes its partial sums to a buffer
-// of its own and the GroupNorm kernel that consumes them adds the parts in order (same bits whatever ran where; a
-// function of the launch shape only).  Parts of at least 4 k-blocks, at most 8 parts, no more units than SMs, and
-// only where the tiles use the plain-store epilogue (widths below 128).
-int conv_ksplit(const tsdp_ctx* c, int M, int N, int K, size_t cap_elems) {
-  if (c->no_ksplit || c->cfg.precision == 0 || M <= 0 || K % GEMM_BK != 0 || N % 32 != 0) return 1;
-  if (c->force_bn == 0 && use_pair_gemm(c, M, N, K)) return 1;
-  const int BN = (c->force_bn > 0 && N % c->force_bn == 0) ? c->force_bn : pick_bn(M, N, c->num_sms);
-  if (gemm_tma_epilogue(BN)) return 1;
-  const int tiles = ((M + GEMM_BM - 1) / GEMM_BM) * (N / BN), kblocks = K / GEMM_BK;
-  int S = 1;
-  while (S < 8 && tiles * S * 2 <= c->num_sms && kblocks / (S * 2) >= 4 && (size_t)(S * 2) * (size_t)(M + 4) * (size_t)N <= cap_elems) S *= 2;
-  return S;
+// A convolution run as a GEMM (see GemmArgs): channels and positions of the padded tensor it reads, offset of its first
+// tap, and how it is cut up: tile width (0: chosen as for a plain GEMM) and parts of the reduction.
+struct ConvSpec { int c, L, off, bn, ksplit; };
+int conv_tile_rows(int L) { return GEMM_BM / L * L; }
+// Rows of one partial-sum buffer of a split reduction: whole tiles, so that a tile leaving through TMA stays inside.
+int conv_split_rows(int M, int L) { const int tr = conv_tile_rows(L); return (M + tr - 1) / tr * tr; }
+
+// Tile width and number of parts of the reduction for a convolution [M x N x K] -> fp32.  The levels of the UNet give few
+// tiles with long reductions (20 - 120 k-blocks), so wide tiles leave most SMs idle and narrow ones read their operands
+// many times; cutting the k range of wider tiles uses the idle SMs instead.  Each part writes a buffer of its own and the
+// GroupNorm kernel that consumes them adds the parts in order (the same bits whatever ran where; a function of
+// the launch shape only).  The choice is the cheapest by measured figures: start and epilogue of a launch, time per
+// k-block (both by tile width), and 8 bytes more per value and part for the partial sums.
+ConvSpec conv_plan(const tsdp_ctx* c, int n_cand, int cch, int L, int off, int N, int taps, size_t cap_elems, bool may_split) {
+  ConvSpec best{cch, L, off, 0, 1};
+  if (c->cfg.precision == 0 || c->force_bn > 0) return best;
+  const int M = n_cand * L, K = taps * cch, kb = K / GEMM_BK, rows = conv_split_rows(M, L), tm = rows / conv_tile_rows(L);
+  if (use_pair_gemm(c, M, N, K)) return best;
+  const int bns[4] = {256, 128, 64, 32};
+  const double start_us[4] = {6.0, 4.4, 3.6, 3.3}, kb_us[4] = {0.30, 0.19, 0.145, 0.135};
+  double best_us = 1e30;
+  for (int i = 0; i < 4; ++i) {
+    if (N % bns[i] != 0) continue;
+    const int tiles = tm * (N / bns[i]);
+    for (int S = 1; S <= 8; ++S) {
+      if (S > 1 && (!may_split || c->no_ksplit || kb / S < 4 || tiles * S > c->num_sms || (size_t)S * rows * N > cap_elems)) break;
+      const int waves = (tiles * S + c->num_sms - 1) / c->num_sms;
+      const double us = start_us[i] + waves * ((kb + S - 1) / S) * kb_us[i] + (S - 1) * 8.0 * M * N / 4.0e6;
+      if (us < best_us) { best_us = us; best.bn = bns[i]; best.ksplit = S; }
+    }
+  }
+  return best;
 }
 
 // Gate of an adaptive-LayerNorm residual (EPI_GATE): gate vectors and the row -> timestep map.
@@ -484,10 +530,10 @@ struct GateSpec {
 };
 
 int gemm(tsdp_ctx* c, const void* A, const void* W, const float* bias, int M, int N, int K, int epi, void* out,
-         int ldo, cudaStream_t s, const GateSpec* gs = nullptr, int conv_c = 0, int ksplit = 1, long long split_stride = 0) {
+         int ldo, cudaStream_t s, const GateSpec* gs = nullptr, const ConvSpec* cv = nullptr) {
   if (M <= 0) return TSDP_OK;
-  GemmArgs g{M, N, K, bias, out, ldo, c->status, nullptr, 0, nullptr, 1, 0, 1, 1, conv_c > 0 ? conv_c : K, conv_c,
-             LiveRows{nullptr, 0, 0}, nullptr, 0, 0, 0};
+  GemmArgs g = gemm_args(c, M, N, K, bias, out, ldo);
+  if (cv) { g.lda = g.conv_c = cv->c; g.conv_l = cv->L; g.conv_off = cv->off; g.tile_rows = conv_tile_rows(cv->L); }
   if (c->dbg_armed && c->dbg_in_test_gemm && c->cfg.precision == 1) {      // one launch: see tsdp_debug_arm_gemm_timeout
     g.wait_cycles = c->dbg_wait_cycles;
     g.withhold_first_stage = 1;
@@ -499,10 +545,9 @@ int gemm(tsdp_ctx* c, const void* A, const void* W, const float* bias, int M, in
     g.Tsteps = gs->Tsteps; g.list = gs->cm->list;
   }
   if (c->live_n != nullptr && c->live_static > 0) {
-    // rows per candidate of this GEMM: M = n rows_per (token rows), or n rows_per - 4 (a convolution over padded tensors)
+    // rows per candidate of this GEMM: M = n rows_per
     const int n = c->live_static;
     if (M % n == 0) g.live = LiveRows{c->live_n, M / n, 0};
-    else if ((M + 4) % n == 0) g.live = LiveRows{c->live_n, (M + 4) / n, -4};
   }
   if (c->cfg.precision == 0) {
     dim3 grid((N + 63) / 64, (M + 63) / 64);
@@ -524,17 +569,18 @@ int gemm(tsdp_ctx* c, const void* A, const void* W, const float* bias, int M, in
     c->last_error = "tensor-core GEMM needs K % 64 == 0 and N % 32 == 0";
     return TSDP_ERR_ARG;
   }
-  const bool pair = c->force_bn == 0 && use_pair_gemm(c, M, N, K);
-  const int BN = pair ? 256 : ((c->force_bn > 0 && N % c->force_bn == 0) ? c->force_bn : pick_bn(M, N, c->num_sms));
-  if (ksplit > 1) {      // see conv_ksplit: narrow tiles with the plain-store epilogue only
-    if (pair || gemm_tma_epilogue(BN) || epi != EPI_F32 || ksplit > K / GEMM_BK) return TSDP_ERR_ARG;
-    g.ksplit = ksplit; g.split_stride = split_stride;
+  const int want_bn = cv ? cv->bn : 0;
+  const bool pair = c->force_bn == 0 && want_bn == 0 && use_pair_gemm(c, M, N, K);
+  const int BN = pair ? 256 : (want_bn > 0 ? want_bn : ((c->force_bn > 0 && N % c->force_bn == 0) ? c->force_bn : pick_bn(M, N, c->num_sms)));
+  if (cv && cv->ksplit > 1) {      // see conv_plan
+    if (pair || epi != EPI_F32 || cv->ksplit > K / GEMM_BK) return TSDP_ERR_ARG;
+    g.ksplit = cv->ksplit; g.split_rows = conv_split_rows(M, cv->L); g.split_stride = (long long)g.split_rows * ldo;
   }
   CUtensorMap ma, mb, mc;
   int r;
-  if (conv_c > 0) {      // kernel-5 convolution: A is the padded tensor [M + 4, conv_c] itself
-    if (conv_c % GEMM_BK != 0 || K != 5 * conv_c) return TSDP_ERR_ARG;
-    if ((r = get_map(c, A, 2, M + 4, conv_c, conv_c, GEMM_BK, GEMM_BM, &ma)) != TSDP_OK) return r;
+  if (cv) {
+    if (cv->c % GEMM_BK != 0 || K % cv->c != 0 || M % cv->L != 0) return TSDP_ERR_ARG;
+    if ((r = get_map_conv(c, A, M / cv->L, cv->L + 4, cv->c, cv->L, g.tile_rows / cv->L, &ma)) != TSDP_OK) return r;
   } else if ((r = get_map(c, A, 2, M, K, K, GEMM_BK, GEMM_BM, &ma)) != TSDP_OK) return r;
   if ((r = get_map(c, W, 2, N, K, K, GEMM_BK, pair ? BN / 2 : BN, &mb)) != TSDP_OK) return r;
   mc = ma;
@@ -544,7 +590,7 @@ int gemm(tsdp_ctx* c, const void* A, const void* W, const float* bias, int M, in
       c->last_error = "GEMM output must be 16-byte aligned with a row pitch that is a multiple of 16 bytes";
       return TSDP_ERR_ARG;
     }
-    if ((r = get_map(c, out, esz, M, N, ldo, 128 / esz, GEMM_BM, &mc)) != TSDP_OK) return r;
+    if ((r = get_map(c, out, esz, g.ksplit > 1 ? g.ksplit * g.split_rows : M, N, ldo, 128 / esz, g.tile_rows, &mc)) != TSDP_OK) return r;
   }
   if (pair) return launch_tc_pair_epi(c, ma, mb, mc, g, epi, s);
   switch (BN) {
@@ -558,7 +604,7 @@ int gemm(tsdp_ctx* c, const void* A, const void* W, const float* bias, int M, in
 // fp32 CUDA-core GEMM whatever the precision mode: the timestep-conditioning tables built at weight load.
 int gemm_f32(tsdp_ctx* c, const float* A, const float* W, const float* bias, int M, int N, int K, int epi, float* out,
              cudaStream_t s) {
-  GemmArgs g{M, N, K, bias, out, N, c->status, nullptr, 0, nullptr, 1, 0, 1, 1, K, 0, LiveRows{nullptr, 0, 0}, nullptr, 0, 0, 0};
+  const GemmArgs g = gemm_args(c, M, N, K, bias, out, N);
   dim3 grid((N + 63) / 64, (M + 63) / 64);
   if (epi == EPI_MISH) TSDP_LAUNCH(c, (gemm_simt_kernel<EPI_MISH>), grid, 256, 0, s, A, W, g);
   else if (epi == EPI_SILU) TSDP_LAUNCH(c, (gemm_simt_kernel<EPI_SILU>), grid, 256, 0, s, A, W, g);
@@ -689,7 +735,8 @@ bool fused_attn_ok(const tsdp_config_t& cfg, const tsdp_net_t& net) {
 // the GEMM's epilogue.  M is a multiple of 16 (whole candidates).
 int gemm_qkv_attn(tsdp_ctx* c, const void* A, const XfmrLayer& w, int M, int d, void* out, cudaStream_t s) {
   const int N = 3 * d, K = d, BN = GEMM_ATTN_BN;
-  GemmArgs g{M, N, K, w.bqkv_hm, out, d, c->status, nullptr, 0, nullptr, 1, 0, 1, 1, K, 0, LiveRows{nullptr, 0, 0}, nullptr, 0, 0, 1};
+  GemmArgs g = gemm_args(c, M, N, K, w.bqkv_hm, out, d);
+  g.causal = 1;
   if (c->live_n != nullptr && c->live_static > 0 && M % c->live_static == 0) g.live = LiveRows{c->live_n, M / c->live_static, 0};
   CUtensorMap ma, mb;
   int r;
@@ -991,98 +1038,106 @@ int dit_prepare_ctx_t(tsdp_ctx* c, Net& n, int B, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------------------------------ conv UNet
+// Where a GroupNorm's result goes (see GnArgs).
+struct GnOut { void* dst; int pitch, coff; void* up; int up_pitch; void* pool; };
 template <typename T>
 int unet_gn(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, const float* gam, const float* bet, int foff, const T* res_t,
-            int res_pitch, const float* res_f, T* dst, int dst_pitch, int coff, int L, int C, cudaStream_t s, int n_split = 1,
-            long long split_stride = 0) {
+            int res_pitch, const float* res_f, const GnOut& o, int L, int C, cudaStream_t s, const ConvSpec& cv) {
+  GnArgs g{};
+  g.Y = n.uw.Y; g.n_split = cv.ksplit; g.split_stride = (long long)conv_split_rows(n_cand * L, L) * C;
+  g.gam = gam; g.bet = bet; g.groups = n.cfg.heads;
+  if (foff >= 0) { g.film_time = n.film_time; g.film_obs = n.film_obs; g.F = n.F; g.foff = foff; }
+  g.Tsteps = c->cfg.T;
+  g.res_t = res_t; g.res_pitch = res_pitch; g.res_f = res_f;
+  g.dst = o.dst; g.dst_pitch = o.pitch; g.coff = o.coff; g.up = o.up; g.up_pitch = o.up_pitch; g.pool = o.pool;
+  g.L = L; g.C = C;
+  const int Cg = C / g.groups, items = L * Cg / 4, all = n_cand * g.groups;
   prof_begin(c, s, 1, 0.0);
-  TSDP_LAUNCH(c, (gn_mish_kernel<T>), n_cand * n.cfg.heads, 256, 0, s, n.uw.Y, gam, bet, n.cfg.heads,
-              foff >= 0 ? n.film_time : nullptr, n.film_obs, n.F, foff >= 0 ? foff : 0, cm, c->cfg.T, res_t, res_pitch, res_f, dst,
-              dst_pitch, coff, L, C, n_split, split_stride);
+  // a warp per group while that gives every SM a few, four warps where groups are scarce (or long)
+  if (Cg % 4 != 0 || items > GN_ITEMS * 128) TSDP_LAUNCH(c, (gn_mish_any_kernel<T>), all, 256, 0, s, g, cm, n_cand);
+  else if (items > GN_ITEMS * 32 || all < 4 * c->num_sms) {
+    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 8>), all, 128, 0, s, g, cm, n_cand);
+    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 2>), all, 128, 0, s, g, cm, n_cand);
+  } else {
+    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 8>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
+    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 2>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
+  }
   prof_end(c, s);
   c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
   return TSDP_OK;
 }
 
-// One FiLM residual block: xin [n, L+4, cin] -> dst[n, L+4, coff .. coff+cout) of a tensor of pitch dst_pitch.
+// One FiLM residual block: xin [n, L+4, cin] -> `out`.
 template <typename T>
-int unet_resblock(tsdp_ctx* c, Net& n, const Net::UBlock& b, const CandMap& cm, int n_cand, const T* xin, T* tmp, T* dst,
-                  int dst_pitch, int coff, int L, cudaStream_t s) {
-  const int rows = n_cand * (L + 4);
+int unet_resblock(tsdp_ctx* c, Net& n, const Net::UBlock& b, const CandMap& cm, int n_cand, const T* xin, T* tmp, const GnOut& out,
+                  int L, cudaStream_t s) {
+  const int M = n_cand * L;
   int r;
-  const long long ystr = (long long)rows * b.cout;      // distance of the partial-sum buffers of a split reduction
-  const int s1 = conv_ksplit(c, rows - 4, b.cout, 5 * b.cin, n.uw.Y_cap), s2 = conv_ksplit(c, rows - 4, b.cout, 5 * b.cout, n.uw.Y_cap);
+  const ConvSpec c1 = conv_plan(c, n_cand, b.cin, L, 0, b.cout, 5, n.uw.Y_cap, true), c2 = conv_plan(c, n_cand, b.cout, L, 0, b.cout, 5, n.uw.Y_cap, true);
   const bool fork = b.Wr != nullptr && c->aux_on && !c->prof_on;      // (per-launch timing keeps one stream)
+  auto residual = [&](cudaStream_t st) {
+    const ConvSpec cr = conv_plan(c, n_cand, b.cin, L, 2, b.cout, 1, 0, false);
+    return gemm(c, xin, b.Wr, b.br, M, b.cout, b.cin, EPI_F32, n.uw.R, b.cout, st, nullptr, &cr);
+  };
   if (fork) {      // the residual projection only needs xin: beside the two convolutions, on the second stream
     CU_TRY(c, cudaEventRecord(c->ev_aux_fork, s));
     CU_TRY(c, cudaStreamWaitEvent(c->aux_stream, c->ev_aux_fork, 0));
-    if ((r = gemm(c, xin, b.Wr, b.br, rows, b.cout, b.cin, EPI_F32, n.uw.R, b.cout, c->aux_stream))) return r;
+    if ((r = residual(c->aux_stream))) return r;
     CU_TRY(c, cudaEventRecord(c->ev_aux_join, c->aux_stream));
   }
-  if ((r = gemm(c, xin, b.W1, b.b1, rows - 4, b.cout, 5 * b.cin, EPI_F32, n.uw.Y, b.cout, s, nullptr, b.cin, s1, ystr))) return r;
-  if ((r = unet_gn<T>(c, n, cm, n_cand, b.g1, b.be1, b.foff, nullptr, 0, nullptr, tmp, b.cout, 0, L, b.cout, s, s1, ystr))) return r;
-  if ((r = gemm(c, tmp, b.W2, b.b2, rows - 4, b.cout, 5 * b.cout, EPI_F32, n.uw.Y, b.cout, s, nullptr, b.cout, s2, ystr))) return r;
+  if ((r = gemm(c, xin, b.W1, b.b1, M, b.cout, 5 * b.cin, EPI_F32, n.uw.Y, b.cout, s, nullptr, &c1))) return r;
+  if ((r = unet_gn<T>(c, n, cm, n_cand, b.g1, b.be1, b.foff, nullptr, 0, nullptr, GnOut{tmp, b.cout, 0, nullptr, 0, nullptr}, L, b.cout, s, c1))) return r;
+  if ((r = gemm(c, tmp, b.W2, b.b2, M, b.cout, 5 * b.cout, EPI_F32, n.uw.Y, b.cout, s, nullptr, &c2))) return r;
   if (b.Wr) {
     if (fork) CU_TRY(c, cudaStreamWaitEvent(s, c->ev_aux_join, 0));
-    else if ((r = gemm(c, xin, b.Wr, b.br, rows, b.cout, b.cin, EPI_F32, n.uw.R, b.cout, s))) return r;
-    return unet_gn<T>(c, n, cm, n_cand, b.g2, b.be2, -1, nullptr, 0, n.uw.R, dst, dst_pitch, coff, L, b.cout, s, s2, ystr);
+    else if ((r = residual(s))) return r;
+    return unet_gn<T>(c, n, cm, n_cand, b.g2, b.be2, -1, nullptr, 0, n.uw.R, out, L, b.cout, s, c2);
   }
-  return unet_gn<T>(c, n, cm, n_cand, b.g2, b.be2, -1, xin, b.cin, nullptr, dst, dst_pitch, coff, L, b.cout, s, s2, ystr);
+  return unet_gn<T>(c, n, cm, n_cand, b.g2, b.be2, -1, xin, b.cin, nullptr, out, L, b.cout, s, c2);
 }
 
 template <typename T>
 int unet_forward_t(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, cudaStream_t s) {
   const int H = c->cfg.H, A = c->cfg.A, ch = n.cfg.d, LV = n.cfg.layers, last = LV - 1;
   auto P = [](void* p) { return reinterpret_cast<T*>(p); };
+  auto plain = [](void* p, int C) { return GnOut{p, C, 0, nullptr, 0, nullptr}; };
+  // the last block of a level on the way up: its result, repeated, is the first part of the next finer level's input
+  auto raised = [&](int lv) { return GnOut{nullptr, 0, 0, n.uw.CAT[lv - 1], (ch << lv) + (ch << (lv - 1)), nullptr}; };
   int r, bi = 0;
   prof_begin(c, s, 3, 0.0);
-  TSDP_LAUNCH(c, (unet_embed_kernel<T>), n_cand * H, ch < 256 ? ch : 256, 0, s, cm, n.W_in, n.b_in, P(n.uw.X0), H, A, ch);
+  TSDP_LAUNCH(c, (unet_embed_kernel<T>), n_cand, 256, 0, s, cm, n.W_in, n.b_in, P(n.uw.X0), H, A, ch);
   prof_end(c, s);
   c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
   const T* x = P(n.uw.X0);
   for (int lv = 0; lv < LV; ++lv) {
     const int L = H >> lv, C = ch << lv;
-    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, x, P(n.uw.TMP[lv]), P(n.uw.D[lv]), C, 0, L, s))) return r;
-    if (lv < last) {
-      const int Cup = ch << (lv + 1), Ccat = Cup + C;
-      if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.D[lv]), P(n.uw.TMP[lv]), P(n.uw.CAT[lv]), Ccat, Cup, L, s))) return r;
-      const long long tot = (long long)n_cand * (L / 2) * C;
-      prof_begin(c, s, 3, 0.0);
-      TSDP_LAUNCH(c, (unet_pool_kernel<T>), (unsigned)((tot + 255) / 256), 256, 0, s, P(n.uw.CAT[lv]), Ccat, Cup, P(n.uw.P[lv]),
-                  n_cand, L / 2, C, live_desc(c, 1));
-      prof_end(c, s);
-      c->launches_per_round_tmp++;
-      CU_TRY(c, cudaGetLastError());
+    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, x, P(n.uw.TMP[lv]), plain(n.uw.D[lv], C), L, s))) return r;
+    if (lv < last) {      // kept for the way up behind the channels that come from below, and pooled for the next level
+      const int Cup = ch << (lv + 1);
+      const GnOut o{n.uw.CAT[lv], Cup + C, Cup, nullptr, 0, n.uw.P[lv]};
+      if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.D[lv]), P(n.uw.TMP[lv]), o, L, s))) return r;
       x = P(n.uw.P[lv]);
     } else {
-      if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.D[lv]), P(n.uw.TMP[lv]), P(n.uw.E), C, 0, L, s))) return r;
+      if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.D[lv]), P(n.uw.TMP[lv]), plain(n.uw.E, C), L, s))) return r;
     }
   }
   {
     const int L = H >> last, C = ch << last;
-    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.E), P(n.uw.TMP[last]), P(n.uw.M1), C, 0, L, s))) return r;
-    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.M1), P(n.uw.TMP[last]), P(n.uw.M2), C, 0, L, s))) return r;
+    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.E), P(n.uw.TMP[last]), plain(n.uw.M1, C), L, s))) return r;
+    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.M1), P(n.uw.TMP[last]), last > 0 ? raised(last) : plain(n.uw.M2, C), L, s))) return r;
   }
   const T* cur = P(n.uw.M2);
   for (int lv = last - 1; lv >= 0; --lv) {
-    const int L = H >> lv, C = ch << lv, Cup = ch << (lv + 1), Ccat = Cup + C;
-    const long long tot = (long long)n_cand * L * Cup;
-    prof_begin(c, s, 3, 0.0);
-    TSDP_LAUNCH(c, (unet_upsample_kernel<T>), (unsigned)((tot + 255) / 256), 256, 0, s, cur, P(n.uw.CAT[lv]), Ccat, n_cand, L, Cup, live_desc(c, 1));
-    prof_end(c, s);
-    c->launches_per_round_tmp++;
-    CU_TRY(c, cudaGetLastError());
-    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.CAT[lv]), P(n.uw.TMP[lv]), P(n.uw.U1[lv]), C, 0, L, s))) return r;
-    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.U1[lv]), P(n.uw.TMP[lv]), P(n.uw.U2[lv]), C, 0, L, s))) return r;
-    cur = P(n.uw.U2[lv]);
+    const int L = H >> lv, C = ch << lv;
+    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.CAT[lv]), P(n.uw.TMP[lv]), plain(n.uw.U1[lv], C), L, s))) return r;
+    if ((r = unet_resblock<T>(c, n, n.ub[bi++], cm, n_cand, P(n.uw.U1[lv]), P(n.uw.TMP[lv]), lv > 0 ? raised(lv) : plain(n.uw.U2, C), L, s))) return r;
+    cur = P(n.uw.U2);
   }
-  const int rows = n_cand * (H + 4);
-  const long long ystr = (long long)rows * ch;
-  const int sh = conv_ksplit(c, rows - 4, ch, 5 * ch, n.uw.Y_cap);
-  if ((r = gemm(c, cur, n.Wh, n.bh, rows - 4, ch, 5 * ch, EPI_F32, n.uw.Y, ch, s, nullptr, ch, sh, ystr))) return r;
-  if ((r = unet_gn<T>(c, n, cm, n_cand, n.gh, n.beh, -1, nullptr, 0, nullptr, P(n.uw.HB), ch, 0, H, ch, s, sh, ystr))) return r;
+  const ConvSpec ch5 = conv_plan(c, n_cand, ch, H, 0, ch, 5, n.uw.Y_cap, true);
+  if ((r = gemm(c, cur, n.Wh, n.bh, n_cand * H, ch, 5 * ch, EPI_F32, n.uw.Y, ch, s, nullptr, &ch5))) return r;
+  if ((r = unet_gn<T>(c, n, cm, n_cand, n.gh, n.beh, -1, nullptr, 0, nullptr, plain(n.uw.HB, ch), H, ch, s, ch5))) return r;
   prof_begin(c, s, 3, 0.0);
   TSDP_LAUNCH(c, (unet_head_kernel<T>), (n_cand * H + 7) / 8, 256, 0, s, P(n.uw.HB), n.W_outT, n.b_out, cm, n_cand * H, H, A, ch);
   prof_end(c, s);
@@ -1099,8 +1154,13 @@ int unet_prepare_obs(tsdp_ctx* c, Net& n, int N, cudaStream_t s) {
   TSDP_LAUNCH(c, (mish_kernel), (unsigned)((tot + 255) / 256), 256, 0, s, c->obs, n.obs_m, tot);
   c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
+  const size_t smem = (size_t)UF_N * ((dobs + 3) & ~3) * sizeof(float);
   c->launches_per_round_tmp++;
-  return gemm_f32(c, n.obs_m, n.WfT_obs, nullptr, N, n.F, dobs, EPI_F32, n.film_obs, s);
+  if (smem > UF_MAX_SMEM) return gemm_f32(c, n.obs_m, n.WfT_obs, nullptr, N, n.F, dobs, EPI_F32, n.film_obs, s);
+  TSDP_LAUNCH(c, film_obs_kernel, dim3((n.F + 8 * UF_F - 1) / (8 * UF_F), (N + UF_N - 1) / UF_N), 256, smem, s, n.obs_m, n.WfT_obs,
+              n.film_obs, N, n.F, dobs);
+  CU_TRY(c, cudaGetLastError());
+  return TSDP_OK;
 }
 
 int prepare_obs(tsdp_ctx* c, Net& n, int B, cudaStream_t s) {
@@ -1689,6 +1749,7 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
     fprintf(stderr, "tsdp_init: the persistent cluster drafter does not fit this configuration\n");
     return fail(TSDP_ERR_UNSUPPORTED);
   }
+  INIT_TRY(cudaFuncSetAttribute(film_obs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UF_MAX_SMEM));
   for (const void* fn : {(const void*)mlp_forward_kernel<1>, (const void*)mlp_forward_kernel<4>, (const void*)mlp_rollout_kernel<1>,
                          (const void*)mlp_rollout_kernel<4>})
     INIT_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_MAX_SMEM));
@@ -1715,17 +1776,19 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
     auto pad = [&](void** p, size_t lv, size_t C) { return alloc_bytes(c, c->allocs, p, nc * ((cfg->H >> lv) + 4) * C * esz); };
     int e = 0;
     e |= pad(&n.uw.X0, 0, ch); e |= pad(&n.uw.HB, 0, ch);
-    e |= pad(&n.uw.E, last, ch << last); e |= pad(&n.uw.M1, last, ch << last); e |= pad(&n.uw.M2, last, ch << last);
+    e |= pad(&n.uw.E, last, ch << last); e |= pad(&n.uw.M1, last, ch << last);
+    if (last > 0) e |= pad(&n.uw.U2, 0, ch); else e |= pad(&n.uw.M2, 0, ch);
     for (size_t lv = 0; lv < LV; ++lv) {
       e |= pad(&n.uw.TMP[lv], lv, ch << lv); e |= pad(&n.uw.D[lv], lv, ch << lv);
       if (lv < last) {
         e |= pad(&n.uw.CAT[lv], lv, (ch << (lv + 1)) + (ch << lv)); e |= pad(&n.uw.P[lv], lv + 1, ch << lv);
-        e |= pad(&n.uw.U1[lv], lv, ch << lv); e |= pad(&n.uw.U2[lv], lv, ch << lv);
+        e |= pad(&n.uw.U1[lv], lv, ch << lv);
       }
     }
-    n.uw.Y_cap = 4 * nc * (cfg->H + 4) * (ch << last);      // room for the partial sums of a split reduction (conv_ksplit)
+    // room for the partial sums of a split reduction (conv_plan): at most one tile of 128 x 256 per SM
+    n.uw.Y_cap = std::max(nc * cfg->H * (ch << last), (size_t)c->num_sms * GEMM_BM * 256);
     e |= dev_alloc(c, c->allocs, &n.uw.Y, n.uw.Y_cap);
-    e |= dev_alloc(c, c->allocs, &n.uw.R, nc * (cfg->H + 4) * (ch << last));
+    e |= dev_alloc(c, c->allocs, &n.uw.R, nc * cfg->H * (ch << last));
     if (e) return fail(TSDP_ERR_CUDA);
   }
   INIT_TRY(cudaDeviceSynchronize());
