@@ -81,10 +81,18 @@ __device__ __forceinline__ float posterior_mean(const DdpmTables& S, float x, fl
 // x_{t-1} = mu + sigma xi
 __device__ __forceinline__ float ddpm_sample(float mu, float sigma, float xi) { return __fmaf_rn(sigma, xi, mu); }
 
-// Programmatic dependent launch: a kernel signals early that its successor in the stream may be
-// scheduled, and waits (after whatever set-up touches no shared data) until every kernel it depends on
-// has completed and its memory is visible.  Both are no-ops for a kernel launched without the attribute.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Programmatic dependent launch: a kernel signals that its successor in the stream may be scheduled, and waits (after
+// whatever set-up touches no shared data) until every kernel it depends on has completed and its memory is visible.
+// Both are no-ops for a kernel launched without the attribute.
+// The signal is given only by grids that leave half the chip free.  The successor's blocks are placed when it is given: on a
+// nearly full chip they crowd onto the few free SMs and run two or three to an SM with others idle, which costs more
+// than the launch latency saved.  Measured, signal at the start of every kernel -> this rule: 96 environments vanilla 56.2 ->
+// 53.9 ms, 32 of the UNet workload 25.0 -> 23.0, 24 of the Push-T-shaped one 11.05 -> 10.46 (no signal at all: 53.9,
+// 24.3, 10.65).  The GEMM signals when its last operand loads are issued, the others when they start.
+constexpr unsigned PDL_MAX_GRID = 74;
+__device__ __forceinline__ void pdl_trigger() {
+  if (gridDim.x <= PDL_MAX_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ float warp_sum(float v) {

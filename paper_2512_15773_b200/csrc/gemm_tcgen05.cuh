@@ -122,6 +122,7 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
   return p != 0;
 }
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory"); }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
@@ -404,7 +405,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   static_assert((EPI == EPI_ATTN) == (BN == GEMM_ATTN_BN), "the fused attention epilogue has its own tile width");
 
   extern __shared__ uint8_t smem_raw[];
-  pdl_trigger();
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   constexpr bool TMA_EPI = gemm_tma_epilogue(BN);
   const uint32_t staging = base + STAGES * STAGE_BYTES;    // 1024-byte aligned: every stage is a multiple of 1 KB
@@ -424,6 +424,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   const uint32_t rank = CG == 2 ? ptx::cluster_rank() : 0u;     // 0: the pair's leader
 
   if (threadIdx.x == 0) {
+    ptx::prefetch_map(&tmA); ptx::prefetch_map(&tmB);
+    if (TMA_EPI) ptx::prefetch_map(&tmC);
     for (int s = 0; s < STAGES; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
     for (int s = 0; s < 2; ++s) { ptx::mbar_init(tfull_bar(s), 1); ptx::mbar_init(tempty_bar(s), GEMM_EPI_WARPS * CG); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -498,6 +500,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
     }
+    pdl_trigger();
   } else if (warp == 1) {
     if (rank == 0 && ptx::elect_one()) {      // in a pair only the leader issues
       int stage = 0; uint32_t phase = 0; int it = 0;
