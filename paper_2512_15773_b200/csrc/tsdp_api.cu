@@ -65,6 +65,9 @@ struct Net {
   XfoldLayerW* fold_lw = nullptr;             // [L] device
   __nv_bfloat16 *fold_kq_time = nullptr, *fold_ut_time = nullptr, *fold_kq_obs = nullptr, *fold_ut_obs = nullptr;
   float *fold_c_time = nullptr, *fold_c_obs = nullptr;
+  // XFMR small enough for the cluster kernel: weights in the order its lanes read them, per-CTA parameters (drafter_cluster.cuh)
+  __nv_bfloat16* dc_w = nullptr;
+  float* dc_par = nullptr;
   float* mod = nullptr;                       // DIT: [T, L*6d + 2d] shift / scale / gate vectors of every timestep
   int mod_ld = 0;
   // UNET: residual blocks in execution order, FiLM tables, head
@@ -1259,15 +1262,16 @@ int forward_arch(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, cudaStream_
 }
 
 // ------------------------------------------------------------------------------------------ drafter
+constexpr int DC_SMEM_LIMIT = 227 * 1024;
 // Whether the persistent cluster kernel can run this context's drafter at all (shapes, shared memory).
 bool cluster_drafter_fits(const tsdp_config_t& cfg, const tsdp_net_t& n, int* smem_bytes, bool* resident) {
   if (cfg.precision != 1 || n.arch != TSDP_ARCH_XFMR || (n.d != 128 && n.d != 256) || n.layers > DC_MAX_LAYERS ||
       cfg.H > DC_ROWS || 1 + cfg.obs_tokens > DC_MAX_NK || cfg.H * cfg.A > 256 || (n.d / n.heads) % 4 != 0)
     return false;
-  // weight slices resident in shared memory if they fit beside the activations, otherwise read through the L2
+  // weight slices resident in shared memory if they fit beside the activations, otherwise through a ring of chunks
   for (int res = 1; res >= 0; --res) {
-    const DcSmem pl = dc_smem_plan(n.d, n.layers, cfg.A, res != 0);
-    if (pl.total <= 227 * 1024) { *smem_bytes = pl.total; *resident = res != 0; return true; }
+    const DcSmem pl = dc_smem_plan(n.d, n.layers, cfg.A, res != 0, DC_SMEM_LIMIT);
+    if (pl.total <= DC_SMEM_LIMIT) { *smem_bytes = pl.total; *resident = res != 0; return true; }
   }
   return false;
 }
@@ -1291,14 +1295,7 @@ bool use_cluster_verifier(const tsdp_ctx* c, int B, int K) {
 int launch_cluster_forward(tsdp_ctx* c, int which, int mode, int B, int K, cudaStream_t s) {
   const Net& n = c->net[which];
   DcParams P{};
-  for (int l = 0; l < n.cfg.layers; ++l) {
-    const XfmrLayer& w = n.L[l];
-    DcLayer& o = P.L[l];
-    o.Wqkv = (const __nv_bfloat16*)w.Wqkv; o.Wo = (const __nv_bfloat16*)w.Wo; o.Wq2 = (const __nv_bfloat16*)w.Wq2;
-    o.Wo2 = (const __nv_bfloat16*)w.Wo2; o.W1 = (const __nv_bfloat16*)w.W1; o.W2 = (const __nv_bfloat16*)w.W2;
-    o.bqkv = w.bqkv; o.bo = w.bo; o.bq2 = w.bq2; o.bo2 = w.bo2; o.b1 = w.b1; o.b2 = w.b2;
-    o.ln1_g = w.ln1_g; o.ln1_b = w.ln1_b; o.ln2_g = w.ln2_g; o.ln2_b = w.ln2_b; o.ln3_g = w.ln3_g; o.ln3_b = w.ln3_b;
-  }
+  P.Wf = n.dc_w; P.parf = n.dc_par;
   P.layers = n.cfg.layers; P.heads = n.cfg.heads; P.H = c->cfg.H; P.A = c->cfg.A; P.To = c->cfg.obs_tokens; P.T = c->cfg.T;
   P.W_in = n.W_in; P.b_in = n.b_in; P.pos = n.pos;
   P.lnf_g = n.lnf_g; P.lnf_b = n.lnf_b; P.W_outT = n.W_outT; P.b_out = n.b_out;
@@ -1318,6 +1315,7 @@ int launch_cluster_forward(tsdp_ctx* c, int which, int mode, int B, int K, cudaS
   P.item = c->item;
   const bool verify = mode == 1;
   P.resident = (verify ? c->cv_resident : c->dc_resident) ? 1 : 0;
+  P.n_slots = dc_smem_plan(n.cfg.d, n.cfg.layers, c->cfg.A, P.resident != 0, DC_SMEM_LIMIT).n_slots;
   const int maxc = verify ? c->cv_max_clusters : c->dc_max_clusters, smem = verify ? c->cv_smem : c->dc_smem;
   const int work = verify ? B * (K + 1) : B;
   const int ncl = work < maxc ? work : maxc;
@@ -2220,6 +2218,23 @@ int tsdp_load_weights(tsdp_ctx* c, int which, const float* blob, size_t n) {
       if (st) return TSDP_ERR_CUDA;
       CU_TRY(c, cudaMemcpy(net.fold_lw, lw.data(), sizeof(XfoldLayerW) * L, cudaMemcpyHostToDevice));
       if ((r = xfold_build(c, net, net.kv_time, T, net.fold_kq_time, net.fold_ut_time, net.fold_c_time, 0))) return r;
+    }
+    int smem_unused; bool res_unused;
+    if (cluster_drafter_fits(cfg, net.cfg, &smem_unused, &res_unused)) {
+      const size_t lw = (size_t)DC_CS * dc_layer_bytes((int)d) / 2, lp = (size_t)DC_CS * dc_par_floats((int)d);
+      if (dev_alloc(c, net.allocs, &net.dc_w, L * lw)) return TSDP_ERR_CUDA;
+      if (dev_alloc(c, net.allocs, &net.dc_par, L * lp)) return TSDP_ERR_CUDA;
+      for (size_t l = 0; l < L; ++l) {
+        const XfmrLayer& w = net.L[l];
+        const void* slabs[6] = {w.Wqkv, w.Wo, w.W1, w.W2, w.Wq2, w.Wo2};
+        for (int s = 0; s < 6; ++s) {
+          const long long nel = (long long)dc_slab_rows((int)d, s) * DC_CS * dc_slab_k((int)d, s);
+          dc_pack_kernel<<<(unsigned)((nel + 255) / 256), 256>>>(reinterpret_cast<const __nv_bfloat16*>(slabs[s]), net.dc_w + l * lw, (int)d, s);
+        }
+        const DcParSrc ps{{w.ln1_g, w.ln1_b, w.ln2_g, w.ln2_b, w.ln3_g, w.ln3_b}, {w.bqkv, w.bo, w.bq2, w.bo2, w.b1, w.b2}};
+        dc_pack_par_kernel<<<DC_CS, 256>>>(ps, net.dc_par + l * lp, (int)d);
+      }
+      CU_TRY(c, cudaGetLastError());
     }
     CU_TRY(c, cudaDeviceSynchronize());
     if ((r = check_status(c))) return r;
