@@ -1,31 +1,33 @@
 // Persistent drafter: the whole K-step draft rollout of one environment (Sec. 3.2 "Draft Generation
 // Procedure", Eq. (3)) in ONE kernel launch, for small batches where the rollout is latency-bound.
 //
-// One thread-block cluster of DC_CS CTAs serves one environment at a time.  Every CTA owns a 1/DC_CS
-// slice (a block of output columns) of every weight matrix of the drafter and a full replica of the activations of the
-// 16-token sequence.  A linear layer is computed as Y[:, slice] = X W_slice^T on mma.sync m16n8k16 (the sequence is one
-// 16-row tile), and each CTA writes its slice of Y into the replicas of all CTAs through distributed shared
-// memory (4 such exchanges per block: qkv, attention projection, MLP up, MLP down; 6 when the
-// cross-attention is not folded into the memory tokens).  LayerNorm, the attentions, the folded
-// cross-attention products, the head, the DDPM posterior and the noise are cheap enough to be
-// recomputed by every CTA, which saves their broadcasts.  Reductions are warp shuffles.
+// One thread-block cluster of DC_CS = 8 CTAs serves one environment at a time; the sequence is one 16-row tile of mma.sync
+// m16n8k16.  The work is split so that little has to travel and nothing is computed twice that matters:
+//   * the residual stream belongs to rows: CTA r keeps token rows 2r, 2r + 1 in registers (128 threads a row) and does everything
+//     that is local to a token -- embedding, LayerNorms, the folded cross-attention, output head, scheduler step;
+//   * the weights belong to columns: CTA r computes queries and keys of its head, the d / 8 value columns and the MLP
+//     columns [r d/2, +d/2) for all 16 rows, and the products that follow (attention projection, MLP down) over
+//     just those columns as k: 8 partial sums per output, added by the row's owner in a fixed order.
+// So a block exchanges four times: normalised rows to everyone (1 KB per CTA and peer at d = 256), partial sums to their row
+// owners (2 KB), and the same again for the MLP; queries, keys, values and MLP activations never leave a CTA.
+// An exchange costs about 770 clocks plus 390 per KB (measured); the layout before this one (every activation
+// replicated in every CTA, LayerNorms and the cross-attention recomputed by all) exchanged 2.4 KB four times on average
+// and needed 33 k clocks per d = 256 block.
 //
 // Weights are laid out once, when they are loaded, in the order in which the lanes of a warp consume them (dc_pack_kernel):
 // a lane's operand of two MMAs is one 16-byte word, a warp reads 512 contiguous bytes, and a CTA's slice of a matrix is
 // one contiguous piece.  A producer warp brings the pieces to shared memory by bulk copies: all of them once per launch
 // where a CTA's share of the whole network fits, otherwise in 16 KB chunks through a ring that runs ahead of the
-// computation across layers and forwards (the weights do not depend on it), so that a linear layer never waits for the L2.
-// Each layer's LayerNorm parameters and bias slices travel the same way.  Eight warps compute.
+// computation across layers and forwards (the weights do not depend on it), so that a linear layer rarely waits for the L2.
+// Each layer's LayerNorm parameters and biases and the memory tokens' folded tables travel the same way.  Eight warps compute.
 //
-// A stage's slices travel as 16-byte st.async stores that also count their bytes on an mbarrier of the receiving
-// CTA; a CTA goes on as soon as the bytes of all eight slices have arrived (a bounded mbarrier wait), with no
+// What a stage exchanges travels as 16-byte st.async stores that also count their bytes on an mbarrier of the receiving
+// CTA; a CTA goes on as soon as the bytes of all eight CTAs have arrived (a bounded mbarrier wait), with no
 // release fence and no cluster-wide barrier per stage.  Two mbarriers alternate between consecutive stages: a CTA
-// can run at most one stage ahead of the slowest one (it needs everybody's slice of the previous stage), so the
+// can run at most one stage ahead of the slowest one (it needs everybody's bytes of the previous stage), so the
 // bytes of stage s + 1 never land on the barrier that still counts stage s.  The same reasoning covers the
 // buffers: what a fast CTA writes remotely in stage s + 1 is never what a slower one still reads in stage s.
 // (TSDP_NO_ASYNC_BCAST selects plain distributed-shared-memory stores and one remote arrival per CTA and stage.)
-// Measured: an exchange takes 770 clocks plus 390 per KB of slice; a block of the d = 128 drafter ~16.7 k clocks before this
-// layout, one of a streamed d = 256 network 31 k.
 // All CTAs of a cluster make the same sequence of stages because the control flow depends only on (t[b], k).
 #pragma once
 #include <cooperative_groups.h>
@@ -41,11 +43,12 @@ constexpr int DC_COMPUTE = 256;   // compute threads; one producer warp behind t
 constexpr int DC_THREADS = DC_COMPUTE + 32;
 constexpr int DC_WARPS = DC_COMPUTE / 32;
 constexpr int DC_ROWS = 16;       // one m16 tile: H <= 16
+constexpr int DC_OWN = DC_ROWS / DC_CS;   // token rows a CTA owns
 constexpr int DC_MAX_LAYERS = 8;
 constexpr int DC_MAX_NK = 4;      // memory tokens: time token + at most 3 observation tokens
-constexpr int DC_PU = 40;         // folded cross-attention: row pitch (bf16) of the softmax weights
+constexpr int DC_MAX_NKH = 16;    // folded cross-attention: (memory token, head) pairs
 constexpr int DC_CHUNK = 16384;   // bytes of a ring slot
-constexpr int DC_MIN_SLOTS = 4;   // the four chunks of the widest stage must be resident together
+constexpr int DC_MIN_SLOTS = 4;   // the chunks of one pass over a matrix must be resident together
 constexpr int DC_MAX_SLOTS = 8;
 
 __device__ __forceinline__ uint32_t dc_mapa(uint32_t addr, uint32_t rank) {
@@ -66,52 +69,69 @@ __device__ __forceinline__ void dc_bulk_load(uint32_t dst, const void* src, uint
 }
 __device__ __forceinline__ void dc_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }      // the compute warps
 
-template <int BYTES>
-__device__ __forceinline__ void dc_cp_async(void* smem_dst, const void* gsrc) {
-  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gsrc) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(gsrc) : "memory");
-}
+__device__ __forceinline__ void dc_row_sync(int row) { asm volatile("bar.sync %0, 128;" ::"r"(2 + row) : "memory"); }      // the four warps of an owned row
 
-// ---- weight layout.  A CTA's share of a layer is its slices of the six matrices, one behind the other:
-//   0 qkv [3d/8 x d] | 1 attention projection [d/8 x d] | 2 MLP up [4d/8 x d] | 3 MLP down [d/8 x 4d] | 4 query, 5 output projection
-//   of the cross-attention [d/8 x d] each (last: not needed when it is folded)
-// and a slice [n x K] is [K / KC][n / 8 column tiles][KC / 32][32 lanes] 16-byte words, KC = min(K, 256): the word of lane
+// ---- weight layout.  A CTA's share of a layer, one piece ("slab") behind the other (dh = head width, v = d / 8 columns):
+//   0 [query dh | key dh of its head | its value columns v] x d | 1 attention projection, d x (its v columns, padded to 32) |
+//   2 MLP up d/2 x d | 3 MLP down d x (its d/2 columns) | not needed when the cross-attention is folded: 4 its query dh x d |
+//   5 output projection, d x (its v columns, padded to 32)
+// and a slab [n x K] is [K / KC][n / 8 column tiles][KC / 32][32 lanes] 16-byte words, KC = min(K, 256): the word of lane
 // (g, tg) = (lane / 4, lane % 4) holds W[8 tile + g][k0 + {0, 8, 16, 24} + 2 tg .. + 1], the B operands of two MMAs.
-__host__ __device__ constexpr int dc_slab_rows(int d, int s) { return s == 0 ? 3 * d / DC_CS : (s == 2 ? 4 * d / DC_CS : d / DC_CS); }
-__host__ __device__ constexpr int dc_slab_k(int d, int s) { return s == 3 ? 4 * d : d; }
-__host__ __device__ constexpr int dc_slab_bytes(int d, int s) { return dc_slab_rows(d, s) * dc_slab_k(d, s) * 2; }
-__host__ __device__ constexpr int dc_slab_off(int d, int s) { int o = 0; for (int i = 0; i < s; ++i) o += dc_slab_bytes(d, i); return o; }
-__host__ __device__ constexpr int dc_layer_bytes(int d) { return dc_slab_off(d, 6); }
-// floats of a layer's parameters in a CTA: 6 LayerNorm vectors, this CTA's bias slices, the whole bo2
-__host__ __device__ constexpr int dc_par_floats(int d) { return 7 * d + 11 * d / DC_CS; }
-// element offset of weight (n, k) inside its slice
+__host__ __device__ constexpr int dc_kv(int d) { return d / DC_CS < 32 ? 32 : d / DC_CS; }
+__host__ __device__ constexpr int dc_slab_rows(int d, int dh, int s) {
+  return s == 0 ? 2 * dh + d / DC_CS : (s == 2 ? d / 2 : (s == 4 ? dh : d));
+}
+__host__ __device__ constexpr int dc_slab_k(int d, int s) { return s == 1 || s == 5 ? dc_kv(d) : (s == 3 ? d / 2 : d); }
+__host__ __device__ constexpr int dc_slab_bytes(int d, int dh, int s) { return dc_slab_rows(d, dh, s) * dc_slab_k(d, s) * 2; }
+__host__ __device__ constexpr int dc_slab_off(int d, int dh, int s) { int o = 0; for (int i = 0; i < s; ++i) o += dc_slab_bytes(d, dh, i); return o; }
+__host__ __device__ constexpr int dc_layer_bytes(int d, int dh) { return dc_slab_off(d, dh, 6); }
+// floats of a layer's parameters in a CTA: 6 LayerNorm vectors, bo, bo2, b2 (whole), its biases of slab 0, of slab 2, of slab 4
+__host__ __device__ constexpr int dc_par_floats(int d, int dh) { return 9 * d + 2 * dh + d / DC_CS + d / 2 + dh; }
+// element offset of weight (n, k) inside its slab
 __host__ __device__ inline int dc_frag_index(int n, int k, int rows, int K) {
   const int KC = K < 256 ? K : 256, kc = k / KC, kk = k % KC, tile = n >> 3, g = n & 7, kb = kk >> 5, r = kk & 31;
   const int tg = (r & 7) >> 1;
   return (((kc * (rows >> 3) + tile) * (KC >> 5) + kb) * 32 + (g * 4 + tg)) * 8 + ((r >> 3) << 1) + (r & 1);
 }
-// W [n_out, K] bf16 -> slab `s` of every rank's share of a layer
-__global__ void dc_pack_kernel(const __nv_bfloat16* __restrict__ W, __nv_bfloat16* __restrict__ layer, int d, int s) {
-  const int rows = dc_slab_rows(d, s), K = dc_slab_k(d, s);
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)rows * DC_CS * K) return;
-  const int n = (int)(i / K), k = (int)(i % K), rank = n / rows;
-  layer[(size_t)rank * (dc_layer_bytes(d) / 2) + dc_slab_off(d, s) / 2 + dc_frag_index(n % rows, k, rows, K)] = W[i];
+// where element (n, k) of slab s of CTA `rank` comes from: row and column of the full matrix [out, in]; false: padding
+__host__ __device__ inline bool dc_slab_source(int d, int dh, int rank, int s, int n, int k, int* row, int* col) {
+  const int heads = d / dh, hd = rank * heads / DC_CS, v = d / DC_CS;      // 8 / heads CTAs share a head
+  *row = n; *col = k;
+  if (s == 0) *row = n < dh ? hd * dh + n : (n < 2 * dh ? d + hd * dh + (n - dh) : 2 * d + rank * v + (n - 2 * dh));
+  else if (s == 1 || s == 5) { *col = rank * v + k; return k < v; }
+  else if (s == 2) *row = rank * (d / 2) + n;
+  else if (s == 3) *col = rank * (d / 2) + k;
+  else *row = hd * dh + n;
+  return true;
 }
-struct DcParSrc { const float* ln[6]; const float* bias[6]; };      // ln1 g, b, ln2 g, b, ln3 g, b; bqkv, bo, bq2, bo2, b1, b2
-__global__ void dc_pack_par_kernel(DcParSrc src, float* __restrict__ layer, int d) {
-  const int PL = dc_par_floats(d), rank = blockIdx.x;
-  const int ns[6] = {3 * d / DC_CS, d / DC_CS, d / DC_CS, d / DC_CS, 4 * d / DC_CS, d / DC_CS};
-  float* o = layer + (size_t)rank * PL;
-  for (int j = 0; j < 6; ++j)
-    for (int i = threadIdx.x; i < d; i += blockDim.x) o[j * d + i] = src.ln[j][i];
-  int off = 6 * d;
-  for (int j = 0; j < 6; ++j) {
-    for (int i = threadIdx.x; i < ns[j]; i += blockDim.x) o[off + i] = src.bias[j][rank * ns[j] + i];
-    off += ns[j];
+// W [out, in] bf16 of row pitch ld -> slab `s` of every CTA's share of a layer
+__global__ void dc_pack_kernel(const __nv_bfloat16* __restrict__ W, int ld, __nv_bfloat16* __restrict__ layer, int d, int dh, int s) {
+  const int rows = dc_slab_rows(d, dh, s), K = dc_slab_k(d, s);
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)rows * K * DC_CS) return;
+  const int rank = (int)(i / ((long long)rows * K)), n = (int)(i / K % rows), k = (int)(i % K);
+  int row, col;
+  const bool real = dc_slab_source(d, dh, rank, s, n, k, &row, &col);
+  layer[(size_t)rank * (dc_layer_bytes(d, dh) / 2) + dc_slab_off(d, dh, s) / 2 + dc_frag_index(n, k, rows, K)] =
+      real ? W[(size_t)row * ld + col] : __float2bfloat16_rn(0.f);
+}
+struct DcParSrc { const float* whole[9]; const float *bqkv, *b1, *bq2; };      // ln1 g, b, ln2 g, b, ln3 g, b, bo, bo2, b2
+__global__ void dc_pack_par_kernel(DcParSrc src, float* __restrict__ layer, int d, int dh) {
+  const int rank = blockIdx.x;
+  float* o = layer + (size_t)rank * dc_par_floats(d, dh);
+  for (int j = 0; j < 9; ++j, o += d)
+    for (int i = threadIdx.x; i < d; i += blockDim.x) o[i] = src.whole[j][i];
+  const int slabs[3] = {0, 2, 4};
+  const float* bias[3] = {src.bqkv, src.b1, src.bq2};
+  for (int j = 0; j < 3; ++j) {
+    const int n = dc_slab_rows(d, dh, slabs[j]);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      int row, col;
+      dc_slab_source(d, dh, rank, slabs[j], i, 0, &row, &col);
+      o[i] = bias[j][row];
+    }
+    o += n;
   }
-  for (int i = threadIdx.x; i < d; i += blockDim.x) o[off + i] = src.bias[3][i];
 }
 
 struct DcParams {
@@ -143,222 +163,53 @@ struct DcParams {
   int B, K;
 };
 
-// Shared-memory plan of one CTA (bytes), for model width d.
+// Shared-memory plan of one CTA (bytes), for model width d and head width dh.
 struct DcSmem {
   int n_slots;      // ring slots (0: resident)
-  int off_w, off_par, off_h, off_a, off_qkv, off_q2, off_f, off_kv, off_x, off_head, off_bar, total;
+  int off_w, off_par, off_xa, off_q, off_o, off_f, off_recv, off_kq, off_u, off_x, off_xr, off_red, off_head, off_bar, total;
 };
-__host__ __device__ inline int dc_hpitch(int d) { return d + 8; }      // fp32 words per row of the stream (no bank conflicts between rows)
-__host__ __device__ inline DcSmem dc_smem_plan(int d, int layers, int A, bool resident, int limit) {
+__host__ __device__ inline DcSmem dc_smem_plan(int d, int dh, int layers, int A, bool resident, int limit) {
   DcSmem p{};
   int o = 0;
   auto take = [&](int bytes) { int r = o; o += (bytes + 127) & ~127; return r; };
-  p.off_h = take(DC_ROWS * dc_hpitch(d) * 4);
-  p.off_a = take(DC_ROWS * (d + 8) * 2);
-  // (between a block's attention and the next block also: partial sums of split reductions, one 16 x 8 fp32 tile per warp;
-  // partial scores [8][16][16] and softmax weights of the folded cross-attention)
-  p.off_qkv = take(DC_ROWS * (3 * d + 8) * 2);
-  p.off_q2 = take(DC_ROWS * (d + 8) * 2);
-  p.off_f = take(DC_ROWS * (4 * d + 8) * 2);
-  p.off_kv = take(8 * (d + 8) * 4);                 // folded: u rows [8][d + 8] words; otherwise keys / values [4][2d] fp32 of the block
-  p.off_x = take(DC_ROWS * ((A + 3) & ~3) * 4 * 2); // latent and eps, rows padded to 16 bytes
+  p.off_xa = take(DC_ROWS * (d + 8) * 2);                        // normalised rows of everyone
+  p.off_q = take(DC_ROWS * (2 * dh + d / DC_CS + 8) * 2);        // queries, keys of the head, value columns (all 16 rows)
+  p.off_o = take(DC_ROWS * (dc_kv(d) + 8) * 2);                  // attention output, this CTA's columns
+  p.off_f = take(DC_ROWS * (d / 2 + 8) * 2);                     // MLP activations, this CTA's columns
+  p.off_recv = take(DC_CS * DC_OWN * d * 4);                     // partial sums of the owned rows
+  p.off_kq = take(DC_MAX_NKH * d * 2);                           // folded cross-attention: kq rows; otherwise keys, values of the head
+  p.off_u = take(DC_MAX_NKH / 2 * d * 4);                        // u rows (head pairs in one word)
+  p.off_x = take(DC_OWN * ((A + 3) & ~3) * 4 * 2);               // latent and eps of the owned rows
+  p.off_xr = take(DC_OWN * d * 4);                               // an owned row's normalised values, fp32
+  p.off_red = take(512);                                         // row statistics [2][2][4] (mean, M2), scores [2][16]
   p.off_head = take((2 * d + A * d + 64) * 4);
-  p.off_par = take((resident ? layers : 2) * dc_par_floats(d) * 4);
+  p.off_par = take((resident ? layers : 2) * dc_par_floats(d, dh) * 4);
   p.off_bar = take(256);
   p.off_w = o;
-  if (resident) { p.total = o + layers * dc_layer_bytes(d); return p; }
-  int n = (limit - o) / DC_CHUNK;
+  if (resident) { p.total = o + layers * dc_layer_bytes(d, dh); return p; }
+  const int n = (limit - o) / DC_CHUNK;
   p.n_slots = n > DC_MAX_SLOTS ? DC_MAX_SLOTS : n;
   p.total = p.n_slots >= DC_MIN_SLOTS ? o + p.n_slots * DC_CHUNK : limit + 1;
   return p;
 }
 
-// LayerNorm of the 16 replicated rows: each half-warp normalises one row (warp w: rows 2w and 2w + 1), so
-// the 16 rows go through in one pass; fp32 in, bf16 out.
-__device__ __forceinline__ float half_warp_sum(float v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-template <int D_MODEL, bool AFFINE = true>
-__device__ __forceinline__ void dc_layernorm(const float* h, const float* gam, const float* bet,
-                                             __nv_bfloat16* out, int pitch) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = 2 * warp + (lane >> 4), l16 = lane & 15;
-  constexpr int V = D_MODEL / 64;          // float4 per lane
-  float4 v[V], gg[V], bb[V];
-  float s = 0.f;
-#pragma unroll
-  for (int j = 0; j < V; ++j) {
-    v[j] = *reinterpret_cast<const float4*>(h + row * dc_hpitch(D_MODEL) + (j * 16 + l16) * 4);
-    s += v[j].x + v[j].y + v[j].z + v[j].w;
-  }
-  if (AFFINE) {
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-      gg[j] = *reinterpret_cast<const float4*>(gam + (j * 16 + l16) * 4);
-      bb[j] = *reinterpret_cast<const float4*>(bet + (j * 16 + l16) * 4);
-    }
-  }
-  const float mean = half_warp_sum(s) / D_MODEL;
-  float q = 0.f;
-#pragma unroll
-  for (int j = 0; j < V; ++j) {
-    v[j].x -= mean; v[j].y -= mean; v[j].z -= mean; v[j].w -= mean;
-    q += v[j].x * v[j].x + v[j].y * v[j].y + v[j].z * v[j].z + v[j].w * v[j].w;
-  }
-  const float rstd = rsqrtf(half_warp_sum(q) / D_MODEL + 1e-5f);
-#pragma unroll
-  for (int j = 0; j < V; ++j) {
-    const int c = (j * 16 + l16) * 4;
-    if (AFFINE)
-      store4(out + row * pitch + c, v[j].x * rstd * gg[j].x + bb[j].x, v[j].y * rstd * gg[j].y + bb[j].y,
-             v[j].z * rstd * gg[j].z + bb[j].z, v[j].w * rstd * gg[j].w + bb[j].w);
-    else
-      store4(out + row * pitch + c, v[j].x * rstd, v[j].y * rstd, v[j].z * rstd, v[j].w * rstd);
-  }
-}
-
-// Attention of the replicated sequence, recomputed by every CTA: four lanes own one (head, query row),
-// each a quarter of the head width.  SELF: causal over the H tokens in qkv; otherwise over NK memory
-// tokens whose keys/values are the fp32 rows kv[kx] = [K (d) | V (d)].
-template <int D_MODEL, bool SELF>
-__device__ __forceinline__ void dc_attention(const __nv_bfloat16* qsrc, int pq, const __nv_bfloat16* qkv, int pqkv,
-                                             const float* kv, int NK, __nv_bfloat16* out, int po, int heads, int H) {
-  const int dh = D_MODEL / heads, seg = dh >> 2;
-  const int sub = threadIdx.x & 3;
-  const float scale = rsqrtf((float)dh);
-  for (int p = threadIdx.x >> 2; p < heads * DC_ROWS; p += DC_COMPUTE / 4) {
-    const int head = p / DC_ROWS, row = p % DC_ROWS;
-    const int c0 = head * dh + sub * seg;
-    constexpr int NKEY = SELF ? DC_ROWS : DC_MAX_NK;
-    float sc[NKEY];
-    float m = -INFINITY;
-#pragma unroll
-    for (int j = 0; j < NKEY; ++j) {
-      float a = 0.f;
-      if (SELF) {
-        for (int i = 0; i < seg; ++i)
-          a += __bfloat162float(qsrc[row * pq + c0 + i]) * __bfloat162float(qkv[j * pqkv + D_MODEL + c0 + i]);
-      } else if (j < NK) {
-        for (int i = 0; i < seg; ++i) a += __bfloat162float(qsrc[row * pq + c0 + i]) * kv[j * 2 * D_MODEL + c0 + i];
-      }
-      a += __shfl_xor_sync(0xffffffffu, a, 1);
-      a += __shfl_xor_sync(0xffffffffu, a, 2);
-      const bool vis = SELF ? (j <= row && j < H) : (j < NK);
-      sc[j] = vis ? a * scale : -INFINITY;
-      m = fmaxf(m, sc[j]);
-    }
-    if (m == -INFINITY) m = 0.f;            // padding rows see nothing; keep them finite
-    float l = 0.f;
-#pragma unroll
-    for (int j = 0; j < NKEY; ++j) { sc[j] = __expf(sc[j] - m); l += sc[j]; }
-    const float inv = l > 0.f ? 1.0f / l : 0.f;
-    for (int i = 0; i < seg; ++i) {
-      float o = 0.f;
-#pragma unroll
-      for (int j = 0; j < NKEY; ++j) {
-        if (SELF) o += sc[j] * __bfloat162float(qkv[j * pqkv + 2 * D_MODEL + c0 + i]);
-        else if (j < NK) o += sc[j] * kv[j * 2 * D_MODEL + D_MODEL + c0 + i];
-      }
-      out[row * po + c0 + i] = __float2bfloat16_rn(o * inv);
-    }
-  }
-}
-
-// Causal self-attention of the replicated 16-token sequence on mma.sync, operands through ldmatrix from the qkv replica.
-// With at most four heads two warps share one: both compute its scores, each half of its output columns.
-template <int D_MODEL, int DH>
-__device__ __forceinline__ void dc_self_attn_mma(const __nv_bfloat16* qkv, int pqkv, __nv_bfloat16* out, int po, int heads, int H) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, tg = lane & 3;
-  constexpr int KS = DH / 16;
-  const float scale = rsqrtf((float)DH);
-  const int parts = heads * 2 <= DC_WARPS ? 2 : 1;
-  for (int u = warp; u < heads * parts; u += DC_WARPS) {
-    const int hd = u / parts, part = u - hd * parts;
-    const __nv_bfloat16* qb = qkv + hd * DH;
-    const __nv_bfloat16* kb = qb + D_MODEL;
-    const __nv_bfloat16* vb = kb + D_MODEL;
-    float s[2][4];
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      uint32_t a[4], b[4];
-      ldmatrix_x4(a, qb + (lane & 15) * pqkv + ks * 16 + 8 * (lane >> 4));
-      ldmatrix_x4(b, kb + ((lane & 7) + 8 * (lane >> 4)) * pqkv + ks * 16 + 8 * ((lane >> 3) & 1));
-      mma_bf16_16816(s[0], a, b[0], b[1]);
-      mma_bf16_16816(s[1], a, b[2], b[3]);
-    }
-    const int r0 = g, r1 = g + 8;
-    float m0 = -INFINITY, m1 = -INFINITY;
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int col = nt * 8 + 2 * tg;
-      s[nt][0] = (col <= r0 && col < H) ? s[nt][0] * scale : -INFINITY;
-      s[nt][1] = (col + 1 <= r0 && col + 1 < H) ? s[nt][1] * scale : -INFINITY;
-      s[nt][2] = (col <= r1 && col < H) ? s[nt][2] * scale : -INFINITY;
-      s[nt][3] = (col + 1 <= r1 && col + 1 < H) ? s[nt][3] * scale : -INFINITY;
-      m0 = fmaxf(m0, fmaxf(s[nt][0], s[nt][1]));
-      m1 = fmaxf(m1, fmaxf(s[nt][2], s[nt][3]));
-    }
-    m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 1)); m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 1));
-    m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 2)); m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 2));
-    if (m0 == -INFINITY) m0 = 0.f;
-    if (m1 == -INFINITY) m1 = 0.f;
-    float l0 = 0.f, l1 = 0.f;
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      s[nt][0] = __expf(s[nt][0] - m0); s[nt][1] = __expf(s[nt][1] - m0);
-      s[nt][2] = __expf(s[nt][2] - m1); s[nt][3] = __expf(s[nt][3] - m1);
-      l0 += s[nt][0] + s[nt][1]; l1 += s[nt][2] + s[nt][3];
-    }
-    l0 += __shfl_xor_sync(0xffffffffu, l0, 1); l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-    l0 += __shfl_xor_sync(0xffffffffu, l0, 2); l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-    const float inv0 = l0 > 0.f ? 1.0f / l0 : 0.f, inv1 = l1 > 0.f ? 1.0f / l1 : 0.f;
-    uint32_t pa[4];
-    pa[0] = pack_bf16x2(s[0][0], s[0][1]); pa[1] = pack_bf16x2(s[0][2], s[0][3]);
-    pa[2] = pack_bf16x2(s[1][0], s[1][1]); pa[3] = pack_bf16x2(s[1][2], s[1][3]);
-    const int c_end = (part + 1) * (DH / parts);
-    for (int c0 = part * (DH / parts); c0 < c_end; c0 += 16) {
-      float o0[4] = {0.f, 0.f, 0.f, 0.f}, o1[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t b[4];
-      ldmatrix_x4_trans(b, vb + ((lane & 7) + 8 * ((lane >> 3) & 1)) * pqkv + c0 + 8 * (lane >> 4));
-      mma_bf16_16816(o0, pa, b[0], b[1]);
-      mma_bf16_16816(o1, pa, b[2], b[3]);
-      const int oc = hd * DH + c0 + 2 * tg;
-      *reinterpret_cast<uint32_t*>(out + r0 * po + oc) = pack_bf16x2(o0[0] * inv0, o0[1] * inv0);
-      *reinterpret_cast<uint32_t*>(out + r1 * po + oc) = pack_bf16x2(o0[2] * inv1, o0[3] * inv1);
-      *reinterpret_cast<uint32_t*>(out + r0 * po + oc + 8) = pack_bf16x2(o1[0] * inv0, o1[1] * inv0);
-      *reinterpret_cast<uint32_t*>(out + r1 * po + oc + 8) = pack_bf16x2(o1[2] * inv1, o1[3] * inv1);
-    }
-  }
-}
-
-__host__ __device__ constexpr int dc_ksplit(int KD, int n_tiles) {
-  int ksplit = 1;
-  while (n_tiles * ksplit * 2 <= DC_WARPS && (KD / 32) % (ksplit * 2) == 0) ksplit *= 2;     // parts of whole 32-k blocks
-  return ksplit;
-}
-// One warp's k loop of a linear layer: c[t] = X[16, k32 blocks kb0 .. +NKB) * (column tile nt[t])^T, two accumulator chains per
+// One warp's k loop of a linear layer: c[t] = X[16, k32 blocks 0 .. NKB) * (column tile nt[t])^T, two accumulator chains per
 // tile.  `frag(tile, kb)` is the address of the tile's 512-byte piece for one block of 32 k.
 template <int TPW, int NKB, typename Frag>
-__device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, int kb0, const int (&nt)[TPW], float (&c)[TPW][4], Frag frag) {
+__device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, const int (&nt)[TPW], float (&c)[TPW][4], Frag frag) {
   const int lane = threadIdx.x & 31;
   float e[TPW][4];
 #pragma unroll
   for (int t = 0; t < TPW; ++t) { c[t][0] = c[t][1] = c[t][2] = c[t][3] = 0.f; e[t][0] = e[t][1] = e[t][2] = e[t][3] = 0.f; }
   const __nv_bfloat16* xa = X + (lane & 15) * px + 8 * (lane >> 4);
-#pragma unroll 8
-  for (int i = 0; i < NKB; ++i) {
-    const int kb = kb0 + i;
+#pragma unroll
+  for (int kb = 0; kb < NKB; ++kb) {
     uint32_t a1[4], a2[4];
     ldmatrix_x4(a1, xa + kb * 32);
     ldmatrix_x4(a2, xa + kb * 32 + 16);
 #pragma unroll
     for (int t = 0; t < TPW; ++t) {
-      const uint4 w = *reinterpret_cast<const uint4*>(frag(nt[t], kb) + lane * 16);
+      const uint4 w = *reinterpret_cast<const uint4*>(frag(t, nt[t], kb) + lane * 16);
       mma_bf16_16816(c[t], a1, w.x, w.y);
       mma_bf16_16816(e[t], a2, w.z, w.w);
     }
@@ -367,7 +218,7 @@ __device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, int kb0
   for (int t = 0; t < TPW; ++t) { c[t][0] += e[t][0]; c[t][1] += e[t][1]; c[t][2] += e[t][2]; c[t][3] += e[t][3]; }
 }
 
-template <int D_MODEL>
+template <int D_MODEL, int DH>
 __global__ void __cluster_dims__(DC_CS, 1, 1) __launch_bounds__(DC_THREADS, 1)
 drafter_cluster_kernel(const __grid_constant__ DcParams P) {
   extern __shared__ __align__(128) uint8_t dc_smem[];
@@ -375,33 +226,37 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int cid = blockIdx.x / DC_CS, ncl = gridDim.x / DC_CS;
-  constexpr int d = D_MODEL;
-  constexpr int HP = d + 8, PA = d + 8, PQKV = 3 * d + 8, PF = 4 * d + 8;
-  constexpr int NS_D = d / DC_CS, NS_3D = 3 * d / DC_CS, NS_4D = 4 * d / DC_CS;   // slice widths
-  constexpr int PL = dc_par_floats(d);
+  constexpr int d = D_MODEL, V2 = d / 128;                       // columns of an owned row per thread
+  constexpr int VW = d / DC_CS, NQ = 2 * DH + VW;                // value columns of this CTA; columns of slab 0
+  constexpr int PX = d + 8, PQ = NQ + 8, PO = dc_kv(d) + 8, PF = d / 2 + 8;
+  constexpr int PL = dc_par_floats(d, DH), HEADS = d / DH;
   const bool resident = P.resident != 0, use_async = P.async_bcast != 0;
-  const DcSmem pl = dc_smem_plan(d, P.layers, P.A, resident, DC_CHUNK * 1024);      // (offsets only: the number of slots is the host's)
+  const DcSmem pl = dc_smem_plan(d, DH, P.layers, P.A, resident, DC_CHUNK * 1024);      // (offsets only: the number of slots is the host's)
   const int n_slots = P.n_slots;
-  float* h = reinterpret_cast<float*>(dc_smem + pl.off_h);
-  __nv_bfloat16* a = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_a);
-  __nv_bfloat16* qkv = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_qkv);
-  __nv_bfloat16* q2 = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_q2);
-  __nv_bfloat16* f = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_f);
-  float* red = reinterpret_cast<float*>(qkv);
-  const int H = P.H, A = P.A, AP = (A + 3) & ~3, D = H * A, L = P.layers, NK = 1 + P.To;
-  float* sx = reinterpret_cast<float*>(dc_smem + pl.off_x);          // [16][AP]
-  float* seps = sx + DC_ROWS * AP;                                   // [16][AP]
+  __nv_bfloat16* xa = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_xa);
+  __nv_bfloat16* qs = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_q);
+  __nv_bfloat16* os = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_o);
+  __nv_bfloat16* fs = reinterpret_cast<__nv_bfloat16*>(dc_smem + pl.off_f);
+  float* recv = reinterpret_cast<float*>(dc_smem + pl.off_recv);
+  const __nv_bfloat16* skq = reinterpret_cast<const __nv_bfloat16*>(dc_smem + pl.off_kq);
+  const uint32_t* su = reinterpret_cast<const uint32_t*>(dc_smem + pl.off_u);
+  const int H = P.H, A = P.A, AP = (A + 3) & ~3, D = H * A, L = P.layers, NK = 1 + P.To, NKH = NK * HEADS;
+  float* sx = reinterpret_cast<float*>(dc_smem + pl.off_x);          // [2][AP]
+  float* seps = sx + DC_OWN * AP;                                    // [2][AP]
+  float* sxr = reinterpret_cast<float*>(dc_smem + pl.off_xr);        // [2][d]
+  float2* sstat = reinterpret_cast<float2*>(dc_smem + pl.off_red);   // [2 uses][2 rows][4 warps]
+  float* sscore = reinterpret_cast<float*>(dc_smem + pl.off_red + 128);   // [2][16]
   float* shead = reinterpret_cast<float*>(dc_smem + pl.off_head);
   float* spar = reinterpret_cast<float*>(dc_smem + pl.off_par);
   const uint32_t sbase = ptx::smem_u32(dc_smem), bar0 = sbase + pl.off_bar, ring = sbase + pl.off_w;
-  // barriers: stage hand-over 0, 1 | resident weights 2 | parameters full 3, 4, empty 5, 6 | ring full 8 .., empty 16 ..
+  // barriers: stage hand-over 0, 1 | resident weights 2 | parameters full 3, 4, empty 5, 6 | tables full 7, empty 24 |
+  // ring full 8 .., empty 16 ..
   auto bar_of = [&](int i) { return bar0 + 8u * (uint32_t)i; };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) ptx::mbar_init(bar_of(i), use_async ? 1 : DC_CS);
-    ptx::mbar_init(bar_of(2), 1);
-    for (int i = 3; i < 5; ++i) ptx::mbar_init(bar_of(i), 1);
-    for (int i = 5; i < 7; ++i) ptx::mbar_init(bar_of(i), DC_WARPS);
+    for (int i : {2, 3, 4, 7}) ptx::mbar_init(bar_of(i), 1);
+    for (int i : {5, 6, 24}) ptx::mbar_init(bar_of(i), DC_WARPS);
     for (int i = 0; i < DC_MAX_SLOTS; ++i) { ptx::mbar_init(bar_of(8 + i), 1); ptx::mbar_init(bar_of(16 + i), DC_WARPS); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -412,19 +267,19 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
     if (!ptx::mbar_wait_thread(bar, parity)) { failed = true; atomicExch(P.status, 5); }
   };
   const int n_slabs = P.fold ? 4 : 6;
-  constexpr int order[6] = {0, 1, 4, 5, 2, 3};                       // the order in which a block uses its slabs
   int chunks_layer = 0;
+#pragma unroll
   for (int s = 0; s < 6; ++s)
-    if (s < 4 || n_slabs == 6) chunks_layer += (dc_slab_bytes(d, s) + DC_CHUNK - 1) / DC_CHUNK;
+    if (s < 4 || n_slabs == 6) chunks_layer += (dc_slab_bytes(d, DH, s) + DC_CHUNK - 1) / DC_CHUNK;
 
   // ---- once per launch (compute warps): head parameters; zeroed activations
   if (warp < DC_WARPS) {
     for (int i = threadIdx.x; i < d; i += DC_COMPUTE) { shead[i] = P.lnf_g[i]; shead[d + i] = P.lnf_b[i]; }
     for (int i = threadIdx.x; i < A * d; i += DC_COMPUTE) shead[2 * d + i] = P.W_outT[i];
     for (int i = threadIdx.x; i < A; i += DC_COMPUTE) shead[2 * d + A * d + i] = P.b_out[i];
-    uint32_t* z = reinterpret_cast<uint32_t*>(dc_smem);              // h, a, qkv, q2, f: one behind the other
-    for (int i = threadIdx.x; i < pl.off_kv / 4; i += DC_COMPUTE) z[i] = 0u;
-    for (int i = threadIdx.x; i < 2 * DC_ROWS * AP; i += DC_COMPUTE) sx[i] = 0.f;
+    uint32_t* z = reinterpret_cast<uint32_t*>(dc_smem);              // xa, q, o, f: one behind the other
+    for (int i = threadIdx.x; i < pl.off_recv / 4; i += DC_COMPUTE) z[i] = 0u;
+    for (int i = threadIdx.x; i < 2 * DC_OWN * AP; i += DC_COMPUTE) sx[i] = 0.f;
   }
   cluster.sync();
   const float *lnf_g = shead, *lnf_b = shead + d, *woutT = shead + 2 * d, *bout = shead + 2 * d + A * d;
@@ -437,67 +292,87 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
   auto live_cand = [&](int w) { const int tb = P.t[w / P.C]; return tb >= 0 && w % P.C <= tb; };
 
   if (warp == DC_WARPS) {
-    // ================================================================ producer: weights and parameters, ahead of the computation
+    // ================================================================ producer: weights, parameters, tables, ahead of the computation
     if (ptx::elect_one()) {
-      auto wsrc = [&](int l) { return reinterpret_cast<const uint8_t*>(P.Wf) + ((size_t)l * DC_CS + rank) * dc_layer_bytes(d); };
+      auto wsrc = [&](int l) { return reinterpret_cast<const uint8_t*>(P.Wf) + ((size_t)l * DC_CS + rank) * dc_layer_bytes(d, DH); };
       auto psrc = [&](int l) { return P.parf + ((size_t)l * DC_CS + rank) * PL; };
+      int slot = 0, pre_chunks = 0;
+      uint32_t round = 0, n_layer = 0;          // rounds through the ring; layers whose parameters have been asked for
+      auto par_load = [&](int l) {
+        const uint32_t n = n_layer++, b = n & 1u;
+        if (n >= 2) wait_bar(bar_of(5 + (int)b), ((n >> 1) - 1u) & 1u);
+        if (failed) return;
+        ptx::mbar_expect_tx(bar_of(3 + (int)b), PL * 4u);
+        dc_bulk_load(sbase + pl.off_par + b * PL * 4u, psrc(l), PL * 4u, bar_of(3 + (int)b));
+      };
+      auto chunk_load = [&](const uint8_t* src, int bytes) {
+        if (round > 0) wait_bar(bar_of(16 + slot), (round - 1) & 1u);
+        if (failed) return;
+        ptx::mbar_expect_tx(bar_of(8 + slot), (uint32_t)bytes);
+        dc_bulk_load(ring + (uint32_t)slot * DC_CHUNK, src, (uint32_t)bytes, bar_of(8 + slot));
+        if (++slot == n_slots) { slot = 0; ++round; }
+      };
+      auto layer_load = [&](int l, int skip, int most) {      // chunks skip .. of layer l, at most `most` of them, in the order of use
+        int at = 0;
+        const uint8_t* src = wsrc(l);
+        constexpr int order[6] = {0, 1, 4, 5, 2, 3};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          const int s = order[i];
+          if (s >= 4 && n_slabs == 4) continue;
+          for (int o = 0; o < dc_slab_bytes(d, DH, s); o += DC_CHUNK, ++at)
+            if (at >= skip && at < skip + most) chunk_load(src + dc_slab_off(d, DH, s) + o, min(DC_CHUNK, dc_slab_bytes(d, DH, s) - o));
+        }
+      };
       if (resident) {
-        const uint32_t wb = (uint32_t)(P.fold ? dc_slab_off(d, 4) : dc_layer_bytes(d));
+        const uint32_t wb = (uint32_t)(P.fold ? dc_slab_off(d, DH, 4) : dc_layer_bytes(d, DH));
         ptx::mbar_expect_tx(bar_of(2), (uint32_t)L * (wb + PL * 4u));
         for (int l = 0; l < L; ++l) {
-          dc_bulk_load(ring + (uint32_t)l * dc_layer_bytes(d), wsrc(l), wb, bar_of(2));
+          dc_bulk_load(ring + (uint32_t)(l * dc_layer_bytes(d, DH)), wsrc(l), wb, bar_of(2));
           dc_bulk_load(sbase + pl.off_par + (uint32_t)l * PL * 4u, psrc(l), PL * 4u, bar_of(2));
         }
-        pdl_wait();
-      } else {
-        // chunk by chunk in the order of use; the first layer's chunks are on their way before the predecessor has finished
-        int slot = 0, pre_chunks = 0;
-        uint32_t round = 0;
-        auto par_load = [&](int l, uint32_t n) {       // n: layers before this one
-          if (n >= 2) wait_bar(bar_of(5 + (int)(n & 1u)), ((n >> 1) - 1u) & 1u);
-          if (failed) return;
-          ptx::mbar_expect_tx(bar_of(3 + (int)(n & 1u)), PL * 4u);
-          dc_bulk_load(sbase + pl.off_par + (n & 1u) * PL * 4u, psrc(l), PL * 4u, bar_of(3 + (int)(n & 1u)));
-        };
-        auto chunk_load = [&](const uint8_t* src, int bytes) {
-          if (round > 0) wait_bar(bar_of(16 + slot), (round - 1) & 1u);
-          if (failed) return;
-          ptx::mbar_expect_tx(bar_of(8 + slot), (uint32_t)bytes);
-          dc_bulk_load(ring + (uint32_t)slot * DC_CHUNK, src, (uint32_t)bytes, bar_of(8 + slot));
-          if (++slot == n_slots) { slot = 0; ++round; }
-        };
-        uint32_t n_layer = 1;                     // layers whose parameters have been asked for
-        auto layer_load = [&](int l, int skip, int most) {      // chunks skip .. of layer l, at most `most` of them
-          int at = 0;
-          const uint8_t* src = wsrc(l);
-#pragma unroll
-          for (int i = 0; i < 6; ++i) {
-            const int s = order[i];
-            if (s >= 4 && n_slabs == 4) continue;
-            for (int o = 0; o < dc_slab_bytes(d, s); o += DC_CHUNK, ++at) {
-              if (at < skip || at >= skip + most) continue;
-              chunk_load(src + dc_slab_off(d, s) + o, min(DC_CHUNK, dc_slab_bytes(d, s) - o));
-            }
-          }
-        };
-        par_load(0, 0);
+      } else {      // the first layer's pieces are on their way before the predecessor has finished
+        par_load(0);
         pre_chunks = min(n_slots, chunks_layer);
         layer_load(0, 0, pre_chunks);
-        pdl_wait();
-        long long n_fwd = 0;
-        if (P.mode == 1) { for (int w = cid; w < P.B * P.C; w += ncl) n_fwd += live_cand(w) ? 1 : 0; }
-        else for (int s = cid; s < P.B; s += ncl) n_fwd += window(s);
-        if (n_fwd == 0) {                         // nothing to do: let the copies land
-          wait_bar(bar_of(3), 0);
-          for (int i = 0; i < pre_chunks; ++i) wait_bar(bar_of(8 + i), 0);
-        }
-        for (long long fw = 0; fw < n_fwd && !failed; ++fw)
-          for (int l = 0; l < L && !failed; ++l) {
-            const bool first = fw == 0 && l == 0;
-            if (!first) par_load(l, n_layer++);
-            layer_load(l, first ? pre_chunks : 0, chunks_layer);
-          }
       }
+      pdl_wait();
+      uint32_t n_tab = 0;
+      bool first = true;
+      auto serve = [&](int tau, int env) {      // everything one forward consumes
+        for (int l = 0; l < L && !failed; ++l) {
+          if (!resident && !first) par_load(l);
+          if (P.fold) {
+            if (n_tab > 0) wait_bar(bar_of(24), (n_tab - 1) & 1u);
+            if (failed) return;
+            ++n_tab;
+            const uint32_t tok = (uint32_t)(HEADS * d * 2);      // bytes of a memory token's kq rows, and of its u rows
+            const size_t stride = (size_t)L * HEADS * d, lay = (size_t)l * HEADS * d;
+            ptx::mbar_expect_tx(bar_of(7), 2u * (uint32_t)NK * tok);
+            for (int j = 0; j < NK; ++j) {
+              const size_t at = (j == 0 ? (size_t)tau : (size_t)env * P.To + (j - 1)) * stride + lay;
+              dc_bulk_load(sbase + pl.off_kq + (uint32_t)j * tok, (j == 0 ? P.kq_time : P.kq_obs) + at, tok, bar_of(7));
+              dc_bulk_load(sbase + pl.off_u + (uint32_t)j * tok, (j == 0 ? P.ut_time : P.ut_obs) + at, tok, bar_of(7));
+            }
+          }
+          if (!resident) layer_load(l, first ? pre_chunks : 0, chunks_layer);
+          first = false;
+        }
+      };
+      if (P.mode == 1) {
+        for (int w = cid; w < P.B * P.C && !failed; w += ncl)
+          if (live_cand(w)) serve(P.t[w / P.C] - w % P.C, item_of(P.item, w / P.C));
+      } else {
+        for (int s = cid; s < P.B && !failed; s += ncl) {
+          const int ke = window(s);
+          for (int k = 1; k <= ke && !failed; ++k) serve(P.t[s] - k + 1, item_of(P.item, s));
+        }
+      }
+      if (first && !resident) {                 // nothing to do: let the copies land
+        wait_bar(bar_of(3), 0);
+        for (int i = 0; i < pre_chunks; ++i) wait_bar(bar_of(8 + i), 0);
+      }
+      if (first && resident) wait_bar(bar_of(2), 0);
       if (failed) { const long long t0 = clock64(); while (clock64() - t0 < 400000ll) { } }
     }
     __syncwarp();
@@ -508,42 +383,95 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
   // ================================================================== compute warps
   pdl_wait();      // t, the latents and the obs K/V come from earlier kernels
   const uint64_t seed = *P.seed;
-  const size_t ldkv = (size_t)L * 2 * d;
   const int g = lane >> 2, tg = lane & 3;
+  const int row = threadIdx.x >> 7, ct = threadIdx.x & 127, c0 = ct * V2;      // owned row 0 / 1 of this thread, its columns
   uint32_t stage_no = 0, stage_phase = 0;      // stages so far; bit b = parity this CTA waits for next on barrier b
-  // this thread's four destinations of a broadcast (its partner thread serves the other four): shared::cluster address
-  // of their shared memory
-  uint32_t rb[2][4];
-#pragma unroll
-  for (int hf = 0; hf < 2; ++hf)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) rb[hf][j] = dc_mapa(sbase, (uint32_t)((rank + hf * 4 + j) & 7));
   auto stage_begin = [&](uint32_t bytes) {     // thread 0 announces the bytes this CTA will receive in the stage that begins
-    if (use_async && threadIdx.x == 0) ptx::mbar_expect_tx(bar_of(stage_no & 1u), bytes);
+    if (use_async && threadIdx.x == 0) ptx::mbar_expect_tx(bar_of((int)(stage_no & 1u)), bytes);
   };
-  // 16 bytes to the same shared-memory offset in four CTAs of the cluster (half hf of them)
-  auto bcast16 = [&](uint32_t off, const uint4& v, int hf) {
-    const uint32_t bo = (uint32_t)pl.off_bar + 8u * (stage_no & 1u);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t r = hf ? rb[1][j] : rb[0][j];
-      if (use_async) dc_st_async16(r + off, v, r + bo); else dc_st_cluster16(r + off, v);
-    }
+  // 16 bytes to shared-memory offset `off` of the CTA whose shared memory starts at `r`
+  auto send16 = [&](uint32_t r, uint32_t off, const uint4& v) {
+    if (use_async) dc_st_async16(r + off, v, r + (uint32_t)pl.off_bar + 8u * (stage_no & 1u));
+    else dc_st_cluster16(r + off, v);
   };
-  // every slice of the stage has arrived in this CTA (bounded wait)
+  // everything of the stage has arrived in this CTA (bounded wait)
   auto stage_end = [&]() {
     const uint32_t b = stage_no & 1u;
     if (!use_async) {
       asm volatile("fence.acq_rel.cluster;" ::: "memory");
       dc_sync();
-      if (threadIdx.x < DC_CS) ptx::mbar_arrive_cluster(dc_mapa(bar_of(b), threadIdx.x));
+      if (threadIdx.x < DC_CS) ptx::mbar_arrive_cluster(dc_mapa(bar_of((int)b), threadIdx.x));
     }
-    wait_bar(bar_of(b), (stage_phase >> b) & 1u);
+    wait_bar(bar_of((int)b), (stage_phase >> b) & 1u);
     if (!use_async) asm volatile("fence.acq_rel.cluster;" ::: "memory");
     stage_phase ^= 1u << b;
     ++stage_no;
   };
-  // ---- ring, consumer side: chunk i of the stage that begins sits in slot (cslot + i) % n_slots
+  // ---- all-gather of the owned rows' values (as bf16) into everyone's xa: 8 columns of a row are 8 / V2 neighbouring lanes,
+  // each of which sends the 16 bytes to V2 of the CTAs
+  constexpr int GL = 8 / V2;
+  uint32_t gdst[V2];
+#pragma unroll
+  for (int j = 0; j < V2; ++j) gdst[j] = dc_mapa(sbase, (uint32_t)((lane % GL) * V2 + j));
+  auto gather_rows = [&](const float (&v)[V2]) {
+    const float up = V2 == 1 ? __shfl_down_sync(0xffffffffu, v[0], 1) : v[V2 - 1];
+    const uint32_t w = pack_bf16x2(v[0], up);                          // V2 = 1: even lanes hold a pair
+    uint4 o;
+    uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ow[j] = __shfl_sync(0xffffffffu, w, (lane & ~(GL - 1)) | (j * (GL / 4)));
+    const uint32_t off = (uint32_t)pl.off_xa + (uint32_t)((DC_OWN * rank + row) * PX + (c0 & ~7)) * 2u;
+#pragma unroll
+    for (int j = 0; j < V2; ++j) send16(gdst[j], off, o);
+  };
+  // ---- partial sums of an output tile (8 columns, 16 rows) to the owners of the rows: lanes pair up, the even one sends four
+  // columns of row g, the odd one of row g + 8
+  const uint32_t pdst = dc_mapa(sbase, (uint32_t)((tg & 1) * 4 + (g >> 1)));
+  const uint32_t poff = (uint32_t)pl.off_recv + (uint32_t)((rank * DC_OWN + (g & 1)) * d + 4 * (tg >> 1)) * 4u;
+  auto send_partial = [&](int tile, const float (&c)[4]) {
+    const bool odd = tg & 1;
+    const float r0 = __shfl_xor_sync(0xffffffffu, odd ? c[0] : c[2], 1), r1 = __shfl_xor_sync(0xffffffffu, odd ? c[1] : c[3], 1);
+    const uint4 o = odd ? make_uint4(__float_as_uint(r0), __float_as_uint(r1), __float_as_uint(c[2]), __float_as_uint(c[3]))
+                        : make_uint4(__float_as_uint(c[0]), __float_as_uint(c[1]), __float_as_uint(r0), __float_as_uint(r1));
+    send16(pdst, poff + (uint32_t)tile * 32u, o);
+  };
+  float hv[V2];      // the stream: this thread's columns of its row
+  auto add_partials = [&](const float* bias) {      // stream += sum of the eight parts (in order) + bias
+#pragma unroll
+    for (int j = 0; j < V2; ++j) {
+      float s = 0.f;
+#pragma unroll
+      for (int r = 0; r < DC_CS; ++r) s += recv[(r * DC_OWN + row) * d + c0 + j];
+      hv[j] += s + bias[c0 + j];
+    }
+  };
+  // LayerNorm of the owned rows without the affine part: mean and squared deviations per warp, then combined over the row's four
+  uint32_t n_stat = 0;
+  auto normalise = [&](float (&x)[V2]) {
+    float s = 0.f, q = 0.f;
+#pragma unroll
+    for (int j = 0; j < V2; ++j) s += hv[j];
+    const float mw = warp_sum(s) * (1.0f / (32 * V2));
+#pragma unroll
+    for (int j = 0; j < V2; ++j) { const float e = hv[j] - mw; q += e * e; }
+    q = warp_sum(q);
+    float2* st = sstat + ((n_stat & 1u) * DC_OWN + row) * 4;
+    if (lane == 0) st[warp & 3] = make_float2(mw, q);
+    ++n_stat;
+    dc_row_sync(row);
+    const float2 a0 = st[0], a1 = st[1], a2 = st[2], a3 = st[3];
+    const float mean = 0.25f * ((a0.x + a1.x) + (a2.x + a3.x));
+    const float e0 = a0.x - mean, e1 = a1.x - mean, e2 = a2.x - mean, e3 = a3.x - mean;
+    const float m2 = ((a0.y + a1.y) + (a2.y + a3.y)) + (32 * V2) * ((e0 * e0 + e1 * e1) + (e2 * e2 + e3 * e3));
+    const float rstd = rsqrtf(m2 / d + 1e-5f);
+#pragma unroll
+    for (int j = 0; j < V2; ++j) x[j] = (hv[j] - mean) * rstd;
+  };
+  auto affine = [&](float (&x)[V2], const float* gam, const float* bet) {
+#pragma unroll
+    for (int j = 0; j < V2; ++j) x[j] = x[j] * gam[c0 + j] + bet[c0 + j];
+  };
+  // ---- ring, consumer side: chunk i of the pass that begins sits in slot (cslot + i) % n_slots
   int cslot = 0;
   uint32_t cround = 0;
   auto chunk_wait = [&](int i) {
@@ -551,404 +479,329 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
     wait_bar(bar_of(8 + (s >= n_slots ? s - n_slots : s)), (cround + (s >= n_slots ? 1u : 0u)) & 1u);
   };
   auto chunk_addr = [&](int i) { const int s = cslot + i; return dc_smem + pl.off_w + (size_t)(s >= n_slots ? s - n_slots : s) * DC_CHUNK; };
-  auto chunks_release = [&](int n) {           // this warp is done with the stage's n chunks
+  auto chunks_release = [&](int n) {           // this warp is done with the pass's n chunks
     __syncwarp();
     for (int i = 0; i < n; ++i) {
-      if (lane == 0) ptx::mbar_arrive(bar_of(16 + cslot));
+      if (lane == 0) {      // having seen the chunk, whether or not this warp read it: a warp without tiles stays within the round
+        wait_bar(bar_of(8 + cslot), cround & 1u);
+        ptx::mbar_arrive(bar_of(16 + cslot));
+      }
       if (++cslot == n_slots) { cslot = 0; ++cround; }
     }
   };
-  // k loop of slab S of layer l over this warp's units, then `done(tile index list, accumulators)`
+  // Y = X W^T for slab S of layer l, up to TPW tiles per warp and pass (tile warp + 8 t of the pass), `done(tile, accumulators)`
+  // per finished tile.  A pass is at most four chunks.
   auto linear = [&](auto slab_c, int l, const __nv_bfloat16* X, int px, auto done) {
     constexpr int S = decltype(slab_c)::value;
-    constexpr int K = dc_slab_k(d, S), NT = dc_slab_rows(d, S) / 8, KS = dc_ksplit(K, NT), KC = K < 256 ? K : 256, KBC = KC / 32;
-    constexpr int TPW = KS > 1 ? 1 : (NT + DC_WARPS - 1) / DC_WARPS, NCH = (dc_slab_bytes(d, S) + DC_CHUNK - 1) / DC_CHUNK;
-    constexpr int NKB = K / 32 / KS;
-    int nt[TPW];
-    int kb0 = 0;
-    if (KS > 1) { nt[0] = warp % NT; kb0 = (warp / NT) * NKB; }      // unit (tile, part of k); warps beyond the last unit idle
-    else {
+    constexpr int K = dc_slab_k(d, S), NT = dc_slab_rows(d, DH, S) / 8, NKB = K / 32, TB = K * 16;      // TB: bytes of a tile
+    constexpr int TPW = NT >= 32 && K <= 128 ? 4 : 2, PT = TPW * DC_WARPS;                                          // tiles of a pass
+    static_assert(K <= 256 && PT * TB <= 4 * DC_CHUNK, "a pass is at most four chunks");
+    const uint8_t* wres = dc_smem + pl.off_w + (size_t)l * dc_layer_bytes(d, DH) + dc_slab_off(d, DH, S);
 #pragma unroll
-      for (int t = 0; t < TPW; ++t) nt[t] = min(warp + t * DC_WARPS, NT - 1);      // past the last tile: computed again, not used
-    }
-    const bool busy = KS == 1 || warp < NT * KS;
-    float c[TPW][4];
-    const uint8_t* wres = dc_smem + pl.off_w + (size_t)l * dc_layer_bytes(d) + dc_slab_off(d, S);
-    if (!resident && busy) {
+    for (int t0 = 0; t0 < NT; t0 += PT) {
+      constexpr int FULL = PT;
+      const int n_pass = NT - t0 < FULL ? NT - t0 : FULL;                                               // compile-time after unrolling
+      const int nch = (n_pass * TB + DC_CHUNK - 1) / DC_CHUNK;
+      const uint8_t* base[TPW];
+      int nt[TPW];
 #pragma unroll
-      for (int i = 0; i < NCH; ++i) {          // the chunks that hold this warp's pieces
-        bool mine = false;
-#pragma unroll
-        for (int t = 0; t < TPW; ++t)
-#pragma unroll
-          for (int kc = 0; kc < K / KC; ++kc)
-            mine |= (((kc * NT + nt[t]) * KC * 16) >> 14) == i && (kc + 1) * KBC > kb0 && kc * KBC < kb0 + NKB;
-        if (mine) chunk_wait(i);
+      for (int t = 0; t < TPW; ++t) {
+        nt[t] = warp + t * DC_WARPS;
+        if (nt[t] < n_pass) {
+          const int o = nt[t] * TB;
+          if (resident) base[t] = wres + t0 * TB + o;
+          else { chunk_wait(o / DC_CHUNK); base[t] = chunk_addr(o / DC_CHUNK) + o % DC_CHUNK; }
+        } else base[t] = nullptr;
       }
       __syncwarp();
+      auto frag = [&](int t, int, int kb) { return base[t] + kb * 512; };
+      float c[TPW][4];
+      int have = 0;
+#pragma unroll
+      for (int t = 0; t < TPW; ++t) have += nt[t] < n_pass ? 1 : 0;                                    // warp-uniform
+      if (have == TPW) dc_kloop<TPW, NKB>(X, px, nt, c, frag);
+      else if (have > 0) {      // a ragged pass: tile by tile
+#pragma unroll
+        for (int t = 0; t < TPW; ++t)
+          if (t < have) {
+            const int one[1] = {nt[t]};
+            float c1[1][4];
+            dc_kloop<1, NKB>(X, px, one, c1, [&](int, int, int kb) { return base[t] + kb * 512; });
+            c[t][0] = c1[0][0]; c[t][1] = c1[0][1]; c[t][2] = c1[0][2]; c[t][3] = c1[0][3];
+          }
+      }
+      if (!resident) chunks_release(nch);
+#pragma unroll
+      for (int t = 0; t < TPW; ++t)
+        if (nt[t] < n_pass) done(t0 + nt[t], c[t]);
     }
-    if (busy) {
-      auto frag = [&](int tile, int kb) -> const uint8_t* {
-        const int o = ((kb / KBC) * NT + tile) * KC * 16 + (kb % KBC) * 512;
-        return resident ? wres + o : chunk_addr(o >> 14) + (o & (DC_CHUNK - 1));
-      };
-      dc_kloop<TPW, NKB>(X, px, kb0, nt, c, frag);
-    }
-    if (!resident) chunks_release(NCH);
-    done(nt, c, busy);
   };
-  // a finished fragment with bias (and GELU) as bf16 into every replica of `dst`: the quads gather rows of 8 columns
-  auto emit_bf16 = [&](int tile, float (&c)[4], const float* bias, bool gelu, uint32_t dst_off, int pitch, int col0) {
+  // a finished tile with bias (and GELU) as bf16 into a local buffer
+  auto keep = [&](__nv_bfloat16* dst, int pitch, int tile, const float (&c)[4], const float* bias, bool gelu) {
     const float2 bb = *reinterpret_cast<const float2*>(bias + tile * 8 + 2 * tg);
     float v0 = c[0] + bb.x, v1 = c[1] + bb.y, v2 = c[2] + bb.x, v3 = c[3] + bb.y;
     if (gelu) { v0 = ptx::gelu_fast(v0); v1 = ptx::gelu_fast(v1); v2 = ptx::gelu_fast(v2); v3 = ptx::gelu_fast(v3); }
-    const uint32_t p0 = pack_bf16x2(v0, v1), p1 = pack_bf16x2(v2, v3);
-    // lanes tg 0, 2: row g; tg 1, 3: row g + 8; the two lanes of a row serve four destinations each
-    uint4 o;
-    uint32_t* ow = reinterpret_cast<uint32_t*>(&o);
+    *reinterpret_cast<uint32_t*>(dst + g * pitch + tile * 8 + 2 * tg) = pack_bf16x2(v0, v1);
+    *reinterpret_cast<uint32_t*>(dst + (g + 8) * pitch + tile * 8 + 2 * tg) = pack_bf16x2(v2, v3);
+  };
+  // dot products of the owned rows' fp32 values (sxr) with `n` vectors per row, one per warp and turn: out(row, i, value) in lane 0
+  auto row_dots = [&](int n, auto load4, auto out) {
+    for (int p0 = warp; p0 < DC_OWN * n; p0 += 4 * DC_WARPS) {
+      float acc[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t x = __shfl_sync(0xffffffffu, p0, (lane & ~3) | j), y = __shfl_sync(0xffffffffu, p1, (lane & ~3) | j);
-      ow[j] = (tg & 1) ? y : x;
+      for (int u = 0; u < 4; ++u) {
+        const int p = min(p0 + u * DC_WARPS, DC_OWN * n - 1), r = p & 1, i = p >> 1;
+        acc[u] = 0.f;
+#pragma unroll
+        for (int j = 0; j < d / 128; ++j) {
+          const int c = j * 128 + lane * 4;
+          const float4 x = *reinterpret_cast<const float4*>(sxr + r * d + c), w = load4(i, c);
+          acc[u] += (x.x * w.x + x.y * w.y) + (x.z * w.z + x.w * w.w);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int p = p0 + u * DC_WARPS;
+        if (lane == u && p < DC_OWN * n) out(p & 1, p >> 1, acc[u]);
+      }
     }
-    bcast16(dst_off + (uint32_t)((g + 8 * (tg & 1)) * pitch + col0 + tile * 8) * 2u, o, tg >> 1);
   };
-  // parts of a split reduction (16 x 8 tiles in `red`) of NT tiles, KS parts: four columns of a row per pair of threads
-  auto put_part = [&](float (&c)[4]) {
-    float* r = red + (size_t)warp * (DC_ROWS * 8);
-    *reinterpret_cast<float2*>(r + g * 8 + 2 * tg) = make_float2(c[0], c[1]);
-    *reinterpret_cast<float2*>(r + (g + 8) * 8 + 2 * tg) = make_float2(c[2], c[3]);
-  };
-  auto sum_parts = [&](int NT, int KS, int piece) {      // piece: (tile, row, half of the 8 columns)
-    const int tile = piece / 32, rem = piece % 32;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int kp = 0; kp < KS; ++kp) {
-      const float4 q = *reinterpret_cast<const float4*>(red + (size_t)(tile + kp * NT) * (DC_ROWS * 8) + rem * 4);
-      v.x += q.x; v.y += q.y; v.z += q.z; v.w += q.w;
-    }
-    return v;
-  };
-  // y + bias + stream -> the stream, every replica (fp32)
-  auto emit_stream = [&](int NT, int KS, const float* bias, uint32_t slice0) {
-    for (int i = threadIdx.x; i < NT * 64; i += DC_COMPUTE) {
-      const int piece = i >> 1, tile = piece / 32, row = (piece % 32) >> 1, c4 = tile * 8 + (piece & 1) * 4;
-      const float4 v = sum_parts(NT, KS, piece), b4 = *reinterpret_cast<const float4*>(bias + c4);
-      const float4 ho = *reinterpret_cast<const float4*>(h + row * HP + slice0 + c4);
-      const uint4 o = make_uint4(__float_as_uint(ho.x + v.x + b4.x), __float_as_uint(ho.y + v.y + b4.y), __float_as_uint(ho.z + v.z + b4.z),
-                                 __float_as_uint(ho.w + v.w + b4.w));
-      bcast16((uint32_t)pl.off_h + (uint32_t)(row * HP + slice0 + c4) * 4u, o, i & 1);
-    }
+  auto put_rows = [&](const float (&x)[V2]) {
+#pragma unroll
+    for (int j = 0; j < V2; ++j) sxr[row * d + c0 + j] = x[j];
   };
 
-  uint32_t n_layer = 0;      // layers so far (parameter buffers)
+  uint32_t n_layer = 0, n_tab = 0;      // layers so far (parameter buffers), tables so far
   if (resident) wait_bar(bar_of(2), 0);
-  // One forward of the network on the latent in sx at timestep tau for request env; leaves eps in seps.  `hook` runs while the
-  // last stage's slices are on their way.
-  auto forward = [&](int tau, int env, auto hook) {
-    {   // token embedding into the residual stream: a thread owns one column of 16 (d = 256) or 8 rows
-      constexpr int RPT = DC_ROWS * d / DC_COMPUTE;
-      const int col = threadIdx.x % d, r0 = (threadIdx.x / d) * RPT;
-      float acc[RPT];
-      const float bi = __ldg(P.b_in + col);
+  // One forward of the network on the owned rows' latent in sx at timestep tau for request env; leaves their eps in seps.  `rest`
+  // is run once, by the upper four warps, which have nothing to do during the first layer's attention.
+  auto forward = [&](int tau, int env, auto rest) {
+    {   // token embedding into the residual stream
+      const int tok = DC_OWN * rank + row;
+      const bool live = tok < H;
 #pragma unroll
-      for (int r = 0; r < RPT; ++r) acc[r] = r0 + r < H ? bi + __ldg(P.pos + (r0 + r) * d + col) : 0.f;
-      for (int c0 = 0; c0 < A; c0 += 4) {
-        float w[4];
+      for (int j = 0; j < V2; ++j) hv[j] = live ? __ldg(P.b_in + c0 + j) + __ldg(P.pos + tok * d + c0 + j) : 0.f;
+      if (live)
+#pragma unroll 4
+        for (int i = 0; i < A; ++i) {
+          const float xv = sx[row * AP + i];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = c0 + j < A ? __ldg(P.W_in + (c0 + j) * d + col) : 0.f;
-#pragma unroll
-        for (int r = 0; r < RPT; ++r) {
-          const float4 xv = *reinterpret_cast<const float4*>(sx + (r0 + r) * AP + c0);      // rows past H and columns past A are zero
-          acc[r] = __fmaf_rn(xv.x, w[0], acc[r]); acc[r] = __fmaf_rn(xv.y, w[1], acc[r]);
-          acc[r] = __fmaf_rn(xv.z, w[2], acc[r]); acc[r] = __fmaf_rn(xv.w, w[3], acc[r]);
+          for (int j = 0; j < V2; ++j) hv[j] = __fmaf_rn(xv, __ldg(P.W_in + i * d + c0 + j), hv[j]);
         }
-      }
-#pragma unroll
-      for (int r = 0; r < RPT; ++r) h[(r0 + r) * HP + col] = acc[r];
     }
-    dc_sync();
-    const int heads = P.heads, hp = heads >> 1, NKH = NK * heads;
-    uint32_t* sU = reinterpret_cast<uint32_t*>(dc_smem + pl.off_kv);       // folded: [NKH / 2][d + 8] words
-    float* skv = reinterpret_cast<float*>(dc_smem + pl.off_kv);            // otherwise [NK][2d]
     for (int l = 0; l < L; ++l) {
-      if (!resident) wait_bar(bar_of(3 + (n_layer & 1u)), (n_layer >> 1) & 1u);
+      if (!resident) wait_bar(bar_of(3 + (int)(n_layer & 1u)), (n_layer >> 1) & 1u);
       const float* pb = spar + (size_t)(resident ? l : (int)(n_layer & 1u)) * PL;
-      const float* bb = pb + 6 * d;                      // bias slices: columns of this CTA only
-      struct { const float *ln1_g, *ln1_b, *ln2_g, *ln2_b, *ln3_g, *ln3_b, *bqkv, *bo, *bq2, *bo2, *b1, *b2; } W =
-          {pb, pb + d, pb + 2 * d, pb + 3 * d, pb + 4 * d, pb + 5 * d, bb, bb + NS_3D, bb + NS_3D + NS_D,
-           bb + NS_3D + 2 * NS_D, bb + NS_3D + 3 * NS_D, bb + NS_3D + 3 * NS_D + NS_4D};
-      // ---- causal self-attention
-      dc_layernorm<d>(h, W.ln1_g, W.ln1_b, a, PA);
+      const float *ln1 = pb, *ln2 = pb + 2 * d, *ln3 = pb + 4 * d, *bo = pb + 6 * d, *bo2 = pb + 7 * d, *b2 = pb + 8 * d,
+                  *bqkv = pb + 9 * d, *b1 = bqkv + NQ, *bq2 = b1 + d / 2;
+      float x[V2];
+      // ---- causal self-attention of this CTA's head
+      normalise(x);
+      affine(x, ln1, ln1 + d);
+      stage_begin(DC_ROWS * d * 2);
+      gather_rows(x);
+      stage_end();
+      linear(std::integral_constant<int, 0>{}, l, xa, PX, [&](int tile, const float (&c)[4]) { keep(qs, PQ, tile, c, bqkv, false); });
       dc_sync();
-      stage_begin(DC_ROWS * 3 * d * 2);
-      linear(std::integral_constant<int, 0>{}, l, a, PA, [&](auto& nt, auto& c, bool) {
-        constexpr int TPW = sizeof(nt) / sizeof(int);
+      if (warp < VW / 16) {
+        // scores of all 16 rows by each of these warps, then 16 of the CTA's value columns
+        const float scale = rsqrtf((float)DH);
+        float s[2][4];
 #pragma unroll
-        for (int t = 0; t < TPW; ++t)
-          if (warp + t * DC_WARPS < NS_3D / 8) emit_bf16(nt[t], c[t], W.bqkv, false, (uint32_t)pl.off_qkv, PQKV, rank * NS_3D);
-      });
-      // while the slices travel: the memory tokens' folded tables of this block start their way into shared memory, kq rows into the
-      // q2 buffer, u rows (head pairs in one word, as stored) into the u buffer, the constants into registers
-      float cst[DC_MAX_NK];
+        for (int nt = 0; nt < 2; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < DH / 16; ++ks) {
+          uint32_t a4[4], b4[4];
+          ldmatrix_x4(a4, qs + (lane & 15) * PQ + ks * 16 + 8 * (lane >> 4));
+          ldmatrix_x4(b4, qs + ((lane & 7) + 8 * (lane >> 4)) * PQ + DH + ks * 16 + 8 * ((lane >> 3) & 1));
+          mma_bf16_16816(s[0], a4, b4[0], b4[1]);
+          mma_bf16_16816(s[1], a4, b4[2], b4[3]);
+        }
+        const int r0 = g, r1 = g + 8;
+        float m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          const int col = nt * 8 + 2 * tg;
+          s[nt][0] = (col <= r0 && col < H) ? s[nt][0] * scale : -INFINITY;
+          s[nt][1] = (col + 1 <= r0 && col + 1 < H) ? s[nt][1] * scale : -INFINITY;
+          s[nt][2] = (col <= r1 && col < H) ? s[nt][2] * scale : -INFINITY;
+          s[nt][3] = (col + 1 <= r1 && col + 1 < H) ? s[nt][3] * scale : -INFINITY;
+          m0 = fmaxf(m0, fmaxf(s[nt][0], s[nt][1]));
+          m1 = fmaxf(m1, fmaxf(s[nt][2], s[nt][3]));
+        }
+        m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 1)); m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 1));
+        m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 2)); m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 2));
+        float l0 = 0.f, l1 = 0.f;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          s[nt][0] = __expf(s[nt][0] - m0); s[nt][1] = __expf(s[nt][1] - m0);
+          s[nt][2] = __expf(s[nt][2] - m1); s[nt][3] = __expf(s[nt][3] - m1);
+          l0 += s[nt][0] + s[nt][1]; l1 += s[nt][2] + s[nt][3];
+        }
+        l0 += __shfl_xor_sync(0xffffffffu, l0, 1); l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
+        l0 += __shfl_xor_sync(0xffffffffu, l0, 2); l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
+        const float inv0 = 1.0f / l0, inv1 = 1.0f / l1;      // every row sees at least key 0 (H >= 1)
+        uint32_t pa[4];
+        pa[0] = pack_bf16x2(s[0][0], s[0][1]); pa[1] = pack_bf16x2(s[0][2], s[0][3]);
+        pa[2] = pack_bf16x2(s[1][0], s[1][1]); pa[3] = pack_bf16x2(s[1][2], s[1][3]);
+        float o0[4] = {0.f, 0.f, 0.f, 0.f}, o1[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t b4[4];
+        ldmatrix_x4_trans(b4, qs + ((lane & 7) + 8 * ((lane >> 3) & 1)) * PQ + 2 * DH + warp * 16 + 8 * (lane >> 4));
+        mma_bf16_16816(o0, pa, b4[0], b4[1]);
+        mma_bf16_16816(o1, pa, b4[2], b4[3]);
+        __nv_bfloat16* o = os + warp * 16 + 2 * tg;
+        *reinterpret_cast<uint32_t*>(o + r0 * PO) = pack_bf16x2(o0[0] * inv0, o0[1] * inv0);
+        *reinterpret_cast<uint32_t*>(o + r1 * PO) = pack_bf16x2(o0[2] * inv1, o0[3] * inv1);
+        *reinterpret_cast<uint32_t*>(o + r0 * PO + 8) = pack_bf16x2(o1[0] * inv0, o1[1] * inv0);
+        *reinterpret_cast<uint32_t*>(o + r1 * PO + 8) = pack_bf16x2(o1[2] * inv1, o1[3] * inv1);
+      } else if (l == 0 && warp >= 4) rest();
+      dc_sync();
+      stage_begin(DC_CS * DC_OWN * d * 4);
+      linear(std::integral_constant<int, 1>{}, l, os, PO, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
+      float cst = 0.f;      // constant of the score that this lane will finish (at most 32 scores: four per warp)
       if (P.fold) {
-        const size_t tok_stride = (size_t)L * heads * d, lay = (size_t)l * heads * d;
-        for (int i = threadIdx.x; i < NKH * (d / 8); i += DC_COMPUTE) {
-          const int n = i / (d / 8), ch = i % (d / 8);
-          const int j = n / heads, hh = n - j * heads;
-          const __nv_bfloat16* src = (j == 0 ? P.kq_time + (size_t)tau * tok_stride : P.kq_obs + ((size_t)env * P.To + (j - 1)) * tok_stride) +
-                                     lay + (size_t)hh * d + ch * 8;
-          dc_cp_async<16>(q2 + n * PA + ch * 8, src);
-        }
-        for (int i = threadIdx.x; i < (NKH / 2) * (d / 4); i += DC_COMPUTE) {
-          const int pr = i / (d / 4), ch = i - pr * (d / 4);
-          const int j = pr / hp, q = pr - j * hp;
-          const __nv_bfloat16* src = (j == 0 ? P.ut_time + (size_t)tau * tok_stride : P.ut_obs + ((size_t)env * P.To + (j - 1)) * tok_stride) +
-                                     lay + (size_t)q * d * 2 + ch * 8;
-          dc_cp_async<16>(sU + pr * (d + 8) + ch * 4, src);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-#pragma unroll
-        for (int j = 0; j < DC_MAX_NK; ++j) {
-          cst[j] = 0.f;
-          if (j < NK && threadIdx.x < DC_ROWS * heads)
-            cst[j] = __ldg((j == 0 ? P.c_time + (size_t)tau * L * heads : P.c_obs + ((size_t)env * P.To + (j - 1)) * L * heads) +
-                           (size_t)l * heads + threadIdx.x % heads);
+        const int p = warp + lane * DC_WARPS, n = p >> 1, j = n / HEADS;
+        if (lane < 4 && p < DC_OWN * NKH)
+          cst = __ldg((j == 0 ? P.c_time + (size_t)tau * L * HEADS : P.c_obs + ((size_t)env * P.To + (j - 1)) * L * HEADS) +
+                      (size_t)l * HEADS + n % HEADS);
+      } else {      // keys and value columns of the memory tokens for this CTA's head
+        float* skv = reinterpret_cast<float*>(dc_smem + pl.off_kq);      // [NK][DH + VW]
+        const size_t ldkv = (size_t)L * 2 * d;
+        for (int i = threadIdx.x; i < NK * (DH + VW); i += DC_COMPUTE) {
+          const int kx = i / (DH + VW), c = i % (DH + VW);
+          const float* src = (kx == 0 ? P.kv_time + (size_t)tau * ldkv : P.kv_obs + ((size_t)env * P.To + (kx - 1)) * ldkv) + (size_t)l * 2 * d;
+          skv[i] = __ldg(src + (c < DH ? rank * HEADS / DC_CS * DH + c : d + rank * VW + (c - DH)));
         }
       }
       stage_end();
-      switch (d / P.heads) {
-        case 32: dc_self_attn_mma<d, 32>(qkv, PQKV, a, PA, P.heads, H); break;
-        case 64: dc_self_attn_mma<d, 64>(qkv, PQKV, a, PA, P.heads, H); break;
-        case 128: dc_self_attn_mma<d, 128>(qkv, PQKV, a, PA, P.heads, H); break;
-        default: dc_attention<d, true>(qkv, PQKV, qkv, PQKV, nullptr, 0, a, PA, P.heads, H); break;
-      }
-      dc_sync();
-      stage_begin(DC_ROWS * d * 4);
-      linear(std::integral_constant<int, 1>{}, l, a, PA, [&](auto&, auto& c, bool busy) {
-        if (busy) put_part(c[0]);
-        dc_sync();
-        emit_stream(NS_D / 8, dc_ksplit(d, NS_D / 8), W.bo, (uint32_t)rank * NS_D);
-      });
-      if (!P.fold) {   // keys / values of the memory tokens for this block: time token of tau, then the obs tokens
-        for (int i = threadIdx.x; i < NK * 2 * d; i += DC_COMPUTE) {
-          const int kx = i / (2 * d), c = i % (2 * d);
-          const float* src = kx == 0 ? P.kv_time + (size_t)tau * ldkv : P.kv_obs + ((size_t)env * P.To + (kx - 1)) * ldkv;
-          skv[i] = __ldg(src + (size_t)l * 2 * d + c);
-        }
-      }
-      stage_end();
+      add_partials(bo);
       // ---- cross-attention to [time token | obs tokens]
+      normalise(x);
       if (P.fold) {
-        // Folded form: scores = xhat . kq + c, out = P . u + bo2, both so small that every CTA computes them whole
-        // on its own replica: no slices to exchange, two linear stages fewer per block.
-        float* sS = reinterpret_cast<float*>(qkv);                                 // [8][16][16] partial scores
-        __nv_bfloat16* sP = reinterpret_cast<__nv_bfloat16*>(sS + DC_WARPS * DC_ROWS * 16);   // [16][DC_PU] softmax weights
-        dc_layernorm<d, false>(h, nullptr, nullptr, a, PA);
-        for (int i = threadIdx.x; i < DC_ROWS * DC_PU / 2; i += DC_COMPUTE) reinterpret_cast<uint32_t*>(sP)[i] = 0u;
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        // Folded form, on the owned rows alone: scores = xhat . kq + c, out = P . u + bo2 (fp32)
+        put_rows(x);
+        wait_bar(bar_of(7), n_tab & 1u);
+        ++n_tab;
         dc_sync();
-        {   // warp w: a part of the d input columns, all 16 score columns (those past the last one repeat it and are not read)
-          float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
-          const __nv_bfloat16* ka = q2 + (size_t)min((lane & 7) + 8 * (lane >> 4), NKH - 1) * PA + 8 * ((lane >> 3) & 1);
+        row_dots(NKH, [&](int n, int c) {
+          const uint2 w = *reinterpret_cast<const uint2*>(skq + n * d + c);
+          const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x)), hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.y));
+          return make_float4(lo.x, lo.y, hi.x, hi.y);
+        }, [&](int r, int n, float v) { sscore[r * DC_MAX_NKH + n] = v + cst; });
+        dc_sync();
+        float pr[DC_MAX_NKH];
 #pragma unroll
-          for (int kk = 0; kk < d / 128; ++kk) {
-            const int k = (warp * (d / 128) + kk) * 16;
-            uint32_t x4[4], b4[4];
-            ldmatrix_x4(x4, a + (lane & 15) * PA + k + 8 * (lane >> 4));
-            ldmatrix_x4(b4, ka + k);
-            mma_bf16_16816(s0, x4, b4[0], b4[1]);
-            mma_bf16_16816(s1, x4, b4[2], b4[3]);
-          }
-          float* o = sS + (size_t)warp * DC_ROWS * 16 + g * 16 + 2 * tg;
-          *reinterpret_cast<float2*>(o) = make_float2(s0[0], s0[1]);
-          *reinterpret_cast<float2*>(o + 8) = make_float2(s1[0], s1[1]);
-          *reinterpret_cast<float2*>(o + 128) = make_float2(s0[2], s0[3]);
-          *reinterpret_cast<float2*>(o + 136) = make_float2(s1[2], s1[3]);
+        for (int n = 0; n < DC_MAX_NKH; ++n) pr[n] = n < NKH ? sscore[row * DC_MAX_NKH + n] : -INFINITY;
+#pragma unroll
+        for (int hh = 0; hh < HEADS && hh < DC_MAX_NKH; ++hh) {
+          float m = -INFINITY, s = 0.f;
+#pragma unroll
+          for (int n = hh; n < DC_MAX_NKH; n += HEADS) m = fmaxf(m, pr[n]);
+#pragma unroll
+          for (int n = hh; n < DC_MAX_NKH; n += HEADS) { pr[n] = __expf(pr[n] - m); s += pr[n]; }
+          const float inv = 1.0f / s;
+#pragma unroll
+          for (int n = hh; n < DC_MAX_NKH; n += HEADS) pr[n] *= inv;
         }
-        dc_sync();
-        if (threadIdx.x < DC_ROWS * heads) {      // heads <= 16: one (row, head) per thread
-          const int row = threadIdx.x / heads, hh = threadIdx.x % heads;
-          float sc[DC_MAX_NK];
-          float m = -INFINITY;
+        float o[V2];
 #pragma unroll
-          for (int j = 0; j < DC_MAX_NK; ++j)
-            if (j < NK) {
-              float v = 0.f;
+        for (int j = 0; j < V2; ++j) o[j] = 0.f;
 #pragma unroll
-              for (int w = 0; w < DC_WARPS; ++w) v += sS[(w * DC_ROWS + row) * 16 + j * heads + hh];
-              sc[j] = v + cst[j];
-              m = fmaxf(m, sc[j]);
+        for (int q = 0; q < DC_MAX_NKH / 2; ++q)
+          if (2 * q < NKH) {
+#pragma unroll
+            for (int j = 0; j < V2; ++j) {
+              const float2 u2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(su + q * d + c0 + j));
+              o[j] = __fmaf_rn(pr[2 * q], u2.x, __fmaf_rn(pr[2 * q + 1], u2.y, o[j]));
             }
-          float lsum = 0.f;
-#pragma unroll
-          for (int j = 0; j < DC_MAX_NK; ++j)
-            if (j < NK) { sc[j] = __expf(sc[j] - m); lsum += sc[j]; }
-          const float inv = 1.0f / lsum;
-#pragma unroll
-          for (int j = 0; j < DC_MAX_NK; ++j)
-            if (j < NK) sP[row * DC_PU + j * heads + hh] = __float2bfloat16_rn(sc[j] * inv);
-        }
-        dc_sync();
-        const float* bo2_full = pb + 6 * d + 11 * d / DC_CS;
-        {
-          // out = P . u: warp w the output columns [w d/8, (w+1) d/8), every row; a word of the u rows is one B
-          // fragment register (k = heads 2q, 2q+1 of a memory token), so nothing is transposed.
-          uint32_t pa[4];
-          ldmatrix_x4(pa, sP + (lane & 15) * DC_PU + 8 * (lane >> 4));
-          const uint32_t* pu[2];
-          uint32_t ulive[2];
-#pragma unroll
-          for (int rg = 0; rg < 2; ++rg) {
-            const int pr = 4 * rg + tg;
-            ulive[rg] = 2 * pr < NKH ? 0xffffffffu : 0u;
-            pu[rg] = sU + (size_t)min(pr, NKH / 2 - 1) * (d + 8) + g;
           }
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(bar_of(24));      // this warp is done with the tables
 #pragma unroll
-          for (int nt = 0; nt < d / 64; ++nt) {
-            const int col = warp * (d / 8) + nt * 8;
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_bf16_16816(acc, pa, pu[0][col] & ulive[0], pu[1][col] & ulive[1]);
-            // every CTA updates its own replica of the stream: straight from the fragment, two columns per lane and row
-            const float2 b2 = *reinterpret_cast<const float2*>(bo2_full + col + 2 * tg);
-            float2* h0 = reinterpret_cast<float2*>(h + g * HP + col + 2 * tg);
-            float2* h1 = reinterpret_cast<float2*>(h + (g + 8) * HP + col + 2 * tg);
-            float2 a0 = *h0, a1 = *h1;
-            a0.x += acc[0] + b2.x; a0.y += acc[1] + b2.y; a1.x += acc[2] + b2.x; a1.y += acc[3] + b2.y;
-            *h0 = a0; *h1 = a1;
-          }
-        }
-        dc_sync();
+        for (int j = 0; j < V2; ++j) hv[j] += o[j] + bo2[c0 + j];
       } else {
-        dc_layernorm<d>(h, W.ln2_g, W.ln2_b, a, PA);
-        dc_sync();                               // also: the keys / values above were written by other threads
+        affine(x, ln2, ln2 + d);
         stage_begin(DC_ROWS * d * 2);
-        linear(std::integral_constant<int, 4>{}, l, a, PA, [&](auto&, auto& c, bool busy) {
-          constexpr int NT = NS_D / 8, KS = dc_ksplit(d, NT);
-          if (busy) put_part(c[0]);
-          dc_sync();
-          for (int i = threadIdx.x; i < NT * 32; i += DC_COMPUTE) {      // 8 columns of a row per pair of threads
-            const int tile = i / 32, row = (i % 32) >> 1;
-            const float4 lo = sum_parts(NT, KS, tile * 32 + row * 2), hi = sum_parts(NT, KS, tile * 32 + row * 2 + 1);
-            const float* bq = W.bq2 + tile * 8;
-            bcast16((uint32_t)pl.off_q2 + (uint32_t)(row * PA + rank * NS_D + tile * 8) * 2u,
-                    make_uint4(pack_bf16x2(lo.x + bq[0], lo.y + bq[1]), pack_bf16x2(lo.z + bq[2], lo.w + bq[3]),
-                               pack_bf16x2(hi.x + bq[4], hi.y + bq[5]), pack_bf16x2(hi.z + bq[6], hi.w + bq[7])), i & 1);
-          }
-        });
+        gather_rows(x);
         stage_end();
-        dc_attention<d, false>(q2, PA, nullptr, 0, skv, NK, a, PA, P.heads, H);
+        dc_sync();                                         // the keys / values above were written by other threads
+        linear(std::integral_constant<int, 4>{}, l, xa, PX, [&](int tile, const float (&c)[4]) { keep(qs, PQ, tile, c, bq2, false); });
         dc_sync();
-        stage_begin(DC_ROWS * d * 4);
-        linear(std::integral_constant<int, 5>{}, l, a, PA, [&](auto&, auto& c, bool busy) {
-          if (busy) put_part(c[0]);
-          dc_sync();
-          emit_stream(NS_D / 8, dc_ksplit(d, NS_D / 8), W.bo2, (uint32_t)rank * NS_D);
-        });
+        if (threadIdx.x < 4 * DC_ROWS) {                   // four lanes per query row, each a quarter of the head and of the value columns
+          const float* skv = reinterpret_cast<const float*>(dc_smem + pl.off_kq);
+          const int r = threadIdx.x >> 2, sub = threadIdx.x & 3;
+          const float scale = rsqrtf((float)DH);
+          float sc[DC_MAX_NK], m = -INFINITY, s = 0.f;
+#pragma unroll
+          for (int j = 0; j < DC_MAX_NK; ++j) {
+            float v = 0.f;
+            if (j < NK)
+              for (int i = sub * (DH / 4); i < (sub + 1) * (DH / 4); ++i) v += __bfloat162float(qs[r * PQ + i]) * skv[j * (DH + VW) + i];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            sc[j] = j < NK ? v * scale : -INFINITY;
+            m = fmaxf(m, sc[j]);
+          }
+#pragma unroll
+          for (int j = 0; j < DC_MAX_NK; ++j) { sc[j] = __expf(sc[j] - m); s += sc[j]; }
+          const float inv = 1.0f / s;
+          for (int i = sub * (VW / 4); i < (sub + 1) * (VW / 4); ++i) {
+            float v = 0.f;
+#pragma unroll
+            for (int j = 0; j < DC_MAX_NK; ++j)
+              if (j < NK) v += sc[j] * skv[j * (DH + VW) + DH + i];
+            os[r * PO + i] = __float2bfloat16_rn(v * inv);
+          }
+        }
+        dc_sync();
+        stage_begin(DC_CS * DC_OWN * d * 4);
+        linear(std::integral_constant<int, 5>{}, l, os, PO, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
         stage_end();
+        add_partials(bo2);
       }
       // ---- MLP
-      dc_layernorm<d>(h, W.ln3_g, W.ln3_b, a, PA);
+      normalise(x);
+      affine(x, ln3, ln3 + d);
+      stage_begin(DC_ROWS * d * 2);
+      gather_rows(x);
+      stage_end();
+      linear(std::integral_constant<int, 2>{}, l, xa, PX, [&](int tile, const float (&c)[4]) { keep(fs, PF, tile, c, b1, true); });
       dc_sync();
-      stage_begin(DC_ROWS * 4 * d * 2);
-      linear(std::integral_constant<int, 2>{}, l, a, PA, [&](auto& nt, auto& c, bool) {
-        constexpr int TPW = sizeof(nt) / sizeof(int);
-#pragma unroll
-        for (int t = 0; t < TPW; ++t)
-          if (warp + t * DC_WARPS < NS_4D / 8) emit_bf16(nt[t], c[t], W.b1, true, (uint32_t)pl.off_f, PF, rank * NS_4D);
-      });
+      stage_begin(DC_CS * DC_OWN * d * 4);
+      linear(std::integral_constant<int, 3>{}, l, fs, PF, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
       stage_end();
-      stage_begin(DC_ROWS * d * 4);
-      linear(std::integral_constant<int, 3>{}, l, f, PF, [&](auto&, auto& c, bool busy) {
-        if (busy) put_part(c[0]);
-        dc_sync();
-        emit_stream(NS_D / 8, dc_ksplit(4 * d, NS_D / 8), W.b2, (uint32_t)rank * NS_D);
-      });
-      if (!resident) { __syncwarp(); if (lane == 0) ptx::mbar_arrive(bar_of(5 + (n_layer & 1u))); }
+      add_partials(b2);
+      if (!resident) { __syncwarp(); if (lane == 0) ptx::mbar_arrive(bar_of(5 + (int)(n_layer & 1u))); }
       ++n_layer;
-      if (l == L - 1) hook();
-      stage_end();
     }
-    // ---- head: eps = LN_f(h) W_out + b_out   (every CTA, rows 2w, 2w + 1 of warp w side by side)
-    {
-      constexpr int V = d / 128;
-      float4 v[2][V];
-#pragma unroll
-      for (int rr = 0; rr < 2; ++rr)
-#pragma unroll
-        for (int j = 0; j < V; ++j) v[rr][j] = *reinterpret_cast<const float4*>(h + (2 * warp + rr) * HP + j * 128 + lane * 4);
-      float s[2] = {0.f, 0.f}, q[2] = {0.f, 0.f};
-#pragma unroll
-      for (int rr = 0; rr < 2; ++rr)
-#pragma unroll
-        for (int j = 0; j < V; ++j) s[rr] += v[rr][j].x + v[rr][j].y + v[rr][j].z + v[rr][j].w;
-      s[0] = warp_sum(s[0]); s[1] = warp_sum(s[1]);
-#pragma unroll
-      for (int rr = 0; rr < 2; ++rr) {
-        const float mean = s[rr] / d;
-#pragma unroll
-        for (int j = 0; j < V; ++j) {
-          float4& e = v[rr][j];
-          e.x -= mean; e.y -= mean; e.z -= mean; e.w -= mean;
-          q[rr] += e.x * e.x + e.y * e.y + e.z * e.z + e.w * e.w;
-        }
-      }
-      q[0] = warp_sum(q[0]); q[1] = warp_sum(q[1]);
-#pragma unroll
-      for (int rr = 0; rr < 2; ++rr) {
-        const float rstd = rsqrtf(q[rr] / d + 1e-5f);
-#pragma unroll
-        for (int j = 0; j < V; ++j) {
-          const int c = j * 128 + lane * 4;
-          const float4 gg = *reinterpret_cast<const float4*>(lnf_g + c), be = *reinterpret_cast<const float4*>(lnf_b + c);
-          float4& e = v[rr][j];
-          e.x = e.x * rstd * gg.x + be.x; e.y = e.y * rstd * gg.y + be.y;
-          e.z = e.z * rstd * gg.z + be.z; e.w = e.w * rstd * gg.w + be.w;
-        }
-      }
-      for (int c0 = 0; c0 < A; c0 += 4) {      // four actions of both rows at a time: eight reductions in flight
-        float acc[4][2];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[i][0] = acc[i][1] = 0.f;
-#pragma unroll
-          for (int j = 0; j < V; ++j) {
-            const float4 w = *reinterpret_cast<const float4*>(woutT + (size_t)min(c0 + i, A - 1) * d + j * 128 + lane * 4);
-#pragma unroll
-            for (int rr = 0; rr < 2; ++rr) acc[i][rr] += v[rr][j].x * w.x + v[rr][j].y * w.y + v[rr][j].z * w.z + v[rr][j].w * w.w;
-          }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            acc[i][0] += __shfl_xor_sync(0xffffffffu, acc[i][0], o);
-            acc[i][1] += __shfl_xor_sync(0xffffffffu, acc[i][1], o);
-          }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (lane == i && c0 + i < A) {
-            seps[(2 * warp) * AP + c0 + i] = acc[i][0] + bout[c0 + i];
-            seps[(2 * warp + 1) * AP + c0 + i] = acc[i][1] + bout[c0 + i];
-          }
-      }
-    }
+    // ---- head: eps = LN_f(h) W_out + b_out of the owned rows
+    float x[V2];
+    normalise(x);
+    affine(x, lnf_g, lnf_b);
+    put_rows(x);
+    dc_sync();
+    row_dots(A, [&](int i, int c) { return *reinterpret_cast<const float4*>(woutT + (size_t)i * d + c); },
+             [&](int r, int i, float v) { seps[r * AP + i] = v + bout[i]; });
     dc_sync();
   };
-  auto at = [&](int i) { return (i / A) * AP + i % A; };      // element i of a latent in the padded rows
+  // one element of the owned rows per thread of the upper four warps (A <= 64): its index in the latent, -1 if there is none
+  const int e_own = (int)threadIdx.x - 128, e_row = e_own >= 0 ? e_own / A : 0;
+  const int e_idx = e_own >= 0 && e_row < DC_OWN && DC_OWN * rank + e_row < H ? (DC_OWN * rank + e_row) * A + e_own % A : -1;
+  float* e_x = sx + e_row * AP + (e_own >= 0 ? e_own % A : 0);
+  const float* e_eps = seps + e_row * AP + (e_own >= 0 ? e_own % A : 0);
 
   if (P.mode == 1) {      // verification: one forward per (slot, candidate), the whole batch in one wave of clusters
     for (int w = cid; w < P.B * P.C; w += ncl) {
       if (!live_cand(w)) continue;                // finished slot, or a candidate beyond t = 0 (same for every CTA)
       const int slot = w / P.C, cand = w % P.C;
-      const int tb = P.t[slot];
-      const int env = item_of(P.item, slot);
-      const float* xin = P.xt + slot * P.xs_b + (long long)cand * D;
-      for (int i = threadIdx.x; i < D; i += DC_COMPUTE) sx[at(i)] = xin[i];
+      if (e_idx >= 0) *e_x = P.xt[slot * P.xs_b + (long long)cand * D + e_idx];
       dc_sync();
-      forward(tb - cand, env, [] {});
-      if (rank == 0)
-        for (int i = threadIdx.x; i < D; i += DC_COMPUTE) P.eps[slot * P.es_b + (long long)cand * D + i] = seps[at(i)];
-      dc_sync();
+      forward(P.t[slot] - cand, item_of(P.item, slot), [] {});
+      if (e_idx >= 0) P.eps[slot * P.es_b + (long long)cand * D + e_idx] = *e_eps;
     }
   } else {
     for (int slot = cid; slot < P.B; slot += ncl) {
@@ -956,39 +809,34 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       const int env = item_of(P.item, slot);     // request served by this slot: its noise streams, obs K/V, parameters
       float* xt_b = P.xt + slot * P.xs_b;
       float* mh_b = P.muhat + slot * P.ms_b;
-      for (int i = threadIdx.x; i < D; i += DC_COMPUTE) sx[at(i)] = xt_b[i];
+      float xv = 0.f;
+      if (e_idx >= 0) { xv = xt_b[e_idx]; *e_x = xv; }
       dc_sync();
-      const int q = threadIdx.x;                 // D <= 256: at most one group of four elements per thread
-      const bool mine = q < (D + 3) >> 2;
       for (int k = 1; k <= P.K; ++k) {
         const int tau = tb - k + 1;
         if (k > ke) {                            // beyond K_eff: carry the latent along (same for every CTA)
-          if (rank == 0)
-            for (int i = threadIdx.x; i < D; i += DC_COMPUTE) {
-              mh_b[(size_t)(k - 1) * D + i] = sx[at(i)];
-              xt_b[(size_t)k * D + i] = sx[at(i)];
-            }
+          if (e_idx >= 0) { mh_b[(size_t)(k - 1) * D + e_idx] = xv; xt_b[(size_t)k * D + e_idx] = xv; }
           continue;
         }
-        float z[4];
-        forward(tau, env, [&] { if (mine) normal4(seed, (uint32_t)env, STREAM_XI, (uint32_t)tau, (uint32_t)q, z); });
-        // ---- scheduler step: mu^_k, x~_k = mu^_k + sigma_tau xi_tau
-        if (mine) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int i = 4 * q + j;
-            if (i < D) {
-              const int p = at(i);
-              const float m = posterior_mean(P.S, sx[p], seps[p], tau);
-              const float xn = ddpm_sample(m, P.S.sigma[tau], z[j]);
-              sx[p] = xn;
-              if (rank == 0) { mh_b[(size_t)(k - 1) * D + i] = m; xt_b[(size_t)k * D + i] = xn; }
-            }
+        float z = 0.f, sig = 0.f;
+        forward(tau, env, [&] {
+          if (e_idx >= 0) {
+            float z4[4];
+            normal4(seed, (uint32_t)env, STREAM_XI, (uint32_t)tau, (uint32_t)(e_idx >> 2), z4);
+            const int j = e_idx & 3;
+            z = j == 0 ? z4[0] : (j == 1 ? z4[1] : (j == 2 ? z4[2] : z4[3]));
+            sig = P.S.sigma[tau];
           }
+        });
+        if (e_idx >= 0) {                        // scheduler step: mu^_k, x~_k = mu^_k + sigma_tau xi_tau
+          const float m = posterior_mean(P.S, xv, *e_eps, tau);
+          xv = ddpm_sample(m, sig, z);
+          *e_x = xv;
+          mh_b[(size_t)(k - 1) * D + e_idx] = m;
+          xt_b[(size_t)k * D + e_idx] = xv;
         }
         dc_sync();
       }
-      dc_sync();
     }
   }
   if (failed) { const long long t0 = clock64(); while (clock64() - t0 < 400000ll) { } }      // copies in flight land first

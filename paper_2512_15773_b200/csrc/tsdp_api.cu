@@ -1263,14 +1263,20 @@ int forward_arch(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, cudaStream_
 
 // ------------------------------------------------------------------------------------------ drafter
 constexpr int DC_SMEM_LIMIT = 227 * 1024;
+typedef void (*ClusterKernel)(const DcParams);
+ClusterKernel cluster_kernel_of(int d, int dh) {
+  if (d == 128) return dh == 32 ? drafter_cluster_kernel<128, 32> : (dh == 64 ? drafter_cluster_kernel<128, 64> : (dh == 128 ? drafter_cluster_kernel<128, 128> : nullptr));
+  if (d == 256) return dh == 32 ? drafter_cluster_kernel<256, 32> : (dh == 64 ? drafter_cluster_kernel<256, 64> : (dh == 128 ? drafter_cluster_kernel<256, 128> : nullptr));
+  return nullptr;
+}
 // Whether the persistent cluster kernel can run this context's drafter at all (shapes, shared memory).
 bool cluster_drafter_fits(const tsdp_config_t& cfg, const tsdp_net_t& n, int* smem_bytes, bool* resident) {
   if (cfg.precision != 1 || n.arch != TSDP_ARCH_XFMR || (n.d != 128 && n.d != 256) || n.layers > DC_MAX_LAYERS ||
-      cfg.H > DC_ROWS || 1 + cfg.obs_tokens > DC_MAX_NK || cfg.H * cfg.A > 256 || (n.d / n.heads) % 4 != 0)
+      cfg.H > DC_ROWS || 1 + cfg.obs_tokens > DC_MAX_NK || cfg.H * cfg.A > 256 || !cluster_kernel_of(n.d, n.d / n.heads))
     return false;
   // weight slices resident in shared memory if they fit beside the activations, otherwise through a ring of chunks
   for (int res = 1; res >= 0; --res) {
-    const DcSmem pl = dc_smem_plan(n.d, n.layers, cfg.A, res != 0, DC_SMEM_LIMIT);
+    const DcSmem pl = dc_smem_plan(n.d, n.d / n.heads, n.layers, cfg.A, res != 0, DC_SMEM_LIMIT);
     if (pl.total <= DC_SMEM_LIMIT) { *smem_bytes = pl.total; *resident = res != 0; return true; }
   }
   return false;
@@ -1315,13 +1321,12 @@ int launch_cluster_forward(tsdp_ctx* c, int which, int mode, int B, int K, cudaS
   P.item = c->item;
   const bool verify = mode == 1;
   P.resident = (verify ? c->cv_resident : c->dc_resident) ? 1 : 0;
-  P.n_slots = dc_smem_plan(n.cfg.d, n.cfg.layers, c->cfg.A, P.resident != 0, DC_SMEM_LIMIT).n_slots;
+  P.n_slots = dc_smem_plan(n.cfg.d, n.cfg.d / n.cfg.heads, n.cfg.layers, c->cfg.A, P.resident != 0, DC_SMEM_LIMIT).n_slots;
   const int maxc = verify ? c->cv_max_clusters : c->dc_max_clusters, smem = verify ? c->cv_smem : c->dc_smem;
   const int work = verify ? B * (K + 1) : B;
   const int ncl = work < maxc ? work : maxc;
   prof_begin(c, s, verify ? 9 : 7, 0.0);
-  if (n.cfg.d == 128) TSDP_LAUNCH(c, (drafter_cluster_kernel<128>), ncl * DC_CS, DC_THREADS, smem, s, P);
-  else TSDP_LAUNCH(c, (drafter_cluster_kernel<256>), ncl * DC_CS, DC_THREADS, smem, s, P);
+  TSDP_LAUNCH(c, cluster_kernel_of(n.cfg.d, n.cfg.d / n.cfg.heads), ncl * DC_CS, DC_THREADS, smem, s, P);
   prof_end(c, s);
   c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
@@ -1724,7 +1729,7 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
     const tsdp_net_t& nn = which == TSDP_BASE ? cfg->base : cfg->draft;
     int smem = 0; bool res = false;
     if (!cluster_drafter_fits(*cfg, nn, &smem, &res)) continue;
-    const void* fn = nn.d == 128 ? (const void*)drafter_cluster_kernel<128> : (const void*)drafter_cluster_kernel<256>;
+    const void* fn = (const void*)cluster_kernel_of(nn.d, nn.d / nn.heads);
     int cur_attr = 0;   // both nets may use the same instantiation: keep the larger request
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess) cur_attr = fa.maxDynamicSharedSizeBytes;
@@ -2221,18 +2226,20 @@ int tsdp_load_weights(tsdp_ctx* c, int which, const float* blob, size_t n) {
     }
     int smem_unused; bool res_unused;
     if (cluster_drafter_fits(cfg, net.cfg, &smem_unused, &res_unused)) {
-      const size_t lw = (size_t)DC_CS * dc_layer_bytes((int)d) / 2, lp = (size_t)DC_CS * dc_par_floats((int)d);
+      const int di = (int)d, dhi = di / net.cfg.heads;
+      const size_t lw = (size_t)DC_CS * dc_layer_bytes(di, dhi) / 2, lp = (size_t)DC_CS * dc_par_floats(di, dhi);
       if (dev_alloc(c, net.allocs, &net.dc_w, L * lw)) return TSDP_ERR_CUDA;
       if (dev_alloc(c, net.allocs, &net.dc_par, L * lp)) return TSDP_ERR_CUDA;
       for (size_t l = 0; l < L; ++l) {
         const XfmrLayer& w = net.L[l];
         const void* slabs[6] = {w.Wqkv, w.Wo, w.W1, w.W2, w.Wq2, w.Wo2};
         for (int s = 0; s < 6; ++s) {
-          const long long nel = (long long)dc_slab_rows((int)d, s) * DC_CS * dc_slab_k((int)d, s);
-          dc_pack_kernel<<<(unsigned)((nel + 255) / 256), 256>>>(reinterpret_cast<const __nv_bfloat16*>(slabs[s]), net.dc_w + l * lw, (int)d, s);
+          const long long nel = (long long)dc_slab_rows(di, dhi, s) * dc_slab_k(di, s) * DC_CS;
+          dc_pack_kernel<<<(unsigned)((nel + 255) / 256), 256>>>(reinterpret_cast<const __nv_bfloat16*>(slabs[s]), s == 3 ? 4 * di : di,
+                                                                 net.dc_w + l * lw, di, dhi, s);
         }
-        const DcParSrc ps{{w.ln1_g, w.ln1_b, w.ln2_g, w.ln2_b, w.ln3_g, w.ln3_b}, {w.bqkv, w.bo, w.bq2, w.bo2, w.b1, w.b2}};
-        dc_pack_par_kernel<<<DC_CS, 256>>>(ps, net.dc_par + l * lp, (int)d);
+        const DcParSrc ps{{w.ln1_g, w.ln1_b, w.ln2_g, w.ln2_b, w.ln3_g, w.ln3_b, w.bo, w.bo2, w.b2}, w.bqkv, w.b1, w.bq2};
+        dc_pack_par_kernel<<<DC_CS, 256>>>(ps, net.dc_par + l * lp, di, dhi);
       }
       CU_TRY(c, cudaGetLastError());
     }
