@@ -48,7 +48,6 @@ constexpr int DC_MAX_LAYERS = 8;
 constexpr int DC_MAX_NK = 4;      // memory tokens: time token + at most 3 observation tokens
 constexpr int DC_MAX_NKH = 16;    // folded cross-attention: (memory token, head) pairs
 constexpr int DC_CHUNK = 16384;   // bytes of a ring slot
-constexpr int DC_MIN_SLOTS = 4;   // the chunks of one pass over a matrix must be resident together
 constexpr int DC_MAX_SLOTS = 8;
 
 __device__ __forceinline__ uint32_t dc_mapa(uint32_t addr, uint32_t rank) {
@@ -87,6 +86,21 @@ __host__ __device__ constexpr int dc_slab_off(int d, int dh, int s) { int o = 0;
 __host__ __device__ constexpr int dc_layer_bytes(int d, int dh) { return dc_slab_off(d, dh, 6); }
 // floats of a layer's parameters in a CTA: 6 LayerNorm vectors, bo, bo2, b2 (whole), its biases of slab 0, of slab 2, of slab 4
 __host__ __device__ constexpr int dc_par_floats(int d, int dh) { return 9 * d + 2 * dh + d / DC_CS + d / 2 + dh; }
+// column tiles of a slab that a warp takes in one pass over it: all of them where that is at most 4 tiles of 128 k or 3 of 256 (the
+// accumulators, and the chunks of a pass, which are resident together)
+__host__ __device__ constexpr int dc_tiles_per_warp(int d, int dh, int s) {
+  const int per = (dc_slab_rows(d, dh, s) / 8 + DC_WARPS - 1) / DC_WARPS, most = dc_slab_k(d, s) <= 128 ? 4 : 3;
+  return per <= most ? per : (most == 3 ? 2 : most);
+}
+__host__ __device__ constexpr int dc_min_slots(int d, int dh) {      // chunks of the largest pass
+  int most = 0;
+  for (int s = 0; s < 6; ++s) {
+    const int nt = dc_slab_rows(d, dh, s) / 8, pt = dc_tiles_per_warp(d, dh, s) * DC_WARPS;
+    const int n = ((nt < pt ? nt : pt) * dc_slab_k(d, s) * 16 + DC_CHUNK - 1) / DC_CHUNK;
+    most = n > most ? n : most;
+  }
+  return most;
+}
 // element offset of weight (n, k) inside its slab
 __host__ __device__ inline int dc_frag_index(int n, int k, int rows, int K) {
   const int KC = K < 256 ? K : 256, kc = k / KC, kk = k % KC, tile = n >> 3, g = n & 7, kb = kk >> 5, r = kk & 31;
@@ -179,7 +193,7 @@ __host__ __device__ inline DcSmem dc_smem_plan(int d, int dh, int layers, int A,
   p.off_recv = take(DC_CS * DC_OWN * d * 4);                     // partial sums of the owned rows
   p.off_kq = take(DC_MAX_NKH * d * 2);                           // folded cross-attention: kq rows; otherwise keys, values of the head
   p.off_u = take(DC_MAX_NKH / 2 * d * 4);                        // u rows (head pairs in one word)
-  p.off_x = take(DC_OWN * ((A + 3) & ~3) * 4 * 2);               // latent and eps of the owned rows
+  p.off_x = take(DC_OWN * ((A + 3) & ~3) * 4 * 4);               // latent, eps, noise and sigma of the owned rows
   p.off_xr = take(DC_OWN * d * 4);                               // an owned row's normalised values, fp32
   p.off_red = take(512);                                         // row statistics [2][2][4] (mean, M2), scores [2][16]
   p.off_head = take((2 * d + A * d + 64) * 4);
@@ -189,14 +203,19 @@ __host__ __device__ inline DcSmem dc_smem_plan(int d, int dh, int layers, int A,
   if (resident) { p.total = o + layers * dc_layer_bytes(d, dh); return p; }
   const int n = (limit - o) / DC_CHUNK;
   p.n_slots = n > DC_MAX_SLOTS ? DC_MAX_SLOTS : n;
-  p.total = p.n_slots >= DC_MIN_SLOTS ? o + p.n_slots * DC_CHUNK : limit + 1;
+  p.total = p.n_slots >= dc_min_slots(d, dh) ? o + p.n_slots * DC_CHUNK : limit + 1;
   return p;
 }
 
-// One warp's k loop of a linear layer: c[t] = X[16, k32 blocks 0 .. NKB) * (column tile nt[t])^T, two accumulator chains per
-// tile.  `frag(tile, kb)` is the address of the tile's 512-byte piece for one block of 32 k.
+template <int I, int N, typename F>
+__device__ __forceinline__ void dc_passes(F f) {      // f(0), f(1), .. f(N - 1) with compile-time arguments
+  if constexpr (I < N) { f(std::integral_constant<int, I>{}); dc_passes<I + 1, N>(f); }
+}
+// One warp's k loop of a linear layer: c[t] = X[16, k32 blocks 0 .. NKB) * (its tile t)^T, two accumulator chains per
+// tile.  `frag(t, kb)` is the address of the tile's 512-byte piece for one block of 32 k.  All warps read all of X, so the loop is bound by
+// shared-memory reads (d = 256, 16 tiles: 64 KB of X and 64 KB of weights, 1024 clocks at 128 B per clock).
 template <int TPW, int NKB, typename Frag>
-__device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, const int (&nt)[TPW], float (&c)[TPW][4], Frag frag) {
+__device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, float (&c)[TPW][4], Frag frag) {
   const int lane = threadIdx.x & 31;
   float e[TPW][4];
 #pragma unroll
@@ -209,7 +228,7 @@ __device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, const i
     ldmatrix_x4(a2, xa + kb * 32 + 16);
 #pragma unroll
     for (int t = 0; t < TPW; ++t) {
-      const uint4 w = *reinterpret_cast<const uint4*>(frag(t, nt[t], kb) + lane * 16);
+      const uint4 w = *reinterpret_cast<const uint4*>(frag(t, kb) + lane * 16);
       mma_bf16_16816(c[t], a1, w.x, w.y);
       mma_bf16_16816(e[t], a2, w.z, w.w);
     }
@@ -279,17 +298,18 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
     for (int i = threadIdx.x; i < A; i += DC_COMPUTE) shead[2 * d + A * d + i] = P.b_out[i];
     uint32_t* z = reinterpret_cast<uint32_t*>(dc_smem);              // xa, q, o, f: one behind the other
     for (int i = threadIdx.x; i < pl.off_recv / 4; i += DC_COMPUTE) z[i] = 0u;
-    for (int i = threadIdx.x; i < 2 * DC_OWN * AP; i += DC_COMPUTE) sx[i] = 0.f;
+    for (int i = threadIdx.x; i < 4 * DC_OWN * AP; i += DC_COMPUTE) sx[i] = 0.f;
   }
   cluster.sync();
   const float *lnf_g = shead, *lnf_b = shead + d, *woutT = shead + 2 * d, *bout = shead + 2 * d + A * d;
 
   // forwards this cluster runs (the same for every CTA and every warp)
-  auto window = [&](int slot) {                // drafted steps of a slot in mode 0
+  const int C = P.mode == 1 ? P.C : 1;
+  auto steps = [&](int slot, int cand) {       // forwards of a work item: 0 for a finished slot or a candidate beyond t = 0
     const int tb = P.t[slot];
+    if (P.mode == 1) return tb >= 0 && cand <= tb ? 1 : 0;
     return tb < 0 ? 0 : min(min(P.K, env_draft_cap(P.envp, item_of(P.item, slot), tb, P.K, P.T)), tb);
   };
-  auto live_cand = [&](int w) { const int tb = P.t[w / P.C]; return tb >= 0 && w % P.C <= tb; };
 
   if (warp == DC_WARPS) {
     // ================================================================ producer: weights, parameters, tables, ahead of the computation
@@ -314,14 +334,15 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       };
       auto layer_load = [&](int l, int skip, int most) {      // chunks skip .. of layer l, at most `most` of them, in the order of use
         int at = 0;
-        const uint8_t* src = wsrc(l);
-        constexpr int order[6] = {0, 1, 4, 5, 2, 3};
-#pragma unroll
+#pragma unroll 1
         for (int i = 0; i < 6; ++i) {
-          const int s = order[i];
-          if (s >= 4 && n_slabs == 4) continue;
-          for (int o = 0; o < dc_slab_bytes(d, DH, s); o += DC_CHUNK, ++at)
-            if (at >= skip && at < skip + most) chunk_load(src + dc_slab_off(d, DH, s) + o, min(DC_CHUNK, dc_slab_bytes(d, DH, s) - o));
+          const int s = i < 2 ? i : (i < 4 ? i + 2 : i - 2);      // 0, 1, (4, 5,) 2, 3
+          if (s >= n_slabs) continue;
+          const uint8_t* src = wsrc(l) + dc_slab_off(d, DH, s);
+          const int bytes = dc_slab_bytes(d, DH, s);
+#pragma unroll 1
+          for (int o = 0; o < bytes; o += DC_CHUNK, ++at)
+            if (at >= skip && at < skip + most) chunk_load(src + o, min(DC_CHUNK, bytes - o));
         }
       };
       if (resident) {
@@ -339,33 +360,29 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       pdl_wait();
       uint32_t n_tab = 0;
       bool first = true;
-      auto serve = [&](int tau, int env) {      // everything one forward consumes
-        for (int l = 0; l < L && !failed; ++l) {
-          if (!resident && !first) par_load(l);
-          if (P.fold) {
-            if (n_tab > 0) wait_bar(bar_of(24), (n_tab - 1) & 1u);
-            if (failed) return;
-            ++n_tab;
-            const uint32_t tok = (uint32_t)(HEADS * d * 2);      // bytes of a memory token's kq rows, and of its u rows
-            const size_t stride = (size_t)L * HEADS * d, lay = (size_t)l * HEADS * d;
-            ptx::mbar_expect_tx(bar_of(7), 2u * (uint32_t)NK * tok);
-            for (int j = 0; j < NK; ++j) {
-              const size_t at = (j == 0 ? (size_t)tau : (size_t)env * P.To + (j - 1)) * stride + lay;
-              dc_bulk_load(sbase + pl.off_kq + (uint32_t)j * tok, (j == 0 ? P.kq_time : P.kq_obs) + at, tok, bar_of(7));
-              dc_bulk_load(sbase + pl.off_u + (uint32_t)j * tok, (j == 0 ? P.ut_time : P.ut_obs) + at, tok, bar_of(7));
+      for (int w = cid; w < P.B * C && !failed; w += ncl) {
+        const int slot_w = w / C, cand = w - slot_w * C, ke = steps(slot_w, cand), env = item_of(P.item, slot_w);
+        for (int k = 1; k <= ke && !failed; ++k) {
+          const int tau = P.t[slot_w] - cand - k + 1;
+          for (int l = 0; l < L && !failed; ++l) {      // everything one forward consumes
+            if (!resident && !first) par_load(l);
+            if (P.fold) {
+              if (n_tab > 0) wait_bar(bar_of(24), (n_tab - 1) & 1u);
+              if (failed) break;
+              ++n_tab;
+              const uint32_t tok = (uint32_t)(HEADS * d * 2);      // bytes of a memory token's kq rows, and of its u rows
+              const size_t stride = (size_t)L * HEADS * d, lay = (size_t)l * HEADS * d;
+              ptx::mbar_expect_tx(bar_of(7), 2u * (uint32_t)NK * tok);
+#pragma unroll 1
+              for (int j = 0; j < NK; ++j) {
+                const size_t at = (j == 0 ? (size_t)tau : (size_t)env * P.To + (j - 1)) * stride + lay;
+                dc_bulk_load(sbase + pl.off_kq + (uint32_t)j * tok, (j == 0 ? P.kq_time : P.kq_obs) + at, tok, bar_of(7));
+                dc_bulk_load(sbase + pl.off_u + (uint32_t)j * tok, (j == 0 ? P.ut_time : P.ut_obs) + at, tok, bar_of(7));
+              }
             }
+            if (!resident) layer_load(l, first ? pre_chunks : 0, chunks_layer);
+            first = false;
           }
-          if (!resident) layer_load(l, first ? pre_chunks : 0, chunks_layer);
-          first = false;
-        }
-      };
-      if (P.mode == 1) {
-        for (int w = cid; w < P.B * P.C && !failed; w += ncl)
-          if (live_cand(w)) serve(P.t[w / P.C] - w % P.C, item_of(P.item, w / P.C));
-      } else {
-        for (int s = cid; s < P.B && !failed; s += ncl) {
-          const int ke = window(s);
-          for (int k = 1; k <= ke && !failed; ++k) serve(P.t[s] - k + 1, item_of(P.item, s));
         }
       }
       if (first && !resident) {                 // nothing to do: let the copies land
@@ -474,67 +491,48 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
   // ---- ring, consumer side: chunk i of the pass that begins sits in slot (cslot + i) % n_slots
   int cslot = 0;
   uint32_t cround = 0;
-  auto chunk_wait = [&](int i) {
-    const int s = cslot + i;
-    wait_bar(bar_of(8 + (s >= n_slots ? s - n_slots : s)), (cround + (s >= n_slots ? 1u : 0u)) & 1u);
-  };
-  auto chunk_addr = [&](int i) { const int s = cslot + i; return dc_smem + pl.off_w + (size_t)(s >= n_slots ? s - n_slots : s) * DC_CHUNK; };
-  auto chunks_release = [&](int n) {           // this warp is done with the pass's n chunks
+  auto slot_of = [&](int i) { const int s = cslot + i; return s >= n_slots ? s - n_slots : s; };
+  auto chunks_wait = [&](int n) {              // the pass's n chunks are there (one lane each)
+    if (lane < n) wait_bar(bar_of(8 + slot_of(lane)), (cround + (cslot + lane >= n_slots ? 1u : 0u)) & 1u);
     __syncwarp();
-    for (int i = 0; i < n; ++i) {
-      if (lane == 0) {      // having seen the chunk, whether or not this warp read it: a warp without tiles stays within the round
-        wait_bar(bar_of(8 + cslot), cround & 1u);
-        ptx::mbar_arrive(bar_of(16 + cslot));
-      }
-      if (++cslot == n_slots) { cslot = 0; ++cround; }
-    }
   };
-  // Y = X W^T for slab S of layer l, up to TPW tiles per warp and pass (tile warp + 8 t of the pass), `done(tile, accumulators)`
-  // per finished tile.  A pass is at most four chunks.
+  auto chunk_addr = [&](int i) { return dc_smem + pl.off_w + (size_t)slot_of(i) * DC_CHUNK; };
+  auto chunks_release = [&](int n) {           // this warp is done with them
+    __syncwarp();
+    if (lane < n) ptx::mbar_arrive(bar_of(16 + slot_of(lane)));
+    cslot += n;
+    if (cslot >= n_slots) { cslot -= n_slots; ++cround; }
+  };
+  // Y = X W^T for slab S of layer l, tile warp + 8 t of a pass; `done(tile, accumulators)` per finished tile
   auto linear = [&](auto slab_c, int l, const __nv_bfloat16* X, int px, auto done) {
     constexpr int S = decltype(slab_c)::value;
     constexpr int K = dc_slab_k(d, S), NT = dc_slab_rows(d, DH, S) / 8, NKB = K / 32, TB = K * 16;      // TB: bytes of a tile
-    constexpr int TPW = NT >= 32 && K <= 128 ? 4 : 2, PT = TPW * DC_WARPS;                                          // tiles of a pass
-    static_assert(K <= 256 && PT * TB <= 4 * DC_CHUNK, "a pass is at most four chunks");
+    constexpr int TPW = dc_tiles_per_warp(d, DH, S), PT = TPW * DC_WARPS;                               // tiles of a pass
     const uint8_t* wres = dc_smem + pl.off_w + (size_t)l * dc_layer_bytes(d, DH) + dc_slab_off(d, DH, S);
+    dc_passes<0, (NT + PT - 1) / PT>([&](auto pass_c) {
+      constexpr int t0 = decltype(pass_c)::value * PT, N = NT - t0 < PT ? NT - t0 : PT, NCH = (N * TB + DC_CHUNK - 1) / DC_CHUNK;
+      constexpr int T1 = (N + DC_WARPS - 1) / DC_WARPS;      // tiles of the busiest warps; the others have one less
+      if (!resident) chunks_wait(NCH);
+      auto run = [&](auto tiles_c) {
+        constexpr int T = decltype(tiles_c)::value;
+        if constexpr (T > 0) {
+          const uint8_t* base[T];
 #pragma unroll
-    for (int t0 = 0; t0 < NT; t0 += PT) {
-      constexpr int FULL = PT;
-      const int n_pass = NT - t0 < FULL ? NT - t0 : FULL;                                               // compile-time after unrolling
-      const int nch = (n_pass * TB + DC_CHUNK - 1) / DC_CHUNK;
-      const uint8_t* base[TPW];
-      int nt[TPW];
-#pragma unroll
-      for (int t = 0; t < TPW; ++t) {
-        nt[t] = warp + t * DC_WARPS;
-        if (nt[t] < n_pass) {
-          const int o = nt[t] * TB;
-          if (resident) base[t] = wres + t0 * TB + o;
-          else { chunk_wait(o / DC_CHUNK); base[t] = chunk_addr(o / DC_CHUNK) + o % DC_CHUNK; }
-        } else base[t] = nullptr;
-      }
-      __syncwarp();
-      auto frag = [&](int t, int, int kb) { return base[t] + kb * 512; };
-      float c[TPW][4];
-      int have = 0;
-#pragma unroll
-      for (int t = 0; t < TPW; ++t) have += nt[t] < n_pass ? 1 : 0;                                    // warp-uniform
-      if (have == TPW) dc_kloop<TPW, NKB>(X, px, nt, c, frag);
-      else if (have > 0) {      // a ragged pass: tile by tile
-#pragma unroll
-        for (int t = 0; t < TPW; ++t)
-          if (t < have) {
-            const int one[1] = {nt[t]};
-            float c1[1][4];
-            dc_kloop<1, NKB>(X, px, one, c1, [&](int, int, int kb) { return base[t] + kb * 512; });
-            c[t][0] = c1[0][0]; c[t][1] = c1[0][1]; c[t][2] = c1[0][2]; c[t][3] = c1[0][3];
+          for (int t = 0; t < T; ++t) {
+            const int o = (warp + t * DC_WARPS) * TB;
+            base[t] = resident ? wres + t0 * TB + o : chunk_addr(o / DC_CHUNK) + o % DC_CHUNK;
           }
-      }
-      if (!resident) chunks_release(nch);
+          float c[T][4];
+          dc_kloop<T, NKB>(X, px, c, [&](int t, int kb) { return base[t] + kb * 512; });
+          if (!resident) chunks_release(NCH);
 #pragma unroll
-      for (int t = 0; t < TPW; ++t)
-        if (nt[t] < n_pass) done(t0 + nt[t], c[t]);
-    }
+          for (int t = 0; t < T; ++t) done(t0 + warp + t * DC_WARPS, c[t]);
+        } else if (!resident) chunks_release(NCH);
+      };
+      if constexpr (N % DC_WARPS == 0) run(std::integral_constant<int, T1>{});
+      else if (warp < N - (T1 - 1) * DC_WARPS) run(std::integral_constant<int, T1>{});
+      else run(std::integral_constant<int, T1 - 1>{});
+    });
   };
   // a finished tile with bias (and GELU) as bf16 into a local buffer
   auto keep = [&](__nv_bfloat16* dst, int pitch, int tile, const float (&c)[4], const float* bias, bool gelu) {
@@ -693,30 +691,26 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
           return make_float4(lo.x, lo.y, hi.x, hi.y);
         }, [&](int r, int n, float v) { sscore[r * DC_MAX_NKH + n] = v + cst; });
         dc_sync();
-        float pr[DC_MAX_NKH];
+        // softmax over the memory tokens of each head, lane n (and n + 16) for (token, head) pair n of the warp's row
+        float p = (lane & 15) < NKH ? sscore[row * DC_MAX_NKH + (lane & 15)] : -INFINITY, m = p;
 #pragma unroll
-        for (int n = 0; n < DC_MAX_NKH; ++n) pr[n] = n < NKH ? sscore[row * DC_MAX_NKH + n] : -INFINITY;
+        for (int o = HEADS; o < DC_MAX_NKH; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        p = __expf(p - m);
+        float sum = p;
 #pragma unroll
-        for (int hh = 0; hh < HEADS && hh < DC_MAX_NKH; ++hh) {
-          float m = -INFINITY, s = 0.f;
-#pragma unroll
-          for (int n = hh; n < DC_MAX_NKH; n += HEADS) m = fmaxf(m, pr[n]);
-#pragma unroll
-          for (int n = hh; n < DC_MAX_NKH; n += HEADS) { pr[n] = __expf(pr[n] - m); s += pr[n]; }
-          const float inv = 1.0f / s;
-#pragma unroll
-          for (int n = hh; n < DC_MAX_NKH; n += HEADS) pr[n] *= inv;
-        }
+        for (int o = HEADS; o < DC_MAX_NKH; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        p /= sum;
         float o[V2];
 #pragma unroll
         for (int j = 0; j < V2; ++j) o[j] = 0.f;
 #pragma unroll
         for (int q = 0; q < DC_MAX_NKH / 2; ++q)
           if (2 * q < NKH) {
+            const float p0 = __shfl_sync(0xffffffffu, p, 2 * q), p1 = __shfl_sync(0xffffffffu, p, 2 * q + 1);
 #pragma unroll
             for (int j = 0; j < V2; ++j) {
               const float2 u2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(su + q * d + c0 + j));
-              o[j] = __fmaf_rn(pr[2 * q], u2.x, __fmaf_rn(pr[2 * q + 1], u2.y, o[j]));
+              o[j] = __fmaf_rn(p0, u2.x, __fmaf_rn(p1, u2.y, o[j]));
             }
           }
         __syncwarp();
@@ -792,52 +786,43 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
   const int e_own = (int)threadIdx.x - 128, e_row = e_own >= 0 ? e_own / A : 0;
   const int e_idx = e_own >= 0 && e_row < DC_OWN && DC_OWN * rank + e_row < H ? (DC_OWN * rank + e_row) * A + e_own % A : -1;
   float* e_x = sx + e_row * AP + (e_own >= 0 ? e_own % A : 0);
-  const float* e_eps = seps + e_row * AP + (e_own >= 0 ? e_own % A : 0);
+  const int e_eps = DC_OWN * AP, e_z = 2 * e_eps, e_sig = 3 * e_eps;      // from there to its eps, noise, sigma
 
-  if (P.mode == 1) {      // verification: one forward per (slot, candidate), the whole batch in one wave of clusters
-    for (int w = cid; w < P.B * P.C; w += ncl) {
-      if (!live_cand(w)) continue;                // finished slot, or a candidate beyond t = 0 (same for every CTA)
-      const int slot = w / P.C, cand = w % P.C;
-      if (e_idx >= 0) *e_x = P.xt[slot * P.xs_b + (long long)cand * D + e_idx];
-      dc_sync();
-      forward(P.t[slot] - cand, item_of(P.item, slot), [] {});
-      if (e_idx >= 0) P.eps[slot * P.es_b + (long long)cand * D + e_idx] = *e_eps;
-    }
-  } else {
-    for (int slot = cid; slot < P.B; slot += ncl) {
-      const int tb = P.t[slot], ke = window(slot);
-      const int env = item_of(P.item, slot);     // request served by this slot: its noise streams, obs K/V, parameters
-      float* xt_b = P.xt + slot * P.xs_b;
-      float* mh_b = P.muhat + slot * P.ms_b;
-      float xv = 0.f;
-      if (e_idx >= 0) { xv = xt_b[e_idx]; *e_x = xv; }
-      dc_sync();
-      for (int k = 1; k <= P.K; ++k) {
-        const int tau = tb - k + 1;
-        if (k > ke) {                            // beyond K_eff: carry the latent along (same for every CTA)
-          if (e_idx >= 0) { mh_b[(size_t)(k - 1) * D + e_idx] = xv; xt_b[(size_t)k * D + e_idx] = xv; }
-          continue;
+  // drafting: one slot after the other, K steps each; verification: one forward per (slot, candidate)
+  const bool verify = P.mode == 1;
+  for (int w = cid; w < P.B * C; w += ncl) {
+    const int slot = w / C, cand = w - slot * C, ke = steps(slot, cand), tb = P.t[slot] - cand;
+    const int env = item_of(P.item, slot);       // request served by this slot: its noise streams, obs K/V, parameters
+    float* xt_b = P.xt + slot * P.xs_b + (long long)cand * D;
+    float* mh_b = P.muhat + slot * P.ms_b;
+    float xv = 0.f;
+    if (e_idx >= 0) { xv = xt_b[e_idx]; *e_x = xv; }
+    dc_sync();
+    for (int k = 1; k <= ke; ++k) {
+      const int tau = tb - k + 1;
+      forward(tau, env, [&] {
+        if (e_idx >= 0 && !verify) {
+          float z4[4];
+          normal4(seed, (uint32_t)env, STREAM_XI, (uint32_t)tau, (uint32_t)(e_idx >> 2), z4);
+          const int j = e_idx & 3;
+          e_x[e_z] = j == 0 ? z4[0] : (j == 1 ? z4[1] : (j == 2 ? z4[2] : z4[3]));      // (kept in registers, it was computed where it is used)
+          e_x[e_sig] = P.S.sigma[tau];
         }
-        float z = 0.f, sig = 0.f;
-        forward(tau, env, [&] {
-          if (e_idx >= 0) {
-            float z4[4];
-            normal4(seed, (uint32_t)env, STREAM_XI, (uint32_t)tau, (uint32_t)(e_idx >> 2), z4);
-            const int j = e_idx & 3;
-            z = j == 0 ? z4[0] : (j == 1 ? z4[1] : (j == 2 ? z4[2] : z4[3]));
-            sig = P.S.sigma[tau];
-          }
-        });
-        if (e_idx >= 0) {                        // scheduler step: mu^_k, x~_k = mu^_k + sigma_tau xi_tau
-          const float m = posterior_mean(P.S, xv, *e_eps, tau);
-          xv = ddpm_sample(m, sig, z);
+      });
+      if (e_idx >= 0) {
+        if (verify) P.eps[slot * P.es_b + (long long)cand * D + e_idx] = e_x[e_eps];
+        else {                                   // scheduler step: mu^_k, x~_k = mu^_k + sigma_tau xi_tau
+          const float m = posterior_mean(P.S, xv, e_x[e_eps], tau);
+          xv = ddpm_sample(m, e_x[e_sig], e_x[e_z]);
           *e_x = xv;
           mh_b[(size_t)(k - 1) * D + e_idx] = m;
           xt_b[(size_t)k * D + e_idx] = xv;
         }
-        dc_sync();
       }
+      dc_sync();
     }
+    if (!verify && e_idx >= 0)                   // beyond K_eff: carry the latent along
+      for (int k = ke + 1; k <= P.K; ++k) { mh_b[(size_t)(k - 1) * D + e_idx] = xv; xt_b[(size_t)k * D + e_idx] = xv; }
   }
   if (failed) { const long long t0 = clock64(); while (clock64() - t0 < 400000ll) { } }      // copies in flight land first
   cluster.sync();      // no CTA leaves while another may still write into its shared memory
