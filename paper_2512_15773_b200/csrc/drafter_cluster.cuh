@@ -212,14 +212,27 @@ __device__ __forceinline__ void dc_passes(F f) {      // f(0), f(1), .. f(N - 1)
   if constexpr (I < N) { f(std::integral_constant<int, I>{}); dc_passes<I + 1, N>(f); }
 }
 // One warp's k loop of a linear layer: c[t] = X[16, k32 blocks 0 .. NKB) * (its tile t)^T, two accumulator chains per
-// tile.  `frag(t, kb)` is the address of the tile's 512-byte piece for one block of 32 k.  All warps read all of X, so the loop is bound by
-// shared-memory reads (d = 256, 16 tiles: 64 KB of X and 64 KB of weights, 1024 clocks at 128 B per clock).
-template <int TPW, int NKB, typename Frag>
-__device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, float (&c)[TPW][4], Frag frag) {
+// tile; base[t] is the shared-memory address of this lane's words of the tile.  All warps read all of X, so the loop is bound by
+// shared-memory reads (d = 256, 16 tiles: 64 KB of X and 64 KB of weights, 1024 clocks at 128 B per clock); `ready` says when X
+// may be read, and the first half of the weights is fetched before that, while X is still on its way from the other CTAs.
+__device__ __forceinline__ uint4 dc_lds16(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+template <int TPW, int NKB, typename Ready>
+__device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, float (&c)[TPW][4], const uint32_t (&base)[TPW], Ready ready) {
+  constexpr int PRE = NKB < 4 ? NKB : 4;
   const int lane = threadIdx.x & 31;
   float e[TPW][4];
+  uint4 pre[TPW][PRE];
 #pragma unroll
-  for (int t = 0; t < TPW; ++t) { c[t][0] = c[t][1] = c[t][2] = c[t][3] = 0.f; e[t][0] = e[t][1] = e[t][2] = e[t][3] = 0.f; }
+  for (int t = 0; t < TPW; ++t) {
+    c[t][0] = c[t][1] = c[t][2] = c[t][3] = 0.f; e[t][0] = e[t][1] = e[t][2] = e[t][3] = 0.f;
+#pragma unroll
+    for (int kb = 0; kb < PRE; ++kb) pre[t][kb] = dc_lds16(base[t] + kb * 512);
+  }
+  ready();
   const __nv_bfloat16* xa = X + (lane & 15) * px + 8 * (lane >> 4);
 #pragma unroll
   for (int kb = 0; kb < NKB; ++kb) {
@@ -228,7 +241,7 @@ __device__ __forceinline__ void dc_kloop(const __nv_bfloat16* X, int px, float (
     ldmatrix_x4(a2, xa + kb * 32 + 16);
 #pragma unroll
     for (int t = 0; t < TPW; ++t) {
-      const uint4 w = *reinterpret_cast<const uint4*>(frag(t, kb) + lane * 16);
+      const uint4 w = kb < PRE ? pre[t][kb < PRE ? kb : 0] : dc_lds16(base[t] + kb * 512);
       mma_bf16_16816(c[t], a1, w.x, w.y);
       mma_bf16_16816(e[t], a2, w.z, w.w);
     }
@@ -489,6 +502,7 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
     for (int j = 0; j < V2; ++j) x[j] = x[j] * gam[c0 + j] + bet[c0 + j];
   };
   // ---- ring, consumer side: chunk i of the pass that begins sits in slot (cslot + i) % n_slots
+  const uint32_t ring_end = resident ? 0xffffffffu : ring + (uint32_t)n_slots * DC_CHUNK;
   int cslot = 0;
   uint32_t cround = 0;
   auto slot_of = [&](int i) { const int s = cslot + i; return s >= n_slots ? s - n_slots : s; };
@@ -496,19 +510,18 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
     if (lane < n) wait_bar(bar_of(8 + slot_of(lane)), (cround + (cslot + lane >= n_slots ? 1u : 0u)) & 1u);
     __syncwarp();
   };
-  auto chunk_addr = [&](int i) { return dc_smem + pl.off_w + (size_t)slot_of(i) * DC_CHUNK; };
   auto chunks_release = [&](int n) {           // this warp is done with them
     __syncwarp();
     if (lane < n) ptx::mbar_arrive(bar_of(16 + slot_of(lane)));
     cslot += n;
     if (cslot >= n_slots) { cslot -= n_slots; ++cround; }
   };
-  // Y = X W^T for slab S of layer l, tile warp + 8 t of a pass; `done(tile, accumulators)` per finished tile
-  auto linear = [&](auto slab_c, int l, const __nv_bfloat16* X, int px, auto done) {
+  // Y = X W^T for slab S of layer l, tile warp + 8 t of a pass; X may be read after `ready()`, which every warp runs once; `done(tile, accumulators)`
+  // per finished tile
+  auto linear = [&](auto slab_c, int l, const __nv_bfloat16* X, int px, auto ready, auto done) {
     constexpr int S = decltype(slab_c)::value;
     constexpr int K = dc_slab_k(d, S), NT = dc_slab_rows(d, DH, S) / 8, NKB = K / 32, TB = K * 16;      // TB: bytes of a tile
     constexpr int TPW = dc_tiles_per_warp(d, DH, S), PT = TPW * DC_WARPS;                               // tiles of a pass
-    const uint8_t* wres = dc_smem + pl.off_w + (size_t)l * dc_layer_bytes(d, DH) + dc_slab_off(d, DH, S);
     dc_passes<0, (NT + PT - 1) / PT>([&](auto pass_c) {
       constexpr int t0 = decltype(pass_c)::value * PT, N = NT - t0 < PT ? NT - t0 : PT, NCH = (N * TB + DC_CHUNK - 1) / DC_CHUNK;
       constexpr int T1 = (N + DC_WARPS - 1) / DC_WARPS;      // tiles of the busiest warps; the others have one less
@@ -516,18 +529,24 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       auto run = [&](auto tiles_c) {
         constexpr int T = decltype(tiles_c)::value;
         if constexpr (T > 0) {
-          const uint8_t* base[T];
+          // a resident slab lies in one piece; a pass in the ring may wrap
+          const uint32_t first = ring + (uint32_t)(warp * TB + lane * 16) +
+                                 (resident ? (uint32_t)(l * dc_layer_bytes(d, DH) + dc_slab_off(d, DH, S) + t0 * TB) : (uint32_t)cslot * DC_CHUNK);
+          uint32_t base[T];
 #pragma unroll
           for (int t = 0; t < T; ++t) {
-            const int o = (warp + t * DC_WARPS) * TB;
-            base[t] = resident ? wres + t0 * TB + o : chunk_addr(o / DC_CHUNK) + o % DC_CHUNK;
+            const uint32_t at = first + t * DC_WARPS * TB;
+            base[t] = at >= ring_end ? at - (uint32_t)n_slots * DC_CHUNK : at;
           }
           float c[T][4];
-          dc_kloop<T, NKB>(X, px, c, [&](int t, int kb) { return base[t] + kb * 512; });
+          dc_kloop<T, NKB>(X, px, c, base, [&] { if constexpr (t0 == 0) ready(); });
           if (!resident) chunks_release(NCH);
 #pragma unroll
           for (int t = 0; t < T; ++t) done(t0 + warp + t * DC_WARPS, c[t]);
-        } else if (!resident) chunks_release(NCH);
+        } else {
+          if constexpr (t0 == 0) ready();
+          if (!resident) chunks_release(NCH);
+        }
       };
       if constexpr (N % DC_WARPS == 0) run(std::integral_constant<int, T1>{});
       else if (warp < N - (T1 - 1) * DC_WARPS) run(std::integral_constant<int, T1>{});
@@ -602,8 +621,7 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       affine(x, ln1, ln1 + d);
       stage_begin(DC_ROWS * d * 2);
       gather_rows(x);
-      stage_end();
-      linear(std::integral_constant<int, 0>{}, l, xa, PX, [&](int tile, const float (&c)[4]) { keep(qs, PQ, tile, c, bqkv, false); });
+      linear(std::integral_constant<int, 0>{}, l, xa, PX, stage_end, [&](int tile, const float (&c)[4]) { keep(qs, PQ, tile, c, bqkv, false); });
       dc_sync();
       if (warp < VW / 16) {
         // scores of all 16 rows by each of these warps, then 16 of the CTA's value columns
@@ -659,7 +677,7 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       } else if (l == 0 && warp >= 4) rest();
       dc_sync();
       stage_begin(DC_CS * DC_OWN * d * 4);
-      linear(std::integral_constant<int, 1>{}, l, os, PO, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
+      linear(std::integral_constant<int, 1>{}, l, os, PO, [] {}, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
       float cst = 0.f;      // constant of the score that this lane will finish (at most 32 scores: four per warp)
       if (P.fold) {
         const int p = warp + lane * DC_WARPS, n = p >> 1, j = n / HEADS;
@@ -721,9 +739,7 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
         affine(x, ln2, ln2 + d);
         stage_begin(DC_ROWS * d * 2);
         gather_rows(x);
-        stage_end();
-        dc_sync();                                         // the keys / values above were written by other threads
-        linear(std::integral_constant<int, 4>{}, l, xa, PX, [&](int tile, const float (&c)[4]) { keep(qs, PQ, tile, c, bq2, false); });
+        linear(std::integral_constant<int, 4>{}, l, xa, PX, stage_end, [&](int tile, const float (&c)[4]) { keep(qs, PQ, tile, c, bq2, false); });
         dc_sync();
         if (threadIdx.x < 4 * DC_ROWS) {                   // four lanes per query row, each a quarter of the head and of the value columns
           const float* skv = reinterpret_cast<const float*>(dc_smem + pl.off_kq);
@@ -753,7 +769,7 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
         }
         dc_sync();
         stage_begin(DC_CS * DC_OWN * d * 4);
-        linear(std::integral_constant<int, 5>{}, l, os, PO, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
+        linear(std::integral_constant<int, 5>{}, l, os, PO, [] {}, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
         stage_end();
         add_partials(bo2);
       }
@@ -762,11 +778,9 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       affine(x, ln3, ln3 + d);
       stage_begin(DC_ROWS * d * 2);
       gather_rows(x);
-      stage_end();
-      linear(std::integral_constant<int, 2>{}, l, xa, PX, [&](int tile, const float (&c)[4]) { keep(fs, PF, tile, c, b1, true); });
-      dc_sync();
+      linear(std::integral_constant<int, 2>{}, l, xa, PX, stage_end, [&](int tile, const float (&c)[4]) { keep(fs, PF, tile, c, b1, true); });
       stage_begin(DC_CS * DC_OWN * d * 4);
-      linear(std::integral_constant<int, 3>{}, l, fs, PF, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
+      linear(std::integral_constant<int, 3>{}, l, fs, PF, dc_sync, [&](int tile, const float (&c)[4]) { send_partial(tile, c); });
       stage_end();
       add_partials(b2);
       if (!resident) { __syncwarp(); if (lane == 0) ptx::mbar_arrive(bar_of(5 + (int)(n_layer & 1u))); }
