@@ -1285,10 +1285,10 @@ bool cluster_drafter_fits(const tsdp_config_t& cfg, const tsdp_net_t& n, int* sm
 bool use_cluster_drafter(const tsdp_ctx* c, int B) {
   if (!c->dc_ok || c->cfg.drafter == 1) return false;
   if (c->cfg.drafter == 2) return true;
-  // Beyond a few waves of clusters the batched tensor-core path wins: measured about 29 us per draft step and wave
-  // with resident weights (PushT drafter) and 70-130 us with L2-streamed ones, against 100-175 us per step for the
-  // layer-by-layer path whatever the batch.
-  return B <= (c->dc_resident ? 3 : 1) * c->dc_max_clusters;
+  // Beyond a few waves of clusters (15 at a time) the layer-by-layer path wins.  Whole calls, cluster / layered: weights streamed
+  // (d = 256, conv-UNet base) 20 environments 16.5 / 21.0 ms, 32 21.8 / 22.6, (d = 512 base) 48 26.4 / 25.4; resident weights (d = 128) 24
+  // environments 8.6 / 10.5 ms, 40 10.7 / 12.5, 64 14.5 / 14.0.
+  return B <= (c->dc_resident ? 4 : 3) * c->dc_max_clusters;
 }
 
 bool use_cluster_verifier(const tsdp_ctx* c, int B, int K) {
