@@ -172,6 +172,44 @@ __host__ __device__ constexpr size_t xf_smem_bytes(int D, int nkh) {
 // `delta` is the output of the self-attention projection (bf16, bias included), which this kernel adds to the
 // residual stream before anything else: that GEMM then writes 2 bytes per element instead of doing an fp32
 // read-modify-write of the stream.
+// Mean and reciprocal standard deviation of the warp's two rows, both rows' shuffles in flight together.
+template <int V>
+__device__ __forceinline__ void xf_row_stats(const float4 (&x)[2][V], float (&mean)[2], float (&rstd)[2]) {
+  constexpr float INV = 1.0f / (128 * V);
+  float s[2], q[2];
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    float2 s2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < V; ++j) s2 = __fadd2_rn(s2, __fadd2_rn(xf_lo(x[rr][j]), xf_hi(x[rr][j])));
+    s[rr] = s2.x + s2.y;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+    s[1] += __shfl_xor_sync(0xffffffffu, s[1], o);
+  }
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    mean[rr] = s[rr] * INV;
+    const float2 nm = xf_dup(-mean[rr]);
+    float2 q2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      const float2 lo = __fadd2_rn(xf_lo(x[rr][j]), nm), hi = __fadd2_rn(xf_hi(x[rr][j]), nm);
+      q2 = __ffma2_rn(lo, lo, q2); q2 = __ffma2_rn(hi, hi, q2);
+    }
+    q[rr] = q2.x + q2.y;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    q[0] += __shfl_xor_sync(0xffffffffu, q[0], o);
+    q[1] += __shfl_xor_sync(0xffffffffu, q[1], o);
+  }
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) rstd[rr] = rsqrtf(q[rr] * INV + 1e-5f);
+}
+
 template <int D>
 __global__ void __launch_bounds__(XF_THREADS, 3)
 xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta, XfoldTables tb, const float* __restrict__ bo2,
@@ -185,6 +223,7 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
   constexpr int V = D / 128;
   extern __shared__ __align__(16) unsigned char xf_smem[];
   const int NK = 1 + To, NKH = NK * heads;
+  const int hs = __ffs(heads) - 1;         // heads divides D: a power of two, at least 2
   __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(xf_smem);
   unsigned char* region = xf_smem + (size_t)16 * LDA * 2;
   __nv_bfloat16* sK = reinterpret_cast<__nv_bfloat16*>(region);
@@ -192,24 +231,38 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
   float* sS = reinterpret_cast<float*>(sU + (size_t)(NKH / 2) * LDU);      // [4][16][XF_MAXN]
   __nv_bfloat16* sP = reinterpret_cast<__nv_bfloat16*>(sS + 4 * 16 * XF_MAXN);
   const int n = blockIdx.x;
-  if (n >= cand_count(cm, gridDim.x)) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, tg = lane & 3;
+  float* xc = x + (size_t)n * H * D;
+  const __nv_bfloat16* dc = delta + (size_t)n * H * D;
+  // The rows of the stream and of delta depend on nothing but the block's number (a block past the live candidates reads rows that
+  // exist): they are asked for first, beside the candidate's place in the list, and what depends on that place comes after.
+  const int listed = cm.list ? cm.list[n] : 0;
+  float4 xr[2][V];                             // rows 2 warp, 2 warp + 1 of the stream with delta added: kept until phase 5
+  uint2 dv[2][V];
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    const int r = min(2 * warp + rr, H - 1);
+#pragma unroll
+    for (int j = 0; j < V; ++j) xr[rr][j] = reinterpret_cast<const float4*>(xc + (size_t)r * D)[j * 32 + lane];
+#pragma unroll
+    for (int j = 0; j < V; ++j) dv[rr][j] = reinterpret_cast<const uint2*>(dc + (size_t)r * D)[j * 32 + lane];
+  }
+  if (n >= cand_count(cm, gridDim.x)) return;
   int b, cnd;
-  cand_decode(cm, n, b, cnd);
+  if (cm.list) { b = listed >> 6; cnd = listed & 63; }
+  else cand_decode(cm, n, b, cnd);
   int tau = cm.t[b] - cm.koff - cnd;
   tau = max(0, min(Tsteps - 1, tau));
   const int item = item_of(cm.item, b);
   const size_t tok_stride = (size_t)L * heads * D;      // kq / ut elements per memory token
   const size_t lay_off = (size_t)layer * heads * D;
-  float* xc = x + (size_t)n * H * D;
-  const __nv_bfloat16* dc = delta + (size_t)n * H * D;
 
   // ---- 0: tables of this candidate's memory tokens, one row per warp at a time
   {
     const int hp = heads >> 1;
     for (int row = warp; row < NKH; row += XF_WARPS) {
-      const int jt = row / heads, h = row - jt * heads;
+      const int jt = row >> hs, h = row & (heads - 1);
       const __nv_bfloat16* sr = (jt == 0 ? tb.kq_time + (size_t)tau * tok_stride : tb.kq_obs + ((size_t)item * To + (jt - 1)) * tok_stride) +
                                 lay_off + (size_t)h * D;
       __nv_bfloat16* dr = sK + (size_t)row * LDA;
@@ -219,7 +272,7 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
     }
     xf_cp_commit();
     for (int row = warp; row < NKH / 2; row += XF_WARPS) {
-      const int jt = row / hp, q = row - jt * hp;
+      const int jt = row >> (hs - 1), q = row & (hp - 1);
       const __nv_bfloat16* sr = (jt == 0 ? tb.ut_time + (size_t)tau * tok_stride : tb.ut_obs + ((size_t)item * To + (jt - 1)) * tok_stride) +
                                 lay_off + (size_t)q * D * 2;
       uint32_t* dr = sU + (size_t)row * LDU;
@@ -231,11 +284,10 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
 
   // ---- 1: LayerNorm statistics, normalised rows to shared memory
   for (int i = threadIdx.x; i < 16 * LDP / 2; i += XF_THREADS) reinterpret_cast<uint32_t*>(sP)[i] = 0u;
-  float4 xr[2][V];                             // rows 2 warp, 2 warp + 1 of the stream with delta added: kept until phase 5
   // the score constants this thread needs in phase 3: in flight from here on
   float cst[XF_MAXNK];
   {
-    const int h = threadIdx.x % heads;
+    const int h = threadIdx.x & (heads - 1);
 #pragma unroll
     for (int j = 0; j < XF_MAXNK; ++j) {
       cst[j] = 0.f;
@@ -246,45 +298,20 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
       }
     }
   }
-  {                                            // two rows per warp: all of their loads are in flight together
-    float4 v[2][V];
-#pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-      const int r = min(2 * warp + rr, H - 1);
-#pragma unroll
-      for (int j = 0; j < V; ++j) v[rr][j] = reinterpret_cast<const float4*>(xc + (size_t)r * D)[j * 32 + lane];
-    }
-    uint2 dv[2][V];
-#pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-      const int r = min(2 * warp + rr, H - 1);
-#pragma unroll
-      for (int j = 0; j < V; ++j) dv[rr][j] = reinterpret_cast<const uint2*>(dc + (size_t)r * D)[j * 32 + lane];
-    }
+  {
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr)
 #pragma unroll
-      for (int j = 0; j < V; ++j) { xf_add_bf16x4(v[rr][j], dv[rr][j]); xr[rr][j] = v[rr][j]; }
+      for (int j = 0; j < V; ++j) xf_add_bf16x4(xr[rr][j], dv[rr][j]);
+    float mean[2], rstd[2];
+    xf_row_stats<V>(xr, mean, rstd);
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
       const int r = 2 * warp + rr;
-      float2 s2 = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int j = 0; j < V; ++j) s2 = __fadd2_rn(s2, __fadd2_rn(xf_lo(v[rr][j]), xf_hi(v[rr][j])));
-      const float mean = warp_sum(s2.x + s2.y) / D;
-      const float2 nm = xf_dup(-mean);
-      float2 q2 = make_float2(0.f, 0.f);
-      float2 lo[V], hi[V];
+      const float2 nm = xf_dup(-mean[rr]), rs2 = xf_dup(r < H ? rstd[rr] : 0.f);      // rows past H enter the products as zeros
 #pragma unroll
       for (int j = 0; j < V; ++j) {
-        lo[j] = __fadd2_rn(xf_lo(v[rr][j]), nm); hi[j] = __fadd2_rn(xf_hi(v[rr][j]), nm);
-        q2 = __ffma2_rn(lo[j], lo[j], q2); q2 = __ffma2_rn(hi[j], hi[j], q2);
-      }
-      const float rstd = r < H ? rsqrtf(warp_sum(q2.x + q2.y) / D + 1e-5f) : 0.f;      // rows past H enter the products as zeros
-      const float2 rs2 = xf_dup(rstd);
-#pragma unroll
-      for (int j = 0; j < V; ++j) {
-        const float2 a = __fmul2_rn(lo[j], rs2), b = __fmul2_rn(hi[j], rs2);
+        const float2 a = __fmul2_rn(__fadd2_rn(xf_lo(xr[rr][j]), nm), rs2), b = __fmul2_rn(__fadd2_rn(xf_hi(xr[rr][j]), nm), rs2);
         uint2 pk2;
         pk2.x = pack_bf16(a.x, a.y);
         pk2.y = pack_bf16(b.x, b.y);
@@ -330,7 +357,7 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
   // ---- 3: softmax over the NK memory tokens for every (row, head)
   if (threadIdx.x < 16 * heads) {              // heads <= 16: one (row, head) per thread
     const int idx = threadIdx.x;
-    const int r = idx / heads, h = idx % heads;
+    const int r = idx >> hs, h = idx & (heads - 1);
     float s[XF_MAXNK];
 #pragma unroll
     for (int j = 0; j < XF_MAXNK; ++j) s[j] = cst[j];
@@ -355,6 +382,12 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
   }
   xf_cp_wait<0>();                             // this thread's u chunks have landed
   __syncthreads();                             // also: every warp is done with the normalised rows and the kq rows, whose memory the product reuses
+  // bo2 and the LayerNorm parameters of phase 5 start for the (now dead) partial scores: 3 D floats, each thread its own words
+  float* sB = sS;
+  static_assert(3 * D <= 4 * 16 * XF_MAXN, "phase 5 parameters fit over the partial scores");
+  for (int i = threadIdx.x; i < 3 * D / 4; i += XF_THREADS)
+    xf_cp16(sB + 4 * i, (i < D / 4 ? bo2 : (i < D / 2 ? ln3_g - D : ln3_b - 2 * D)) + 4 * i);
+  xf_cp_commit();
 
   // ---- 4: P . U for all 16 rows, warp w the output columns [w D/8, (w+1) D/8), into shared memory over the
   //         (now dead) normalised rows and kq rows
@@ -387,10 +420,7 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
       *reinterpret_cast<float2*>(sO + (g + 8) * LDO + o_base + 8 * nt + 2 * tg) = make_float2(acc[2], acc[3]);
     }
   }
-  // bo2 of this lane's columns: in flight across the barrier
-  float4 bb[V];
-#pragma unroll
-  for (int j = 0; j < V; ++j) bb[j] = __ldg(reinterpret_cast<const float4*>(bo2) + j * 32 + lane);
+  xf_cp_wait<0>();
   __syncthreads();
 
   // ---- 5: rows 2 warp, 2 warp + 1: stream + delta (registers) + product + bo2 -> the stream; LayerNorm -> ln3_out
@@ -401,39 +431,25 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
 #pragma unroll
       for (int j = 0; j < V; ++j) {
         const float4 t = *reinterpret_cast<const float4*>(sO + r * LDO + (j * 32 + lane) * 4);
+        const float4 bb = reinterpret_cast<const float4*>(sB)[j * 32 + lane];
         float4& e = xr[rr][j];
-        e = xf_join(__fadd2_rn(xf_lo(e), __fadd2_rn(xf_lo(t), xf_lo(bb[j]))), __fadd2_rn(xf_hi(e), __fadd2_rn(xf_hi(t), xf_hi(bb[j]))));
+        e = xf_join(__fadd2_rn(xf_lo(e), __fadd2_rn(xf_lo(t), xf_lo(bb))), __fadd2_rn(xf_hi(e), __fadd2_rn(xf_hi(t), xf_hi(bb))));
         if (r < H) reinterpret_cast<float4*>(xc + (size_t)r * D)[j * 32 + lane] = e;
       }
     }
-    float4 gg[V], be[V];
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-      gg[j] = __ldg(reinterpret_cast<const float4*>(ln3_g) + j * 32 + lane);
-      be[j] = __ldg(reinterpret_cast<const float4*>(ln3_b) + j * 32 + lane);
-    }
     __nv_bfloat16* oc = ln3_out + (size_t)n * H * D;
+    float mean[2], rstd[2];
+    xf_row_stats<V>(xr, mean, rstd);
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
       const int r = 2 * warp + rr;
-      float2 s2 = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int j = 0; j < V; ++j) s2 = __fadd2_rn(s2, __fadd2_rn(xf_lo(xr[rr][j]), xf_hi(xr[rr][j])));
-      const float mean = warp_sum(s2.x + s2.y) / D;
-      const float2 nm = xf_dup(-mean);
-      float2 q2 = make_float2(0.f, 0.f);
-      float2 lo[V], hi[V];
-#pragma unroll
-      for (int j = 0; j < V; ++j) {
-        lo[j] = __fadd2_rn(xf_lo(xr[rr][j]), nm); hi[j] = __fadd2_rn(xf_hi(xr[rr][j]), nm);
-        q2 = __ffma2_rn(lo[j], lo[j], q2); q2 = __ffma2_rn(hi[j], hi[j], q2);
-      }
-      const float2 rs2 = xf_dup(rsqrtf(warp_sum(q2.x + q2.y) / D + 1e-5f));
+      const float2 nm = xf_dup(-mean[rr]), rs2 = xf_dup(rstd[rr]);
       if (r < H) {
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-          const float2 a = __ffma2_rn(__fmul2_rn(lo[j], rs2), xf_lo(gg[j]), xf_lo(be[j]));
-          const float2 b = __ffma2_rn(__fmul2_rn(hi[j], rs2), xf_hi(gg[j]), xf_hi(be[j]));
+          const float4 gg = reinterpret_cast<const float4*>(sB + D)[j * 32 + lane], be = reinterpret_cast<const float4*>(sB + 2 * D)[j * 32 + lane];
+          const float2 a = __ffma2_rn(__fmul2_rn(__fadd2_rn(xf_lo(xr[rr][j]), nm), rs2), xf_lo(gg), xf_lo(be));
+          const float2 b = __ffma2_rn(__fmul2_rn(__fadd2_rn(xf_hi(xr[rr][j]), nm), rs2), xf_hi(gg), xf_hi(be));
           uint2 o2;
           o2.x = pack_bf16(a.x, a.y);
           o2.y = pack_bf16(b.x, b.y);
