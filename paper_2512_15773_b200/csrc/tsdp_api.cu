@@ -896,6 +896,18 @@ int draft_tail_launch(tsdp_ctx* c, Net& n, int B, int k, int K, bool embed_next,
   return TSDP_OK;
 }
 
+template <typename T>
+void memtok_launch(tsdp_ctx* c, const Net& n, int rows, int cpos_mod, int cpos_off, T* out, cudaStream_t s) {
+  const int d = n.cfg.d, nt = d / MT_N;
+  // 64-row tiles from half a wave of them on: below that the 16-row ones, four times as many, end sooner
+  if ((rows + 63) / 64 * nt * 2 >= c->num_sms)
+    TSDP_LAUNCH(c, (memtok_kernel<T, 64>), dim3(nt, (rows + 63) / 64), MT_THREADS, 0, s, c->obs, rows, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos,
+                cpos_mod, cpos_off, out, d);
+  else
+    TSDP_LAUNCH(c, (memtok_kernel<T, 16>), dim3(nt, (rows + 15) / 16), MT_THREADS, 0, s, c->obs, rows, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos,
+                cpos_mod, cpos_off, out, d);
+}
+
 // Observation tokens -> their cross-attention keys/values for every block (once per chunk).
 template <typename T>
 int xfmr_prepare_obs_t(tsdp_ctx* c, Net& n, int B, cudaStream_t s) {
@@ -903,7 +915,7 @@ int xfmr_prepare_obs_t(tsdp_ctx* c, Net& n, int B, cudaStream_t s) {
   if (To == 0) return TSDP_OK;
   T* mt = reinterpret_cast<T*>(c->memtok);
   prof_begin(c, s, 3, 0.0);
-  TSDP_LAUNCH(c, (memtok_kernel<T>), B * To, d < 256 ? d : 256, 0, s, c->obs, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos, To, 1, mt, d);
+  memtok_launch<T>(c, n, B * To, To, 1, mt, s);
   prof_end(c, s);
   c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
@@ -1032,7 +1044,7 @@ int dit_prepare_ctx_t(tsdp_ctx* c, Net& n, int B, cudaStream_t s) {
   const int Tc = c->cfg.obs_tokens, d = n.cfg.d, L = n.cfg.layers;
   T* mt = reinterpret_cast<T*>(c->memtok);
   prof_begin(c, s, 3, 0.0);
-  TSDP_LAUNCH(c, (memtok_kernel<T>), B * Tc, d < 256 ? d : 256, 0, s, c->obs, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos, Tc, 0, mt, d);
+  memtok_launch<T>(c, n, B * Tc, Tc, 0, mt, s);
   prof_end(c, s);
   c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
@@ -2196,11 +2208,9 @@ int tsdp_load_weights(tsdp_ctx* c, int which, const float* blob, size_t n) {
     // keys/values of the time token for every timestep: (sinusoidal(tau) + cpos[0]) Wkv2 + bkv2, all blocks
     c->launches_per_round_tmp = 0;
     if (cfg.precision == 0) {
-      memtok_kernel<float><<<T, d < 256 ? (int)d : 256>>>(net.temb_table, (int)d, nullptr, nullptr, net.cpos, 0, 0,
-                                                           reinterpret_cast<float*>(c->memtok), (int)d);
+      timetok_kernel<float><<<T, d < 256 ? (int)d : 256>>>(net.temb_table, net.cpos, reinterpret_cast<float*>(c->memtok), (int)d);
     } else {
-      memtok_kernel<__nv_bfloat16><<<T, d < 256 ? (int)d : 256>>>(net.temb_table, (int)d, nullptr, nullptr, net.cpos, 0, 0,
-                                                                   reinterpret_cast<__nv_bfloat16*>(c->memtok), (int)d);
+      timetok_kernel<__nv_bfloat16><<<T, d < 256 ? (int)d : 256>>>(net.temb_table, net.cpos, reinterpret_cast<__nv_bfloat16*>(c->memtok), (int)d);
     }
     CU_TRY(c, cudaGetLastError());
     if ((r = gemm(c, c->memtok, net.Wkv_all, net.bkv_all, T, (int)(L * 2 * d), (int)d, EPI_F32, net.kv_time, (int)(L * 2 * d), 0)))

@@ -129,10 +129,6 @@ xfold_build_kernel(const float* __restrict__ kv, long long ldkv, int rows, const
   }
 }
 
-__device__ __forceinline__ void xf_cp16(void* smem_dst, const void* gsrc) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
-}
 __device__ __forceinline__ void xf_add_bf16x4(float4& a, const uint2 d) {
   const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&d.x));
   const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&d.y));
@@ -267,8 +263,8 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
                                 lay_off + (size_t)h * D;
       __nv_bfloat16* dr = sK + (size_t)row * LDA;
 #pragma unroll
-      for (int ch = 0; ch < D / 256; ++ch) xf_cp16(dr + (ch * 32 + lane) * 8, sr + (ch * 32 + lane) * 8);
-      if (D % 256 && lane < (D % 256) / 8) xf_cp16(dr + (D / 256 * 32 + lane) * 8, sr + (D / 256 * 32 + lane) * 8);
+      for (int ch = 0; ch < D / 256; ++ch) cp_async16(dr + (ch * 32 + lane) * 8, sr + (ch * 32 + lane) * 8);
+      if (D % 256 && lane < (D % 256) / 8) cp_async16(dr + (D / 256 * 32 + lane) * 8, sr + (D / 256 * 32 + lane) * 8);
     }
     xf_cp_commit();
     for (int row = warp; row < NKH / 2; row += XF_WARPS) {
@@ -277,7 +273,7 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
                                 lay_off + (size_t)q * D * 2;
       uint32_t* dr = sU + (size_t)row * LDU;
 #pragma unroll
-      for (int ch = 0; ch < D / 128; ++ch) xf_cp16(dr + (ch * 32 + lane) * 4, sr + (ch * 32 + lane) * 8);
+      for (int ch = 0; ch < D / 128; ++ch) cp_async16(dr + (ch * 32 + lane) * 4, sr + (ch * 32 + lane) * 8);
     }
     xf_cp_commit();
   }
@@ -386,7 +382,7 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
   float* sB = sS;
   static_assert(3 * D <= 4 * 16 * XF_MAXN, "phase 5 parameters fit over the partial scores");
   for (int i = threadIdx.x; i < 3 * D / 4; i += XF_THREADS)
-    xf_cp16(sB + 4 * i, (i < D / 4 ? bo2 : (i < D / 2 ? ln3_g - D : ln3_b - 2 * D)) + 4 * i);
+    cp_async16(sB + 4 * i, (i < D / 4 ? bo2 : (i < D / 2 ? ln3_g - D : ln3_b - 2 * D)) + 4 * i);
   xf_cp_commit();
 
   // ---- 4: P . U for all 16 rows, warp w the output columns [w D/8, (w+1) D/8), into shared memory over the
