@@ -673,9 +673,9 @@ int self_attn_launch(tsdp_ctx* c, const T* qkv, T* out, int n_cand, int H, int d
     const int grid = (n_cand * heads * QT + SA_WARPS - 1) / SA_WARPS;
     if (H > 16 && (dh == 32 || dh == 64 || dh == 128)) {     // several query tiles share a head's K/V: stage them once
       const int g2 = n_cand * heads;
-      if (dh == 32) TSDP_LAUNCH(c, (self_attn_staged_kernel<32>), g2, 128, 0, s, qkv, out, n_cand, H, d, heads, causal, lv);
-      else if (dh == 64) TSDP_LAUNCH(c, (self_attn_staged_kernel<64>), g2, 128, 0, s, qkv, out, n_cand, H, d, heads, causal, lv);
-      else TSDP_LAUNCH(c, (self_attn_staged_kernel<128>), g2, 128, 0, s, qkv, out, n_cand, H, d, heads, causal, lv);
+      if (dh == 32) TSDP_LAUNCH(c, (self_attn_staged_kernel<32>), g2, 128, sa_smem_bytes<32>(), s, qkv, out, n_cand, H, d, heads, causal, lv);
+      else if (dh == 64) TSDP_LAUNCH(c, (self_attn_staged_kernel<64>), g2, 128, sa_smem_bytes<64>(), s, qkv, out, n_cand, H, d, heads, causal, lv);
+      else TSDP_LAUNCH(c, (self_attn_staged_kernel<128>), g2, 128, sa_smem_bytes<128>(), s, qkv, out, n_cand, H, d, heads, causal, lv);
     } else if (H <= 16 && (dh == 32 || dh == 64 || dh == 128)) {   // one 16-row tile: operands staged per warp
       const int tw = dh > 64 ? 2 : 4, g3 = (n_cand * heads + tw - 1) / tw;
       if (dh == 32) TSDP_LAUNCH(c, (self_attn_tile_kernel<32>), g3, tw * 32, 0, s, qkv, out, n_cand, H, d, heads, causal, lv);
@@ -1772,6 +1772,7 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
   INIT_TRY(cudaFuncSetAttribute(cross_attn_ctx_mma_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, cx_smem_bytes<32>(256)));
   INIT_TRY(cudaFuncSetAttribute(cross_attn_ctx_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, cx_smem_bytes<64>(256)));
   INIT_TRY(cudaFuncSetAttribute(cross_attn_ctx_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, cx_smem_bytes<128>(256)));
+  INIT_TRY(cudaFuncSetAttribute(self_attn_staged_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, sa_smem_bytes<128>()));
   INIT_TRY(cudaFuncSetAttribute(cross_attn_ctx_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CXT_SMEM_BYTES));
   INIT_TRY(cudaFuncSetAttribute(xfold_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   INIT_TRY(cudaFuncSetAttribute(xattn_fold_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xf_smem_bytes(128, XF_MAXN)));
