@@ -18,6 +18,7 @@
 // 256 columns of it and under 100 KB of shared memory, so two CTAs share an SM and one's products run under the
 // other's softmax (within a CTA the four steps of a tile are strictly serial).  Rows past the group's end are
 // computed on whatever the tile fetched (other rows of the buffer, or zeros past its end) and never stored.
+// With few groups (a handful of robots) a group's tiles are dealt to `splits` CTAs, which fetch the same keys and values.
 // Every mbarrier wait is bounded; on expiry the CTA records TSDP_ERR_TIMEOUT (5) in `status`, frees its tensor
 // memory and returns.
 #pragma once
@@ -31,6 +32,8 @@ __device__ __forceinline__ void tmem_st8(uint32_t addr, const uint32_t v[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
 }
+// 2^x by the hardware instruction: exp2f spends three more on results below the smallest normal number, weights of nothing here
+__device__ __forceinline__ float ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // D (tensor memory) (+)= A (tensor memory: lane = row, one 32-bit column = two consecutive k) x B (shared memory)
 __device__ __forceinline__ void tc_mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t db, uint32_t idesc, uint32_t acc) {
@@ -55,7 +58,7 @@ constexpr uint32_t CXT_O_COL = 192;
 __global__ void __launch_bounds__(CXT_THREADS, 2)
 cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV,
                          __nv_bfloat16* __restrict__ out, int kv_off, CandMap cm, int rows_per_slot, int d, int heads, int Tc,
-                         const int* __restrict__ slot_start, int H, int* __restrict__ status) {
+                         const int* __restrict__ slot_start, int H, int splits, int* __restrict__ status) {
   extern __shared__ uint8_t cxt_raw[];
   pdl_trigger();
   const uint32_t base = (ptx::smem_u32(cxt_raw) + 1023u) & ~1023u;
@@ -78,8 +81,9 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
   pdl_wait();
 
   // rows of this group (see cross_attn_ctx_mma_kernel: dense slots, compacted slots, or one list entry per group)
-  int b = blockIdx.x / heads;
-  const int hd = blockIdx.x % heads;
+  const int group = blockIdx.x / splits, split = blockIdx.x - group * splits;      // this CTA's tiles of the group: split, split + splits, ..
+  int b = group / heads;
+  const int hd = group % heads;
   long long row0 = (long long)b * rows_per_slot;
   int rows = rows_per_slot;
   bool live = true;
@@ -88,10 +92,11 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     rows = (slot_start[b + 1] - slot_start[b]) * H;
     live = rows > 0;
   } else if (cm.list != nullptr) {
-    live = b < cand_count(cm, (int)(gridDim.x / heads));
+    live = b < cand_count(cm, (int)(gridDim.x / (heads * splits)));
     if (live) b = cm.list[b] >> 6;
   }
-  const int n_tiles = live ? (rows + 127) / 128 : 0;
+  const int tiles = live ? (rows + 127) / 128 : 0, n_tiles = tiles > split ? (tiles - split + splits - 1) / splits : 0;
+  auto tile_row = [&](int i) { return (split + i * splits) * 128; };      // first row, in the group, of this CTA's i-th tile
   bool ok = true;
   const uint32_t kv_bytes = (uint32_t)Tc * 128u;
 
@@ -125,7 +130,7 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
     __syncthreads();
     if (ok && warp == 8 && lane == 0) {                    // the first Q tile, now that the staging tile is free
       ptx::mbar_expect_tx(bar_q0, CXT_Q_BYTES);
-      ptx::tma_load_2d(sQ, &tmQ, hd * 64, (int)row0, bar_q0);
+      ptx::tma_load_2d(sQ, &tmQ, hd * 64, (int)row0 + tile_row(0), bar_q0);
     }
   }
 
@@ -148,7 +153,7 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
           if (i + 1 < n_tiles) {      // the other Q buffer was last read by the first product of tile i - 1: complete
             const uint32_t nb = bar_q0 + 8u * ((i + 1) & 1);
             ptx::mbar_expect_tx(nb, CXT_Q_BYTES);
-            ptx::tma_load_2d(sQ + (uint32_t)((i + 1) & 1) * CXT_Q_BYTES, &tmQ, hd * 64, (int)row0 + (i + 1) * 128, nb);
+            ptx::tma_load_2d(sQ + (uint32_t)((i + 1) & 1) * CXT_Q_BYTES, &tmQ, hd * 64, (int)row0 + tile_row(i + 1), nb);
           }
           if (!ptx::mbar_wait_thread(bar_p, (uint32_t)(i & 1))) { ok = false; break; }
           ptx::tc_fence_after();
@@ -193,8 +198,8 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
           uint32_t pk[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float p0 = exp2f(__fmaf_rn(__uint_as_float(v[2 * j]), c, -mc));
-            const float p1 = exp2f(__fmaf_rn(__uint_as_float(v[2 * j + 1]), c, -mc));
+            const float p0 = ptx::ex2(__fmaf_rn(__uint_as_float(v[2 * j]), c, -mc));
+            const float p1 = ptx::ex2(__fmaf_rn(__uint_as_float(v[2 * j + 1]), c, -mc));
             sum += p0 + p1;
             pk[j] = pack_bf16x2(p0, p1);
           }
@@ -214,7 +219,7 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
         ptx::tmem_ld_wait();
         ptx::tc_fence_before();
         ptx::mbar_arrive(bar_or);                           // O (and P) may be overwritten by the next tile's scores
-        const int row = i * 128 + r;
+        const int row = tile_row(i) + r;
         if (row < rows) {
           const float inv = 1.0f / sum;
           uint4* o = reinterpret_cast<uint4*>(out + (size_t)(row0 + row) * d + hd * 64 + half * 32);
