@@ -25,12 +25,16 @@ __global__ void mish_kernel(const float* in, float* out, long long n) {
   if (i < n) out[i] = mish_f(in[i]);
 }
 
-// v tanh(softplus(v)) = v (w - 1) / (w + 1) with w = (1 + e^v)^2, written without the cancellation: one exponential and
-// one division (log1p, exp and tanh were half of the GroupNorm kernel's instructions).
+// v tanh(softplus(v)) = v n / m with n = e^v (e^v + 2), m = n + 2: one exponential and one division in place of log1p, exp
+// and tanh.  The quotient is taken of the smaller side, n / m = 1 - 2 / m above zero and
+// e^v (1 - (e^2v + e^v) / m) below, where it is at most 0.4, so that the error of the fast division weighs 2/3 at most.
+// Against 64 bits, in units of 2^-24 of the result, largest and rms over [-30, 25]: 4.2 and 0.70; v tanhf(log1pf(expf(v))) 5.4
+// and 0.72, v * __fdividef(n, m) 5.6 and 0.93 (calls of the UNet workload with that one: 0.3 % faster at most).
 __device__ __forceinline__ float mish_fast(float v) {
   if (v > 20.f) return v;
-  const float e = expf(v), n = e * (e + 2.f);
-  return v * __fdividef(n, n + 2.f);
+  const float e = expf(v), m = __fmaf_rn(e, e, e + e) + 2.f;
+  const float c = 1.f - __fdividef(v > 0.f ? 2.f : __fmaf_rn(e, e, e), m);
+  return v * (v > 0.f ? c : e * c);
 }
 
 // Input projection: X[n, l + 2, :] = x[n, l, :] W_in + b_in   (pointwise, A -> C channels).  A block takes the H rows of one

@@ -46,3 +46,32 @@ def test_unet_denoiser_tiles_and_groups(case, N):
             assert err < tol, (precision, n, err)
         assert smp.check_guards() > 0
         smp.close()
+
+
+def test_mish_behind_the_group_norm_keeps_fp32_accuracy():
+    """Every weight but the last norm's shift and a 0/1 output matrix is zero, so eps[l, a] is Mish of shift a, nothing else.
+    Above 9.5 the nearest fp32 number to Mish(v) = v (1 - 2 / (n + 2)), n = e^v (e^v + 2), is v itself (2 / (n + 2) < 2^-25).
+    Elsewhere 10 units of 2^-24: the exponential (1 ulp = 2 units, its weight in the result at most 1); a quotient t <= 0.4 taken
+    from 1, so of weight t / (1 - t) <= 2/3, with 3 units in its parts and 2 ulp of its own; three roundings behind it."""
+    H, A, ch = 2, 64, 128
+    wl = dict(H=H, A=A, To=1, Do=1, T=100, precision=0, gamma=1.0, base=dict(arch="unet", layers=1, d=ch, heads=8, temb=4))
+    smp = binding.Sampler(binding.make_config(H, A, 1, 1, wl["base"], dict(arch="gauss"), max_B=1, max_K=1, precision=0))
+    p = inputs.make_net(1, wl, "base")
+    zero = lambda v: np.zeros_like(np.asarray(v, dtype=np.float64))
+    p = {k: ([{n: zero(w) for n, w in R.items()} for R in v] if k == "blocks" else zero(v) if isinstance(v, np.ndarray) else v)
+         for k, v in p.items()}
+    p["W_out"][:A, :A] = np.eye(A)
+    x = torch.zeros(1, H, A, device="cuda"); obs = torch.zeros(1, 1, 1, device="cuda"); out = torch.zeros_like(x)
+    values = np.linspace(-25.0, 21.0, 24 * A).astype(np.float32).reshape(24, A)
+    got = []
+    for row in values:
+        p["beh"][:A] = row
+        smp.load_weights(binding.BASE, p)
+        smp.denoise(binding.BASE, x, np.array([7], np.int32), obs, 1, out)
+        got.append(out[0, 1].cpu().numpy())
+    smp.close()
+    v, got = values.reshape(-1).astype(np.float64), np.concatenate(got).astype(np.float64)
+    n = np.exp(v) * (np.exp(v) + 2.0)
+    err = np.abs(got - v * n / (n + 2.0)) / np.abs(v * n / (n + 2.0))
+    assert np.max(err) < 10 * 2.0 ** -24
+    assert np.array_equal(got[v >= 9.5], v[v >= 9.5])
