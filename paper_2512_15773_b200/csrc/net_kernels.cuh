@@ -109,7 +109,8 @@ memtok_kernel(const float* __restrict__ in, int rows, int Din, const float* __re
   __shared__ __align__(16) float Bs[MT_BK * MT_N];
   pdl_trigger();
   pdl_wait();
-  const int r0 = blockIdx.y * TM, c0 = blockIdx.x * MT_N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nt = d / MT_N, r0 = (int)(blockIdx.x / nt) * TM, c0 = (int)(blockIdx.x % nt) * MT_N;      // (a long queue has more row tiles than grid.y may)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tid & 15, ty = tid >> 4;
   float ra[NA], rb[NB];
   auto fetch = [&](int k0) {

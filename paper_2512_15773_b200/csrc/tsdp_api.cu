@@ -901,10 +901,10 @@ void memtok_launch(tsdp_ctx* c, const Net& n, int rows, int cpos_mod, int cpos_o
   const int d = n.cfg.d, nt = d / MT_N;
   // 64-row tiles from half a wave of them on: below that the 16-row ones, four times as many, end sooner
   if ((rows + 63) / 64 * nt * 2 >= c->num_sms)
-    TSDP_LAUNCH(c, (memtok_kernel<T, 64>), dim3(nt, (rows + 63) / 64), MT_THREADS, 0, s, c->obs, rows, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos,
+    TSDP_LAUNCH(c, (memtok_kernel<T, 64>), (rows + 63) / 64 * nt, MT_THREADS, 0, s, c->obs, rows, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos,
                 cpos_mod, cpos_off, out, d);
   else
-    TSDP_LAUNCH(c, (memtok_kernel<T, 16>), dim3(nt, (rows + 15) / 16), MT_THREADS, 0, s, c->obs, rows, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos,
+    TSDP_LAUNCH(c, (memtok_kernel<T, 16>), (rows + 15) / 16 * nt, MT_THREADS, 0, s, c->obs, rows, c->cfg.obs_dim, n.W_obs, n.b_obs, n.cpos,
                 cpos_mod, cpos_off, out, d);
 }
 
@@ -1175,7 +1175,7 @@ int unet_prepare_obs(tsdp_ctx* c, Net& n, int N, cudaStream_t s) {
   const size_t smem = (size_t)UF_N * ((dobs + 3) & ~3) * sizeof(float);
   c->launches_per_round_tmp++;
   if (smem > UF_MAX_SMEM) return gemm_f32(c, n.obs_m, n.WfT_obs, nullptr, N, n.F, dobs, EPI_F32, n.film_obs, s);
-  TSDP_LAUNCH(c, film_obs_kernel, dim3((n.F + 8 * UF_F - 1) / (8 * UF_F), (N + UF_N - 1) / UF_N), 256, smem, s, n.obs_m, n.WfT_obs,
+  TSDP_LAUNCH(c, film_obs_kernel, (n.F + 8 * UF_F - 1) / (8 * UF_F) * ((N + UF_N - 1) / UF_N), 256, smem, s, n.obs_m, n.WfT_obs,
               n.film_obs, N, n.F, dobs);
   CU_TRY(c, cudaGetLastError());
   return TSDP_OK;

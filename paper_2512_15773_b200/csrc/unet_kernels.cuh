@@ -85,7 +85,8 @@ film_obs_kernel(const float* __restrict__ x, const float* __restrict__ W, float*
   pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(16) float sx_film[];      // [UF_N][Kp], zero beyond K and N
-  const int Kp = (K + 3) & ~3, n0 = blockIdx.y * UF_N, nn = min(UF_N, N - n0);
+  const int fx = (F + 8 * UF_F - 1) / (8 * UF_F);      // blocks along the features (row blocks of a long queue exceed grid.y)
+  const int Kp = (K + 3) & ~3, n0 = (int)(blockIdx.x / fx) * UF_N, nn = min(UF_N, N - n0);
   for (int i = threadIdx.x; i < UF_N * Kp; i += blockDim.x) {
     const int r = i / Kp, k = i - r * Kp;
     sx_film[i] = (r < nn && k < K) ? x[(size_t)(n0 + r) * K + k] : 0.f;
@@ -93,7 +94,8 @@ film_obs_kernel(const float* __restrict__ x, const float* __restrict__ W, float*
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool vec = (K & 3) == 0;
-  for (int f0 = (blockIdx.x * (blockDim.x >> 5) + warp) * UF_F; f0 < F; f0 += gridDim.x * (blockDim.x >> 5) * UF_F) {
+  const int f0 = ((int)(blockIdx.x % fx) * 8 + warp) * UF_F;
+  if (f0 < F) {
     float acc[UF_F][UF_N];
 #pragma unroll
     for (int i = 0; i < UF_F; ++i)
