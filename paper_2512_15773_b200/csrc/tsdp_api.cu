@@ -10,6 +10,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <thread>
 #include <tuple>
 #include <type_traits>
 #include <utility>
@@ -1517,13 +1518,24 @@ int upload_params(tsdp_ctx* c, int K, const tsdp_accept_t& acc, uint64_t seed, i
   return TSDP_OK;
 }
 
+inline void spin_hint() {
+#if defined(__x86_64__)
+  __builtin_ia32_pause();
+#endif
+}
+
 // Wait until at least `rounds` rounds of the running call are complete and return the progress word.  The word is
-// polled, so that the host reacts within a microsecond; the stream is asked now and then in case it failed.
-int wait_progress(tsdp_ctx* c, cudaStream_t s, unsigned long long rounds, unsigned long long* out) {
+// polled, so that the host reacts within a few microseconds; other threads that are ready to run get the core every 64 polls, and
+// the stream is asked now and then in case it failed.  In a process that asked for blocking waits (`block`) the
+// thread sleeps until everything issued has finished instead.
+int wait_progress(tsdp_ctx* c, cudaStream_t s, bool block, unsigned long long rounds, unsigned long long* out) {
   volatile unsigned long long* p = c->host_prog;
+  if (block) CU_TRY(c, cudaStreamSynchronize(s));
   for (unsigned i = 1;; ++i) {
     unsigned long long v = *p;
     if ((v >> 32) >= rounds) { *out = v; return TSDP_OK; }
+    if (i % 64 != 0) { spin_hint(); continue; }
+    std::this_thread::yield();
     if (i % 4096 != 0) continue;
     const cudaError_t e = cudaStreamQuery(s);
     if (e == cudaErrorNotReady) continue;
@@ -2416,6 +2428,9 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
   // furthest behind after the last completed round the host knows of needs more steps than the rounds in flight can
   // take.  Only where neither holds does the host wait for a newer result; the GPU idles between two rounds only
   // near the end of a call.
+  unsigned dev_flags = 0;
+  CU_TRY(c, cudaGetDeviceFlags(&dev_flags));
+  const bool block = (dev_flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
   const int n_sched = (int)c->sched_K.size();
   auto round_K = [&](long long r) { return n_sched > 0 ? c->sched_K[r < n_sched ? r : n_sched - 1] : K; };
   const long long waves = ((long long)N + B - 1) / B;
@@ -2432,7 +2447,7 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
     }
     if (known == round) break;                       // left == 0: every request is finished
     unsigned long long v = 0;
-    if ((r = wait_progress(c, s, (unsigned long long)known + 1, &v))) return r;
+    if ((r = wait_progress(c, s, block, (unsigned long long)known + 1, &v))) return r;
     for (; known < (long long)(v >> 32); ++known) in_flight -= round_K(known) + 1;
     left = (long long)(v & 0xffffffffull);
   }
