@@ -284,6 +284,12 @@ int tsdp_debug_check_guards(tsdp_ctx* ctx, int* h_checked);
  * incomplete), the status word is cleared, and the context stays usable.  One-shot.  Errors: ARG. */
 int tsdp_debug_arm_gemm_timeout(tsdp_ctx* ctx, long long wait_cycles);
 
+/* Make a sampling call end early on the host (test interface): of the rounds that the following tsdp_sample_chunk(_host) or
+ * tsdp_serve calls issue, the n-th (n >= 1) is refused before anything of it reaches the device, and the call
+ * returns TSDP_ERR_CUDA.  The rounds issued before it are waited for; the context stays usable.  One-shot.
+ * Errors: ARG. */
+int tsdp_debug_arm_round_failure(tsdp_ctx* ctx, int n);
+
 /* The same GEMM launched `reps` times back to back between one pair of CUDA events on `cuda_stream`
  * (after one untimed launch); *h_ms (HOST) receives the mean device time of one launch in milliseconds.
  * With EPI 2 the output accumulates over the launches.  Measurement interface; synchronous. */

@@ -175,6 +175,7 @@ struct tsdp_ctx {
   int pair_mode = 1;                          // TSDP_GEMM_PAIR: 0 never, 1 (default) by shape (use_pair_gemm), 2 wherever it applies
   bool dbg_armed = false, dbg_in_test_gemm = false;   // tsdp_debug_arm_gemm_timeout
   long long dbg_wait_cycles = 0;
+  int dbg_fail_round = 0;                             // tsdp_debug_arm_round_failure
   uint64_t cand_static = 0;                   // candidates the dense layout would have evaluated since the last reset
   // optional per-kernel-family timing with CUDA events (plain launches, no graph)
   bool prof_on = false;
@@ -1448,6 +1449,10 @@ int enqueue_round(tsdp_ctx* c, int B, int K, cudaStream_t s, bool dbg) {
 }
 
 int run_round(tsdp_ctx* c, int B, int K, cudaStream_t s) {
+  if (c->dbg_fail_round > 0 && --c->dbg_fail_round == 0) {
+    c->last_error = "round refused: see tsdp_debug_arm_round_failure";
+    return TSDP_ERR_CUDA;
+  }
   c->cand_static += (uint64_t)B * (K + 1);
   if (!c->cfg.use_graph || c->prof_on) {
     c->launches_per_round_tmp = 0;
@@ -1517,6 +1522,20 @@ int upload_params(tsdp_ctx* c, int K, const tsdp_accept_t& acc, uint64_t seed, i
   CU_TRY(c, cudaMemcpyAsync(c->params, c->params_host, PARAMS_BYTES, cudaMemcpyHostToDevice, s));
   return TSDP_OK;
 }
+
+// Waits, when a call returns before it has seen its rounds finish (an error after the first enqueue), for what it has
+// issued: rounds in flight read the pinned parameters and write the progress word that the next call uses.
+struct DrainOnError {
+  tsdp_ctx* c;
+  cudaStream_t s;
+  bool done = false;                         // the call has synchronised by itself
+  ~DrainOnError() {
+    if (done) return;
+    cudaStreamSynchronize(s);
+    cudaStreamSynchronize(c->side_stream);
+    cudaStreamSynchronize(c->aux_stream);
+  }
+};
 
 inline void spin_hint() {
 #if defined(__x86_64__)
@@ -2397,11 +2416,12 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
   const int D = c->D, T = c->cfg.T;
   int r;
   if ((r = ensure_items(c, (size_t)N))) return r;
+  DrainOnError drain{c, s};
   CU_TRY(c, cudaEventRecord(c->ev_chunk0, s));
   if (obs_n)
     CU_TRY(c, cudaMemcpyAsync(c->obs, obs, obs_n * sizeof(float), obs_on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
   c->items_last = N;
-  *c->host_prog = 0;                         // nothing of an earlier call is in flight: every call ends with a synchronise
+  *c->host_prog = 0;                         // nothing of an earlier call is in flight: every way out of a call waits for its rounds
   if ((r = upload_params(c, K, *acc, seed, N, s, false))) return r;
   if (c->sched_on) {
     // the scheduler network reads the new observation, the previous chunk's actions and the progress; it
@@ -2456,6 +2476,7 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
   CU_TRY(c, cudaMemcpyAsync(c->status_host, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU_TRY(c, cudaEventRecord(c->ev_chunk1, s));
   CU_TRY(c, cudaStreamSynchronize(s));
+  drain.done = true;
   {   // device time of this call, copies included, into the latency ring
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, c->ev_chunk0, c->ev_chunk1) == cudaSuccess) {
@@ -2497,6 +2518,7 @@ int tsdp_round(tsdp_ctx* c, const float* d_obs, int B, int K, const tsdp_accept_
   const int D = c->D;
   const size_t K1 = c->cfg.max_K + 1, Km = c->cfg.max_K > 0 ? c->cfg.max_K : 1;
   int r;
+  DrainOnError drain{c, s};
   if (obs_n) CU_TRY(c, cudaMemcpyAsync(c->obs, d_obs, obs_n * sizeof(float), cudaMemcpyDeviceToDevice, s));
   if ((r = upload_params(c, K, *acc, seed, B, s, true))) return r;
   CU_TRY(c, cudaMemsetAsync(c->round_idx, 0, sizeof(int), s));
@@ -2537,6 +2559,7 @@ int tsdp_round(tsdp_ctx* c, const float* d_obs, int B, int K, const tsdp_accept_
   CU_TRY(c, cudaMemcpyAsync(h_t, c->t, sizeof(int) * B, cudaMemcpyDeviceToHost, s));
   if (h_jstar) CU_TRY(c, cudaMemcpyAsync(h_jstar, c->dbg_jstar, sizeof(int) * B, cudaMemcpyDeviceToHost, s));
   CU_TRY(c, cudaStreamSynchronize(s));
+  drain.done = true;
   return check_status(c);
 }
 
@@ -2694,6 +2717,12 @@ int tsdp_debug_arm_gemm_timeout(tsdp_ctx* c, long long wait_cycles) {
   if (!c || wait_cycles < 1000 || wait_cycles > 2000000000ll || c->cfg.precision != 1) return TSDP_ERR_ARG;
   c->dbg_armed = true;
   c->dbg_wait_cycles = wait_cycles;
+  return TSDP_OK;
+}
+
+int tsdp_debug_arm_round_failure(tsdp_ctx* c, int n) {
+  if (!c || n < 1) return TSDP_ERR_ARG;
+  c->dbg_fail_round = n;
   return TSDP_OK;
 }
 

@@ -4,6 +4,10 @@ import subprocess
 import sys
 
 import pytest
+import torch
+
+from paper_2512_15773_b200 import binding, inputs
+from tests import helpers as hp
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +40,35 @@ def test_a_process_that_asked_for_blocking_waits_does_not_spin():
     """100 rounds of a full batch (tens of milliseconds of GPU work): issuing them takes the host a few, the rest it sleeps."""
     r = subprocess.run([sys.executable, "-c", BLOCKING], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("call", ["chunk", "round"])
+def test_a_call_after_one_that_failed_half_way_sees_nothing_of_it(call):
+    """99 rounds of plain DDPM are in flight when the 100th is refused on the host.  The next call has other parameters; its result
+    and, for a chunk, its number of rounds are those of a context that never failed."""
+    wl = dict(inputs.WORKLOADS["serving_xfmr"], base=dict(arch="xfmr", layers=4, d=512, heads=8))
+    B, K, D = 64, 4, wl["H"] * wl["A"]
+    obs = torch.tensor(inputs.make_obs(3, B, wl["To"], wl["Do"]), dtype=torch.float32, device="cuda")
+    outs = []
+    for fail in (False, True):
+        smp, *_ = hp.setup(wl, max_B=B, max_K=K)
+        out = torch.zeros(B, wl["H"], wl["A"], device="cuda")
+        smp.sample_chunk(obs, B, K, hp.accept_t(), 1, out)                  # graphs exist
+        before = smp.stats()["rounds"]
+        if fail:
+            smp.arm_round_failure(100)
+            with pytest.raises(binding.TsdpError) as e:
+                smp.sample_chunk(obs, B, 0, hp.accept_t(), 2, out)
+            assert e.value.status == 4                                      # TSDP_ERR_CUDA
+            before += 99
+        if call == "chunk":
+            smp.sample_chunk(obs, B, K, hp.accept_t(), 9, out)
+            outs.append((out.clone(), smp.stats()["rounds"] - before))
+        else:
+            x = torch.tensor(inputs.make_obs(7, B, wl["H"], wl["A"]), dtype=torch.float32, device="cuda").reshape(B, D)
+            h_t = (torch.arange(B, dtype=torch.int32) + 20).numpy()
+            smp.round(obs, B, K, hp.accept_t(), 9, x, h_t)
+            outs.append((x.clone(), h_t.tolist()))
+        smp.close()
+    assert torch.equal(outs[0][0], outs[1][0])
+    assert outs[0][1] == outs[1][1]
