@@ -20,13 +20,19 @@ gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ W, GemmA
   g.M = live_rows(g.live, g.M);
   if (m0 >= g.M) return;
   float acc[4][4] = {};
+  const int lr = threadIdx.x >> 4, lk = threadIdx.x & 15;      // this thread loads rows lr, lr + 16, .. at k = lk
+  size_t arow[4];                                              // where they start (kept out of the k loop: a convolution's take a division)
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int row = m0 + lr + 16 * j;
+    arow[j] = (g.conv_c ? (size_t)(row / g.conv_l) * (g.conv_l + 4) + row % g.conv_l + g.conv_off : (size_t)row) * g.lda;
+  }
   for (int k0 = 0; k0 < g.K; k0 += 16) {
-    for (int i = threadIdx.x; i < 64 * 16; i += 256) {
-      const int r = i >> 4, k = i & 15;
-      const int row = m0 + r;
-      const size_t arow = g.conv_c ? (size_t)(row / g.conv_l) * (g.conv_l + 4) + row % g.conv_l + g.conv_off : row;
-      As[k][r] = (row < g.M && k0 + k < g.K) ? A[arow * g.lda + k0 + k] : 0.f;
-      Ws[k][r] = (n0 + r < g.N && k0 + k < g.K) ? W[(size_t)(n0 + r) * g.K + k0 + k] : 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = lr + 16 * j;
+      As[lk][r] = (m0 + r < g.M && k0 + lk < g.K) ? A[arow[j] + k0 + lk] : 0.f;
+      Ws[lk][r] = (n0 + r < g.N && k0 + lk < g.K) ? W[(size_t)(n0 + r) * g.K + k0 + lk] : 0.f;
     }
     __syncthreads();
 #pragma unroll
