@@ -89,9 +89,9 @@ __device__ __forceinline__ float ddpm_sample(float mu, float sigma, float xi) { 
 // than the launch latency saved.  Measured, signal at the start of every kernel -> this rule: 96 environments vanilla 56.2 ->
 // 53.9 ms, 32 of the UNet workload 25.0 -> 23.0, 24 of the Push-T-shaped one 11.05 -> 10.46 (no signal at all: 53.9,
 // 24.3, 10.65).  The GEMM signals when its last operand loads are issued, the others when they start.
-constexpr unsigned PDL_MAX_GRID = 74;
+constexpr unsigned PDL_MAX_GRID = 74;      // half of a B200's SMs
 __device__ __forceinline__ void pdl_trigger() {
-  if (gridDim.x <= PDL_MAX_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (gridDim.x * gridDim.y <= PDL_MAX_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
