@@ -254,14 +254,13 @@ __device__ __forceinline__ void cand_decode(const CandMap& cm, int n, int& b, in
 __device__ __forceinline__ int cand_count(const CandMap& cm, int n_static) {
   return cm.n_live ? min(*cm.n_live, n_static) : n_static;
 }
-// The same for kernels that only see rows: rows = *n * mul + add, never more than the launch was sized for.
+// The same for kernels that only see rows: rows = *n * mul, never more than the launch was sized for.
 struct LiveRows {
-  const int* n;  int mul;  int add;
+  const int* n;  int mul;
 };
 __device__ __forceinline__ int live_rows(const LiveRows& lv, int rows_static) {
   if (lv.n == nullptr) return rows_static;
-  const int v = *lv.n * lv.mul + lv.add;
-  return v < 0 ? 0 : (v < rows_static ? v : rows_static);
+  return min(*lv.n * lv.mul, rows_static);
 }
 
 // Per-round speculative parameters (the scheduler's action space, Sec. 3.3: draft steps, acceptance

@@ -317,7 +317,7 @@ struct GemmArgs {
   // at channel (64 kb) % conv_c, position conv_off + (64 kb) / conv_c; the padding rows cost nothing.
   int conv_c, conv_l, conv_off;
   int tile_rows;        // rows of an output tile: 128, or the largest multiple of conv_l that is not larger
-  // Rows that really exist when the forward runs on a compacted candidate list: min(M, *live.n * live.mul + live.add)
+  // Rows that really exist when the forward runs on a compacted candidate list: min(M, *live.n * live.mul)
   // (live.n null: M).  The tensor maps keep their full extent; tiles beyond the live rows are simply not visited.
   LiveRows live;
   const int* list;      // EPI_GATE with a compacted list: candidate n of a row is (list[n] >> 6, list[n] & 63)

@@ -13,7 +13,7 @@ constexpr int TSDP_PLAN_MAXK = 32;      // = TSDP_MAX_K of the C ABI
 // x_T ~ N(0, I), t = T-1 for every environment.  xt holds the round's candidate latents
 // [B, Kmax+1, D]; slot 0 is the current latent x.
 __global__ void init_chunk_kernel(float* __restrict__ xt, long long xs_b, int* __restrict__ t, int B, int D,
-                                  int T, const uint64_t* __restrict__ seedp, int* __restrict__ round_idx, int* __restrict__ n_done,
+                                  int T, const uint64_t* __restrict__ seedp, int* __restrict__ round_idx,
                                   int* __restrict__ item, int* __restrict__ queue_head, int* __restrict__ item_counts, int n_requests) {
   pdl_trigger();
   pdl_wait();
@@ -31,7 +31,7 @@ __global__ void init_chunk_kernel(float* __restrict__ xt, long long xs_b, int* _
   if (threadIdx.x == 0) {
     t[b] = T - 1;
     item[b] = b;                         // slot b starts on request b; further requests are taken from queue_head on
-    if (b == 0) { *round_idx = 0; *n_done = 0; *queue_head = B; }
+    if (b == 0) { *round_idx = 0; *queue_head = B; }
   }
 }
 
@@ -236,7 +236,7 @@ __global__ void accept_kernel(DdpmTables S, float* __restrict__ xt, long long xs
                               const float* __restrict__ eps, long long es_b, int* __restrict__ t, int K, int D,
                               const uint64_t* __restrict__ seedp, const RoundParams* __restrict__ sched, int n_sched,
                               const int* round_idx, float* __restrict__ actions,
-                              int* __restrict__ n_done, DevStats* __restrict__ stats, float draft_nfe,
+                              DevStats* __restrict__ stats, float draft_nfe,
                               float* __restrict__ dbg_logalpha, int* __restrict__ dbg_jstar,
                               const EnvParams* __restrict__ envp, int* __restrict__ item, int* __restrict__ queue_head,
                               const int* __restrict__ n_items, int* __restrict__ item_counts, RoundEnd rend) {
@@ -383,10 +383,7 @@ __global__ void accept_kernel(DdpmTables S, float* __restrict__ xt, long long xs
       int* ic = item_counts + 4 * (long long)env;
       ic[0] += K_eff; ic[1] += n_acc; ic[2] += 1; ic[3] += adv;
     }
-    if (t_new < 0) {
-      atomicAdd(&stats->chunks_done, 1ull);
-      atomicAdd(n_done, 1);
-    }
+    if (t_new < 0) atomicAdd(&stats->chunks_done, 1ull);
   }
   // Continuous batching: a slot whose request has finished takes the next waiting request, if any --
   // fresh x_T ~ N(0, I) from that request's own noise stream, t = T - 1.

@@ -101,7 +101,7 @@ struct tsdp_ctx {
   int *item = nullptr, *queue_head = nullptr, *n_items = nullptr;
   size_t items_cap = 0;
   uint64_t* seed = nullptr;
-  int *round_idx = nullptr, *n_done = nullptr, *status = nullptr;
+  int *round_idx = nullptr, *status = nullptr;
   int *round_blocks = nullptr, *t_left = nullptr;        // end-of-round bookkeeping of the acceptance kernel (RoundEnd)
   unsigned long long* host_prog = nullptr;    // mapped pinned: rounds complete << 32 | reverse steps still needed
   int* status_host = nullptr;                 // pinned copy of the status word at the end of a chunk call
@@ -272,7 +272,7 @@ void prof_end(tsdp_ctx* c, cudaStream_t s) {
 }
 
 // Live-row descriptor for a kernel whose launch was sized for `per` rows per candidate of the current forward.
-LiveRows live_desc(const tsdp_ctx* c, int per, int add = 0) { return LiveRows{c->live_n, per, add}; }
+LiveRows live_desc(const tsdp_ctx* c, int per) { return LiveRows{c->live_n, per}; }
 
 // (C_in, C_out) of the residual blocks of the conv UNet in execution order: two per level down, two in the
 // middle, two per level up (the first of which takes the concatenation [upsampled | skip]).
@@ -394,8 +394,7 @@ int get_map_conv(tsdp_ctx* c, const void* ptr, int n, int positions, int C, int 
 // round's plan back); otherwise the dense count.
 int gemm_rows_known(const tsdp_ctx* c, const GemmArgs& g) {
   if (g.live.n == nullptr || c->prof_live_count < 0) return g.M;
-  const int v = c->prof_live_count * g.live.mul + g.live.add;
-  return v < 0 ? 0 : (v < g.M ? v : g.M);
+  return std::min(c->prof_live_count * g.live.mul, g.M);
 }
 
 GemmArgs gemm_args(tsdp_ctx* c, int M, int N, int K, const float* bias, void* out, int ldo) {
@@ -552,7 +551,7 @@ int gemm(tsdp_ctx* c, const void* A, const void* W, const float* bias, int M, in
   if (c->live_n != nullptr && c->live_static > 0) {
     // rows per candidate of this GEMM: M = n rows_per
     const int n = c->live_static;
-    if (M % n == 0) g.live = LiveRows{c->live_n, M / n, 0};
+    if (M % n == 0) g.live = LiveRows{c->live_n, M / n};
   }
   if (c->cfg.precision == 0) {
     dim3 grid((N + 63) / 64, (M + 63) / 64);
@@ -742,7 +741,7 @@ int gemm_qkv_attn(tsdp_ctx* c, const void* A, const XfmrLayer& w, int M, int d, 
   const int N = 3 * d, K = d, BN = GEMM_ATTN_BN;
   GemmArgs g = gemm_args(c, M, N, K, w.bqkv_hm, out, d);
   g.causal = 1;
-  if (c->live_n != nullptr && c->live_static > 0 && M % c->live_static == 0) g.live = LiveRows{c->live_n, M / c->live_static, 0};
+  if (c->live_n != nullptr && c->live_static > 0 && M % c->live_static == 0) g.live = LiveRows{c->live_n, M / c->live_static};
   CUtensorMap ma, mb;
   int r;
   if ((r = get_map(c, A, 2, M, K, K, GEMM_BK, GEMM_BM, &ma)) != TSDP_OK) return r;
@@ -1438,7 +1437,7 @@ int enqueue_round(tsdp_ctx* c, int B, int K, cudaStream_t s, bool dbg) {
   if (warps > 16) warps = 16;
   prof_begin(c, s, 8, 0.0);
   TSDP_LAUNCH(c, (accept_kernel), B, warps * 32, 0, s, c->S, c->xt, xs_b, c->muhat, ms_b, c->eps, xs_b, c->t, K, D, c->seed, c->sched,
-                                         TSDP_MAX_T + 1, c->round_idx, c->actions, c->n_done, c->stats, c->cfg.draft_nfe,
+                                         TSDP_MAX_T + 1, c->round_idx, c->actions, c->stats, c->cfg.draft_nfe,
                                          dbg ? c->dbg_logalpha : nullptr, dbg ? c->dbg_jstar : nullptr,
                                          c->sched_on ? c->envp : nullptr, c->item, c->queue_head, c->n_items, c->item_counts,
                                          RoundEnd{c->round_blocks, c->t_left, c->round_idx, c->host_prog});
@@ -1671,7 +1670,6 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
   st |= dev_alloc(c, c->allocs, &c->t, B);
   st |= dev_alloc(c, c->allocs, &c->params, PARAMS_BYTES);
   st |= dev_alloc(c, c->allocs, &c->round_idx, 1);
-  st |= dev_alloc(c, c->allocs, &c->n_done, 1);
   st |= dev_alloc(c, c->allocs, &c->status, 1);
   st |= dev_alloc(c, c->allocs, &c->round_blocks, 1);
   st |= dev_alloc(c, c->allocs, &c->t_left, 1);
@@ -2435,7 +2433,7 @@ static int sample_chunk_impl(tsdp_ctx* c, const float* obs, bool obs_on_host, in
     c->launches++;
   }
   const long long xs_b = (long long)(c->cfg.max_K + 1) * D;
-  init_chunk_kernel<<<B, 128, 0, s>>>(c->xt, xs_b, c->t, B, D, T, c->seed, c->round_idx, c->n_done, c->item, c->queue_head,
+  init_chunk_kernel<<<B, 128, 0, s>>>(c->xt, xs_b, c->t, B, D, T, c->seed, c->round_idx, c->item, c->queue_head,
                                     c->item_counts, N);
   CU_TRY(c, cudaGetLastError());
   c->launches_per_round_tmp = 0;
@@ -2522,7 +2520,6 @@ int tsdp_round(tsdp_ctx* c, const float* d_obs, int B, int K, const tsdp_accept_
   if (obs_n) CU_TRY(c, cudaMemcpyAsync(c->obs, d_obs, obs_n * sizeof(float), cudaMemcpyDeviceToDevice, s));
   if ((r = upload_params(c, K, *acc, seed, B, s, true))) return r;
   CU_TRY(c, cudaMemsetAsync(c->round_idx, 0, sizeof(int), s));
-  CU_TRY(c, cudaMemsetAsync(c->n_done, 0, sizeof(int), s));
   {   // every slot serves the request of its own index and nothing is waiting
     std::vector<int> ident(B);
     for (int b = 0; b < B; ++b) ident[b] = b;
@@ -2850,7 +2847,7 @@ constexpr size_t ST_OFF_STATS = 0;                                            //
 constexpr size_t ST_OFF_TAB = 24832;                                          // 5 x TSDP_STATIC_MAX_T floats
 constexpr size_t ST_OFF_T = ST_OFF_TAB + 5 * TSDP_STATIC_MAX_T * 4;           // t[B]
 constexpr size_t ST_OFF_J = ST_OFF_T + TSDP_STATIC_MAX_B * 4;                 // j*[B]
-constexpr size_t ST_OFF_MISC = ST_OFF_J + TSDP_STATIC_MAX_B * 4;              // seed, round index, done count, round parameters
+constexpr size_t ST_OFF_MISC = ST_OFF_J + TSDP_STATIC_MAX_B * 4;              // seed, round index, round parameters
 constexpr size_t ST_BYTES = ST_OFF_MISC + 256;
 static_assert(sizeof(DevStats) <= ST_OFF_TAB, "statistics block overlaps the tables");
 static_assert(ST_OFF_TAB % 256 == 0 && ST_OFF_T % 256 == 0 && ST_OFF_J % 256 == 0 && ST_OFF_MISC % 256 == 0, "alignment");
@@ -2900,7 +2897,6 @@ int tsdp_verify_commit_static(int device, int T, float beta0, float beta1, float
   int* dj = reinterpret_cast<int*>(base + ST_OFF_J);
   uint64_t* dseed = reinterpret_cast<uint64_t*>(base + ST_OFF_MISC);
   int* dround = reinterpret_cast<int*>(base + ST_OFF_MISC + 8);
-  int* ddone = reinterpret_cast<int*>(base + ST_OFF_MISC + 12);
   RoundParams* drp = reinterpret_cast<RoundParams*>(base + ST_OFF_MISC + 16);
 
   float tab[5 * TSDP_STATIC_MAX_T];
@@ -2933,7 +2929,7 @@ int tsdp_verify_commit_static(int device, int T, float beta0, float beta1, float
   if (warps < 4) warps = 4;
   if (warps > 16) warps = 16;
   accept_kernel<<<B, warps * 32, 0, s>>>(S, d_xt, xs_b, d_muhat, ms_b, d_eps, xs_b, dt, K, D, dseed, drp, 1, dround,
-                                         d_actions, ddone, st, draft_nfe, d_logalpha, dj, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                         d_actions, st, draft_nfe, d_logalpha, dj, nullptr, nullptr, nullptr, nullptr, nullptr,
                                          RoundEnd{});
   ST_TRY(cudaGetLastError());
   ST_TRY(cudaMemcpyAsync(h_t_new, dt, sizeof(int) * B, cudaMemcpyDeviceToHost, s));

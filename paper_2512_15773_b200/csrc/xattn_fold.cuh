@@ -155,19 +155,6 @@ __host__ __device__ constexpr size_t xf_smem_bytes(int D, int nkh) {
          (size_t)16 * (XF_MAXN + 8) * 2;
 }
 
-// One block per candidate (H <= 16 token rows of width D), 8 warps.
-//   0  the candidate's kq and u rows start their way into shared memory (cp.async, 16 bytes per lane: a
-//      lane-by-lane gather of tensor-core fragments from global memory is bound by the L1 tag rate)
-//   1  xhat = LayerNorm without affine of the candidate's rows, bf16, into shared memory (warp w: rows 2w, 2w+1)
-//   2  partial scores: warp w covers a quarter of the D input columns for two of the 8-wide score tiles
-//   3  softmax over the memory tokens per (row, head) -> P [16 x 32] bf16
-//   4  warp w: output columns [w D/8, (w+1) D/8) of P . U for all 16 rows -> shared memory (fp32)
-//   5  warp w again owns rows 2w, 2w+1, whose residual values (stream + delta) are still in its registers from
-//      phase 1: adds the product and bo2, writes the stream back in full 16-byte lanes, and applies the LayerNorm in
-//      front of the MLP with warp-level statistics -> ln3_out (bf16)
-// `delta` is the output of the self-attention projection (bf16, bias included), which this kernel adds to the
-// residual stream before anything else: that GEMM then writes 2 bytes per element instead of doing an fp32
-// read-modify-write of the stream.
 // Mean and reciprocal standard deviation of the warp's two rows, both rows' shuffles in flight together.
 template <int V>
 __device__ __forceinline__ void xf_row_stats(const float4 (&x)[2][V], float (&mean)[2], float (&rstd)[2]) {
@@ -206,6 +193,19 @@ __device__ __forceinline__ void xf_row_stats(const float4 (&x)[2][V], float (&me
   for (int rr = 0; rr < 2; ++rr) rstd[rr] = rsqrtf(q[rr] * INV + 1e-5f);
 }
 
+// One block per candidate (H <= 16 token rows of width D), 8 warps.
+//   0  the candidate's kq and u rows start their way into shared memory (cp.async, 16 bytes per lane: a
+//      lane-by-lane gather of tensor-core fragments from global memory is bound by the L1 tag rate)
+//   1  xhat = LayerNorm without affine of the candidate's rows, bf16, into shared memory (warp w: rows 2w, 2w+1)
+//   2  partial scores: warp w covers a quarter of the D input columns for two of the 8-wide score tiles
+//   3  softmax over the memory tokens per (row, head) -> P [16 x 32] bf16
+//   4  warp w: output columns [w D/8, (w+1) D/8) of P . U for all 16 rows -> shared memory (fp32)
+//   5  warp w again owns rows 2w, 2w+1, whose residual values (stream + delta) are still in its registers from
+//      phase 1: adds the product and bo2, writes the stream back in full 16-byte lanes, and applies the LayerNorm in
+//      front of the MLP with warp-level statistics -> ln3_out (bf16)
+// `delta` is the output of the self-attention projection (bf16, bias included), which this kernel adds to the
+// residual stream before anything else: that GEMM then writes 2 bytes per element instead of doing an fp32
+// read-modify-write of the stream.
 template <int D>
 __global__ void __launch_bounds__(XF_THREADS, 3)
 xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta, XfoldTables tb, const float* __restrict__ bo2,
