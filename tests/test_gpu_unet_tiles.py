@@ -8,6 +8,7 @@ import torch
 from oracle import ddpm, nets
 from paper_2512_15773_b200 import binding, inputs
 from tests import helpers as hp
+from tests.test_gpu_round import _round_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -46,6 +47,22 @@ def test_unet_denoiser_tiles_and_groups(case, N):
             assert err < tol, (precision, n, err)
         assert smp.check_guards() > 0
         smp.close()
+
+
+# One warp per group, eight groups a block: from 32 groups per SM on (4736), four channels a group at least and at most 128 quads of values.
+# Two and three parts of a reduction, four to six, and none with every lane's registers full and a ragged last block (4740 groups).
+@pytest.mark.parametrize("case,N", [((8, 3, 2, 128, 32, 7), 151), ((4, 5, 2, 256, 64, 12), 75), ((16, 2, 1, 128, 4, 5), 1185)])
+def test_unet_denoiser_with_a_warp_per_group(case, N):
+    test_unet_denoiser_tiles_and_groups(case, N)
+
+
+def test_unet_round_with_a_warp_per_group_and_few_live_candidates():
+    """300 slots x 4 candidates x 4 groups; timesteps near the end leave 837 candidates alive, 3348 groups, the last block half full.
+    A rejected draft's reflection multiplies the error of mu^ - mu (3e-7) by 2 sigma |xi| / |mu^ - mu|: 70 at most for this drafter, so 2e-5
+    of the 6e-5 that the committed latent may be off.  (Frozen-target drafts have 490 here, beyond it.)"""
+    wl = dict(H=4, A=3, To=1, Do=6, T=100, precision=0, gamma=0.05, base=dict(arch="unet", layers=1, d=128, heads=4, temb=8),
+              draft=dict(arch="mlp", layers=1, width=64))
+    _round_parity(wl, 300, 3, hp.accept_t(), 13, 1e-4, 2e-5, [i % 5 for i in range(299)] + [0])
 
 
 def test_mish_behind_the_group_norm_keeps_fp32_accuracy():
