@@ -819,7 +819,7 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
           float z4[4];
           normal4(seed, (uint32_t)env, STREAM_XI, (uint32_t)tau, (uint32_t)(e_idx >> 2), z4);
           const int j = e_idx & 3;
-          e_x[e_z] = j == 0 ? z4[0] : (j == 1 ? z4[1] : (j == 2 ? z4[2] : z4[3]));      // (kept in registers, it was computed where it is used)
+          e_x[e_z] = j == 0 ? z4[0] : (j == 1 ? z4[1] : (j == 2 ? z4[2] : z4[3]));
           e_x[e_sig] = P.S.sigma[tau];
         }
       });

@@ -44,7 +44,7 @@ constexpr long long GEMM_WAIT_CYCLES = 2000000000ll;   // about one second of SM
 // k-blocks per pipeline stage.  A round of the issue loops (wait, loads or MMAs, arrive) takes about 336 clocks, the tensor
 // core 160 - 192 clocks per k-block for tiles up to 64 wide (operand reads from shared memory), so there a stage holds two
 // k-blocks and a round issues twice as much: 0.177 -> 0.135 us per k-block at BN = 64 (0.177 -> 0.130 at BN = 32).  At 128 two of
-// them leave only three stages and tie, wider tiles are bound by the MMAs (512 clocks per k-block at BN = 256).
+// them leave only three stages and tie; at 256 the MMAs of a k-block take 520 - 560 clocks, longer than a round of issuing.
 __host__ __device__ constexpr int gemm_stage_kb(int BN) { return BN <= 64 ? 2 : 1; }
 __host__ __device__ constexpr int gemm_stages(int BN) { return BN >= 192 ? 4 : (BN == 128 ? 6 : (BN == 64 ? 4 : 5)); }
 __host__ __device__ constexpr int gemm_stage_bytes(int BN) { return gemm_stage_kb(BN) * (GEMM_BM * GEMM_BK * 2 + BN * GEMM_BK * 2); }
@@ -100,8 +100,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 // Bounded wait: false when the barrier did not flip within `limit` SM clock cycles.  The first try stands alone and the loop
-// behind it is kept rolled: unrolled by the compiler it made 6 KB of code per wait, which the instruction caches paid for (code of
-// the cluster kernel 636 -> 134 KB, of a GEMM 38 -> 16; layered rounds 2 to 4 % faster, the cluster kernel's 9 to 13 %).
+// behind it is not unrolled: layered rounds are 2 to 4 % faster that way, the cluster kernel's 9 to 13 %.
 __device__ __forceinline__ bool mbar_wait_thread(uint32_t bar, uint32_t parity, long long limit = GEMM_WAIT_CYCLES) {
   if (mbar_try_wait(bar, parity)) return true;
 #pragma unroll 1
@@ -118,9 +117,8 @@ __device__ __forceinline__ bool mbar_wait_thread(uint32_t bar, uint32_t parity, 
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, long long limit = GEMM_WAIT_CYCLES) {
   return __all_sync(0xffffffffu, mbar_wait_thread(bar, parity, limit)) != 0;
 }
-// One lane of a converged warp, chosen by the hardware.  Under this predicate the compiler knows that a single thread
-// runs and issues tcgen05 / TMA instructions directly; under `lane == 0` it wraps each of them in a loop over the active
-// lanes (measured per k-block of four MMAs, wait and commit: 231 clocks against 467 for tiles up to 64 wide).
+// One lane of a converged warp, chosen by the hardware, to issue tcgen05 and TMA instructions: a k-block of four MMAs, wait and
+// commit takes 231 clocks, 467 under `lane == 0` (tiles up to 64 wide).
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));

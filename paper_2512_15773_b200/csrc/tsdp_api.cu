@@ -481,9 +481,9 @@ cudaError_t set_smem_attr_all() {
 
 // Tile width: the widest BN in {256, 128, 64, 32} dividing N whose tiles still fill 60 % of the SMs, else the
 // narrowest that divides N (small-batch calls are latency-bound and want many CTAs).  Measured on the block's
-// shapes at 4 k - 45 k rows: per flop a 128-wide tile costs 1.24x and a 64-wide one 2.15x of a 256-wide one (the
-// k-loop of a narrow tile is bound by loading the 128-row A block, which does not shrink), so a wide tile that
-// leaves a third of the SMs idle still beats two waves of narrow ones; below about half occupancy it does not.
+// shapes at 4 k - 45 k rows: per flop a 128-wide tile costs 1.16x, a 64-wide one 1.70x and a 32-wide one 2.5x of a 256-wide
+// one (45 056 x 1536 x 512: 66.3, 76.7, 112.7, 165.7 us), so a wide tile that leaves a third of the SMs idle still beats
+// two waves of narrow ones; below about half occupancy it does not.
 int pick_bn(int M, int N, int num_sms) {
   const int tm = (M + GEMM_BM - 1) / GEMM_BM;
   const int cands[4] = {256, 128, 64, 32};
@@ -506,7 +506,7 @@ int conv_split_rows(int M, int L) { const int tr = conv_tile_rows(L); return (M 
 // many times; cutting the k range of wider tiles uses the idle SMs instead.  Each part writes a buffer of its own and the
 // GroupNorm kernel that consumes them adds the parts in order (the same bits whatever ran where; a function of
 // the launch shape only).  The choice is the cheapest by measured figures: start and epilogue of a launch, time per
-// k-block (both by tile width), and 8 bytes more per value and part for the partial sums.
+// k-block (both by tile width; 256: 557 clocks, the MMAs' own time), and 8 bytes more per value and part for the partial sums.
 ConvSpec conv_plan(const tsdp_ctx* c, int n_cand, int cch, int L, int off, int N, int taps, size_t cap_elems, bool may_split) {
   ConvSpec best{cch, L, off, 0, 1};
   if (c->cfg.precision == 0 || c->force_bn > 0) return best;
