@@ -388,7 +388,8 @@ __device__ __forceinline__ void epilogue_store16(const GemmArgs& g, int row, int
 // warp issues for both; stage and accumulator hand-over barriers are signalled in both CTAs by multicast commits, the
 // stage-full and accumulator-empty barriers live in the leader and are signalled from both CTAs.  Per flop each SM
 // pulls a third fewer operand bytes from the L2, which is what bounds the 128 x 256 form at K = 512.
-template <int BN, int EPI, int CG = 1>
+// LONG: the form of the fused attention kernel for launches of more than two tiles per CTA (see the MMA warp).
+template <int BN, int EPI, int CG = 1, bool LONG = false>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmC, GemmArgs g) {
@@ -504,7 +505,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
     pdl_trigger();
   } else if (warp == 1) {
-    auto issue = [&] {
+    // In a pair only the leader issues.  The fused attention's epilogue multiplies on the tensor cores too, and beside a long stream of
+    // MMAs at the elected lane's pace it falls behind: in its LONG form lane 0 issues, which is slower (d = 512, us at 1, 2, 3, 7 and 16
+    // tiles per CTA: elected 6.55, 9.8, 16.2, 29.7, 58.6, lane 0 6.96, 10.2, 15.5, 26.7, 53.7; equal at 2.5).
+    if (rank == 0 && (LONG ? lane == 0 : ptx::elect_one())) {
       int stage = 0; uint32_t phase = 0; int it = 0;
       for (int unit = tile0; unit < n_tiles && ok; unit += tile_step, ++it) {
         const int part = unit % S;
@@ -534,14 +538,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (!ok) break;
         if (CG == 2) ptx::tc_commit_pair(tfull_bar(as)); else ptx::tc_commit(tfull_bar(as));
       }
-    };
-    // In a pair only the leader issues.  The fused attention's epilogue multiplies on the tensor cores too, and beside a long stream of
-    // MMAs at the elected lane's pace it falls behind: there lane 0 issues, which is slower (d = 512, us at 1, 2, 3, 7 and 16 tiles per
-    // CTA: elected 6.55, 9.8, 16.2, 29.7, 58.6, lane 0 6.96, 10.2, 15.5, 26.7, 53.7; equal at 2.5).
-    if (EPI == EPI_ATTN && n_tiles > 2 * tile_step) {
-      if (rank == 0 && lane == 0) issue();
-    } else if (rank == 0 && ptx::elect_one()) {
-      issue();
     }
   } else {
     const int ew = warp - 2;

@@ -756,7 +756,8 @@ int gemm_qkv_attn(tsdp_ctx* c, const void* A, const XfmrLayer& w, int M, int d, 
   } else {
     const int tiles = ((M + GEMM_BM - 1) / GEMM_BM) * (N / BN);
     const int grid = tiles < c->num_sms ? tiles : c->num_sms;
-    TSDP_LAUNCH(c, (gemm_tcgen05_kernel<GEMM_ATTN_BN, EPI_ATTN>), grid, GEMM_THREADS, gemm_smem_bytes(BN), s, ma, mb, ma, g);
+    if (tiles > 2 * grid) TSDP_LAUNCH(c, (gemm_tcgen05_kernel<GEMM_ATTN_BN, EPI_ATTN, 1, true>), grid, GEMM_THREADS, gemm_smem_bytes(BN), s, ma, mb, ma, g);
+    else TSDP_LAUNCH(c, (gemm_tcgen05_kernel<GEMM_ATTN_BN, EPI_ATTN>), grid, GEMM_THREADS, gemm_smem_bytes(BN), s, ma, mb, ma, g);
   }
   prof_end(c, s);
   c->launches_per_round_tmp++;
@@ -1743,6 +1744,8 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
     INIT_TRY(set_smem_attr_all<64>());
     INIT_TRY(set_smem_attr_all<32>());
     INIT_TRY(cudaFuncSetAttribute(gemm_tcgen05_kernel<GEMM_ATTN_BN, EPI_ATTN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  gemm_smem_bytes(GEMM_ATTN_BN)));
+    INIT_TRY(cudaFuncSetAttribute(gemm_tcgen05_kernel<GEMM_ATTN_BN, EPI_ATTN, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   gemm_smem_bytes(GEMM_ATTN_BN)));
     if (const char* pm = getenv("TSDP_GEMM_PAIR")) c->pair_mode = atoi(pm);
     if (c->pair_mode != 0) {      // CTA-pair kernels: shared-memory opt-in and how many clusters of 2 the device holds at once
