@@ -67,8 +67,8 @@ struct Net {
   __nv_bfloat16 *fold_kq_time = nullptr, *fold_ut_time = nullptr, *fold_kq_obs = nullptr, *fold_ut_obs = nullptr;
   float *fold_c_time = nullptr, *fold_c_obs = nullptr;
   // XFMR small enough for the cluster kernel: weights in the order its lanes read them, per-CTA parameters (drafter_cluster.cuh)
-  __nv_bfloat16* dc_w = nullptr;
-  float* dc_par = nullptr;
+  __nv_bfloat16* dc_w[2] = {};                // for clusters of 8 and of 4
+  float* dc_par[2] = {};
   float* mod = nullptr;                       // DIT: [T, L*6d + 2d] shift / scale / gate vectors of every timestep
   int mod_ld = 0;
   // UNET: residual blocks in execution order, FiLM tables, head
@@ -150,13 +150,9 @@ struct tsdp_ctx {
   bool pdl = true;                            // programmatic dependent launch between the kernels of a round
   int tc_attn = 1;                            // context cross-attention on tcgen05: 0 never (TSDP_NO_TC_ATTN), 1 large groups, 2 always (TSDP_TC_ATTN=2)
   bool async_bcast = true;                    // cluster kernel: st.async + mbarrier stage hand-over (TSDP_NO_ASYNC_BCAST unset)
-  bool dc_ok = false;
+  // the cluster kernel for a net: clusters of 8 CTAs [0] and of 4 [1]
+  struct ClusterPlan { bool ok = false, resident = false; int smem = 0, max_clusters = 0; } dc[2], cv[2];      // drafter; base model (verification)
   bool no_ksplit = false;                      // TSDP_NO_KSPLIT: convolution GEMMs never split their reduction
-  int dc_smem = 0, dc_max_clusters = 0;
-  bool dc_resident = false;
-  // the same cluster kernel running the BASE model's verification forward (small batches of small transformers)
-  bool cv_ok = false, cv_resident = false;
-  int cv_smem = 0, cv_max_clusters = 0;
   uint64_t rounds = 0, launches = 0;
   int launches_per_round_tmp = 0;
   // plan of a round (round_plan_kernel): compacted candidate list of the verification forward, slot order and
@@ -1280,44 +1276,63 @@ int forward_arch(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, cudaStream_
 // ------------------------------------------------------------------------------------------ drafter
 constexpr int DC_SMEM_LIMIT = 227 * 1024;
 typedef void (*ClusterKernel)(const DcParams);
-ClusterKernel cluster_kernel_of(int d, int dh) {
-  if (d == 128) return dh == 32 ? drafter_cluster_kernel<128, 32> : (dh == 64 ? drafter_cluster_kernel<128, 64> : (dh == 128 ? drafter_cluster_kernel<128, 128> : nullptr));
-  if (d == 256) return dh == 32 ? drafter_cluster_kernel<256, 32> : (dh == 64 ? drafter_cluster_kernel<256, 64> : (dh == 128 ? drafter_cluster_kernel<256, 128> : nullptr));
-  return nullptr;
+constexpr int DC_SIZES[2] = {8, 4};      // CTAs per cluster
+template <int D>
+ClusterKernel cluster_kernel_of(int dh, int cs) {
+  if (dh != 32 && dh != 64 && dh != 128) return nullptr;
+  if (cs == 8) return dh == 32 ? drafter_cluster_kernel<D, 32, 8> : (dh == 64 ? drafter_cluster_kernel<D, 64, 8> : drafter_cluster_kernel<D, 128, 8>);
+  if (D / dh > 4) return nullptr;        // a CTA works on one head
+  return dh == D / 4 ? drafter_cluster_kernel<D, D / 4, 4> : (dh == D / 2 ? drafter_cluster_kernel<D, D / 2, 4> : nullptr);
 }
-// Whether the persistent cluster kernel can run this context's drafter at all (shapes, shared memory).
-bool cluster_drafter_fits(const tsdp_config_t& cfg, const tsdp_net_t& n, int* smem_bytes, bool* resident) {
+ClusterKernel cluster_kernel_of(int d, int dh, int cs) {
+  return d == 128 ? cluster_kernel_of<128>(dh, cs) : (d == 256 ? cluster_kernel_of<256>(dh, cs) : nullptr);
+}
+// Whether the persistent cluster kernel can run this net at all in clusters of `cs` (shapes, shared memory).
+bool cluster_drafter_fits(const tsdp_config_t& cfg, const tsdp_net_t& n, int cs, int* smem_bytes, bool* resident) {
   if (cfg.precision != 1 || n.arch != TSDP_ARCH_XFMR || (n.d != 128 && n.d != 256) || n.layers > DC_MAX_LAYERS ||
-      cfg.H > DC_ROWS || 1 + cfg.obs_tokens > DC_MAX_NK || cfg.H * cfg.A > 256 || !cluster_kernel_of(n.d, n.d / n.heads))
+      cfg.H > DC_ROWS || 1 + cfg.obs_tokens > DC_MAX_NK || cfg.H * cfg.A > 256 || (cs < 8 && dc_own(cs) * cfg.A > 128) ||
+      !cluster_kernel_of(n.d, n.d / n.heads, cs))
     return false;
   // weight slices resident in shared memory if they fit beside the activations, otherwise through a ring of chunks
   for (int res = 1; res >= 0; --res) {
-    const DcSmem pl = dc_smem_plan(n.d, n.d / n.heads, n.layers, cfg.A, res != 0, DC_SMEM_LIMIT);
+    const DcSmem pl = dc_smem_plan(n.d, n.d / n.heads, cs, n.layers, cfg.A, res != 0, DC_SMEM_LIMIT);
     if (pl.total <= DC_SMEM_LIMIT) { *smem_bytes = pl.total; *resident = res != 0; return true; }
   }
   return false;
 }
 
+// Cluster size for `work` rollouts or candidates: 0 for clusters of 8, 1 for clusters of 4.  A forward in a cluster of 4 takes about 1.25 times as long
+// (the exchanges take the same time, the k loops twice), but 33 of them run at once instead of 15; both give the same bits.  32 environments,
+// 8 steps of a d = 256 drafter of 4 blocks: 914 us in three waves of clusters of 8, calls of the conv-UNet policy 21.8 -> 15.0 ms.
+int cluster_size_of(const tsdp_ctx::ClusterPlan (&pl)[2], int work) {
+  if (!pl[1].ok) return 0;
+  const int w8 = (work + pl[0].max_clusters - 1) / pl[0].max_clusters, w4 = (work + pl[1].max_clusters - 1) / pl[1].max_clusters;
+  return 5 * w4 < 4 * w8 ? 1 : 0;
+}
+
 bool use_cluster_drafter(const tsdp_ctx* c, int B) {
-  if (!c->dc_ok || c->cfg.drafter == 1) return false;
+  if (!c->dc[0].ok || c->cfg.drafter == 1) return false;
   if (c->cfg.drafter == 2) return true;
-  // Beyond a few waves of clusters (15 at a time) the layer-by-layer path wins.  Whole calls, cluster / layered: weights streamed
-  // (d = 256, conv-UNet base) 20 environments 16.5 / 21.0 ms, 32 21.8 / 22.6, (d = 512 base) 48 26.4 / 25.4; resident weights (d = 128) 24
-  // environments 8.6 / 10.5 ms, 40 10.7 / 12.5, 64 14.5 / 14.0.
-  return B <= (c->dc_resident ? 4 : 3) * c->dc_max_clusters;
+  // Beyond a few waves of clusters (15 of 8 CTAs or 33 of 4 at a time) the layer-by-layer path wins.  Whole calls, cluster / layered, ms:
+  // d = 256 (conv-UNet base) 33 environments 16.9 / 23.6, 48 23.9 / 25.5, 64 25.2 / 27.0, 96 34.2 / 32.1, (d = 512 base) 64 25.3 / 26.1, 96 32.4 / 31.2;
+  // d = 128 40 environments 9.0 / 10.3, 64 11.5 / 13.1, 96 13.3 / 13.8, 128 17.0 / 16.7.
+  if (c->dc[1].ok) return B <= (c->cfg.draft.d <= 128 ? 3 : 2) * c->dc[1].max_clusters;
+  return B <= (c->dc[0].resident ? 4 : 3) * c->dc[0].max_clusters;
 }
 
 bool use_cluster_verifier(const tsdp_ctx* c, int B, int K) {
-  if (!c->cv_ok || c->cfg.verifier == 1) return false;
+  if (!c->cv[0].ok || c->cfg.verifier == 1) return false;
   if (c->cfg.verifier == 2) return true;
-  return B * (K + 1) <= c->cv_max_clusters;     // every candidate gets its own cluster in one wave
+  // Every candidate gets its own cluster of 8 in one wave.  Clusters of 4 would be faster up to 66 candidates (whole calls of a d = 256 base of 8
+  // blocks, cluster / layered, ms: 18 candidates 2.97 / 4.21, 32 3.27 / 4.72, 64 4.79 / 4.95, 81 5.71 / 4.84), but the two forwards
+  // round differently, and a queue through a few slots keeps the bits of the same requests in one batch from 16 candidates on.
+  return B * (K + 1) <= c->cv[0].max_clusters;
 }
 
 // mode 0: K-step draft rollout with the drafter; mode 1: verification forward of the base model on K+1 candidates.
 int launch_cluster_forward(tsdp_ctx* c, int which, int mode, int B, int K, cudaStream_t s) {
   const Net& n = c->net[which];
   DcParams P{};
-  P.Wf = n.dc_w; P.parf = n.dc_par;
   P.layers = n.cfg.layers; P.heads = n.cfg.heads; P.H = c->cfg.H; P.A = c->cfg.A; P.To = c->cfg.obs_tokens; P.T = c->cfg.T;
   P.W_in = n.W_in; P.b_in = n.b_in; P.pos = n.pos;
   P.lnf_g = n.lnf_g; P.lnf_b = n.lnf_b; P.W_outT = n.W_outT; P.b_out = n.b_out;
@@ -1336,13 +1351,15 @@ int launch_cluster_forward(tsdp_ctx* c, int which, int mode, int B, int K, cudaS
   P.envp = c->sched_on ? c->envp : nullptr;
   P.item = c->item;
   const bool verify = mode == 1;
-  P.resident = (verify ? c->cv_resident : c->dc_resident) ? 1 : 0;
-  P.n_slots = dc_smem_plan(n.cfg.d, n.cfg.d / n.cfg.heads, n.cfg.layers, c->cfg.A, P.resident != 0, DC_SMEM_LIMIT).n_slots;
-  const int maxc = verify ? c->cv_max_clusters : c->dc_max_clusters, smem = verify ? c->cv_smem : c->dc_smem;
   const int work = verify ? B * (K + 1) : B;
-  const int ncl = work < maxc ? work : maxc;
+  const int sz = cluster_size_of(verify ? c->cv : c->dc, work), cs = DC_SIZES[sz], dh = n.cfg.d / n.cfg.heads;
+  const tsdp_ctx::ClusterPlan& pl = (verify ? c->cv : c->dc)[sz];
+  P.Wf = n.dc_w[sz]; P.parf = n.dc_par[sz];
+  P.resident = pl.resident ? 1 : 0;
+  P.n_slots = dc_smem_plan(n.cfg.d, dh, cs, n.cfg.layers, c->cfg.A, pl.resident, DC_SMEM_LIMIT).n_slots;
+  const int ncl = work < pl.max_clusters ? work : pl.max_clusters;
   prof_begin(c, s, verify ? 9 : 7, 0.0);
-  TSDP_LAUNCH(c, cluster_kernel_of(n.cfg.d, n.cfg.d / n.cfg.heads), ncl * DC_CS, DC_THREADS, smem, s, P);
+  TSDP_LAUNCH(c, cluster_kernel_of(n.cfg.d, dh, cs), ncl * cs, DC_THREADS, pl.smem, s, P);
   prof_end(c, s);
   c->launches_per_round_tmp++;
   CU_TRY(c, cudaGetLastError());
@@ -1771,31 +1788,33 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
                 c->pair_clusters_attn);
     }
   }
-  for (int which = 0; which < 2; ++which) {
+  for (int i = 0; i < 4; ++i) {
+    const int which = i >> 1, sz = i & 1, cs = DC_SIZES[sz];
     const tsdp_net_t& nn = which == TSDP_BASE ? cfg->base : cfg->draft;
     int smem = 0; bool res = false;
-    if (!cluster_drafter_fits(*cfg, nn, &smem, &res)) continue;
-    const void* fn = (const void*)cluster_kernel_of(nn.d, nn.d / nn.heads);
+    if (!cluster_drafter_fits(*cfg, nn, cs, &smem, &res)) continue;
+    const void* fn = (const void*)cluster_kernel_of(nn.d, nn.d / nn.heads, cs);
     int cur_attr = 0;   // both nets may use the same instantiation: keep the larger request
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, fn) == cudaSuccess) cur_attr = fa.maxDynamicSharedSizeBytes;
     if (smem > cur_attr) INIT_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(DC_CS * 64); lc.blockDim = dim3(DC_THREADS); lc.dynamicSmemBytes = (size_t)smem;
+    lc.gridDim = dim3(cs * 64); lc.blockDim = dim3(DC_THREADS); lc.dynamicSmemBytes = (size_t)smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = DC_CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     lc.attrs = at; lc.numAttrs = 1;
     int ncl = 0;
     if (cudaOccupancyMaxActiveClusters(&ncl, fn, &lc) != cudaSuccess || ncl < 1) { cudaGetLastError(); ncl = 0; }
-    if (which == TSDP_DRAFT) { c->dc_smem = smem; c->dc_resident = res; c->dc_max_clusters = ncl; c->dc_ok = ncl >= 1; }
-    else { c->cv_smem = smem; c->cv_resident = res; c->cv_max_clusters = ncl; c->cv_ok = ncl >= 1; }
+    tsdp_ctx::ClusterPlan& pl = (which == TSDP_DRAFT ? c->dc : c->cv)[sz];
+    pl.smem = smem; pl.resident = res; pl.max_clusters = ncl; pl.ok = ncl >= 1;
+    if (getenv("TSDP_VERBOSE")) fprintf(stderr, "tsdp_init: net %d, clusters of %d: %d bytes, resident %d, %d at once\n", which, cs, smem, (int)res, ncl);
   }
-  if (cfg->verifier == 2 && !c->cv_ok) {
+  if (cfg->verifier == 2 && !c->cv[0].ok) {
     fprintf(stderr, "tsdp_init: the cluster verification kernel does not fit this configuration\n");
     return fail(TSDP_ERR_UNSUPPORTED);
   }
-  if (cfg->drafter == 2 && !c->dc_ok) {
+  if (cfg->drafter == 2 && !c->dc[0].ok) {
     fprintf(stderr, "tsdp_init: the persistent cluster drafter does not fit this configuration\n");
     return fail(TSDP_ERR_UNSUPPORTED);
   }
@@ -2270,21 +2289,23 @@ int tsdp_load_weights(tsdp_ctx* c, int which, const float* blob, size_t n) {
       if ((r = xfold_build(c, net, net.kv_time, T, net.fold_kq_time, net.fold_ut_time, net.fold_c_time, 0))) return r;
     }
     int smem_unused; bool res_unused;
-    if (cluster_drafter_fits(cfg, net.cfg, &smem_unused, &res_unused)) {
+    for (int sz = 0; sz < 2; ++sz) {
+      const int cs = DC_SIZES[sz];
+      if (!cluster_drafter_fits(cfg, net.cfg, cs, &smem_unused, &res_unused)) continue;
       const int di = (int)d, dhi = di / net.cfg.heads;
-      const size_t lw = (size_t)DC_CS * dc_layer_bytes(di, dhi) / 2, lp = (size_t)DC_CS * dc_par_floats(di, dhi);
-      if (dev_alloc(c, net.allocs, &net.dc_w, L * lw)) return TSDP_ERR_CUDA;
-      if (dev_alloc(c, net.allocs, &net.dc_par, L * lp)) return TSDP_ERR_CUDA;
+      const size_t lw = (size_t)cs * dc_layer_bytes(di, dhi, cs) / 2, lp = (size_t)cs * dc_par_floats(di, dhi, cs);
+      if (dev_alloc(c, net.allocs, &net.dc_w[sz], L * lw)) return TSDP_ERR_CUDA;
+      if (dev_alloc(c, net.allocs, &net.dc_par[sz], L * lp)) return TSDP_ERR_CUDA;
       for (size_t l = 0; l < L; ++l) {
         const XfmrLayer& w = net.L[l];
         const void* slabs[6] = {w.Wqkv, w.Wo, w.W1, w.W2, w.Wq2, w.Wo2};
         for (int s = 0; s < 6; ++s) {
-          const long long nel = (long long)dc_slab_rows(di, dhi, s) * dc_slab_k(di, s) * DC_CS;
+          const long long nel = (long long)dc_slab_rows(di, dhi, s, cs) * dc_slab_k(di, s, cs) * cs;
           dc_pack_kernel<<<(unsigned)((nel + 255) / 256), 256>>>(reinterpret_cast<const __nv_bfloat16*>(slabs[s]), s == 3 ? 4 * di : di,
-                                                                 net.dc_w + l * lw, di, dhi, s);
+                                                                 net.dc_w[sz] + l * lw, di, dhi, s, cs);
         }
         const DcParSrc ps{{w.ln1_g, w.ln1_b, w.ln2_g, w.ln2_b, w.ln3_g, w.ln3_b, w.bo, w.bo2, w.b2}, w.bqkv, w.b1, w.bq2};
-        dc_pack_par_kernel<<<DC_CS, 256>>>(ps, net.dc_par + l * lp, di, dhi);
+        dc_pack_par_kernel<<<cs, 256>>>(ps, net.dc_par[sz] + l * lp, di, dhi, cs);
       }
       CU_TRY(c, cudaGetLastError());
     }
