@@ -2,6 +2,7 @@
 // warp reductions.  Written for sm_100a; nothing here is shared with the CPU oracle.
 #pragma once
 #include <cuda_bf16.h>
+#include <type_traits>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -84,14 +85,17 @@ __device__ __forceinline__ float ddpm_sample(float mu, float sigma, float xi) { 
 // Programmatic dependent launch: a kernel signals that its successor in the stream may be scheduled, and waits (after
 // whatever set-up touches no shared data) until every kernel it depends on has completed and its memory is visible.
 // Both are no-ops for a kernel launched without the attribute.
-// The signal is given only by grids that leave half the chip free.  The successor's blocks are placed when it is given: on a
-// nearly full chip they crowd onto the few free SMs and run two or three to an SM with others idle, which costs more
-// than the launch latency saved.  Measured, signal at the start of every kernel -> this rule: 96 environments vanilla 56.2 ->
+// The signal is given by grids that leave half the chip free, and by kernels whose successor is a tensor-core GEMM (`always`: bf16 LayerNorms,
+// attentions, GroupNorms, the cross-attention sub-block, the GEMMs in front of another GEMM).  The successor's blocks are placed when it is
+// given: on a nearly full chip small blocks crowd onto the few free SMs and run two or three to an SM with others idle, which costs more
+// than the launch latency saved.  A GEMM has one CTA on an SM whatever happens, so its launch and its set-up (barriers, tensor memory, descriptors)
+// pass while the kernel before it runs.  Measured, signal at the start of every kernel -> by the grid alone: 96 environments vanilla 56.2 ->
 // 53.9 ms, 32 of the UNet workload 25.0 -> 23.0, 24 of the Push-T-shaped one 11.05 -> 10.46 (no signal at all: 53.9,
-// 24.3, 10.65).  The GEMM signals when its last operand loads are issued, the others when they start.
+// 24.3, 10.65); by the grid alone -> in front of GEMMs too: 96 vanilla 49.7 -> 48.5, 21 UNet frozen 9.08 -> 8.78, 3 VLA 62.5 -> 60.6.
+// The GEMM signals when its last operand loads are issued, the others when they start.
 constexpr unsigned PDL_MAX_GRID = 74;      // half of a B200's SMs
-__device__ __forceinline__ void pdl_trigger() {
-  if (gridDim.x * gridDim.y <= PDL_MAX_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+__device__ __forceinline__ void pdl_trigger(bool always = false) {
+  if (always || gridDim.x * gridDim.y <= PDL_MAX_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -61,7 +61,7 @@ cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_c
                          __nv_bfloat16* __restrict__ out, int kv_off, CandMap cm, int rows_per_slot, int d, int heads, int Tc,
                          const int* __restrict__ slot_start, int H, int splits, int* __restrict__ status) {
   extern __shared__ uint8_t cxt_raw[];
-  pdl_trigger();
+  pdl_trigger(true);
   const uint32_t base = (ptx::smem_u32(cxt_raw) + 1023u) & ~1023u;
   uint8_t* gbase = cxt_raw + (base - ptx::smem_u32(cxt_raw));
   const uint32_t sQ = base, sK = base + CXT_OFF_K, sVt = base + CXT_OFF_VT, bar0 = base + CXT_OFF_BAR;

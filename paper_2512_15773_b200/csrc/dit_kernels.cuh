@@ -28,7 +28,7 @@ __device__ __forceinline__ int row_tau(const CandMap& cm, int row, int H, int Ts
 template <typename T, int VEC>
 __global__ void ln_mod_kernel(const float* __restrict__ h, const float* __restrict__ mod, int mod_ld, int off_shift,
                               int off_scale, CandMap cm, int H, int Tsteps, T* __restrict__ out, int M) {
-  pdl_trigger();
+  pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
   constexpr int d = VEC * 128;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(CX_WARPS * 32)
 cross_attn_ctx_mma_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ out,
                           const __nv_bfloat16* __restrict__ kv, long long ld_kv, int kv_off, CandMap cm, int rows_per_slot,
                           int d, int heads, int Tc, const int* __restrict__ slot_start, int H) {
-  pdl_trigger();
+  pdl_trigger(true);
   pdl_wait();
   extern __shared__ __align__(16) uint8_t cx_raw[];
   constexpr int P = DH + 8, KS = DH / 16, NO = DH / 8;

@@ -21,7 +21,7 @@ __global__ void draft_tail_kernel(float* __restrict__ h, const float* __restrict
                                   const float* __restrict__ pos, const float* __restrict__ ln1_g, const float* __restrict__ ln1_b,
                                   T* __restrict__ a_out, int embed_next, int M, int H, int A,
                                   const int* __restrict__ order, const int* __restrict__ n_live) {
-  pdl_trigger();
+  pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
   constexpr int d = VEC * 128;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);

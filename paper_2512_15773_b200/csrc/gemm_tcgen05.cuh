@@ -503,7 +503,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         }
       }
     }
-    pdl_trigger();
+    pdl_trigger(EPI == EPI_ATTN || EPI == EPI_GELU);      // the product behind them is a GEMM too
   } else if (warp == 1) {
     // In a pair only the leader issues.  The fused attention's epilogue multiplies on the tensor cores too, and beside a long stream of
     // MMAs at the elected lane's pace it falls behind: in its LONG form lane 0 issues, which is slower (d = 512, us at 1, 2, 3, 7 and 16

@@ -182,7 +182,7 @@ __device__ __forceinline__ void store4(__nv_bfloat16* o, float a, float b, float
 template <typename T, int VEC>
 __global__ void ln_kernel(const float* __restrict__ h, const float* __restrict__ gam, const float* __restrict__ bet,
                           T* __restrict__ out, int M, LiveRows lv) {
-  pdl_trigger();
+  pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
   constexpr int d = VEC * 128;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -266,7 +266,7 @@ template <typename T, int VEC>
 __global__ void embed_ln_kernel(CandMap cm, const float* __restrict__ W_in, const float* __restrict__ b_in,
                                 const float* __restrict__ pos, float* __restrict__ h, const float* __restrict__ gam,
                                 const float* __restrict__ bet, T* __restrict__ out, int M, int H, int A) {
-  pdl_trigger();
+  pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
   constexpr int d = VEC * 128;
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -402,7 +402,7 @@ template <int DH>
 __global__ void __launch_bounds__(SA_WARPS * 32)
 self_attn_mma_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
                      int heads, int causal, LiveRows lv) {
-  pdl_trigger();
+  pdl_trigger(true);
   pdl_wait();
   n_cand = live_rows(lv, n_cand);
   constexpr int KS = DH / 16;        // k-steps of Q K^T
@@ -528,7 +528,7 @@ template <int DH>
 __global__ void __launch_bounds__((DH > 64 ? 2 : 4) * 32)
 self_attn_tile_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
                       int heads, int causal, LiveRows lv) {
-  pdl_trigger();
+  pdl_trigger(true);
   pdl_wait();
   n_cand = live_rows(lv, n_cand);
   constexpr int TW = DH > 64 ? 2 : 4;
@@ -586,7 +586,7 @@ template <int DH>
 __global__ void __launch_bounds__(128)
 self_attn_staged_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
                         int heads, int causal, LiveRows lv) {
-  pdl_trigger();
+  pdl_trigger(true);
   pdl_wait();
   constexpr int KS = DH / 16, NO = DH / 8, P = DH + 8, VPR = DH / 8;
   extern __shared__ __align__(16) uint8_t sa_raw[];

@@ -45,7 +45,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 unet_embed_kernel(CandMap cm, const float* __restrict__ W_in, const float* __restrict__ b_in,
                   T* __restrict__ X, int H, int A, int C) {
-  pdl_trigger();
+  pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
   const int n = blockIdx.x;
   if (n >= cand_count(cm, gridDim.x)) return;
@@ -171,7 +171,7 @@ constexpr int GN_ITEMS = 4;
 template <typename T, int TPG, int MAXS>
 __global__ void __launch_bounds__(TPG == 32 ? 256 : TPG)
 gn_mish_kernel(GnArgs g, CandMap cm, int n_static) {
-  pdl_trigger();
+  pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
   constexpr int GPB = TPG == 32 ? 8 : 1;                  // groups per block
   __shared__ float s_red[2][TPG / 32];
