@@ -1072,11 +1072,12 @@ int unet_gn(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, const float* gam
   // beyond
   if (Cg % 4 != 0 || items > GN_ITEMS * 128) TSDP_LAUNCH(c, (gn_mish_any_kernel<T>), all, 256, 0, s, g, cm, n_cand);
   else if (items > GN_ITEMS * 32 || all < 32 * c->num_sms) {
-    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 8>), all, 128, 0, s, g, cm, n_cand);
-    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 2>), all, 128, 0, s, g, cm, n_cand);
+    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 8, true>), all, 128, 0, s, g, cm, n_cand);
+    else if (all < 14 * c->num_sms) TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 2, true>), all, 128, 0, s, g, cm, n_cand);
+    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 2, false>), all, 128, 0, s, g, cm, n_cand);
   } else {
-    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 8>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
-    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 2>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
+    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 8, true>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
+    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 2, true>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
   }
   prof_end(c, s);
   c->launches_per_round_tmp++;

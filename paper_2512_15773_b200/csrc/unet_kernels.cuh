@@ -167,9 +167,13 @@ __device__ __forceinline__ float4 gn_load4(const __nv_bfloat16* p) {
 // all values in flight together), statistics in two steps in registers, 8-byte bf16 stores.  One warp per group (no
 // block barrier) where there are enough groups to fill the chip, four where there are not.  MAXS: parts.
 // 288 candidates x 8 groups of 512 values: 12.6 us with 256 scalar threads per group and two passes over Y.
+// PRE: the sums (those of a candidate past the live ones exist) are on their way beside the live count and the candidate, whose timestep and
+// request follow and then, beside the statistics, the affine and FiLM vectors, in place of one behind the other.  64 registers a thread
+// in place of 56, which costs blocks of four warps more than it gives on a full chip: whole UNet calls without and with it, 1 environment 8.81 / 8.64 ms,
+// 6 10.18 / 9.98, 21 with frozen drafts 8.63 / 8.47, 28 9.05 / 9.01, 32 15.29 / 15.40, 100 (a warp per group) 31.2 / 31.0.
 constexpr int GN_ITEMS = 4;
-template <typename T, int TPG, int MAXS>
-__global__ void __launch_bounds__(TPG == 32 ? 256 : TPG)
+template <typename T, int TPG, int MAXS, bool PRE>
+__global__ void __launch_bounds__(TPG == 32 ? 256 : TPG, MAXS == 2 ? (TPG == 32 ? 4 : (PRE ? 8 : 9)) : 1)
 gn_mish_kernel(GnArgs g, CandMap cm, int n_static) {
   pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
@@ -178,7 +182,7 @@ gn_mish_kernel(GnArgs g, CandMap cm, int n_static) {
   __shared__ float4 s_pool[GPB][GN_ITEMS * TPG];
   const int sub = TPG == 32 ? (threadIdx.x >> 5) : 0, t = TPG == 32 ? (threadIdx.x & 31) : threadIdx.x;
   const int gid = blockIdx.x * GPB + sub, n = gid / g.groups, grp = gid - n * g.groups;
-  if (n >= cand_count(cm, n_static)) return;              // the whole warp (TPG 32) or block
+  if (n >= (PRE ? n_static : cand_count(cm, n_static))) return;      // the whole warp (TPG 32) or block
   const int Cg = g.C / g.groups, quads = Cg >> 2, items = g.L * quads, cnt = g.L * Cg;
   const int q_step = TPG % quads, l_step = TPG / quads;
   int lj[GN_ITEMS], qj[GN_ITEMS];
@@ -196,14 +200,28 @@ gn_mish_kernel(GnArgs g, CandMap cm, int n_static) {
       const float* y = g.Y + ((size_t)n * g.L + lj[j]) * g.C + grp * Cg + 4 * qj[j];
       float4 p[MAXS];
 #pragma unroll
-      for (int s = 0; s < MAXS; ++s) if (s < g.n_split) p[s] = *reinterpret_cast<const float4*>(y + (size_t)s * (size_t)g.split_stride);
+      for (int s = 0; s < MAXS; ++s) if (s < g.n_split) p[s] = load_now(y + (size_t)s * (size_t)g.split_stride);
       v[j] = p[0];
 #pragma unroll
       for (int s = 1; s < MAXS; ++s) if (s < g.n_split) { v[j].x += p[s].x; v[j].y += p[s].y; v[j].z += p[s].z; v[j].w += p[s].w; }
     }
   }
+  int cb, cc;
+  cand_decode(cm, n, cb, cc);
+  if (PRE && n >= cand_count(cm, n_static)) return;
   const float *ft = nullptr, *fo = nullptr;
-  if (g.film_time) gn_film_rows(g, cm, n, ft, fo);
+  if (g.film_time) {
+    ft = g.film_time + (size_t)max(0, min(g.Tsteps - 1, cm.t[cb] - cm.koff - cc)) * g.F + g.foff;
+    fo = g.film_obs + (size_t)item_of(cm.item, cb) * g.F + g.foff;
+  }
+  // (PRE: where a lane's values are all of the same four channels, the thread count being a multiple of the group's quads)
+  const bool same = PRE && q_step == 0;
+  float4 ga0, be0, fs0, fs1, fb0, fb1;
+  auto vectors = [&](int c) {
+    ga0 = load_now(g.gam + c); be0 = load_now(g.bet + c);
+    if (ft) { fs0 = load_now(ft + c); fs1 = load_now(fo + c); fb0 = load_now(ft + g.C + c); fb1 = load_now(fo + g.C + c); }
+  };
+  if (same) vectors(grp * Cg + 4 * qj[0]);
   auto group_sum = [&](float x, int slot) {
     x = warp_sum(x);
     if (TPG == 32) return x;
@@ -230,15 +248,13 @@ gn_mish_kernel(GnArgs g, CandMap cm, int n_static) {
   for (int j = 0; j < GN_ITEMS; ++j) {
     if (j * TPG + t >= items) continue;
     const int l = lj[j], c = grp * Cg + 4 * qj[j];
-    const float4 ga = __ldg(reinterpret_cast<const float4*>(g.gam + c)), be = __ldg(reinterpret_cast<const float4*>(g.bet + c));
+    if (!same) vectors(c);
     float4 o;
-    o.x = mish_fast(v[j].x * rstd * ga.x + be.x); o.y = mish_fast(v[j].y * rstd * ga.y + be.y);
-    o.z = mish_fast(v[j].z * rstd * ga.z + be.z); o.w = mish_fast(v[j].w * rstd * ga.w + be.w);
+    o.x = mish_fast(v[j].x * rstd * ga0.x + be0.x); o.y = mish_fast(v[j].y * rstd * ga0.y + be0.y);
+    o.z = mish_fast(v[j].z * rstd * ga0.z + be0.z); o.w = mish_fast(v[j].w * rstd * ga0.w + be0.w);
     if (ft) {
-      const float4 s0 = __ldg(reinterpret_cast<const float4*>(ft + c)), s1 = *reinterpret_cast<const float4*>(fo + c);
-      const float4 b0 = __ldg(reinterpret_cast<const float4*>(ft + g.C + c)), b1 = *reinterpret_cast<const float4*>(fo + g.C + c);
-      o.x = (s0.x + s1.x) * o.x + (b0.x + b1.x); o.y = (s0.y + s1.y) * o.y + (b0.y + b1.y);
-      o.z = (s0.z + s1.z) * o.z + (b0.z + b1.z); o.w = (s0.w + s1.w) * o.w + (b0.w + b1.w);
+      o.x = (fs0.x + fs1.x) * o.x + (fb0.x + fb1.x); o.y = (fs0.y + fs1.y) * o.y + (fb0.y + fb1.y);
+      o.z = (fs0.z + fs1.z) * o.z + (fb0.z + fb1.z); o.w = (fs0.w + fs1.w) * o.w + (fb0.w + fb1.w);
     }
     const size_t prow = (size_t)n * (g.L + 4) + l + 2;
     if (g.res_t) {

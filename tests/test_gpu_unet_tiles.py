@@ -56,6 +56,12 @@ def test_unet_denoiser_with_a_warp_per_group(case, N):
     test_unet_denoiser_tiles_and_groups(case, N)
 
 
+# Four warps per group: the last launch whose GroupNorms fetch everything early (14 groups per SM, 2072) and the first that does not.
+@pytest.mark.parametrize("N", [258, 259])
+def test_unet_denoiser_on_both_sides_of_the_early_fetch(N):
+    test_unet_denoiser_tiles_and_groups((16, 2, 1, 128, 8, 5), N)
+
+
 def test_unet_round_with_a_warp_per_group_and_few_live_candidates():
     """300 slots x 4 candidates x 4 groups; timesteps near the end leave 837 candidates alive, 3348 groups, the last block half full.
     A rejected draft's reflection multiplies the error of mu^ - mu (3e-7) by 2 sigma |xi| / |mu^ - mu|: 70 at most for this drafter, so 2e-5
