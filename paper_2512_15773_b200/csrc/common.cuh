@@ -99,11 +99,12 @@ __device__ __forceinline__ void pdl_trigger(bool always = false) {
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// 16 bytes that nothing writes while the kernel runs, asked for where the call stands: the compiler would move a plain load down to its
-// use, behind the reductions that its latency is meant to pass under.
+// 16 bytes, asked for where the call stands: the compiler would move an ordinary load down to its use, behind the reductions that its
+// latency is meant to pass under.  Coherent (no .nc): a kernel that is launched early is resident, in pdl_wait, while its predecessors
+// still write what it will read.
 __device__ __forceinline__ float4 load_now(const float* p) {
   float4 v;
-  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
   return v;
 }
 
