@@ -59,7 +59,7 @@ constexpr uint32_t CXT_O_COL = 192;
 __global__ void __launch_bounds__(CXT_THREADS, 2)
 cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV,
                          __nv_bfloat16* __restrict__ out, int kv_off, CandMap cm, int rows_per_slot, int d, int heads, int Tc,
-                         const int* __restrict__ slot_start, int H, int splits, int* __restrict__ status) {
+                         const int* slot_start, int H, int splits, int* __restrict__ status) {
   extern __shared__ uint8_t cxt_raw[];
   pdl_trigger(true);
   const uint32_t base = (ptx::smem_u32(cxt_raw) + 1023u) & ~1023u;

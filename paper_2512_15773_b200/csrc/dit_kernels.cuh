@@ -26,7 +26,7 @@ __device__ __forceinline__ int row_tau(const CandMap& cm, int row, int H, int Ts
 // out[row] = LN0(h[row]) * (1 + scale(tau)) + shift(tau); LN0 = LayerNorm without gain and bias.
 // One warp per row, d = VEC * 128; shift / scale are columns [off_shift, +d) and [off_scale, +d) of mod[tau].
 template <typename T, int VEC>
-__global__ void ln_mod_kernel(const float* __restrict__ h, const float* __restrict__ mod, int mod_ld, int off_shift,
+__global__ void ln_mod_kernel(const float* h, const float* __restrict__ mod, int mod_ld, int off_shift,
                               int off_scale, CandMap cm, int H, int Tsteps, T* __restrict__ out, int M) {
   pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
@@ -62,7 +62,7 @@ __global__ void ln_mod_kernel(const float* __restrict__ h, const float* __restri
 
 // eps[n, i, :] = (LN0(h[row]) (1 + scale_f(tau)) + shift_f(tau)) W_out + b_out; one warp per row.
 template <int VEC>
-__global__ void head_mod_kernel(const float* __restrict__ h, const float* __restrict__ mod, int mod_ld, int off_shift,
+__global__ void head_mod_kernel(const float* h, const float* __restrict__ mod, int mod_ld, int off_shift,
                                 int off_scale, const float* __restrict__ W_outT, const float* __restrict__ b_out,
                                 CandMap cm, int M, int H, int A, int Tsteps) {
   pdl_trigger();
@@ -117,7 +117,7 @@ __global__ void head_mod_kernel(const float* __restrict__ h, const float* __rest
 // q, out [M, d]; kv [items * Tc, ld_kv] with this block's [K (d) | V (d)] at column kv_off.
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void cross_attn_ctx_simt_kernel(const T* __restrict__ q, T* __restrict__ out, const T* __restrict__ kv,
+__global__ void cross_attn_ctx_simt_kernel(const T* q, T* __restrict__ out, const T* kv,
                                            long long ld_kv, int kv_off, CandMap cm, int M, int H, int d, int heads, int Tc) {
   pdl_trigger();
   pdl_wait();
@@ -174,9 +174,9 @@ __host__ __device__ constexpr int cx_smem_bytes(int Tc) {      // keys and value
 
 template <int DH>
 __global__ void __launch_bounds__(CX_WARPS * 32)
-cross_attn_ctx_mma_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ out,
-                          const __nv_bfloat16* __restrict__ kv, long long ld_kv, int kv_off, CandMap cm, int rows_per_slot,
-                          int d, int heads, int Tc, const int* __restrict__ slot_start, int H) {
+cross_attn_ctx_mma_kernel(const __nv_bfloat16* q, __nv_bfloat16* __restrict__ out,
+                          const __nv_bfloat16* kv, long long ld_kv, int kv_off, CandMap cm, int rows_per_slot,
+                          int d, int heads, int Tc, const int* slot_start, int H) {
   pdl_trigger(true);
   pdl_wait();
   extern __shared__ __align__(16) uint8_t cx_raw[];

@@ -15,12 +15,12 @@ template <typename T, int VEC>
 __global__ void draft_tail_kernel(float* __restrict__ h, const float* __restrict__ lnf_g, const float* __restrict__ lnf_b,
                                   const float* __restrict__ W_outT, const float* __restrict__ b_out, DdpmTables S,
                                   float* __restrict__ xt, long long xs_b, float* __restrict__ muhat, long long ms_b,
-                                  float* __restrict__ eps_d, const int* __restrict__ t, int k, int K, int Tsteps,
-                                  const uint64_t* __restrict__ seedp, const EnvParams* __restrict__ envp,
-                                  const int* __restrict__ item, const float* __restrict__ W_in, const float* __restrict__ b_in,
+                                  float* __restrict__ eps_d, const int* t, int k, int K, int Tsteps,
+                                  const uint64_t* __restrict__ seedp, const EnvParams* envp,
+                                  const int* item, const float* __restrict__ W_in, const float* __restrict__ b_in,
                                   const float* __restrict__ pos, const float* __restrict__ ln1_g, const float* __restrict__ ln1_b,
                                   T* __restrict__ a_out, int embed_next, int M, int H, int A,
-                                  const int* __restrict__ order, const int* __restrict__ n_live) {
+                                  const int* order, const int* n_live) {
   pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
   constexpr int d = VEC * 128;

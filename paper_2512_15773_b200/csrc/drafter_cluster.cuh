@@ -738,15 +738,14 @@ drafter_cluster_kernel(const __grid_constant__ DcParams P) {
       if (P.fold) {
         const int p = warp + lane * DC_WARPS, n = p / OWN, j = n / HEADS;
         if (p < OWN * NKH)
-          cst = __ldg((j == 0 ? P.c_time + (size_t)tau * L * HEADS : P.c_obs + ((size_t)env * P.To + (j - 1)) * L * HEADS) +
-                      (size_t)l * HEADS + n % HEADS);
+          cst = (j == 0 ? P.c_time + (size_t)tau * L * HEADS : P.c_obs + ((size_t)env * P.To + (j - 1)) * L * HEADS)[(size_t)l * HEADS + n % HEADS];
       } else {      // keys and value columns of the memory tokens for this CTA's head
         float* skv = reinterpret_cast<float*>(dc_smem + pl.off_kq);      // [NK][DH + VW]
         const size_t ldkv = (size_t)L * 2 * d;
         for (int i = threadIdx.x; i < NK * (DH + VW); i += DC_COMPUTE) {
           const int kx = i / (DH + VW), c = i % (DH + VW);
           const float* src = (kx == 0 ? P.kv_time + (size_t)tau * ldkv : P.kv_obs + ((size_t)env * P.To + (kx - 1)) * ldkv) + (size_t)l * 2 * d;
-          skv[i] = __ldg(src + (c < DH ? rank * HEADS / CS * DH + c : d + rank * VW + (c - DH)));
+          skv[i] = src[c < DH ? rank * HEADS / CS * DH + c : d + rank * VW + (c - DH)];
         }
       }
       stage_end();

@@ -167,8 +167,8 @@ mlp_forward_kernel(const __grid_constant__ MlpWeights w, CandMap cm, const float
 template <int R>
 __global__ void __launch_bounds__(MLP_THREADS)
 mlp_rollout_kernel(const __grid_constant__ MlpWeights w, DdpmTables S, float* __restrict__ xt, long long xs_b, float* __restrict__ muhat,
-                   long long ms_b, const int* __restrict__ t, const uint64_t* __restrict__ seedp, const EnvParams* __restrict__ envp,
-                   const int* __restrict__ item, const float* __restrict__ obs, int obs_len, int D, int B, int K, int Tsteps, int cs) {
+                   long long ms_b, const int* t, const uint64_t* __restrict__ seedp, const EnvParams* envp,
+                   const int* item, const float* __restrict__ obs, int obs_len, int D, int B, int K, int Tsteps, int cs) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(16) float mlp_sm[];

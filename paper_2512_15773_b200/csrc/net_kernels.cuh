@@ -11,7 +11,7 @@ namespace tsdp {
 // ------------------------------------------------------------------------------------------------
 template <int EPI>
 __global__ void __launch_bounds__(256)
-gemm_simt_kernel(const float* __restrict__ A, const float* __restrict__ W, GemmArgs g) {
+gemm_simt_kernel(const float* A, const float* __restrict__ W, GemmArgs g) {
   pdl_trigger();
   pdl_wait();
   __shared__ float As[16][65], Ws[16][65];
@@ -108,7 +108,7 @@ __global__ void timetok_kernel(const float* __restrict__ in, const float* __rest
 constexpr int MT_BK = 32, MT_N = 64, MT_THREADS = 256;
 template <typename T, int TM>
 __global__ void __launch_bounds__(MT_THREADS)
-memtok_kernel(const float* __restrict__ in, int rows, int Din, const float* __restrict__ W, const float* __restrict__ bias,
+memtok_kernel(const float* in, int rows, int Din, const float* __restrict__ W, const float* __restrict__ bias,
               const float* __restrict__ cpos, int cpos_mod, int cpos_off, T* __restrict__ out, int d) {
   constexpr int RT = TM / 16, NA = TM * MT_BK / MT_THREADS, NB = MT_BK * MT_N / MT_THREADS, PA = TM + 4;      // rows a thread, loads a step
   __shared__ __align__(16) float As[MT_BK * PA];
@@ -123,7 +123,7 @@ memtok_kernel(const float* __restrict__ in, int rows, int Din, const float* __re
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
       const int r = r0 + warp + 8 * j, k = k0 + lane;
-      ra[j] = r < rows && k < Din ? __ldg(in + (size_t)r * Din + k) : 0.f;
+      ra[j] = r < rows && k < Din ? in[(size_t)r * Din + k] : 0.f;
     }
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
@@ -180,7 +180,7 @@ __device__ __forceinline__ void store4(__nv_bfloat16* o, float a, float b, float
 }
 
 template <typename T, int VEC>
-__global__ void ln_kernel(const float* __restrict__ h, const float* __restrict__ gam, const float* __restrict__ bet,
+__global__ void ln_kernel(const float* h, const float* __restrict__ gam, const float* __restrict__ bet,
                           T* __restrict__ out, int M, LiveRows lv) {
   pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
@@ -286,7 +286,7 @@ __global__ void embed_ln_kernel(CandMap cm, const float* __restrict__ W_in, cons
 // qkv [M, 3d] -> out [M, d].  H <= 64, dh = d / heads a multiple of 32 and <= 128.
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void self_attn_kernel(const T* __restrict__ qkv, T* __restrict__ out, int n_cand, int H, int d,
+__global__ void self_attn_kernel(const T* qkv, T* __restrict__ out, int n_cand, int H, int d,
                                  int heads, int causal, LiveRows lv) {
   pdl_trigger();
   pdl_wait();
@@ -345,8 +345,8 @@ __global__ void self_attn_kernel(const T* __restrict__ qkv, T* __restrict__ out,
 // kv_obs [B*To, L*2d] (built once per chunk); layer l occupies columns [l*2d, (l+1)*2d) = [K | V].
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void cross_attn_kernel(const T* __restrict__ q, T* __restrict__ out, const float* __restrict__ kv_time,
-                                  const float* __restrict__ kv_obs, CandMap cm, int M, int H, int d, int heads,
+__global__ void cross_attn_kernel(const T* q, T* __restrict__ out, const float* __restrict__ kv_time,
+                                  const float* kv_obs, CandMap cm, int M, int H, int d, int heads,
                                   int To, int layer, int L, int Tsteps) {
   pdl_trigger();
   pdl_wait();
@@ -400,7 +400,7 @@ constexpr int SA_WARPS = 4;
 
 template <int DH>
 __global__ void __launch_bounds__(SA_WARPS * 32)
-self_attn_mma_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
+self_attn_mma_kernel(const __nv_bfloat16* qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
                      int heads, int causal, LiveRows lv) {
   pdl_trigger(true);
   pdl_wait();
@@ -419,7 +419,7 @@ self_attn_mma_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __res
   const __nv_bfloat16* base = qkv + (size_t)n * H * ld + (size_t)hd * DH;
   const int r0 = qt * 16 + g, r1 = r0 + 8;
   auto ld32 = [&](int row, int col) -> uint32_t {
-    return row < H ? __ldg(reinterpret_cast<const uint32_t*>(base + (size_t)row * ld + col)) : 0u;
+    return row < H ? *reinterpret_cast<const uint32_t*>(base + (size_t)row * ld + col) : 0u;
   };
   uint32_t qa[KS][4];
 #pragma unroll
@@ -492,7 +492,7 @@ self_attn_mma_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __res
       for (int no = 0; no < NO; ++no) {
         const int col = no * 8 + g;
         auto v16 = [&](int key) -> uint32_t {
-          return key < H ? (uint32_t)__ldg(vraw + (size_t)key * ld + col) : 0u;
+          return key < H ? (uint32_t)vraw[(size_t)key * ld + col] : 0u;
         };
         const uint32_t b0 = v16(k0) | (v16(k0 + 1) << 16);
         const uint32_t b1 = v16(k0 + 8) | (v16(k0 + 9) << 16);
@@ -526,7 +526,7 @@ self_attn_mma_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __res
 // ------------------------------------------------------------------------------------------------
 template <int DH>
 __global__ void __launch_bounds__((DH > 64 ? 2 : 4) * 32)
-self_attn_tile_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
+self_attn_tile_kernel(const __nv_bfloat16* qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
                       int heads, int causal, LiveRows lv) {
   pdl_trigger(true);
   pdl_wait();
@@ -552,7 +552,7 @@ self_attn_tile_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __re
     for (int i = 0; i < CH; ++i) {
       const int idx = (c0 + i) * 32 + lane;
       const int which = idx / (16 * VPR), rem = idx % (16 * VPR), r = rem / VPR, v = rem % VPR;
-      buf[i] = r < H ? __ldg(reinterpret_cast<const uint4*>(base + (size_t)r * ld + (size_t)which * d) + v) : make_uint4(0u, 0u, 0u, 0u);
+      buf[i] = r < H ? reinterpret_cast<const uint4*>(base + (size_t)r * ld + (size_t)which * d)[v] : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
@@ -584,7 +584,7 @@ template <int DH>
 __host__ __device__ constexpr int sa_smem_bytes() { return 3 * 64 * (DH + 8) * 2; }
 template <int DH>
 __global__ void __launch_bounds__(128)
-self_attn_staged_kernel(const __nv_bfloat16* __restrict__ qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
+self_attn_staged_kernel(const __nv_bfloat16* qkv, __nv_bfloat16* __restrict__ out, int n_cand, int H, int d,
                         int heads, int causal, LiveRows lv) {
   pdl_trigger(true);
   pdl_wait();
@@ -706,8 +706,8 @@ constexpr int CA_ROWS = 4;
 
 template <int DH>
 __global__ void __launch_bounds__(256)
-cross_attn_group_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ out,
-                        const float* __restrict__ kv_time, const float* __restrict__ kv_obs, CandMap cm, int n_cand,
+cross_attn_group_kernel(const __nv_bfloat16* q, __nv_bfloat16* __restrict__ out,
+                        const float* __restrict__ kv_time, const float* kv_obs, CandMap cm, int n_cand,
                         int H, int d, int heads, int To, int layer, int L, int Tsteps) {
   pdl_trigger();
   pdl_wait();
@@ -735,8 +735,8 @@ cross_attn_group_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __re
     if (kx < NK) {
       const float* kp = (kx == 0 ? kv_time + (size_t)tau * ldkv : kv_obs + ((size_t)item_of(cm.item, b) * To + (kx - 1)) * ldkv) +
                         (size_t)layer * 2 * d + hd * DH + sub * 8;
-      const float4 k0 = __ldg(reinterpret_cast<const float4*>(kp)), k1 = __ldg(reinterpret_cast<const float4*>(kp) + 1);
-      const float4 v0 = __ldg(reinterpret_cast<const float4*>(kp + d)), v1 = __ldg(reinterpret_cast<const float4*>(kp + d) + 1);
+      const float4 k0 = reinterpret_cast<const float4*>(kp)[0], k1 = reinterpret_cast<const float4*>(kp)[1];
+      const float4 v0 = reinterpret_cast<const float4*>(kp + d)[0], v1 = reinterpret_cast<const float4*>(kp + d)[1];
       kreg[kx][0] = k0.x; kreg[kx][1] = k0.y; kreg[kx][2] = k0.z; kreg[kx][3] = k0.w;
       kreg[kx][4] = k1.x; kreg[kx][5] = k1.y; kreg[kx][6] = k1.z; kreg[kx][7] = k1.w;
       vreg[kx][0] = v0.x; vreg[kx][1] = v0.y; vreg[kx][2] = v0.z; vreg[kx][3] = v0.w;
@@ -794,7 +794,7 @@ cross_attn_group_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __re
 // ------------------------------------------------------------------------------------------------
 // Final LayerNorm of one row by one warp, result left in v (lane owns columns (j*32 + lane)*4 .. +3).
 template <int VEC>
-__device__ __forceinline__ void head_ln_row(const float* __restrict__ h_row, const float* __restrict__ gam,
+__device__ __forceinline__ void head_ln_row(const float* h_row, const float* __restrict__ gam,
                                             const float* __restrict__ bet, float4 (&v)[VEC], int lane) {
   constexpr int d = VEC * 128;
   float s = 0.f;
@@ -834,7 +834,7 @@ __device__ __forceinline__ float head_out(const float4 (&v)[VEC], const float* _
 }
 
 template <int VEC>
-__global__ void head_kernel(const float* __restrict__ h, const float* __restrict__ gam, const float* __restrict__ bet,
+__global__ void head_kernel(const float* h, const float* __restrict__ gam, const float* __restrict__ bet,
                             const float* __restrict__ W_outT, const float* __restrict__ b_out, CandMap cm, int M,
                             int H, int A) {
   pdl_trigger();

@@ -53,8 +53,8 @@ constexpr int PLAN_MAX_B = 4096;
 constexpr int PLAN_PER_THREAD = PLAN_MAX_B / PLAN_THREADS;
 
 __global__ void __launch_bounds__(PLAN_THREADS)
-round_plan_kernel(const int* __restrict__ t, int B, int K, const RoundParams* __restrict__ sched, int n_sched,
-                  const int* __restrict__ round_idx, const EnvParams* __restrict__ envp, const int* __restrict__ item,
+round_plan_kernel(const int* t, int B, int K, const RoundParams* __restrict__ sched, int n_sched,
+                  const int* round_idx, const EnvParams* envp, const int* item,
                   int Tsteps, int* __restrict__ live_n, int* __restrict__ live_list, int* __restrict__ slot_start,
                   int* __restrict__ order, int* __restrict__ dn, DevStats* __restrict__ stats) {
   pdl_trigger();
@@ -143,9 +143,9 @@ round_plan_kernel(const int* __restrict__ t, int B, int K, const RoundParams* __
 // x~_k = mu^_k + sigma_tau xi_tau.  Slots beyond K_eff = min(K, t) copy the previous latent so that
 // every buffer stays finite.  eps^ of slot b is the D values at eps_d + b * es_b.
 __global__ void draft_step_kernel(DdpmTables S, float* __restrict__ xt, long long xs_b, float* __restrict__ muhat,
-                                  long long ms_b, const float* __restrict__ eps_d, long long es_b, const int* __restrict__ t,
-                                  int k, int D, const uint64_t* __restrict__ seedp, const EnvParams* __restrict__ envp,
-                                  int K, int Tsteps, const int* __restrict__ item) {
+                                  long long ms_b, const float* eps_d, long long es_b, const int* t,
+                                  int k, int D, const uint64_t* __restrict__ seedp, const EnvParams* envp,
+                                  int K, int Tsteps, const int* item) {
   pdl_trigger();
   pdl_wait();
   const uint64_t seed = *seedp;
@@ -182,7 +182,7 @@ __global__ void draft_step_kernel(DdpmTables S, float* __restrict__ xt, long lon
 
 // Four consecutive latent values starting at element 4q: one 16-byte load when D is a multiple of 4 (every row of
 // the round's buffers then starts on a 16-byte boundary), element by element with a bounds check otherwise.
-__device__ __forceinline__ void load_quad(const float* __restrict__ p, int q, int D, bool vec, float v[4]) {
+__device__ __forceinline__ void load_quad(const float* p, int q, int D, bool vec, float v[4]) {
   if (vec) {
     const float4 t = *reinterpret_cast<const float4*>(p + 4 * q);
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
@@ -232,13 +232,13 @@ __device__ __forceinline__ void round_end(const RoundEnd& e, int t_after) {     
 // counters per request -- drafts proposed, drafts accepted, rounds, reverse steps taken -- the inputs of
 // the intermediate reward of Sec. 3.3.  dbg_* may be null.
 __global__ void accept_kernel(DdpmTables S, float* __restrict__ xt, long long xs_b,
-                              const float* __restrict__ muhat, long long ms_b,
-                              const float* __restrict__ eps, long long es_b, int* __restrict__ t, int K, int D,
+                              const float* muhat, long long ms_b,
+                              const float* eps, long long es_b, int* __restrict__ t, int K, int D,
                               const uint64_t* __restrict__ seedp, const RoundParams* __restrict__ sched, int n_sched,
                               const int* round_idx, float* __restrict__ actions,
                               DevStats* __restrict__ stats, float draft_nfe,
                               float* __restrict__ dbg_logalpha, int* __restrict__ dbg_jstar,
-                              const EnvParams* __restrict__ envp, int* __restrict__ item, int* __restrict__ queue_head,
+                              const EnvParams* envp, int* __restrict__ item, int* __restrict__ queue_head,
                               const int* __restrict__ n_items, int* __restrict__ item_counts, RoundEnd rend) {
   pdl_trigger();
   pdl_wait();

@@ -14,7 +14,7 @@ struct SchedWeights {            // W [in, out] fp32, as in the weight blob
 };
 
 __global__ void __launch_bounds__(128)
-sched_mlp_kernel(SchedWeights w, const float* __restrict__ obs, int obs_len, const float* __restrict__ prev_act, int D,
+sched_mlp_kernel(SchedWeights w, const float* __restrict__ obs, int obs_len, const float* prev_act, int D,
                  const float* __restrict__ progress, int K_max, EnvParams* __restrict__ out, float* __restrict__ params_out) {
   pdl_trigger();
   pdl_wait();

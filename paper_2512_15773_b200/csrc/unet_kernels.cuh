@@ -81,7 +81,7 @@ unet_embed_kernel(CandMap cm, const float* __restrict__ W_in, const float* __res
 constexpr int UF_N = 8, UF_F = 4;
 constexpr size_t UF_MAX_SMEM = 200 * 1024;
 __global__ void __launch_bounds__(256)
-film_obs_kernel(const float* __restrict__ x, const float* __restrict__ W, float* __restrict__ out, int N, int F, int K) {
+film_obs_kernel(const float* x, const float* __restrict__ W, float* __restrict__ out, int N, int F, int K) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(16) float sx_film[];      // [UF_N][Kp], zero beyond K and N
@@ -340,7 +340,7 @@ gn_mish_any_kernel(GnArgs g, CandMap cm, int n_static) {
 constexpr int UH_A = 5;
 template <typename T>
 __global__ void __launch_bounds__(256)
-unet_head_kernel(const T* __restrict__ X, const float* __restrict__ W_outT, const float* __restrict__ b_out,
+unet_head_kernel(const T* X, const float* __restrict__ W_outT, const float* __restrict__ b_out,
                  CandMap cm, int M, int H, int A, int C) {
   pdl_trigger();
   pdl_wait();

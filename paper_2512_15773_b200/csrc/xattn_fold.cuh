@@ -208,7 +208,7 @@ __device__ __forceinline__ void xf_row_stats(const float4 (&x)[2][V], float (&me
 // read-modify-write of the stream.
 template <int D>
 __global__ void __launch_bounds__(XF_THREADS, 3)
-xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta, XfoldTables tb, const float* __restrict__ bo2,
+xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* delta, XfoldTables tb, const float* __restrict__ bo2,
                   const float* __restrict__ ln3_g, const float* __restrict__ ln3_b, __nv_bfloat16* __restrict__ ln3_out, CandMap cm,
                   int H, int heads, int To, int layer, int L, int Tsteps) {
   pdl_trigger(L > 0);      // always; behind a branch, without which the compiler spills a register (16-row calls 1 % slower)
@@ -290,7 +290,7 @@ xattn_fold_kernel(float* __restrict__ x, const __nv_bfloat16* __restrict__ delta
       if (j < NK && threadIdx.x < 16 * heads) {
         const float* cp = (j == 0 ? tb.c_time + (size_t)tau * L * heads : tb.c_obs + ((size_t)item * To + (j - 1)) * L * heads) +
                           (size_t)layer * heads;
-        cst[j] = __ldg(cp + h);
+        cst[j] = cp[h];
       }
     }
   }
