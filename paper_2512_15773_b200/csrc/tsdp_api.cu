@@ -1068,16 +1068,16 @@ int unet_gn(tsdp_ctx* c, Net& n, const CandMap& cm, int n_cand, const float* gam
   g.L = L; g.C = C;
   const int Cg = C / g.groups, items = L * Cg / 4, all = n_cand * g.groups;
   prof_begin(c, s, 1, 0.0);
-  // four warps per group up to two waves of them (the kernel is a chain of latencies: 288 candidates 6.3 against 9.1 us), one
-  // beyond
+  // four warps per group below 32 groups per SM (the kernel is a chain of latencies: 288 candidates 6.3 against 9.1 us), one
+  // beyond; everything asked for early (PRE) while all blocks run at once (both sides: see the kernel)
   if (Cg % 4 != 0 || items > GN_ITEMS * 128) TSDP_LAUNCH(c, (gn_mish_any_kernel<T>), all, 256, 0, s, g, cm, n_cand);
   else if (items > GN_ITEMS * 32 || all < 32 * c->num_sms) {
     if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 8, true>), all, 128, 0, s, g, cm, n_cand);
-    else if (all < 14 * c->num_sms) TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 2, true>), all, 128, 0, s, g, cm, n_cand);
+    else if (all <= GN_PRE_BLOCKS * c->num_sms) TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 2, true>), all, 128, 0, s, g, cm, n_cand);
     else TSDP_LAUNCH(c, (gn_mish_kernel<T, 128, 2, false>), all, 128, 0, s, g, cm, n_cand);
   } else {
-    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 8, true>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
-    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 2, true>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
+    if (g.n_split > 2) TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 8, false>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
+    else TSDP_LAUNCH(c, (gn_mish_kernel<T, 32, 2, false>), (all + 7) / 8, 256, 0, s, g, cm, n_cand);
   }
   prof_end(c, s);
   c->launches_per_round_tmp++;

@@ -169,11 +169,14 @@ __device__ __forceinline__ float4 gn_load4(const __nv_bfloat16* p) {
 // 288 candidates x 8 groups of 512 values: 12.6 us with 256 scalar threads per group and two passes over Y.
 // PRE: the sums (those of a candidate past the live ones exist) are on their way beside the live count and the candidate, whose timestep and
 // request follow and then, beside the statistics, the affine and FiLM vectors, in place of one behind the other.  64 registers a thread
-// in place of 56, which costs blocks of four warps more than it gives on a full chip: whole UNet calls without and with it, 1 environment 8.81 / 8.64 ms,
-// 6 10.18 / 9.98, 21 with frozen drafts 8.63 / 8.47, 28 9.05 / 9.01, 32 15.29 / 15.40, 100 (a warp per group) 31.2 / 31.0.
+// in place of 56: eight blocks an SM in place of nine.  Chains of launches of 16 x 256 values in 8 groups a candidate, residual / FiLM form, us a
+// launch without and with it: 2 groups per SM 4.19 / 4.38 -> 3.43 / 3.42, 4 4.73 / 4.97 -> 3.69 / 3.74, 8 4.91 / 5.16 -> 4.71 / 4.86, 10 6.39 / 6.45 -> 6.60 / 6.81,
+// 16 7.78 / 8.03 -> 8.29 / 8.46, 32 13.8 / 14.4 -> 15.3 / 15.5.  With a warp per group it loses on one form what it wins on the other (32 groups per SM
+// 8.70 / 8.96 -> 8.80 / 8.65, 64 16.9 / 16.3 -> 17.2 / 15.6) and spills.
 constexpr int GN_ITEMS = 4;
+constexpr int GN_PRE_BLOCKS = 8;      // of the PRE form on an SM
 template <typename T, int TPG, int MAXS, bool PRE>
-__global__ void __launch_bounds__(TPG == 32 ? 256 : TPG, MAXS == 2 ? (TPG == 32 ? 4 : (PRE ? 8 : 9)) : 1)
+__global__ void __launch_bounds__(TPG == 32 ? 256 : TPG, MAXS == 2 ? (TPG == 32 ? 4 : (PRE ? GN_PRE_BLOCKS : 9)) : 1)
 gn_mish_kernel(GnArgs g, CandMap cm, int n_static) {
   pdl_trigger(std::is_same<T, __nv_bfloat16>::value);
   pdl_wait();
