@@ -1302,6 +1302,13 @@ bool cluster_drafter_fits(const tsdp_config_t& cfg, const tsdp_net_t& n, int cs,
   return false;
 }
 
+// Whether a context ever runs net `which` in clusters of DC_SIZES[sz] (each form has its own copy of the weights): the base model in clusters of 8,
+// unless its verification is layer by layer, and in clusters of 4 only where the cluster kernel is asked for whatever the number
+// of candidates; a drafter in both, unless it runs layer by layer.
+bool cluster_form_used(const tsdp_config_t& cfg, int which, int sz) {
+  return which == TSDP_BASE ? cfg.verifier == 2 || (cfg.verifier == 0 && sz == 0) : cfg.drafter != 1;
+}
+
 // Cluster size for `work` rollouts or candidates: 0 for clusters of 8, 1 for clusters of 4.  A forward in a cluster of 4 takes about 1.25 times as long
 // (the exchanges take the same time, the k loops twice), but 33 of them run at once instead of 15; both give the same bits.  32 environments,
 // 8 steps of a d = 256 drafter of 4 blocks: 914 us in three waves of clusters of 8, calls of the conv-UNet policy 21.8 -> 15.0 ms.
@@ -1793,7 +1800,7 @@ int tsdp_init(const tsdp_config_t* cfg, tsdp_ctx** out) {
     const int which = i >> 1, sz = i & 1, cs = DC_SIZES[sz];
     const tsdp_net_t& nn = which == TSDP_BASE ? cfg->base : cfg->draft;
     int smem = 0; bool res = false;
-    if (!cluster_drafter_fits(*cfg, nn, cs, &smem, &res)) continue;
+    if (!cluster_form_used(*cfg, which, sz) || !cluster_drafter_fits(*cfg, nn, cs, &smem, &res)) continue;
     const void* fn = (const void*)cluster_kernel_of(nn.d, nn.d / nn.heads, cs);
     int cur_attr = 0;   // both nets may use the same instantiation: keep the larger request
     cudaFuncAttributes fa;
@@ -2292,7 +2299,7 @@ int tsdp_load_weights(tsdp_ctx* c, int which, const float* blob, size_t n) {
     int smem_unused; bool res_unused;
     for (int sz = 0; sz < 2; ++sz) {
       const int cs = DC_SIZES[sz];
-      if (!cluster_drafter_fits(cfg, net.cfg, cs, &smem_unused, &res_unused)) continue;
+      if (!cluster_form_used(cfg, which, sz) || !cluster_drafter_fits(cfg, net.cfg, cs, &smem_unused, &res_unused)) continue;
       const int di = (int)d, dhi = di / net.cfg.heads;
       const size_t lw = (size_t)cs * dc_layer_bytes(di, dhi, cs) / 2, lp = (size_t)cs * dc_par_floats(di, dhi, cs);
       if (dev_alloc(c, net.allocs, &net.dc_w[sz], L * lw)) return TSDP_ERR_CUDA;
