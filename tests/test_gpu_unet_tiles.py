@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = [  # H, A, levels, channels, groups, obs width
     (12, 3, 3, 128, 8, 7), (20, 5, 3, 128, 16, 24), (24, 1, 2, 256, 8, 33), (64, 2, 2, 128, 4, 12), (8, 7, 1, 128, 64, 5),
-    (16, 10, 3, 128, 1, 24)]
+    (16, 10, 3, 128, 1, 24), (16, 3, 2, 384, 8, 7)]      # (384 channels in 8 groups: a lane's values are of several channel quads)
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -51,7 +51,7 @@ def test_unet_denoiser_tiles_and_groups(case, N):
 
 # One warp per group, eight groups a block: from 32 groups per SM on (4736), four channels a group at least and at most 128 quads of values.
 # Two and three parts of a reduction, four to six, and none with every lane's registers full and a ragged last block (4740 groups).
-@pytest.mark.parametrize("case,N", [((8, 3, 2, 128, 32, 7), 151), ((4, 5, 2, 256, 64, 12), 75), ((16, 2, 1, 128, 4, 5), 1185)])
+@pytest.mark.parametrize("case,N", [((8, 3, 2, 128, 32, 7), 151), ((4, 5, 2, 256, 64, 12), 75), ((16, 2, 1, 128, 4, 5), 1185), ((8, 3, 1, 384, 8, 7), 593)])
 def test_unet_denoiser_with_a_warp_per_group(case, N):
     test_unet_denoiser_tiles_and_groups(case, N)
 
