@@ -55,6 +55,17 @@ constexpr int CXT_OFF_X = CXT_OFF_BAR + 128;              // row maxima and row 
 constexpr int CXT_SMEM_BYTES = CXT_OFF_X + 2048 + 1024;   // + alignment slack
 constexpr uint32_t CXT_TMEM_COLS = 256;          // scores [0, Tc); P over [0, Tc/4) and [Tc/2, 3Tc/4); O in [192, 256)
 constexpr uint32_t CXT_O_COL = 192;
+// A GEMM may be placed before the blocks of its predecessor have their tensor memory, where that predecessor signals first (this kernel, another
+// GEMM).  Were they to share an SM, it could take the columns that such a block still waits for and itself wait for that block's grid
+// to finish.  They never do: an SM has 228 KB of shared memory, each block takes 1 KB more than it asks for.
+constexpr int gemm_min_smem() {
+  int least = gemm_smem_bytes_cg(256, 2) < gemm_smem_bytes_cg(GEMM_ATTN_BN, 2) ? gemm_smem_bytes_cg(256, 2) : gemm_smem_bytes_cg(GEMM_ATTN_BN, 2);
+  const int bn[5] = {32, 64, 128, GEMM_ATTN_BN, 256};
+  for (int i = 0; i < 5; ++i) least = gemm_smem_bytes(bn[i]) < least ? gemm_smem_bytes(bn[i]) : least;
+  return least;
+}
+static_assert((CXT_SMEM_BYTES < gemm_min_smem() ? CXT_SMEM_BYTES : gemm_min_smem()) + gemm_min_smem() + 2 * 1024 > 228 * 1024,
+              "no GEMM shares an SM with a kernel that holds tensor memory and signals early");
 
 __global__ void __launch_bounds__(CXT_THREADS, 2)
 cross_attn_ctx_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV,
