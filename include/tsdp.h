@@ -106,19 +106,24 @@ typedef struct {
   float draft_nfe;         /* NFE cost of one drafter call; 0 => draft.layers/base.layers
                               (the paper's 1/8 rule, Sec. 4 "Evaluation Metrics")               */
   int use_graph;           /* 1: replay each round from a captured CUDA graph                  */
-  int drafter;             /* how the K draft steps run.  0: chosen from the batch size; 1: layer
-                              by layer (batched tensor-core kernels, one drafter forward per step);
-                              2: one persistent thread-block-cluster kernel per round with the
-                              drafter's weights sliced over the 8 CTAs of the cluster: resident
-                              in shared memory when a 1/8 slice fits beside the activations, read
-                              through the L2 otherwise (transformer drafter, precision 1, d = 128
-                              or 256, <= 4 blocks, H <= 16, obs_tokens <= 3; otherwise tsdp_init
-                              returns UNSUPPORTED)                                               */
+  int drafter;             /* how the K draft steps run.  0: chosen from the batch size (2 up to 66
+                              environments or slots at d = 256 and 99 at d = 128; 45, or 60 with
+                              resident weights, where there are no clusters of 4; 1 beyond);
+                              1: layer by layer (batched tensor-core kernels, one drafter forward
+                              per step); 2: one persistent thread-block-cluster kernel per round
+                              with the drafter's weights sliced over the CTAs of the cluster: 8 of
+                              them, or 4 where more environments wait than clusters of 8 run at
+                              once (2 or 4 heads, A <= 32; the same bits).  A slice is resident in
+                              shared memory when it fits beside the activations and read through
+                              the L2 otherwise (transformer drafter, precision 1, d = 128 or 256,
+                              <= 8 blocks, H <= 16, H * A <= 256, obs_tokens <= 3; otherwise
+                              tsdp_init returns UNSUPPORTED)                                     */
   int verifier;            /* how the base model's verification forward runs.  0: chosen from the
                               number of candidates; 1: batched tensor-core kernels, layer by layer;
                               2: the cluster kernel above, one cluster per candidate, in one launch
-                              (same shape limits, <= 8 blocks; meant for batch 1, where the
-                              layer-by-layer forward is bound by the latency of ~90 small launches) */
+                              (same shape limits; meant for batch 1, where the layer-by-layer
+                              forward is bound by the latency of ~90 small launches; 0 takes it up
+                              to 15 candidates, which is one wave of clusters of 8)               */
 } tsdp_config_t;
 
 /* Speculative parameters of a round -- the scheduler's action space (Sec. 3.3).
@@ -233,7 +238,8 @@ int tsdp_sample_chunk(tsdp_ctx* ctx, const float* d_obs, int B, int K, const tsd
  * tsdp_sample_chunk returns for environment i of a batch of N with the same seed -- bit for bit when both calls run
  * the same kernels with sums in the same order (the networks are evaluated row by row); where the kernel choice or a
  * split reduction depends on the number of slots (cluster kernels at small batches, TSDP_ARCH_UNET convolutions at
- * small batches) the two agree to rounding only.  Per-request buffers grow
+ * small batches) the two agree to rounding only.  So for a queue through few enough slots for the cluster drafter (tsdp_config_t.drafter)
+ * against a batch that is too large for it, and for one whose rounds have few enough candidates for the cluster verification.  Per-request buffers grow
  * on demand (the only call besides tsdp_init / tsdp_load_weights that may allocate).  With a per-round
  * schedule the round index counts batched rounds of the whole call.  Errors as tsdp_sample_chunk. */
 int tsdp_serve(tsdp_ctx* ctx, const float* d_obs, int N, int slots, int K, const tsdp_accept_t* accept,

@@ -13,8 +13,9 @@
 // An exchange costs about 770 clocks plus 390 per KB (measured); the layout before this one (every activation
 // replicated in every CTA, LayerNorms and the cross-attention recomputed by all) exchanged 2.4 KB four times on average
 // and needed 33 k clocks per d = 256 block against 17 k now (9.3 us with the block's share of a draft step, cs = 8).
-// cs = 4 takes longer for one environment and serves 33 at a time instead of 15.  Both give the same bits: what is summed over CTAs is summed
-// pairwise, and a CTA of four forms its two halves' sums apart (dc_kloop); what is summed over a row is summed in four groups of columns.
+// cs = 4 takes longer (12.2 us for the same) and serves 33 environments at a time instead of 15.  Both give the same bits: what is summed
+// over CTAs is summed pairwise, and a CTA of four forms its two halves' sums apart (dc_kloop); what is summed over a row is summed in
+// four groups of columns.
 //
 // Weights are laid out once, when they are loaded, in the order in which the lanes of a warp consume them (dc_pack_kernel):
 // a lane's operand of two MMAs is one 16-byte word, a warp reads 512 contiguous bytes, and a CTA's slice of a matrix is
@@ -24,7 +25,7 @@
 // Each layer's LayerNorm parameters and biases and the memory tokens' folded tables travel the same way.  Eight warps compute.
 //
 // What a stage exchanges travels as 16-byte st.async stores that also count their bytes on an mbarrier of the receiving
-// CTA; a CTA goes on as soon as the bytes of all eight CTAs have arrived (a bounded mbarrier wait), with no
+// CTA; a CTA goes on as soon as the bytes of all CTAs of the cluster have arrived (a bounded mbarrier wait), with no
 // release fence and no cluster-wide barrier per stage.  Two mbarriers alternate between consecutive stages: a CTA
 // can run at most one stage ahead of the slowest one (it needs everybody's bytes of the previous stage), so the
 // bytes of stage s + 1 never land on the barrier that still counts stage s.  The same reasoning covers the
@@ -40,7 +41,7 @@
 namespace tsdp {
 namespace cg = cooperative_groups;
 
-// CTAs per cluster: 8 (the portable maximum), or 4 where there are more environments than clusters of 8
+// CTAs per cluster: 8 (the portable maximum), or 4 where more environments wait than clusters of 8 run at once
 constexpr int DC_COMPUTE = 256;   // compute threads; one producer warp behind them
 constexpr int DC_THREADS = DC_COMPUTE + 32;
 constexpr int DC_WARPS = DC_COMPUTE / 32;
@@ -152,8 +153,8 @@ __global__ void dc_pack_par_kernel(DcParSrc src, float* __restrict__ layer, int 
 }
 
 struct DcParams {
-  const __nv_bfloat16* Wf;                                   // [layers][8 ranks][dc_layer_bytes] in fragment order
-  const float* parf;                                         // [layers][8 ranks][dc_par_floats]
+  const __nv_bfloat16* Wf;                                   // [layers][cs ranks][dc_layer_bytes] in fragment order
+  const float* parf;                                         // [layers][cs ranks][dc_par_floats]
   int layers, heads, H, A, To, T;
   const float *W_in, *b_in, *pos;                            // [A, d], [d], [H, d]
   const float *lnf_g, *lnf_b, *W_outT, *b_out;               // W_outT [A, d]
@@ -198,7 +199,7 @@ __host__ __device__ inline DcSmem dc_smem_plan(int d, int dh, int cs, int layers
   p.off_u = take(DC_MAX_NKH / 2 * d * 4);                        // u rows (head pairs in one word)
   p.off_x = take(dc_own(cs) * ((A + 3) & ~3) * 4 * 4);               // latent, eps, noise and sigma of the owned rows
   p.off_xr = take(dc_own(cs) * d * 4);                               // an owned row's normalised values, fp32
-  p.off_red = take(512);                                         // row statistics [2 uses][own][64-column groups of a row] (mean, M2), scores [own][16]
+  p.off_red = take(512);                                         // row statistics [2 uses][own][4 groups of d / 4 columns] (mean, M2), scores [own][16]
   p.off_head = take((2 * d + A * d + 64) * 4);
   p.off_par = take((resident ? layers : 2) * dc_par_floats(d, dh, cs) * 4);
   p.off_bar = take(256);

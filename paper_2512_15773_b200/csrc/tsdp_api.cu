@@ -1309,9 +1309,10 @@ bool cluster_form_used(const tsdp_config_t& cfg, int which, int sz) {
   return which == TSDP_BASE ? cfg.verifier == 2 || (cfg.verifier == 0 && sz == 0) : cfg.drafter != 1;
 }
 
-// Cluster size for `work` rollouts or candidates: 0 for clusters of 8, 1 for clusters of 4.  A forward in a cluster of 4 takes about 1.25 times as long
-// (the exchanges take the same time, the k loops twice), but 33 of them run at once instead of 15; both give the same bits.  32 environments,
-// 8 steps of a d = 256 drafter of 4 blocks: 914 us in three waves of clusters of 8, calls of the conv-UNet policy 21.8 -> 15.0 ms.
+// Cluster size for `work` rollouts or candidates: 0 for clusters of 8, 1 for clusters of 4, which take longer (the exchanges take the same time, the
+// k loops twice) but run 33 at once instead of 15; both give the same bits.  A wave of rollouts, full windows, clusters of 8 / of 4: d = 256,
+// 4 blocks, 8 steps 313 / 390 us, 2 blocks, 10 steps 211 / 258, d = 128, 2 blocks, 8 steps 124 / 135: 1.25 is taken for all.  32 environments
+// of the first: 914 us in three waves of clusters of 8 -> 390, calls of the conv-UNet policy 21.8 -> 15.0 ms.
 int cluster_size_of(const tsdp_ctx::ClusterPlan (&pl)[2], int work) {
   if (!pl[1].ok) return 0;
   const int w8 = (work + pl[0].max_clusters - 1) / pl[0].max_clusters, w4 = (work + pl[1].max_clusters - 1) / pl[1].max_clusters;
