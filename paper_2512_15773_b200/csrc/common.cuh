@@ -93,7 +93,7 @@ __device__ __forceinline__ float ddpm_sample(float mu, float sigma, float xi) { 
 // 53.9 ms, 32 of the UNet workload 25.0 -> 23.0, 24 of the Push-T-shaped one 11.05 -> 10.46 (no signal at all: 53.9,
 // 24.3, 10.65); by the grid alone -> in front of GEMMs too: 96 vanilla 49.7 -> 48.5, 21 UNet frozen 9.08 -> 8.78, 3 VLA 62.5 -> 60.6.
 // Two of these kernels end a chain and have small blocks behind them: the UNet's last GroupNorm (its head) and the draft tail of the last
-// step (the verification's embedding).  They signal all the same; without it 21 UNet frozen 8.61 -> 8.64, a queue of 600 156.1 -> 156.6.
+// step (the verification's embedding).  They signal all the same: without, 21 UNet frozen 8.84 -> 8.89 (0.3 to 0.6 % in three trials) and the serving shape equal.
 // The GEMM signals when its last operand loads are issued, the others when they start.
 constexpr unsigned PDL_MAX_GRID = 74;      // half of a B200's SMs
 __device__ __forceinline__ void pdl_trigger(bool always = false) {
