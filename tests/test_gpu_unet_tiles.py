@@ -56,8 +56,8 @@ def test_unet_denoiser_with_a_warp_per_group(case, N):
     test_unet_denoiser_tiles_and_groups(case, N)
 
 
-# Four warps per group: the last launch whose GroupNorms fetch everything early (8 groups per SM, 1184) and the first that does not.
-@pytest.mark.parametrize("N", [148, 149])
+# Four warps per group: the last launch whose GroupNorms fetch everything early (8 groups per SM, 1184) and the first that does not; two well past it.
+@pytest.mark.parametrize("N", [148, 149, 258, 259])
 def test_unet_denoiser_on_both_sides_of_the_early_fetch(N):
     test_unet_denoiser_tiles_and_groups((16, 2, 1, 128, 8, 5), N)
 
